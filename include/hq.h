@@ -256,10 +256,10 @@ hq_status hq_conv2d_noalloc(const hq_tensor* in, const hq_conv_desc* desc, hq_te
  * call it serves it allocates nothing; the word it reads is cleared by the next hq_conv2d_noalloc. */
 hq_status hq_conv2d_noalloc_sync(void* stream);
 
-/* Choose the convolution path: 0 = automatic, 1 = CUDA cores only, 2 = tensor cores or fail (HQ_ERR_UNSUPPORTED
- * for a shape they do not take, HQ_ERR_WORKSPACE when scratch memory for a lowered form cannot be had), 3 = like 2 and
- * the tensor-core kernel's launch shapes are chosen by what the layer allows, not by its size (small test cases
- * then reach the shapes of large layers). */
+/* Choose the convolution path: 0 = automatic, 1 = CUDA cores only, 2 = the persistent tensor-core kernel or fail
+ * (HQ_ERR_UNSUPPORTED for a shape it does not take, HQ_ERR_WORKSPACE when scratch memory for a lowered form cannot be
+ * had), 3 = like 2 and its launch shapes are chosen by what the layer allows, not by its size (small test cases
+ * then reach the shapes of large layers), 4 = the one-tile-per-CTA tensor-core kernel for small problems or fail. */
 hq_status hq_set_conv_path(hq_handle* h, int32_t path);
 
 /* Order in which the tensor-core convolutions (pixel tiles) and hq_concat_requant (pixels) of this handle walk their

@@ -35,7 +35,7 @@ inline long long tensor_bytes(int n, int h, int w, int c, int bits) {
 // network); NULL means use (and if needed grow) the handle's own buffer.
 hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, hq_tensor* out, void* stream,
                       void* scratch = nullptr, size_t scratch_bytes = 0, const void* res_narrow = nullptr,
-                      const void* wgt_widened = nullptr) {
+                      const void* wgt_widened = nullptr, bool in_slack = false) {
   if (!h || !d) return HQ_ERR_INVALID_ARG;
   hq_status st = check_tensor(in, true, true, false);
   if (st != HQ_OK) return st;
@@ -62,6 +62,7 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
     }
   }
   ConvArgs a{};
+  a.in_slack = in_slack ? 1 : 0;
   a.in = in->data; a.n = in->n; a.h = in->h; a.w = in->w; a.cin = in->c; a.in_bits = in->bits; a.in_signed = in->is_signed;
   a.wgt = d->w; a.wgt_widened = wgt_widened; a.cout = d->cout; a.kh = d->kh; a.kw = d->kw; a.stride = d->stride; a.pad = d->pad;
   a.bias = d->bias; a.b = d->requant.b; a.c = d->requant.c;
@@ -73,6 +74,10 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
   a.relu = d->relu; a.qmin = d->qmin; a.qmax = d->qmax;
   a.out = out->data; a.ho = ho; a.wo = wo; a.out_bits = out->bits; a.out_signed = out->is_signed;
   cudaStream_t s = (cudaStream_t)stream;
+  if (h->conv_path == 4 || (h->conv_path == 0 && hq_conv_small_wanted(a, h->sm_count))) {
+    const hq_status st4 = hq_launch_conv_small(h, a, s);
+    if (st4 != HQ_ERR_UNSUPPORTED || h->conv_path == 4) return st4;
+  }
   const bool tc_ok = hq_conv_tc_supported(a);
   const bool force_tc = h->conv_path >= 2;
   if (force_tc && !tc_ok && !hq_conv_widen4_applies(a)) return HQ_ERR_UNSUPPORTED;
@@ -187,10 +192,32 @@ static void plan_tile_orders(hq_network* net) {
   }
 }
 
-// Allocate `bytes` for layer `layer` of `net` between two guard bands; NULL when the device is out of memory.
+// Kernels of one pass: one per layer, plus the helpers of convolutions that run in a lowered form.
+static void count_launches(hq_network* net) {
+  net->launches = (int32_t)net->layers.size();
+  for (size_t i = 0; i < net->layers.size(); ++i) {
+    const hq_layer& l = net->layers[i];
+    if (l.op != HQ_OP_CONV) continue;
+    const hq_conv_desc& d = l.conv;
+    const hq_tensor& o = net->outs[i];
+    ConvArgs a{};
+    a.n = net->batch; a.cin = d.cin; a.cout = d.cout; a.kh = d.kh; a.kw = d.kw; a.stride = d.stride; a.pad = d.pad;
+    a.h = l.in0 < 0 ? net->image_h : net->outs[l.in0].h; a.w = l.in0 < 0 ? net->image_w : net->outs[l.in0].w;
+    a.in_bits = l.in0 < 0 || net->stored_wide[l.in0] ? 8 : net->outs[l.in0].bits;
+    a.ho = o.h; a.wo = o.w; a.out_bits = o.bits; a.in_slack = l.in0 >= 0;
+    if (hq_conv_small_wanted(a, net->h->sm_count)) continue;
+    if (a.in_bits == 4) net->launches += hq_conv_widen4_applies(a) ? 1 : 0;     // activations widened (weights were when the network was built)
+    else if (hq_conv_s2d_applies(a)) net->launches += 1;                          // space-to-depth copy
+    else if ((!hq_conv_tc_supported(a) || hq_conv_tc_small_im2col(a)) && hq_conv_lowering_applies(a)) net->launches += 2;   // padded weights, patch matrix
+  }
+}
+
+// Allocate `bytes` for layer `layer` of `net` between two guard bands; NULL when the device is out of memory.  Small
+// buffers get the room behind them that an im2col-mode fetch of a small tensor may read (ConvArgs::in_slack).
 static void* net_alloc(hq_network* net, size_t bytes, int32_t layer) {
   unsigned char* base = nullptr;
-  if (cudaMalloc(&base, bytes + 2 * kGuardBytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  const size_t least = 2 * (size_t)kIm2colMinTensorBytes;
+  if (cudaMalloc(&base, (bytes < least ? least : bytes) + 2 * kGuardBytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
   if (cudaMemset(base, kGuardByte, kGuardBytes) != cudaSuccess ||
       cudaMemset(base + kGuardBytes + bytes, kGuardByte, kGuardBytes) != cudaSuccess) { cudaFree(base); return nullptr; }
   net->buffers.push_back({base, base + kGuardBytes, bytes, layer});
@@ -237,7 +264,7 @@ hq_status hq_create(int32_t device, hq_handle** out) {
   h->sm_count = prop.multiProcessorCount;
   h->workspace = nullptr;
   h->workspace_bytes = 0;
-  if (!hq_conv_tc_init()) { delete h; return HQ_ERR_CUDA; }
+  if (!hq_conv_tc_init() || !hq_conv_small_init()) { delete h; return HQ_ERR_CUDA; }
   if (cudaMalloc(&h->dev_status, sizeof(uint32_t)) != cudaSuccess) { delete h; return HQ_ERR_WORKSPACE; }
   if (cudaMemset(h->dev_status, 0, sizeof(uint32_t)) != cudaSuccess) { cudaFree(h->dev_status); delete h; return HQ_ERR_CUDA; }
   if (cudaMalloc(&h->narrow_pairs, (size_t)2 * kNarrowChannels * 16) != cudaSuccess) {
@@ -257,7 +284,7 @@ hq_status hq_destroy(hq_handle* h) {
 }
 
 hq_status hq_set_conv_path(hq_handle* h, int32_t path) {
-  if (!h || path < 0 || path > 3) return HQ_ERR_INVALID_ARG;
+  if (!h || path < 0 || path > 4) return HQ_ERR_INVALID_ARG;
   h->conv_path = path;
   return HQ_OK;
 }
@@ -392,7 +419,6 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
   net->stored_wide.assign(n_layers, 0);
   net->narrow0.assign(n_layers, nullptr);
   net->narrow1.assign(n_layers, nullptr);
-  net->launches = n_layers;
   hq_status st = HQ_OK;
   auto shape_of = [&](int id, hq_tensor* t) -> bool {
     if (id == -1) { *t = hq_tensor{nullptr, batch, image_h, image_w, image_c, 8, image_signed}; return true; }
@@ -415,11 +441,10 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
         {
           ConvArgs a{};
           a.n = batch; a.h = in.h; a.w = in.w; a.cin = in.c; a.in_bits = in.bits; a.cout = d.cout; a.kh = d.kh; a.kw = d.kw;
-          a.stride = d.stride; a.pad = d.pad; a.ho = o.h; a.wo = o.w; a.out_bits = o.bits;
+          a.stride = d.stride; a.pad = d.pad; a.ho = o.h; a.wo = o.w; a.out_bits = o.bits; a.in_slack = l.in0 >= 0;
           if (hq_conv_widen4_applies(a)) {
             const size_t need = hq_conv_widen4_bytes(a);
             if (need > net->scratch_bytes) net->scratch_bytes = need;
-            net->launches += 1;                 // the activation-widening kernel (the weights are widened once, below)
             const long long wvals = (long long)d.cout * d.kh * d.kw * in.c;
             void* wbuf = net_alloc(net, (size_t)wvals, i);
             if (!wbuf) { st = HQ_ERR_WORKSPACE; break; }
@@ -428,7 +453,6 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
           } else if (hq_conv_s2d_applies(a)) {
             const size_t need = hq_conv_s2d_bytes(a);
             if (need > net->scratch_bytes) net->scratch_bytes = need;
-            net->launches += 1;                 // the space-to-depth kernel (the weights are re-laid out once, here)
             a.wgt = d.w; a.bias = d.bias; a.b = d.requant.b; a.c = d.requant.c;
             void* wbuf = net_alloc(net, hq_conv_s2d_prepared_bytes(a), i);
             if (!wbuf) { st = HQ_ERR_WORKSPACE; break; }
@@ -437,7 +461,6 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
           } else if ((!hq_conv_tc_supported(a) || hq_conv_tc_small_im2col(a)) && hq_conv_lowering_applies(a)) {
             const size_t need = hq_conv_lowering_bytes(a);
             if (need > net->scratch_bytes) net->scratch_bytes = need;
-            net->launches += 2;                 // weight padding + patch matrix kernels
           }
         }
         break;
@@ -510,8 +533,6 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
     void* buf = net_alloc(net, wide, i);
     net->outs[i].data = buf;
     if (!buf) { st = HQ_ERR_WORKSPACE; break; }
-    for (int j = i + 1; j < n_layers; ++j)
-      if (net->layers[j].in0 == i) net->launches -= 1;        // no activation-widening kernel ahead of this conv
   }
   if (st == HQ_OK && net->scratch_bytes) {
     const size_t want = net->scratch_bytes;
@@ -551,7 +572,7 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
       if (hq_launch_residual_narrow(l.rescale1.b, l.rescale1.c, net->outs[l.in1].is_signed, ch, buf1, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
     }
   }
-  if (st == HQ_OK) plan_tile_orders(net);
+  if (st == HQ_OK) { plan_tile_orders(net); count_launches(net); }
   if (st == HQ_OK && cudaDeviceSynchronize() != cudaSuccess) st = HQ_ERR_CUDA;
   if (st != HQ_OK) { hq_network_destroy(net); return st; }
   *out = net;
@@ -582,7 +603,7 @@ static hq_status run_layers(hq_network* net, const hq_tensor* images, hq_tensor*
         const int32_t callers_order = h->tile_order;
         h->tile_order = net->tile_order[i];
         if (l.op == HQ_OP_LINEAR) { in.c = in.h * in.w * in.c; in.h = 1; in.w = 1; st = hq_linear(h, &in, &d, &o, s); }
-        else st = conv_common(h, &in, &d, &o, s, net->scratch, net->scratch_bytes, net->res_narrow[i], in_wide ? nullptr : net->wgt_widened[i]);
+        else st = conv_common(h, &in, &d, &o, s, net->scratch, net->scratch_bytes, net->res_narrow[i], in_wide ? nullptr : net->wgt_widened[i], l.in0 >= 0);
         h->tile_order = callers_order;
         break;
       }

@@ -18,7 +18,7 @@ enum : uint32_t {
 
 struct hq_handle {
   int32_t device;
-  int32_t conv_path;          // 0 auto, 1 CUDA cores only, 2 tensor cores or fail
+  int32_t conv_path;          // see hq_set_conv_path
   int32_t sm_count;
   uint32_t* dev_status;       // one word in device memory, sticky until hq_sync
   void* workspace;            // scratch owned by the handle (grown on demand, never inside a capture)
@@ -27,6 +27,7 @@ struct hq_handle {
   int32_t tile_order;         // tensor-core convolutions walk their pixel tiles 0: first to last, 1: last to first
 };
 constexpr int kNarrowChannels = 4096;
+constexpr long long kIm2colMinTensorBytes = 128 * 1024;   // smaller activation tensors are not fetched in im2col mode
 
 // ------------------------------------------------------------------------------------------
 // Dyadic arithmetic (Eq. 4): dn(q, b, c) = (q*b + 2^(c-1)) >> c, 64-bit product, arithmetic shift.
@@ -73,6 +74,7 @@ struct ConvArgs {
   int32_t res_narrow_fresh;  // nonzero: the pairs come from the launch just before on the same stream (the kernel waits for it)
   const void* wgt_widened;   // weights as the lowered form wants them, prepared once by a network, or NULL: 4-bit weights widened
                              // to one byte per value; for the first-layer form the virtual-channel weights and constants
+  int32_t in_slack;          // nonzero: the allocation behind `in` goes on for at least kIm2colMinTensorBytes + one image
   int32_t pad_after_delta;   // padding after the last row/column minus `pad`
   // byte pitches of the activation tensor along W, H and N when it is not dense (0: dense NHWC).  A W pitch
   // below cin bytes makes neighbouring "pixels" overlap: a pixel is then a window of adjacent stored pixels.
@@ -97,6 +99,11 @@ bool hq_conv_tc_supported(const ConvArgs& a);
 bool hq_conv_tc_small_im2col(const ConvArgs& a);
 // Tensor-core path; returns HQ_OK, HQ_ERR_UNSUPPORTED (nothing was launched) or HQ_ERR_CUDA.
 hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t s);
+// One tile per CTA, reduction split over a cluster: small problems (conv_small.cu).  Same status convention.
+bool hq_conv_small_init();
+bool hq_conv_small_supported(const ConvArgs& a);
+bool hq_conv_small_wanted(const ConvArgs& a, int sm_count);    // the automatic path's choice
+hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t s);
 // Fills `out` (channels x 16 bytes) with the narrow residual pairs of an 8-bit residual branch.
 cudaError_t hq_launch_residual_narrow(const int32_t* rb, const int32_t* rc, int res_signed, int channels, void* out,
                                       cudaStream_t s);
