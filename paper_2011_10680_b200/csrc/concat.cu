@@ -468,6 +468,7 @@ __device__ __forceinline__ int concat_my_branch(const ConcatArgs& a, int width) 
 
 // Branches in the four-channel form (few registers, many warps per SM) ...
 __global__ void __launch_bounds__(256, 4) concat_requant_kernel(const __grid_constant__ ConcatArgs a) {
+  hq_pdl_entry();
   const int i = concat_my_branch(a, 4);
   if (a.br[i].bits == 32) concat_w4<32>(a, i);
   else if (a.br[i].bits == 8) concat_w4<8>(a, i);
@@ -476,6 +477,7 @@ __global__ void __launch_bounds__(256, 4) concat_requant_kernel(const __grid_con
 
 // ... and the others (ragged or very wide branches) in the sixteen-channel form, in a launch of their own.
 __global__ void __launch_bounds__(256, 2) concat_requant_wide_kernel(const __grid_constant__ ConcatArgs a) {
+  hq_pdl_entry();
   concat_branch<16>(a, concat_my_branch(a, 16));
 }
 
@@ -569,7 +571,7 @@ extern "C" hq_status hq_concat_requant(hq_handle* h, int32_t n_branches, const h
     if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;
     a.narrow = tab;
   }
-  if (blocks4) concat_requant_kernel<<<(unsigned)blocks4, 256, 0, (cudaStream_t)stream>>>(a);
-  if (blocks16) concat_requant_wide_kernel<<<(unsigned)blocks16, 256, 0, (cudaStream_t)stream>>>(a);
+  if (blocks4) hq_launch_pdl(concat_requant_kernel, (unsigned)blocks4, 256, 0, (cudaStream_t)stream, a);
+  if (blocks16) hq_launch_pdl(concat_requant_wide_kernel, (unsigned)blocks16, 256, 0, (cudaStream_t)stream, a);
   return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }

@@ -59,6 +59,7 @@ __device__ __forceinline__ void store16(void* base, long long elem, const int (&
 // registers) and walks the pixels with a grid stride.
 template <int MB, int RB, int OB>
 __global__ void __launch_bounds__(256) residual_add_vec_kernel(EltArgs a, int groups, int pix_per_block) {
+  if (a.overlap) hq_pdl_entry();
   const int g = threadIdx.x % groups;
   const int pl = threadIdx.x / groups;
   if (pl >= pix_per_block) return;
@@ -272,6 +273,7 @@ __device__ __forceinline__ void requant8_flat(const EltArgs& a, const Dy8 (&m)[4
 
 template <bool RES, bool MSIGNED, bool RSIGNED, bool OUT4, int SATP, bool FLAT>
 __global__ void __launch_bounds__(256) requant8_kernel(EltArgs a, int words, int lo, int hi) {
+  hq_pdl_entry();
   // word (4 channels) of the pixel
   const int wx = FLAT ? (int)(threadIdx.x & (unsigned)(words - 1)) : (int)(blockIdx.x * blockDim.x + threadIdx.x);
   if (wx >= words) return;
@@ -464,6 +466,7 @@ __device__ __forceinline__ void requant8_chunks(const EltArgs& a, const Dy8 (&m)
 
 template <bool RES, bool MSIGNED, bool RSIGNED, bool OUT4, int SATP>
 __global__ void __launch_bounds__(256, RES ? 3 : 5) requant8_staged_kernel(EltArgs a, int words, int lo, int hi) {
+  hq_pdl_entry();
   extern __shared__ __align__(128) unsigned char stage[];
   __shared__ EltPipe pipe;
   const int tid = threadIdx.x;
@@ -528,12 +531,12 @@ cudaError_t launch_requant8_form(const EltArgs& a, dim3 grid, dim3 block, int wo
     const long long blocks = (total + per_block - 1) / per_block, cap = (long long)sm_count * 16;
     if (total / per_block >= 8ll * sm_count) {      // large: the bulk-copy pipeline, three or five persistent blocks per SM
       const size_t smem = (size_t)kEltStages * per_block * 4 * (RES ? 2 : 1);
-      requant8_staged_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP><<<sm_count * (RES ? 3 : 5), 256, smem, s>>>(a, words, lo, hi);
+      hq_launch_pdl(requant8_staged_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP>, sm_count * (RES ? 3 : 5), 256, smem, s, a, words, lo, hi);
       return cudaGetLastError();
     }
-    requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, true><<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, s>>>(a, words, lo, hi);
+    hq_launch_pdl(requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, true>, (unsigned)(blocks < cap ? blocks : cap), 256, 0, s, a, words, lo, hi);
   } else {
-    requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, false><<<grid, block, 0, s>>>(a, words, lo, hi);
+    hq_launch_pdl(requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, false>, grid, block, 0, s, a, words, lo, hi);
   }
   return cudaGetLastError();
 }
@@ -556,6 +559,7 @@ cudaError_t launch_requant8(const EltArgs& a, dim3 grid, dim3 block, int words, 
 struct Dy32 { int b; long long r0; int sh; };
 template <bool RES, bool RSIGNED, int SATP>
 __global__ void __launch_bounds__(256) requant32_flat_kernel(EltArgs a, int quads, int lo, int hi) {
+  if (a.overlap) hq_pdl_entry();
   constexpr int T = 256, U = 4;
   const int wx = threadIdx.x & (quads - 1);
   const long long total = a.pixels * quads;
@@ -629,15 +633,16 @@ cudaError_t launch_requant32(const EltArgs& a, int quads, int lo, int hi, int sm
   const long long total = a.pixels * quads, per_block = 256 * 4;
   const long long blocks = (total + per_block - 1) / per_block, cap = (long long)sm_count * 16;
   const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
-  if (lo == 0 && hi == 255) requant32_flat_kernel<RES, RSIGNED, 1><<<grid, 256, 0, s>>>(a, quads, lo, hi);
-  else if (lo == -128 && hi == 127) requant32_flat_kernel<RES, RSIGNED, 2><<<grid, 256, 0, s>>>(a, quads, lo, hi);
-  else requant32_flat_kernel<RES, RSIGNED, 0><<<grid, 256, 0, s>>>(a, quads, lo, hi);
+  if (lo == 0 && hi == 255) hq_launch_pdl_if(a.overlap != 0, requant32_flat_kernel<RES, RSIGNED, 1>, grid, 256, 0, s, a, quads, lo, hi);
+  else if (lo == -128 && hi == 127) hq_launch_pdl_if(a.overlap != 0, requant32_flat_kernel<RES, RSIGNED, 2>, grid, 256, 0, s, a, quads, lo, hi);
+  else hq_launch_pdl_if(a.overlap != 0, requant32_flat_kernel<RES, RSIGNED, 0>, grid, 256, 0, s, a, quads, lo, hi);
   return cudaGetLastError();
 }
 
 // INT32 output (the wide residual stream of Fig. 2: the add of Section 3.3 with its result kept in INT32):
 // one thread per element, 64-bit dyadic arithmetic, consecutive threads on consecutive channels.
 __global__ void __launch_bounds__(256) residual_add_out32_kernel(EltArgs a) {
+  if (a.overlap) hq_pdl_entry();
   const long long total = a.pixels * a.ch;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
     const int ch = (int)(e % a.ch);
@@ -652,6 +657,7 @@ __global__ void __launch_bounds__(256) residual_add_out32_kernel(EltArgs a) {
 // 16 bytes of an INT32 operand (4 of an 8-bit one) and writes 16 bytes per step, two steps in flight.
 template <int MB, int RB>   // operand bits: 8 or 32; RB = 0: no second operand
 __global__ void __launch_bounds__(256) residual_add_out32_vec_kernel(EltArgs a) {
+  if (a.overlap) hq_pdl_entry();
   const long long quads = a.pixels * (a.ch >> 2);
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -692,6 +698,7 @@ __global__ void __launch_bounds__(256) residual_add_out32_vec_kernel(EltArgs a) 
 
 // Any channel count: one thread per output byte (one element at 8 bit, two at 4 bit).
 __global__ void residual_add_scalar_kernel(EltArgs a) {
+  hq_pdl_entry();
   const int per = (a.out_bits == 4) ? 2 : 1;
   const long long total = a.pixels * a.ch / per;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -711,8 +718,8 @@ __global__ void residual_add_scalar_kernel(EltArgs a) {
 
 template <int MB, int RB>
 cudaError_t launch_vec_out(const EltArgs& a, int groups, int ppb, int grid, cudaStream_t s) {
-  if (a.out_bits == 8) residual_add_vec_kernel<MB, RB, 8><<<grid, 256, 0, s>>>(a, groups, ppb);
-  else residual_add_vec_kernel<MB, RB, 4><<<grid, 256, 0, s>>>(a, groups, ppb);
+  if (a.out_bits == 8) hq_launch_pdl_if(a.overlap != 0, residual_add_vec_kernel<MB, RB, 8>, grid, 256, 0, s, a, groups, ppb);
+  else hq_launch_pdl_if(a.overlap != 0, residual_add_vec_kernel<MB, RB, 4>, grid, 256, 0, s, a, groups, ppb);
   return cudaGetLastError();
 }
 
@@ -731,6 +738,7 @@ cudaError_t launch_vec_res(const EltArgs& a, int groups, int ppb, int grid, cuda
 __global__ void avgpool_vec4_kernel(const unsigned* __restrict__ in, int n, int hw, int ch, int is_signed,
                                     const int32_t* __restrict__ b, const int32_t* __restrict__ c,
                                     int qmin, int qmax, unsigned* __restrict__ out) {
+  hq_pdl_entry();
   const int cg = ch >> 2;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * cg) return;
@@ -762,6 +770,7 @@ __global__ void avgpool_vec4_kernel(const unsigned* __restrict__ in, int n, int 
 __global__ void __launch_bounds__(256) avgpool_vec4_sliced_kernel(const unsigned* __restrict__ in, int hw, int ch, int is_signed,
                                                                   const int32_t* __restrict__ b, const int32_t* __restrict__ c,
                                                                   int qmin, int qmax, unsigned* __restrict__ out) {
+  hq_pdl_entry();
   __shared__ unsigned part[2][4][64];
   const int cg = ch >> 2;
   const int g = blockIdx.x * 64 + threadIdx.x, img = blockIdx.y;
@@ -801,6 +810,7 @@ template <int SLICES, bool SIGNED>
 __global__ void __launch_bounds__(32 * SLICES) avgpool_vec16_kernel(const uint4* __restrict__ in, int hw, int ch,
                                                                     const int32_t* __restrict__ b, const int32_t* __restrict__ c,
                                                                     int qmin, int qmax, unsigned short* __restrict__ out) {
+  hq_pdl_entry();
   __shared__ unsigned part[SLICES][8][32];            // [slice][even / odd byte sums of the four words][channel group]
   const int cg = ch >> 4;
   const int g = blockIdx.x * 32 + threadIdx.x, img = blockIdx.y;
@@ -854,13 +864,14 @@ template <int SLICES>
 void launch_avgpool_vec16(const void* in, int n, int hw, int ch, int in_signed, const int32_t* b, const int32_t* c,
                           int qmin, int qmax, void* out, cudaStream_t s) {
   const dim3 grid((ch / 16 + 31) / 32, n), block(32, SLICES);
-  if (in_signed) avgpool_vec16_kernel<SLICES, true><<<grid, block, 0, s>>>((const uint4*)in, hw, ch, b, c, qmin, qmax, (unsigned short*)out);
-  else avgpool_vec16_kernel<SLICES, false><<<grid, block, 0, s>>>((const uint4*)in, hw, ch, b, c, qmin, qmax, (unsigned short*)out);
+  if (in_signed) hq_launch_pdl(avgpool_vec16_kernel<SLICES, true>, grid, block, 0, s, (const uint4*)in, hw, ch, b, c, qmin, qmax, (unsigned short*)out);
+  else hq_launch_pdl(avgpool_vec16_kernel<SLICES, false>, grid, block, 0, s, (const uint4*)in, hw, ch, b, c, qmin, qmax, (unsigned short*)out);
 }
 
 __global__ void avgpool_scalar_kernel(const void* in, int n, int hw, int ch, int in_bits, int in_signed,
                                       const int32_t* b, const int32_t* c, int qmin, int qmax,
                                       void* out, int out_bits) {
+  hq_pdl_entry();
   const int per = (out_bits == 4) ? 2 : 1;
   const int total = n * ch / per;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -905,7 +916,8 @@ struct BytePairMax {
 // lies inside the same window (pad < k) and leaves the maximum unchanged.
 template <bool SIGNED, bool K3>
 __global__ void __launch_bounds__(256) maxpool_vec16_kernel(const uint4* __restrict__ in, int h, int w, int cg,
-                                                            int k, int stride, int pad, uint4* __restrict__ out, int ho, int wo) {
+                                                            int k, int stride, int pad, uint4* __restrict__ out, int ho, int wo, int overlap) {
+  if (overlap) hq_pdl_entry();
   const int img = blockIdx.x / ho, oh = blockIdx.x - img * ho;
   const uint4* in_img = in + (long long)img * h * w * cg;
   uint4* out_row = out + ((long long)img * ho + oh) * wo * cg;
@@ -953,6 +965,7 @@ __global__ void __launch_bounds__(256) maxpool_vec16_kernel(const uint4* __restr
 
 __global__ void maxpool_scalar_kernel(const void* in, int n, int h, int w, int ch, int bits, int is_signed,
                                       int k, int stride, int pad, void* out, int ho, int wo) {
+  hq_pdl_entry();
   const long long total = (long long)n * ho * wo * ch;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -979,8 +992,10 @@ __global__ void maxpool_scalar_kernel(const void* in, int n, int h, int w, int c
 
 }  // namespace
 
-cudaError_t hq_launch_residual_add(const EltArgs& a, int sm_count, cudaStream_t s) {
-  if (a.pixels == 0) return cudaSuccess;
+cudaError_t hq_launch_residual_add(const EltArgs& args, int sm_count, cudaStream_t s) {
+  if (args.pixels == 0) return cudaSuccess;
+  EltArgs a = args;
+  a.overlap = a.pixels * a.ch < kOverlapValues ? 1 : 0;
   if (a.out_bits == 32) {
     const int quads = a.ch >> 2;
     const bool vec = a.ch % 4 == 0 && (a.main_bits == 8 || a.main_bits == 32) && (!a.res || a.res_bits == 8 || a.res_bits == 32);
@@ -996,17 +1011,17 @@ cudaError_t hq_launch_residual_add(const EltArgs& a, int sm_count, cudaStream_t 
       if (blocks >= mult) {
         const int g = (int)blocks;
         const int rbits = a.res ? a.res_bits : 0;
-        if (a.main_bits == 32 && rbits == 32) residual_add_out32_vec_kernel<32, 32><<<g, 256, 0, s>>>(a);
-        else if (a.main_bits == 32 && rbits == 8) residual_add_out32_vec_kernel<32, 8><<<g, 256, 0, s>>>(a);
-        else if (a.main_bits == 32) residual_add_out32_vec_kernel<32, 0><<<g, 256, 0, s>>>(a);
-        else if (rbits == 32) residual_add_out32_vec_kernel<8, 32><<<g, 256, 0, s>>>(a);
-        else if (rbits == 8) residual_add_out32_vec_kernel<8, 8><<<g, 256, 0, s>>>(a);
-        else residual_add_out32_vec_kernel<8, 0><<<g, 256, 0, s>>>(a);
+        if (a.main_bits == 32 && rbits == 32) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<32, 32>, g, 256, 0, s, a);
+        else if (a.main_bits == 32 && rbits == 8) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<32, 8>, g, 256, 0, s, a);
+        else if (a.main_bits == 32) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<32, 0>, g, 256, 0, s, a);
+        else if (rbits == 32) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<8, 32>, g, 256, 0, s, a);
+        else if (rbits == 8) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<8, 8>, g, 256, 0, s, a);
+        else hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<8, 0>, g, 256, 0, s, a);
         return cudaGetLastError();
       }
     }
     const long long blocks = (a.pixels * a.ch + 255) / 256, cap = (long long)sm_count * 32;
-    residual_add_out32_kernel<<<(int)(blocks < cap ? blocks : cap), 256, 0, s>>>(a);
+    hq_launch_pdl_if(a.overlap != 0, residual_add_out32_kernel, (int)(blocks < cap ? blocks : cap), 256, 0, s, a);
     return cudaGetLastError();
   }
   // 8-bit operands with a channel count the word mapping covers: 32-bit fast kernel
@@ -1054,7 +1069,7 @@ cudaError_t hq_launch_residual_add(const EltArgs& a, int sm_count, cudaStream_t 
   const long long total = a.pixels * a.ch / (a.out_bits == 4 ? 2 : 1);
   long long blocks = (total + 255) / 256;
   const long long cap = (long long)sm_count * 16;
-  residual_add_scalar_kernel<<<(int)(blocks < cap ? blocks : cap), 256, 0, s>>>(a);
+  hq_launch_pdl(residual_add_scalar_kernel, (int)(blocks < cap ? blocks : cap), 256, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -1064,19 +1079,21 @@ cudaError_t hq_launch_avgpool(const void* in, int n, int h, int w, int ch, int i
   if (n == 0) return cudaSuccess;
   if (in_bits == 8 && out_bits == 8 && ch % 16 == 0 && h * w <= 8 * 257 && n <= 65535) {
     const int hw = h * w;
-    if (hw >= 128) launch_avgpool_vec16<8>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
+    // eight slices for long sums, and where the blocks leave SMs idle: a thread then reads its pixels in one or two batches
+    // (2048 channels at 7x7, one image: two slices 6.9 us, eight 4 us)
+    if (hw >= 128 || (hw >= 16 && (long long)n * ((ch / 16 + 31) / 32) <= 148)) launch_avgpool_vec16<8>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
     else if (hw >= 64) launch_avgpool_vec16<4>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
     else launch_avgpool_vec16<2>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
   } else if (in_bits == 8 && out_bits == 8 && ch % 4 == 0 && h * w <= 257 && n <= 65535) {
     const dim3 grid((ch / 4 + 63) / 64, n), block(64, 4);
-    avgpool_vec4_sliced_kernel<<<grid, block, 0, s>>>((const unsigned*)in, h * w, ch, in_signed, b, c, qmin, qmax, (unsigned*)out);
+    hq_launch_pdl(avgpool_vec4_sliced_kernel, grid, block, 0, s, (const unsigned*)in, h * w, ch, in_signed, b, c, qmin, qmax, (unsigned*)out);
   } else if (in_bits == 8 && out_bits == 8 && ch % 4 == 0) {
     const int total = n * (ch / 4);
-    avgpool_vec4_kernel<<<(total + 127) / 128, 128, 0, s>>>((const unsigned*)in, n, h * w, ch, in_signed,
+    hq_launch_pdl(avgpool_vec4_kernel, (total + 127) / 128, 128, 0, s, (const unsigned*)in, n, h * w, ch, in_signed,
                                                              b, c, qmin, qmax, (unsigned*)out);
   } else {
     const int total = n * ch / (out_bits == 4 ? 2 : 1);
-    avgpool_scalar_kernel<<<(total + 127) / 128, 128, 0, s>>>(in, n, h * w, ch, in_bits, in_signed, b, c,
+    hq_launch_pdl(avgpool_scalar_kernel, (total + 127) / 128, 128, 0, s, in, n, h * w, ch, in_bits, in_signed, b, c,
                                                                qmin, qmax, out, out_bits);
   }
   return cudaGetLastError();
@@ -1092,15 +1109,16 @@ cudaError_t hq_launch_maxpool(const void* in, int n, int h, int w, int ch, int b
     // the unrolled 3x3 form: with pad <= 1 at most one row / column of a window lies outside the image, next to
     // a valid one of the same window
     const bool k3 = k == 3 && pad <= 1;
-    if (is_signed && k3) maxpool_vec16_kernel<true, true><<<n * ho, 256, 0, s>>>(src, h, w, cg, k, stride, pad, dst, ho, wo);
-    else if (is_signed)  maxpool_vec16_kernel<true, false><<<n * ho, 256, 0, s>>>(src, h, w, cg, k, stride, pad, dst, ho, wo);
-    else if (k3)         maxpool_vec16_kernel<false, true><<<n * ho, 256, 0, s>>>(src, h, w, cg, k, stride, pad, dst, ho, wo);
-    else                 maxpool_vec16_kernel<false, false><<<n * ho, 256, 0, s>>>(src, h, w, cg, k, stride, pad, dst, ho, wo);
+    const bool overlap = (long long)n * ho * wo * ch < kOverlapValues;
+    if (is_signed && k3) hq_launch_pdl_if(overlap, maxpool_vec16_kernel<true, true>, n * ho, 256, 0, s, src, h, w, cg, k, stride, pad, dst, ho, wo, overlap ? 1 : 0);
+    else if (is_signed)  hq_launch_pdl_if(overlap, maxpool_vec16_kernel<true, false>, n * ho, 256, 0, s, src, h, w, cg, k, stride, pad, dst, ho, wo, overlap ? 1 : 0);
+    else if (k3)         hq_launch_pdl_if(overlap, maxpool_vec16_kernel<false, true>, n * ho, 256, 0, s, src, h, w, cg, k, stride, pad, dst, ho, wo, overlap ? 1 : 0);
+    else                 hq_launch_pdl_if(overlap, maxpool_vec16_kernel<false, false>, n * ho, 256, 0, s, src, h, w, cg, k, stride, pad, dst, ho, wo, overlap ? 1 : 0);
   } else {
     const long long total = (long long)n * ho * wo * ch;
     long long blocks = (total + 255) / 256;
     if (blocks > (1 << 20)) blocks = 1 << 20;
-    maxpool_scalar_kernel<<<(int)blocks, 256, 0, s>>>(in, n, h, w, ch, bits, is_signed, k, stride, pad, out, ho, wo);
+    hq_launch_pdl(maxpool_scalar_kernel, (int)blocks, 256, 0, s, in, n, h, w, ch, bits, is_signed, k, stride, pad, out, ho, wo);
   }
   return cudaGetLastError();
 }

@@ -176,7 +176,8 @@ hq_status hq_launch_conv_lowered(hq_handle* h, const ConvArgs& a, void* scratch,
 namespace {
 
 __global__ void __launch_bounds__(256) space_to_depth_kernel(const unsigned char* __restrict__ in, int n, int h, int w,
-                                                             uint4* __restrict__ out) {
+                                                             uint4* __restrict__ out, int overlap) {
+  if (overlap) hq_pdl_entry();
   // output: [n][h/2 + 3][w/2 + 3] pixels of 16 bytes, the image surrounded by its zero padding (2 before, 1 after).
   // A thread builds two neighbouring output pixels x0 = 2p - 2, x0 + 1: their 2 x 12 source bytes are three aligned
   // words in each of the two image rows (w % 4 == 0 and a 16-byte aligned image make (2 x0) * 3 a multiple of 4).
@@ -294,7 +295,8 @@ hq_status hq_launch_conv_s2d(hq_handle* h, const ConvArgs& a, void* scratch, cud
   const long long px = l.img_bytes / 16 / 2;          // a thread builds two pixels
   long long blocks = (px + 255) / 256;
   const long long cap = (long long)h->sm_count * 32;
-  space_to_depth_kernel<<<(int)(blocks < cap ? blocks : cap), 256, 0, s>>>((const unsigned char*)a.in, a.n, a.h, a.w, (uint4*)base);
+  const bool overlap = l.img_bytes < kOverlapValues;
+  hq_launch_pdl_if(overlap, space_to_depth_kernel, (int)(blocks < cap ? blocks : cap), 256, 0, s, (const unsigned char*)a.in, a.n, a.h, a.w, (uint4*)base, overlap ? 1 : 0);
   if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;
   return hq_launch_conv_tc(h, s2d_conv_args(a, scratch), s);
 }

@@ -21,6 +21,7 @@ struct SumPoolArgs {
 // K = 0 takes the window size from the arguments.
 template <int K>
 __global__ void __launch_bounds__(256) sumpool_kernel(const __grid_constant__ SumPoolArgs a) {
+  hq_pdl_entry();
   const int k = K ? K : a.k;
   const int cg = a.vec ? a.ch >> 2 : a.ch;                       // channel groups per pixel
   const int col = blockIdx.y * 256 + threadIdx.x;
@@ -90,6 +91,7 @@ __global__ void __launch_bounds__(256) sumpool_kernel(const __grid_constant__ Su
 // the image counts as the biased zero), and 9 * 128 comes off at the end.
 template <int IN8, int SIGNED>
 __global__ void __launch_bounds__(256) sumpool3_rows_kernel(const __grid_constant__ SumPoolArgs a, int strip_rows, int strips) {
+  hq_pdl_entry();
   const int cg = a.ch >> 2;
   const int col = blockIdx.x * 256 + threadIdx.x;
   if (col >= a.w * cg) return;
@@ -178,16 +180,16 @@ extern "C" hq_status hq_sumpool(hq_handle* h, const hq_tensor* in, int32_t k, in
     if ((cols3 + 255) / 256 <= 0x7fffffffLL && (long long)a.n * strips <= 65535) {
       const dim3 grid3((unsigned)((cols3 + 255) / 256), (unsigned)(a.n * strips));
       cudaStream_t st = (cudaStream_t)stream;
-      if (a.vec == 1) sumpool3_rows_kernel<0, 0><<<grid3, 256, 0, st>>>(a, strip_rows, strips);
-      else if (a.is_signed) sumpool3_rows_kernel<1, 1><<<grid3, 256, 0, st>>>(a, strip_rows, strips);
-      else sumpool3_rows_kernel<1, 0><<<grid3, 256, 0, st>>>(a, strip_rows, strips);
+      if (a.vec == 1) hq_launch_pdl(sumpool3_rows_kernel<0, 0>, grid3, 256, 0, st, a, strip_rows, strips);
+      else if (a.is_signed) hq_launch_pdl(sumpool3_rows_kernel<1, 1>, grid3, 256, 0, st, a, strip_rows, strips);
+      else hq_launch_pdl(sumpool3_rows_kernel<1, 0>, grid3, 256, 0, st, a, strip_rows, strips);
       return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
     }
   }
   const long long rows = (long long)a.n * ho, cols = (long long)wo * (a.vec ? a.ch / 4 : a.ch);
   if (rows > 0x7fffffffLL || (cols + 255) / 256 > 65535) return HQ_ERR_UNSUPPORTED;
   const dim3 grid((unsigned)rows, (unsigned)((cols + 255) / 256));
-  if (k == 3) sumpool_kernel<3><<<grid, 256, 0, (cudaStream_t)stream>>>(a);
-  else sumpool_kernel<0><<<grid, 256, 0, (cudaStream_t)stream>>>(a);
+  if (k == 3) hq_launch_pdl(sumpool_kernel<3>, grid, 256, 0, (cudaStream_t)stream, a);
+  else hq_launch_pdl(sumpool_kernel<0>, grid, 256, 0, (cudaStream_t)stream, a);
   return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }
