@@ -35,7 +35,8 @@ inline long long tensor_bytes(int n, int h, int w, int c, int bits) {
 // network); NULL means use (and if needed grow) the handle's own buffer.
 hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, hq_tensor* out, void* stream,
                       void* scratch = nullptr, size_t scratch_bytes = 0, const void* res_narrow = nullptr,
-                      const void* wgt_widened = nullptr, bool in_slack = false) {
+                      const void* wgt_widened = nullptr, bool in_slack = false, const WideArgs* wide = nullptr,
+                      bool wide_sum = true) {
   if (!h || !d) return HQ_ERR_INVALID_ARG;
   hq_status st = check_tensor(in, true, true, false);
   if (st != HQ_OK) return st;
@@ -48,7 +49,7 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
   const int wo = (in->w + 2 * d->pad - d->kw) / d->stride + 1;
   if (out->n != in->n || out->h != ho || out->w != wo || out->c != d->cout) return HQ_ERR_INVALID_ARG;
   if (!aligned16(d->w)) return HQ_ERR_ALIGNMENT;
-  if (out->bits == 32) {
+  if (out->bits == 32 && !wide) {
     if (d->residual) return HQ_ERR_INVALID_ARG;
   } else {
     if (!d->requant.b || !d->requant.c) return HQ_ERR_INVALID_ARG;
@@ -71,9 +72,17 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
     a.rb = d->res_rescale.b; a.rc = d->res_rescale.c;
     a.res_narrow = res_narrow;
   }
+  void* out_data = out->data;
+  if (wide) {                                  // (a network's fused add: `d` carries the add's pairs, `out` its INT32 result)
+    a.wide = wide;
+    if (!wide_sum) out_data = nullptr;
+    a.res = d->residual->data; a.res_bits = d->residual->bits; a.res_signed = d->residual->is_signed;
+    a.rb = d->res_rescale.b; a.rc = d->res_rescale.c;
+  }
   a.relu = d->relu; a.qmin = d->qmin; a.qmax = d->qmax;
-  a.out = out->data; a.ho = ho; a.wo = wo; a.out_bits = out->bits; a.out_signed = out->is_signed;
+  a.out = out_data; a.ho = ho; a.wo = wo; a.out_bits = out->bits; a.out_signed = out->is_signed;
   cudaStream_t s = (cudaStream_t)stream;
+  if (wide) return hq_launch_conv_tc(h, a, s);
   if (h->conv_path == 4 || (h->conv_path == 0 && hq_conv_small_wanted(a, h->sm_count))) {
     const hq_status st4 = hq_launch_conv_small(h, a, s);
     if (st4 != HQ_ERR_UNSUPPORTED || h->conv_path == 4) return st4;
@@ -158,6 +167,10 @@ struct hq_network {
   std::vector<void*> narrow0, narrow1; // per ADD / REQUANT layer with 8-bit operands: narrow pairs of the two branches (owned)
   std::vector<void*> wgt_widened;    // per 4-bit conv layer on the tensor-core path: its weights, one byte per value (owned)
   std::vector<char> stored_wide;     // per layer: its 4-bit output is kept one value per byte (all consumers are such convs)
+  // ADD layers with an INT32 result that run behind the convolution producing their main operand (see plan_wide_adds):
+  // the convolution's layer or -1; the REQUANT layer done along with it or -1; whether somebody else reads the sum
+  std::vector<int32_t> wide_conv, wide_requant;
+  std::vector<char> wide_sum_read, run_by_add;   // run_by_add: conv / requant layers that such an ADD runs
   std::vector<char> tile_order;      // per conv / linear / concat layer: tensors walked from the last pixel to the first (see plan_tile_orders)
   void* scratch;                     // patch matrix of the lowered first layer (owned)
   size_t scratch_bytes;
@@ -179,6 +192,10 @@ static void plan_tile_orders(hq_network* net) {
   auto is_conv = [&](int i) { return net->layers[i].op == HQ_OP_CONV || net->layers[i].op == HQ_OP_LINEAR; };
   auto either_way = [&](int i) { return is_conv(i) || net->layers[i].op == HQ_OP_CONCAT; };
   for (int i = 0; i < n; ++i) {
+    if (net->wide_conv[i] >= 0) {                       // a fused add walks like its convolution, and so does the requantization
+      net->tile_order[i] = net->tile_order[net->wide_conv[i]];
+      if (net->wide_requant[i] >= 0) net->tile_order[net->wide_requant[i]] = net->tile_order[i];
+    }
     if (!either_way(i)) continue;
     char order;
     if (!is_conv(i)) {
@@ -187,8 +204,56 @@ static void plan_tile_orders(hq_network* net) {
       const int src = net->layers[i].in0;
       order = src < 0 ? 0 : !net->tile_order[src];
     }
-    if (i + 1 < n && !either_way(i + 1) && net->layers[i + 1].in0 == i) order = 1;
+    if (i + 1 < n && !either_way(i + 1) && net->layers[i + 1].in0 == i && !net->run_by_add[i]) order = 1;
     net->tile_order[i] = order;
+  }
+}
+
+// The residual add of Fig. 2 on an INT32 stream, fused (WideArgs): an ADD layer whose main operand is the raw INT32 result
+// of a convolution that nobody else reads runs as that convolution's epilogue, and the first REQUANT layer of its result to
+// one byte per value with it.  The raw accumulators then never travel, nor does the stream where only the requantization
+// reads it.  Layer taps need every tensor: with taps the layers run one by one.
+static void plan_wide_adds(hq_network* net) {
+  const int n = (int)net->layers.size();
+  net->wide_conv.assign(n, -1); net->wide_requant.assign(n, -1);
+  net->wide_sum_read.assign(n, 0); net->run_by_add.assign(n, 0);
+  auto reads = [&](int j, int id) {
+    const hq_layer& l = net->layers[j];
+    if (l.op == HQ_OP_CONCAT) { for (int k = 0; k < l.n_in; ++k) if (l.ins[k] == id) return true; return false; }
+    const bool two = l.op == HQ_OP_CONV || l.op == HQ_OP_ADD;
+    return l.in0 == id || (two && l.in1 == id);
+  };
+  for (int i = 0; i < n; ++i) {
+    const hq_layer& l = net->layers[i];
+    if (l.op != HQ_OP_ADD || net->outs[i].bits != 32 || l.in0 < 0 || l.in1 < 0 || l.in1 == l.in0) continue;
+    const int j = l.in0;
+    const hq_layer& cv = net->layers[j];
+    const hq_tensor& o = net->outs[j];
+    if (cv.op != HQ_OP_CONV || o.bits != 32 || cv.in1 >= 0 || cv.in0 < 0 || o.c % 4 != 0 || net->outs[l.in1].bits == 4) continue;
+    if (!l.rescale0.b || !l.rescale0.c || !l.rescale1.b || !l.rescale1.c) continue;
+    bool alone = true;
+    for (int m = j + 1; m < n; ++m) alone = alone && (m == i || !reads(m, j));
+    const hq_tensor& in = net->outs[cv.in0];
+    ConvArgs a{};
+    a.n = in.n; a.h = in.h; a.w = in.w; a.cin = in.c; a.in_bits = net->stored_wide[cv.in0] ? 8 : in.bits; a.cout = o.c;
+    a.kh = cv.conv.kh; a.kw = cv.conv.kw; a.stride = cv.conv.stride; a.pad = cv.conv.pad; a.ho = o.h; a.wo = o.w; a.out_bits = 32;
+    a.in_slack = 1;
+    if (!alone || !hq_conv_tc_supported(a) || (o.c + 127) / 128 > net->h->sm_count) continue;
+    net->wide_conv[i] = j;
+    net->run_by_add[j] = 1;
+    net->wide_sum_read[i] = i == n - 1;
+    for (int m = i + 1; m < n; ++m) {
+      if (!reads(m, i)) continue;
+      const hq_layer& r = net->layers[m];
+      const bool bytes = net->outs[m].bits == 8 || net->stored_wide[m];
+      if (net->wide_requant[i] < 0 && r.op == HQ_OP_REQUANT && bytes && m != n - 1 && r.rescale0.b && r.rescale0.c) {
+        net->wide_requant[i] = m;
+        net->run_by_add[m] = 1;
+      } else {
+        net->wide_sum_read[i] = 1;
+      }
+    }
+    if (net->wide_requant[i] < 0) net->wide_sum_read[i] = 1;
   }
 }
 
@@ -197,6 +262,7 @@ static void count_launches(hq_network* net) {
   net->launches = (int32_t)net->layers.size();
   for (size_t i = 0; i < net->layers.size(); ++i) {
     const hq_layer& l = net->layers[i];
+    if (net->run_by_add[i]) { net->launches -= 1; continue; }
     if (l.op != HQ_OP_CONV) continue;
     const hq_conv_desc& d = l.conv;
     const hq_tensor& o = net->outs[i];
@@ -572,7 +638,7 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
       if (hq_launch_residual_narrow(l.rescale1.b, l.rescale1.c, net->outs[l.in1].is_signed, ch, buf1, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
     }
   }
-  if (st == HQ_OK) { plan_tile_orders(net); count_launches(net); }
+  if (st == HQ_OK) { plan_wide_adds(net); plan_tile_orders(net); count_launches(net); }
   if (st == HQ_OK && cudaDeviceSynchronize() != cudaSuccess) st = HQ_ERR_CUDA;
   if (st != HQ_OK) { hq_network_destroy(net); return st; }
   *out = net;
@@ -583,9 +649,11 @@ static hq_status run_layers(hq_network* net, const hq_tensor* images, hq_tensor*
                             cudaStream_t s, cudaEvent_t* marks = nullptr) {
   hq_handle* h = net->h;
   const int n_layers = (int)net->layers.size();
+  const bool fuse = !taps && h->conv_path == 0;
   for (int i = 0; i < n_layers; ++i) {
     if (marks && cudaEventRecord(marks[i], s) != cudaSuccess) return HQ_ERR_CUDA;
     const hq_layer& l = net->layers[i];
+    if (fuse && net->run_by_add[i]) continue;                 // runs with the ADD layer it feeds, or that feeds it
     hq_tensor in = (l.in0 == -1) ? *images : net->outs[l.in0];
     hq_tensor o = net->outs[i];
     if (i == n_layers - 1) o.data = logits->data;
@@ -612,6 +680,27 @@ static hq_status run_layers(hq_network* net, const hq_tensor* images, hq_tensor*
       case HQ_OP_ADD: {
         if (l.in1 < 0) return HQ_ERR_INVALID_ARG;
         hq_tensor res = net->outs[l.in1];
+        if (fuse && net->wide_conv[i] >= 0) {
+          const int j = net->wide_conv[i], r = net->wide_requant[i];
+          const hq_layer& cv = net->layers[j];
+          hq_tensor cin = net->outs[cv.in0];
+          hq_conv_desc d = cv.conv;
+          const bool cin_wide = net->stored_wide[cv.in0] != 0;
+          if (cin_wide) { cin.bits = 8; d.w_bits = 8; d.w = net->wgt_widened[j]; }
+          d.requant = l.rescale0; d.residual = &res; d.res_rescale = l.rescale1;
+          d.relu = l.relu; d.qmin = l.qmin; d.qmax = l.qmax;
+          WideArgs wa{};
+          if (r >= 0) {
+            const hq_layer& rq = net->layers[r];
+            wa.q = net->outs[r].data; wa.qb = rq.rescale0.b; wa.qc = rq.rescale0.c;
+            wa.q_relu = rq.relu; wa.q_qmin = rq.qmin; wa.q_qmax = rq.qmax;
+          }
+          const int32_t callers_order = h->tile_order;
+          h->tile_order = net->tile_order[j];
+          st = conv_common(h, &cin, &d, &o, s, nullptr, 0, nullptr, nullptr, true, &wa, net->wide_sum_read[i] != 0);
+          h->tile_order = callers_order;
+          break;
+        }
         st = residual_add_impl(h, &in, l.rescale0, &res, l.rescale1, l.relu, l.qmin, l.qmax, &o, s, net->narrow0[i], net->narrow1[i]);
         break;
       }

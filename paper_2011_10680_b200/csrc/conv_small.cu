@@ -87,14 +87,6 @@ __device__ __forceinline__ uint4 widen16(uint2 v, bool is_signed) {
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// 4 x 4 bytes turned round inside each quad of lanes: lane i's word holds bytes (i, 0..3); afterwards (0..3, i).
-__device__ __forceinline__ unsigned quad_transpose(unsigned w, int lane) {
-  unsigned o = __shfl_xor_sync(0xffffffffu, w, 1);
-  w = (lane & 1) ? __byte_perm(w, o, 0x3715) : __byte_perm(w, o, 0x6240);
-  o = __shfl_xor_sync(0xffffffffu, w, 2);
-  return (lane & 2) ? __byte_perm(w, o, 0x3276) : __byte_perm(w, o, 0x5410);
-}
-
 // 4 NG columns x 32 lanes of the accumulator into this lane's registers, one wait for all of them
 template <int NG>
 __device__ __forceinline__ void load_columns(uint32_t taddr, int (&v)[4 * NG]) {

@@ -109,6 +109,7 @@ struct TcParams {
   int32_t narrow_fresh;     // 1: the pairs are written by the kernel launched just before this one
   int32_t relu, qmin, qmax;
   void* out; int32_t out_bits;
+  void* q_out; const int32_t* qb; const int32_t* qc; int32_t q_lo, q_hi;   // wide: the stream requantized to bytes, or NULL
   uint32_t* status;
 };
 
@@ -421,6 +422,134 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
   if (pending) tmem_ld_wait();
 }
 
+// Tile loop of a convolution that ends in the INT32 residual add of Fig. 2 (Section 3.3) and the requantization of the
+// next block (WideArgs): y = clamp(relu(dn(acc + bias, b, c) + dn(res, rb, rc))) to INT32, z = clamp(dn(y, qb, qc)) to bytes.
+// A lane owns one channel and 16 pixels at a time: the INT32 residual of the next 16 pixels and their accumulators are on
+// their way while 16 are processed; every access of a warp to the INT32 tensors is one 128-byte line, bytes leave as
+// words after a turn of 4 x 4 bytes in lane quads.  Nothing passes through shared memory.
+// What bounds it: nine bytes of HBM traffic per value (residual in, stream and bytes out) against about 28 integer
+// instructions, three of them wide multiplies.
+// FAST: every channel of the warp has c >= 32 and qc >= 32.  RNARROW: and rc >= 32, the sum then needs no 64-bit step.
+template <bool FAST, bool RNARROW, bool Q>
+__device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const ChanConst& k_in) {
+  const EpiCtx e = e_in;
+  const ChanConst k = k_in;
+  const TcParams& p = *e.p;
+  SharedCtl& ctl = *e.ctl;
+  const int lane = e.lane, C = p.C;
+  const int qb = Q && e.ch_live ? p.qb[e.ch] : 0, qc = Q && e.ch_live ? p.qc[e.ch] : 32;
+  const long long qr0 = 1LL << (qc - 1);
+  const int qsh = FAST ? qc - 32 : qc, msh = FAST ? k.sh - 32 : k.sh, rsh = RNARROW ? k.rsh - 32 : k.rsh;
+  const uint32_t bmask = (1u << p.lg_bufs) - 1u;
+  const int units = e.px_per_warp >> 4;
+  const bool sum_out = p.out != nullptr;
+  if (e.p_tile0 >= p.p_tiles) return;
+  const uint32_t t_warp = e.tmem_base + ((uint32_t)(e.q * 32) << 16) + (uint32_t)e.col0;
+  const int ch0 = e.c_tile * kTileC + e.cq * 32;                       // first channel of the warp
+  auto wait_bar = [&](unsigned long long* bar, uint32_t ph) -> bool {
+    uint32_t w = 1;
+    if (lane == 0) w = mbar_wait(smem_u32(bar), ph, &ctl, p.status, HQ_DEV_TIMEOUT_EPILOGUE) ? 1u : 0u;
+    return __shfl_sync(0xffffffffu, w, 0) != 0;
+  };
+  // 16 residual values of this lane's channel from pixel px0 on; pixels past the last one read as 0
+  auto load_res = [&](int px0, int (&r)[16]) {
+    const int left = e.ch_live ? p.P - px0 : 0;
+    if (p.res_bits == 32) {
+      const int* base = (const int*)p.res + (long long)px0 * C + ch0;
+      uint32_t off = (uint32_t)lane;
+#pragma unroll
+      for (int j = 0; j < 16; ++j, off += (uint32_t)C) r[j] = j < left ? __ldcg(base + off) : 0;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) r[j] = j < left ? hq_load_elem(p.res, (long long)(px0 + j) * C + e.ch, p.res_bits, p.res_signed) : 0;
+    }
+  };
+  auto unit = [&](const int (&v)[16], const int (&r)[16], int px0) {
+    const int left = p.P - px0;
+    int y[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      long long t;
+      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(v[j]), "r"(k.b), "l"(k.r0));
+      long long u;
+      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(u) : "r"(r[j]), "r"(k.rb), "l"(k.rr0));
+      if (FAST && RNARROW) {
+        y[j] = min(max(((int)(t >> 32) >> msh) + ((int)(u >> 32) >> rsh), e.lo), e.hi);   // both terms below 2^30 in magnitude
+      } else {
+        const long long m = FAST ? (long long)((int)(t >> 32) >> msh) : t >> msh;
+        const long long sum = m + (u >> rsh);
+        y[j] = (int)(sum < (long long)e.lo ? (long long)e.lo : sum > (long long)e.hi ? (long long)e.hi : sum);
+      }
+    }
+    if (sum_out && e.ch_live) {
+      int* base = (int*)p.out + (long long)px0 * C + ch0;
+      uint32_t off = (uint32_t)lane;
+#pragma unroll
+      for (int j = 0; j < 16; ++j, off += (uint32_t)C) if (j < left) base[off] = y[j];
+    }
+    if (Q) {
+      unsigned char* base = (unsigned char*)p.q_out + (long long)px0 * C + ch0;
+      const bool word_live = ch0 + (lane & ~3) < C;
+      uint32_t off = (uint32_t)((lane & 3) * C + (lane & ~3));
+#pragma unroll
+      for (int g = 0; g < 4; ++g, off += 4u * (uint32_t)C) {
+        int z[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          long long t;
+          asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(y[4 * g + j]), "r"(qb), "l"(qr0));
+          if (FAST) z[j] = min(max((int)(t >> 32) >> qsh, p.q_lo), p.q_hi);
+          else { const long long zz = t >> qsh; z[j] = (int)(zz < (long long)p.q_lo ? (long long)p.q_lo : zz > (long long)p.q_hi ? (long long)p.q_hi : zz); }
+        }
+        const unsigned w01 = __byte_perm((unsigned)z[0], (unsigned)z[1], 0x0040), w23 = __byte_perm((unsigned)z[2], (unsigned)z[3], 0x0040);
+        const unsigned w = quad_transpose(__byte_perm(w01, w23, 0x5410), lane);          // four channels of pixel 4 g + lane % 4
+        if (4 * g + (lane & 3) < left && word_live) *(unsigned*)(base + off) = w;
+      }
+    }
+  };
+
+  int va[16], vb[16], ra[16], rb[16];
+  uint32_t tcount = 0, as = 0;
+  int p_tile = e.p_tile0;
+  load_res(tile_at(p, p_tile) * p.pt + e.col0, ra);
+  if (!wait_bar(&ctl.tfull[0], 0)) return;
+  tc_fence_after();
+  tmem_ld16_issue(t_warp, va);
+  bool pending = true;
+  while (true) {
+    const int px_first = tile_at(p, p_tile) * p.pt + e.col0;
+    const bool has_next = p_tile + e.p_step < p.p_tiles;
+    const uint32_t nas = (tcount + 1u) & bmask, naph = ((tcount + 1u) >> p.lg_bufs) & 1u;
+    const uint32_t t_addr = t_warp + as * p.acc_stride;
+    for (int u = 0; u < units; u += 2) {
+      load_res(px_first + 16 * (u + 1), rb);
+      tmem_ld_wait();
+      tie16(va);
+      tmem_ld16_issue(t_addr + 16 * (u + 1), vb);
+      unit(va, ra, px_first + 16 * u);
+      if (u + 2 < units) load_res(px_first + 16 * (u + 2), ra);
+      else if (has_next) load_res(tile_at(p, p_tile + e.p_step) * p.pt + e.col0, ra);
+      tmem_ld_wait();
+      tie16(vb);
+      pending = false;
+      if (u + 2 < units) { tmem_ld16_issue(t_addr + 16 * (u + 2), va); pending = true; }
+      else {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) release_accumulator(p, ctl, as);
+      }
+      unit(vb, rb, px_first + 16 * (u + 1));
+    }
+    if (!has_next) break;
+    if (!wait_bar(&ctl.tfull[nas], naph)) break;
+    tc_fence_after();
+    tmem_ld16_issue(t_warp + nas * p.acc_stride, va);
+    pending = true;
+    p_tile += e.p_step; ++tcount; as = nas;
+  }
+  if (pending) tmem_ld_wait();
+}
+
 // General tile loop: every output type, direct stores, 64-bit arithmetic, INT32 residuals.
 __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanConst& k, uint32_t fast) {
   const TcParams& p = *e.p;
@@ -574,7 +703,8 @@ __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanCo
 // cta_group::2 instructions (a kernel that contains them cannot be launched without clusters).
 // RTM: the instantiation for fused 8-bit residuals that travel through tensor memory; it has one more warp, which
 // stores the finished output tiles.
-template <int EPI_WARPS, int MIN_CTAS, int MMA_WARPS, bool DUO = false, bool RTM = false>
+// WIDE: the instantiation whose epilogue is the INT32 residual add (epilogue_loop_wide).
+template <int EPI_WARPS, int MIN_CTAS, int MMA_WARPS, bool DUO = false, bool RTM = false, bool WIDE = false>
 __global__ void __launch_bounds__(32 * (1 + MMA_WARPS + EPI_WARPS + (RTM ? 1 : 0)), MIN_CTAS)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res,
@@ -996,6 +1126,28 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const bool warp_live = (c_tile * kTileC + cq * 32) < p.C; // warp-uniform
     const int lo = p.relu ? (p.qmin > 0 ? p.qmin : 0) : p.qmin, hi = p.qmax;
 
+    if constexpr (WIDE) {
+      if (half < p.halves) {
+        EpiCtx e;
+        e.p = &p; e.ctl = &ctl; e.tmem_base = tmem_base; e.lane = lane; e.q = q; e.cq = cq; e.ew = ew; e.half = half;
+        e.col0 = col0; e.px_per_warp = px_per_warp; e.ch = ch; e.c_tile = c_tile; e.p_tile0 = p_tile0; e.p_step = p_step;
+        e.lo = lo; e.hi = hi; e.ch_live = ch_live;
+        const ChanConst k = chan_const(p, ch, false);
+        const int qc = p.q_out && ch_live ? p.qc[ch] : 32;
+        const bool wfast = __all_sync(0xffffffffu, k.sh >= 32 && qc >= 32) != 0;
+        const bool rnarrow = wfast && __all_sync(0xffffffffu, k.rsh >= 32) != 0;
+        asm volatile("griddepcontrol.wait;" ::: "memory");             // the residual is the output of an earlier kernel
+        if (p.q_out) {
+          if (rnarrow) epilogue_loop_wide<true, true, true>(e, k);
+          else if (wfast) epilogue_loop_wide<true, false, true>(e, k);
+          else epilogue_loop_wide<false, false, true>(e, k);
+        } else {
+          if (rnarrow) epilogue_loop_wide<true, true, false>(e, k);
+          else if (wfast) epilogue_loop_wide<true, false, false>(e, k);
+          else epilogue_loop_wide<false, false, false>(e, k);
+        }
+      }
+    } else {
     // per-channel constants, once per kernel
     ChanConst k{};
     uint32_t fast = (p.out_bits != 32) ? 1u : 0u;
@@ -1100,6 +1252,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     } else {
       epilogue_loop_general(e, k, fast);
     }
+    }
   }
 
 
@@ -1180,6 +1333,8 @@ bool hq_conv_tc_init() {
          cudaFuncSetAttribute(conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               112 * 1024) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<8, 1, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAttr) == cudaSuccess &&
+         cudaFuncSetAttribute(conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              kSmemAttr) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<kSoloEpilogueWarps, 1, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               kSmemAttr) == cudaSuccess;
 }
@@ -1237,7 +1392,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // epilogue work, e.g. 64 output channels.  Where the layer is large enough for 256-pixel tiles and its residual
   // travels by TMA, the rtm shape below is faster still: 64 -> 256 at 56x56, batch 256: 129 -> 122 us.)
   const bool wide_fits = p.staged_res && a.out_bits == 8 && a.cout > 64 && pick_pt(P, p.c_tiles, h->sm_count, 256) == 256;
-  bool pair = k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !wide_fits;
+  bool pair = !a.wide && k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !wide_fits;
   int stages = 0, stage_bytes = 0, res_tile_bytes = 0, out_tile_bytes = 0, wres_bytes = 0;
   if (pair) {
     // 128-pixel tiles, two accumulator buffers (256 columns), K blocks of at most 64 bytes
@@ -1375,7 +1530,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     // Fourth shape, *duo*: clusters of two CTAs on adjacent SMs share every MMA (cta_group::2, M = 256): each CTA
     // fetches its own 128 weight rows and HALF of the tile's pixel rows, 32 KiB per K block and SM instead of
     // 48 KiB for the same MMA time.  For the long reductions whose weights stream, which the operand fetch bounds.
-    p.duo = (!pair && !wide && !p.strip && !p.wres && !p.fold && p.pt >= 128 && p.bkb == 128 && a.cout % 256 == 0 &&
+    p.duo = (!pair && !wide && !a.wide && !p.strip && !p.wres && !p.fold && p.pt >= 128 && p.bkb == 128 && a.cout % 256 == 0 &&
              k_total >= 2048 && (long long)p.p_tiles * p.c_tiles >= 2LL * h->sm_count) ? 1 : 0;
     if (p.duo) {
       stage_bytes = (kTileC + p.pt / 2) * p.bkb;
@@ -1409,6 +1564,10 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.narrow_fresh = a.res_narrow_fresh;
   p.relu = a.relu; p.qmin = a.qmin; p.qmax = a.qmax;
   p.out = a.out; p.out_bits = a.out_bits; p.out_signed = a.out_signed;
+  if (a.wide) {
+    p.q_out = a.wide->q; p.qb = a.wide->qb; p.qc = a.wide->qc; p.q_hi = a.wide->q_qmax;
+    p.q_lo = a.wide->q_relu ? (a.wide->q_qmin > 0 ? a.wide->q_qmin : 0) : a.wide->q_qmin;
+  }
   {
     const int lo = a.relu ? (a.qmin > 0 ? a.qmin : 0) : a.qmin;
     p.sat_pack = (a.out_bits == 8 && ((!a.out_signed && lo == 0 && a.qmax == 255) ||
@@ -1482,7 +1641,8 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   } else {
     // one CTA per SM (it may allocate all 512 tensor-memory columns): never request less than 120 KiB
     cfg.blockDim = dim3(32 * (1 + kSoloIssuerWarps + kSoloEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
-    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps>, map_x, map_w, map_out, map_res, p);
+    if (a.wide) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps, false, false, true>, map_x, map_w, map_out, map_res, p);
+    else err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps>, map_x, map_w, map_out, map_res, p);
   }
   return err == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }

@@ -89,6 +89,15 @@ __device__ __forceinline__ int hq_clamp_ll(long long y, int relu, int qmin, int 
   return (int)y;
 }
 
+// What may be fused behind a convolution whose raw INT32 result feeds the residual add of Fig. 2 (an INT32 stream) and,
+// through it, the requantization of the next block.  The add's main pair, residual, ReLU, clamp and INT32 result are the
+// b / c / res / relu / qmin / qmax / out fields of ConvArgs (out NULL: nobody reads the stream itself).
+struct WideArgs {
+  void* q;                            // the stream requantized to one byte per value, or NULL
+  const int32_t* qb; const int32_t* qc;
+  int32_t q_relu, q_qmin, q_qmax;
+};
+
 // Launchers implemented in the other translation units.  All return a cudaError_t from the launch.
 struct ConvArgs {
   const void* in; int32_t n, h, w, cin, in_bits, in_signed;
@@ -102,6 +111,7 @@ struct ConvArgs {
   int32_t res_narrow_fresh;  // nonzero: the pairs come from the launch just before on the same stream (the kernel waits for it)
   const void* wgt_widened;   // weights as the lowered form wants them, prepared once by a network, or NULL: 4-bit weights widened
                              // to one byte per value; for the first-layer form the virtual-channel weights and constants
+  const WideArgs* wide;      // non-NULL: the convolution ends in the INT32 residual add (see WideArgs)
   int32_t in_slack;          // nonzero: the allocation behind `in` goes on for at least kIm2colMinTensorBytes + one image
   int32_t pad_after_delta;   // padding after the last row/column minus `pad`
   // byte pitches of the activation tensor along W, H and N when it is not dense (0: dense NHWC).  A W pitch

@@ -50,3 +50,52 @@ def test_small_conv_kernel(cfg, signed):
         assert np.array_equal(got, ref), (int((got != ref).sum()), ref.size)
     finally:
         hq.close()
+
+
+@pytest.mark.parametrize("shifts", ["table", "residual_below_32", "main_below_32", "every"])
+def test_fused_int32_stream_add(shifts):
+    """Graph replay runs the INT32 add and the next block's requantization behind the block's last convolution; with layer
+    taps every layer runs alone.  Both against the oracle on a reduced table, with shifts that select each arithmetic form."""
+    from paper_2011_10680_b200 import binding, build
+    from test_gpu_parity import run_network_and_compare
+    build.build()
+    t = inputs.resnet_table(50, seed=8, image_hw=64, classes=24, width=32, int32_stream=True)
+    g = inputs.rng(77, len(shifts))
+    pick = lambda c, lo, hi: g.integers(lo, hi, size=c, dtype=np.int64).astype(np.int32)
+    for l in t["layers"]:
+        if shifts == "table" or l["op"] not in ("add", "requant"):
+            continue
+        c = l["cout"]
+        if l["op"] == "add":
+            l["c"] = pick(c, *{"residual_below_32": (33, 36), "main_below_32": (28, 34), "every": (30, 60)}[shifts])
+            l["rc"] = pick(c, *{"residual_below_32": (29, 34), "main_below_32": (31, 34), "every": (30, 60)}[shifts])
+        else:
+            l["c"] = pick(c, *((40, 48) if shifts != "every" else (30, 50)))
+    hq = binding.Handle(0)
+    try:
+        run_network_and_compare(hq, t, batch=3, seed=61)
+    finally:
+        hq.close()
+
+
+def test_fused_int32_stream_add_large_tiles():
+    """The same with 256-pixel tiles, folded channel tiles and several tiles per CTA (layers of 40 thousand pixels): the
+    fused run against the layer-by-layer run, whose kernels other tests compare with the oracle."""
+    from paper_2011_10680_b200 import binding, build
+    build.build()
+    t = inputs.resnet_table(50, seed=9, image_hw=96, classes=24, int32_stream=True)
+    hq = binding.Handle(0)
+    net = binding.Network(hq, t, 73)
+    try:
+        images = binding.to_device(inputs.random_images(5, 73, 96))
+        single, fused = (binding.alloc_out(*net.logits_shape, 32, 1) for _ in range(2))
+        assert net.run(images, single, net.alloc_taps()) == binding.HQ_OK
+        hq.sync()
+        with torch.cuda.stream(torch.cuda.Stream()):
+            assert net.run(images, fused, None) == binding.HQ_OK
+            hq.sync()
+        net.check_guards()
+        assert int((single != single[0]).sum()) > 0 and torch.equal(single, fused)
+    finally:
+        net.close()
+        hq.close()
