@@ -229,7 +229,7 @@ static void plan_wide_adds(hq_network* net) {
     const int j = l.in0;
     const hq_layer& cv = net->layers[j];
     const hq_tensor& o = net->outs[j];
-    if (cv.op != HQ_OP_CONV || o.bits != 32 || cv.in1 >= 0 || cv.in0 < 0 || o.c % 4 != 0 || net->outs[l.in1].bits == 4) continue;
+    if (cv.op != HQ_OP_CONV || o.bits != 32 || cv.in1 >= 0 || cv.in0 < 0 || o.c % 16 != 0 || net->outs[l.in1].bits == 4) continue;
     if (!l.rescale0.b || !l.rescale0.c || !l.rescale1.b || !l.rescale1.c) continue;
     bool alone = true;
     for (int m = j + 1; m < n; ++m) alone = alone && (m == i || !reads(m, j));

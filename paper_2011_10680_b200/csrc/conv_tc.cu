@@ -109,7 +109,7 @@ struct TcParams {
   int32_t narrow_fresh;     // 1: the pairs are written by the kernel launched just before this one
   int32_t relu, qmin, qmax;
   void* out; int32_t out_bits;
-  void* q_out; const int32_t* qb; const int32_t* qc; int32_t q_lo, q_hi;   // wide: the stream requantized to bytes, or NULL
+  void* q_out; const int32_t* qb; const int32_t* qc; int32_t q_lo, q_hi, q_sat;   // wide: the stream requantized to bytes, or NULL
   uint32_t* status;
 };
 
@@ -125,6 +125,7 @@ struct SharedCtl {
   unsigned long long drain;
   unsigned long long wfull;              // resident weight slab landed
   unsigned long long pfull[3], pempty[3];  // strip mode: input patches
+  unsigned long long wbox[8][3];         // INT32 results: residual boxes of the epilogue warps (kWideSlots each)
   uint32_t tmem_base;
   volatile uint32_t abort_flag;
 };
@@ -422,132 +423,207 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
   if (pending) tmem_ld_wait();
 }
 
-// Tile loop of a convolution that ends in the INT32 residual add of Fig. 2 (Section 3.3) and the requantization of the
-// next block (WideArgs): y = clamp(relu(dn(acc + bias, b, c) + dn(res, rb, rc))) to INT32, z = clamp(dn(y, qb, qc)) to bytes.
-// A lane owns one channel and 16 pixels at a time: the INT32 residual of the next 16 pixels and their accumulators are on
-// their way while 16 are processed; every access of a warp to the INT32 tensors is one 128-byte line, bytes leave as
-// words after a turn of 4 x 4 bytes in lane quads.  Nothing passes through shared memory.
-// What bounds it: nine bytes of HBM traffic per value (residual in, stream and bytes out) against about 28 integer
-// instructions, three of them wide multiplies.
-// FAST: every channel of the warp has c >= 32 and qc >= 32.  RNARROW: and rc >= 32, the sum then needs no 64-bit step.
-template <bool FAST, bool RNARROW, bool Q>
-__device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const ChanConst& k_in) {
+// Tile loop of the instantiation for INT32 results.  Two uses:
+//   - a convolution that ends in the INT32 residual add of Fig. 2 (Section 3.3) and the requantization of the next block
+//     (WideArgs): y = clamp(relu(dn(acc + bias, b, c) + dn(res, rb, rc))) to INT32, z = clamp(dn(y, qb, qc)) to bytes;
+//   - a raw INT32 result, acc + bias (FORM 3).
+// A warp works on boxes of 32 pixels x 32 channels, one channel per lane.  The residual box arrives by TMA in one of the
+// warp's own three 4 KiB slots (two boxes ahead), the sums are written over it in place and leave by TMA from there;
+// the requantized bytes are turned round in lane quads and leave from a 1 KiB box.  No CTA-wide barrier, no predicates at the
+// tensor's edges (the copies clip), and 64 KiB of loads in flight per SM.
+// What bounds it: nine bytes of HBM traffic per value against three wide multiplies and about fifteen plain instructions.
+// 64 images of 56x56x256: plain loads and stores of a lane (16 KiB in flight per SM) 172-261 us, this form 95-106 us;
+// raw result 110 us with direct stores, 52 us here.
+// FORM 0: every shift of the warp's channels is at least 32 (no 64-bit step).  1: c or rc below 32: bits [c, c + 32) by a funnel
+// shift, and where some value of 16 pixels does not fit 32 bits those 16 again in 64 bits.  2: qc below 32 as well: 64 bits.
+constexpr int kWideSlots = 3;
+constexpr int kWideBox = 32 * 32 * 4, kWideQBox = 32 * 32;
+template <int FORM, bool Q>
+__device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const ChanConst& k_in, const CUtensorMap* map_res, const CUtensorMap* map_q) {
   const EpiCtx e = e_in;
   const ChanConst k = k_in;
   const TcParams& p = *e.p;
   SharedCtl& ctl = *e.ctl;
-  const int lane = e.lane, C = p.C;
+  constexpr bool RAW = FORM == 3;
+  const int lane = e.lane;
   const int qb = Q && e.ch_live ? p.qb[e.ch] : 0, qc = Q && e.ch_live ? p.qc[e.ch] : 32;
   const long long qr0 = 1LL << (qc - 1);
-  const int qsh = FAST ? qc - 32 : qc, msh = FAST ? k.sh - 32 : k.sh, rsh = RNARROW ? k.rsh - 32 : k.rsh;
+  const int qsh = FORM < 2 ? qc - 32 : qc;
+  const int msh1 = min(k.sh, 32), msh2 = k.sh - msh1, mcm = min(k.sh, 31);
+  const int rsh1 = min(k.rsh, 32), rsh2 = k.rsh - rsh1, rcm = min(k.rsh, 31);
   const uint32_t bmask = (1u << p.lg_bufs) - 1u;
-  const int units = e.px_per_warp >> 4;
-  const bool sum_out = p.out != nullptr;
+  const int nb = e.px_per_warp >> 5;                                   // boxes per tile: 2 or 4
+  const bool sum_out = p.out != nullptr, live = e.warp_live;
   if (e.p_tile0 >= p.p_tiles) return;
   const uint32_t t_warp = e.tmem_base + ((uint32_t)(e.q * 32) << 16) + (uint32_t)e.col0;
   const int ch0 = e.c_tile * kTileC + e.cq * 32;                       // first channel of the warp
+  const uint32_t slots = e.out_stage + (uint32_t)(e.ew * kWideSlots * kWideBox);
+  const uint32_t qboxes = e.out_stage + (uint32_t)(kSoloEpilogueWarps * kWideSlots * kWideBox + e.ew * 2 * kWideQBox);
+  const bool res8 = !RAW && p.res_bits == 8;
+  const uint32_t res_bytes = res8 ? kWideQBox : kWideBox, res_at = res8 ? kWideBox - kWideQBox : 0;   // bytes lie at the slot's end
+  const unsigned long long pol = policy_evict_first();
   auto wait_bar = [&](unsigned long long* bar, uint32_t ph) -> bool {
     uint32_t w = 1;
     if (lane == 0) w = mbar_wait(smem_u32(bar), ph, &ctl, p.status, HQ_DEV_TIMEOUT_EPILOGUE) ? 1u : 0u;
     return __shfl_sync(0xffffffffu, w, 0) != 0;
   };
-  // 16 residual values of this lane's channel from pixel px0 on; pixels past the last one read as 0
-  auto load_res = [&](int px0, int (&r)[16]) {
-    const int left = e.ch_live ? p.P - px0 : 0;
-    if (p.res_bits == 32) {
-      const int* base = (const int*)p.res + (long long)px0 * C + ch0;
-      uint32_t off = (uint32_t)lane;
-#pragma unroll
-      for (int j = 0; j < 16; ++j, off += (uint32_t)C) r[j] = j < left ? __ldcg(base + off) : 0;
-    } else {
-#pragma unroll
-      for (int j = 0; j < 16; ++j) r[j] = j < left ? hq_load_elem(p.res, (long long)(px0 + j) * C + e.ch, p.res_bits, p.res_signed) : 0;
-    }
+  // lane 0: the next residual box, in order of use
+  int pf_tile = e.p_tile0, pf_sub = 0, pf_slot = 0, issued = 0;
+  auto prefetch = [&]() {
+    if (RAW || !live || pf_tile >= p.p_tiles) return;
+    const uint32_t bar = smem_u32(&ctl.wbox[e.ew][pf_slot]);
+    mbar_expect_tx(bar, res_bytes);
+    tma_load_2d_hint(slots + (uint32_t)(pf_slot * kWideBox) + res_at, map_res, bar, res8 ? ch0 : ch0 * 4,
+                     tile_at(p, pf_tile) * p.pt + e.col0 + 32 * pf_sub, pol);
+    ++issued;
+    if (++pf_slot == kWideSlots) pf_slot = 0;
+    if (++pf_sub == nb) { pf_sub = 0; pf_tile += e.p_step; }
   };
-  auto unit = [&](const int (&v)[16], const int (&r)[16], int px0) {
-    const int left = p.P - px0;
-    int y[16];
+  if (lane == 0) { prefetch(); prefetch(); }
+
+  int done = 0, slot = 0;
+  uint32_t sph = 0;
+  bool ok = true;
+  auto box = [&](const int (&v)[32], int px0) {
+    if (!live) return;
+    if (!RAW) { ok = wait_bar(&ctl.wbox[e.ew][slot], sph); if (!ok) return; }
+    uint8_t* const sp = e.smem_raw + (slots - e.raw) + slot * kWideBox;
+    const uint32_t qbox = qboxes + (uint32_t)((done & 1) * kWideQBox);
+    int* const words = (int*)sp + lane;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      long long t;
-      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(v[j]), "r"(k.b), "l"(k.r0));
-      long long u;
-      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(u) : "r"(r[j]), "r"(k.rb), "l"(k.rr0));
-      if (FAST && RNARROW) {
-        y[j] = min(max(((int)(t >> 32) >> msh) + ((int)(u >> 32) >> rsh), e.lo), e.hi);   // both terms below 2^30 in magnitude
+    for (int h = 0; h < 2; ++h) {
+      int y[16];
+      if constexpr (RAW) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) y[j] = v[16 * h + j] + k.bias;
       } else {
-        const long long m = FAST ? (long long)((int)(t >> 32) >> msh) : t >> msh;
-        const long long sum = m + (u >> rsh);
-        y[j] = (int)(sum < (long long)e.lo ? (long long)e.lo : sum > (long long)e.hi ? (long long)e.hi : sum);
-      }
-    }
-    if (sum_out && e.ch_live) {
-      int* base = (int*)p.out + (long long)px0 * C + ch0;
-      uint32_t off = (uint32_t)lane;
+        int r[16];
+        if (!res8) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j, off += (uint32_t)C) if (j < left) base[off] = y[j];
-    }
-    if (Q) {
-      unsigned char* base = (unsigned char*)p.q_out + (long long)px0 * C + ch0;
-      const bool word_live = ch0 + (lane & ~3) < C;
-      uint32_t off = (uint32_t)((lane & 3) * C + (lane & ~3));
+          for (int j = 0; j < 16; ++j) r[j] = words[(16 * h + j) * 32];
+        } else {
+          const uint8_t* const bytes = sp + res_at + lane;
 #pragma unroll
-      for (int g = 0; g < 4; ++g, off += 4u * (uint32_t)C) {
-        int z[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          long long t;
-          asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(y[4 * g + j]), "r"(qb), "l"(qr0));
-          if (FAST) z[j] = min(max((int)(t >> 32) >> qsh, p.q_lo), p.q_hi);
-          else { const long long zz = t >> qsh; z[j] = (int)(zz < (long long)p.q_lo ? (long long)p.q_lo : zz > (long long)p.q_hi ? (long long)p.q_hi : zz); }
+          for (int j = 0; j < 16; ++j) r[j] = p.res_signed ? (int)(signed char)bytes[(16 * h + j) * 32] : (int)bytes[(16 * h + j) * 32];
+          __syncwarp();                              // these byte rows may be overwritten by the sums below
         }
-        const unsigned w01 = __byte_perm((unsigned)z[0], (unsigned)z[1], 0x0040), w23 = __byte_perm((unsigned)z[2], (unsigned)z[3], 0x0040);
-        const unsigned w = quad_transpose(__byte_perm(w01, w23, 0x5410), lane);          // four channels of pixel 4 g + lane % 4
-        if (4 * g + (lane & 3) < left && word_live) *(unsigned*)(base + off) = w;
+        int bad = FORM == 2 ? 1 : 0;
+        if constexpr (FORM < 2) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            long long t, u;
+            asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(v[16 * h + j]), "r"(k.b), "l"(k.r0));
+            asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(u) : "r"(r[j]), "r"(k.rb), "l"(k.rr0));
+            if constexpr (FORM == 0) {
+              y[j] = ((int)(t >> 32) >> msh2) + ((int)(u >> 32) >> rsh2);            // each within [-2^30, 2^30)
+            } else {
+              const int th = (int)(t >> 32), uh = (int)(u >> 32);
+              const int t0 = (int)__funnelshift_rc((unsigned)t, (unsigned)th, msh1), u0 = (int)__funnelshift_rc((unsigned)u, (unsigned)uh, rsh1);
+              bad |= ((th >> mcm) ^ (t0 >> 31)) | ((uh >> rcm) ^ (u0 >> 31));
+              asm("add.sat.s32 %0, %1, %2;" : "=r"(y[j]) : "r"(t0 >> msh2), "r"(u0 >> rsh2));
+            }
+            y[j] = min(max(y[j], e.lo), e.hi);
+          }
+        }
+        if (FORM == 2 || (FORM == 1 && __any_sync(0xffffffffu, bad != 0))) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const long long sum = (((long long)v[16 * h + j] * (long long)k.b + k.r0) >> k.sh) + (((long long)r[j] * (long long)k.rb + k.rr0) >> k.rsh);
+            y[j] = (int)(sum < (long long)e.lo ? (long long)e.lo : sum > (long long)e.hi ? (long long)e.hi : sum);
+          }
+        }
+      }
+      if (RAW || sum_out) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) words[(16 * h + j) * 32] = y[j];
+      }
+      if constexpr (Q) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          int z[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            long long t;
+            asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(y[4 * g + j]), "r"(qb), "l"(qr0));
+            if constexpr (FORM < 2) z[j] = (int)(t >> 32) >> qsh;
+            else { const long long zz = t >> qsh; z[j] = (int)(zz < -256 ? -256 : zz > 255 ? 255 : zz); }
+          }
+          unsigned w;
+          if (p.q_sat == 1) w = sat_pack4<false>(z[0], z[1], z[2], z[3]);
+          else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) z[j] = min(max(z[j], p.q_lo), p.q_hi);
+            w = __byte_perm(__byte_perm((unsigned)z[0], (unsigned)z[1], 0x0040), __byte_perm((unsigned)z[2], (unsigned)z[3], 0x0040), 0x5410);
+          }
+          w = quad_transpose(w, lane);                                    // four channels of pixel 16 h + 4 g + lane % 4
+          asm volatile("st.shared.b32 [%0], %1;" ::"r"(qbox + (uint32_t)((16 * h + 4 * g + (lane & 3)) * 32 + (lane & ~3))), "r"(w) : "memory");
+        }
       }
     }
+    fence_async_smem();                              // make this lane's writes visible to the TMA engine
+    __syncwarp();
+    if (lane == 0) {
+      if (px0 < p.P) {
+        if (RAW || sum_out) tma_store_2d(e.map_out, slots + (uint32_t)(slot * kWideBox), ch0 * 4, px0);
+        if (Q) tma_store_2d(map_q, qbox, ch0, px0);
+      }
+      tma_store_commit();
+      // the store before this one has been read: its slot takes the box after next, and the other byte box is free
+      asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      prefetch();
+    }
+    __syncwarp();
+    ++done;
+    if (++slot == kWideSlots) { slot = 0; sph ^= 1u; }
   };
 
-  int va[16], vb[16], ra[16], rb[16];
+  int va[32], vb[32];
   uint32_t tcount = 0, as = 0;
   int p_tile = e.p_tile0;
-  load_res(tile_at(p, p_tile) * p.pt + e.col0, ra);
-  if (!wait_bar(&ctl.tfull[0], 0)) return;
-  tc_fence_after();
-  tmem_ld16_issue(t_warp, va);
-  bool pending = true;
-  while (true) {
-    const int px_first = tile_at(p, p_tile) * p.pt + e.col0;
-    const bool has_next = p_tile + e.p_step < p.p_tiles;
-    const uint32_t nas = (tcount + 1u) & bmask, naph = ((tcount + 1u) >> p.lg_bufs) & 1u;
-    const uint32_t t_addr = t_warp + as * p.acc_stride;
-    for (int u = 0; u < units; u += 2) {
-      load_res(px_first + 16 * (u + 1), rb);
-      tmem_ld_wait();
-      tie16(va);
-      tmem_ld16_issue(t_addr + 16 * (u + 1), vb);
-      unit(va, ra, px_first + 16 * u);
-      if (u + 2 < units) load_res(px_first + 16 * (u + 2), ra);
-      else if (has_next) load_res(tile_at(p, p_tile + e.p_step) * p.pt + e.col0, ra);
-      tmem_ld_wait();
-      tie16(vb);
-      pending = false;
-      if (u + 2 < units) { tmem_ld16_issue(t_addr + 16 * (u + 2), va); pending = true; }
-      else {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) release_accumulator(p, ctl, as);
-      }
-      unit(vb, rb, px_first + 16 * (u + 1));
-    }
-    if (!has_next) break;
-    if (!wait_bar(&ctl.tfull[nas], naph)) break;
+  if (wait_bar(&ctl.tfull[0], 0)) {
     tc_fence_after();
-    tmem_ld16_issue(t_warp + nas * p.acc_stride, va);
-    pending = true;
-    p_tile += e.p_step; ++tcount; as = nas;
+    tmem_ld32_issue(t_warp, va);
+    bool pending = true;
+    while (true) {
+      const int px_first = tile_at(p, p_tile) * p.pt + e.col0;
+      const bool has_next = p_tile + e.p_step < p.p_tiles;
+      const uint32_t nas = (tcount + 1u) & bmask, naph = ((tcount + 1u) >> p.lg_bufs) & 1u;
+      const uint32_t t_addr = t_warp + as * p.acc_stride;
+      for (int c = 0; c < nb; c += 2) {
+        tmem_ld_wait();
+        tie32(va);
+        tmem_ld32_issue(t_addr + 32 * (c + 1), vb);
+        box(va, px_first + 32 * c);
+        tmem_ld_wait();
+        tie32(vb);
+        pending = false;
+        if (c + 2 < nb) { tmem_ld32_issue(t_addr + 32 * (c + 2), va); pending = true; }
+        else {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) release_accumulator(p, ctl, as);
+        }
+        box(vb, px_first + 32 * (c + 1));
+      }
+      if (!ok || !has_next) break;
+      if (!wait_bar(&ctl.tfull[nas], naph)) break;
+      tc_fence_after();
+      tmem_ld32_issue(t_warp + nas * p.acc_stride, va);
+      pending = true;
+      p_tile += e.p_step; ++tcount; as = nas;
+    }
+    if (pending) tmem_ld_wait();
   }
-  if (pending) tmem_ld_wait();
+  if (lane == 0) {
+    // every copy this thread started must have landed before the CTA may exit (all consumed unless a wait ran out)
+    for (int i = done; !RAW && i < issued; ++i) {
+      const uint32_t bar = smem_u32(&ctl.wbox[e.ew][i % kWideSlots]), ph = (uint32_t)(i / kWideSlots) & 1u;
+      const unsigned long long t0 = global_ns();
+      while (!mbar_try_wait(bar, ph))
+        if (global_ns() - t0 > kWaitBudgetNs) { atomicCAS(p.status, 0u, (uint32_t)HQ_DEV_TIMEOUT_DRAIN); break; }
+    }
+    tma_store_wait_all();
+  }
 }
 
 // General tile loop: every output type, direct stores, 64-bit arithmetic, INT32 residuals.
@@ -703,12 +779,12 @@ __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanCo
 // cta_group::2 instructions (a kernel that contains them cannot be launched without clusters).
 // RTM: the instantiation for fused 8-bit residuals that travel through tensor memory; it has one more warp, which
 // stores the finished output tiles.
-// WIDE: the instantiation whose epilogue is the INT32 residual add (epilogue_loop_wide).
+// WIDE: the instantiation for INT32 results, raw or through the residual add of Fig. 2 (epilogue_loop_wide).
 template <int EPI_WARPS, int MIN_CTAS, int MMA_WARPS, bool DUO = false, bool RTM = false, bool WIDE = false>
 __global__ void __launch_bounds__(32 * (1 + MMA_WARPS + EPI_WARPS + (RTM ? 1 : 0)), MIN_CTAS)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res,
-               const __grid_constant__ TcParams p) {
+               const __grid_constant__ CUtensorMap map_q, const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ SharedCtl ctl;
 
@@ -744,6 +820,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     }
     mbar_init(smem_u32(&ctl.drain), p.ni);
     mbar_init(smem_u32(&ctl.wfull), 1);
+    if constexpr (WIDE) for (int s = 0; s < 8 * kWideSlots; ++s) mbar_init(smem_u32(&ctl.wbox[s / kWideSlots][s % kWideSlots]), 1);
     for (int s = 0; s < 3; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), p.ni); }
     ctl.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1129,22 +1206,28 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if constexpr (WIDE) {
       if (half < p.halves) {
         EpiCtx e;
-        e.p = &p; e.ctl = &ctl; e.tmem_base = tmem_base; e.lane = lane; e.q = q; e.cq = cq; e.ew = ew; e.half = half;
+        e.p = &p; e.ctl = &ctl; e.map_out = &map_out; e.smem_raw = smem_raw; e.raw = raw; e.out_stage = out_stage;
+        e.tmem_base = tmem_base; e.lane = lane; e.q = q; e.cq = cq; e.ew = ew; e.half = half;
         e.col0 = col0; e.px_per_warp = px_per_warp; e.ch = ch; e.c_tile = c_tile; e.p_tile0 = p_tile0; e.p_step = p_step;
-        e.lo = lo; e.hi = hi; e.ch_live = ch_live;
-        const ChanConst k = chan_const(p, ch, false);
-        const int qc = p.q_out && ch_live ? p.qc[ch] : 32;
-        const bool wfast = __all_sync(0xffffffffu, k.sh >= 32 && qc >= 32) != 0;
-        const bool rnarrow = wfast && __all_sync(0xffffffffu, k.rsh >= 32) != 0;
-        asm volatile("griddepcontrol.wait;" ::: "memory");             // the residual is the output of an earlier kernel
-        if (p.q_out) {
-          if (rnarrow) epilogue_loop_wide<true, true, true>(e, k);
-          else if (wfast) epilogue_loop_wide<true, false, true>(e, k);
-          else epilogue_loop_wide<false, false, true>(e, k);
+        e.lo = lo; e.hi = hi; e.ch_live = ch_live; e.warp_live = warp_live;
+        if (!p.res) {
+          ChanConst k{};
+          k.bias = (ch_live && p.bias) ? p.bias[ch] : 0;
+          epilogue_loop_wide<3, false>(e, k, &map_res, &map_q);
         } else {
-          if (rnarrow) epilogue_loop_wide<true, true, false>(e, k);
-          else if (wfast) epilogue_loop_wide<true, false, false>(e, k);
-          else epilogue_loop_wide<false, false, false>(e, k);
+          const ChanConst k = chan_const(p, ch, false);
+          const int qc = p.q_out && ch_live ? p.qc[ch] : 32;
+          const bool form1 = __all_sync(0xffffffffu, qc >= 32) != 0;
+          const bool form0 = form1 && __all_sync(0xffffffffu, k.sh >= 32 && k.rsh >= 32) != 0;
+          asm volatile("griddepcontrol.wait;" ::: "memory");           // the residual is the output of an earlier kernel
+          if (p.q_out) {
+            if (form0) epilogue_loop_wide<0, true>(e, k, &map_res, &map_q);
+            else if (form1) epilogue_loop_wide<1, true>(e, k, &map_res, &map_q);
+            else epilogue_loop_wide<2, true>(e, k, &map_res, &map_q);
+          } else {
+            if (form0) epilogue_loop_wide<0, false>(e, k, &map_res, &map_q);
+            else epilogue_loop_wide<1, false>(e, k, &map_res, &map_q);
+          }
         }
       }
     } else {
@@ -1387,6 +1470,10 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.staged_res = (p.staged_out && a.res && a.res_bits == 8 && a.cout % 16 == 0) ? 1 : 0;
   // Launch shape: pair (two CTAs per SM) for short reductions when the tile pipeline fits half an SM.
   const long long k_total = (long long)a.kh * a.kw * a.cin;
+  // INT32 results through TMA boxes (epilogue_loop_wide): every residual add, and raw results but for the long reductions
+  // that the two-CTA shape serves better (and rows that are not whole 16-byte pieces)
+  const bool int32_boxes = a.wide || (a.out_bits == 32 && !a.res && a.cout % 4 == 0 && k_total < 2048);
+  const int box_bytes = kSoloEpilogueWarps * (kWideSlots * kWideBox + (a.wide && a.wide->q ? 2 * kWideQBox : 0));
   // (measured: with the weight slab resident the one-CTA shape catches up for K >= 128; the pair shape still
   // wins on the fused-residual expansions with the shortest reduction, and loses where a tile carries little
   // epilogue work, e.g. 64 output channels.  Where the layer is large enough for 256-pixel tiles and its residual
@@ -1418,7 +1505,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     const int smem_budget = kSmemBudget;                // dynamic bytes after the 1024-byte alignment slack
     // staging: 8 warps x pt/2 pixel rows x 32 bytes (reserved at the 8-bit size), residual 2 or 4 x [pt][128]
     bool chosen = false;
-    for (int cap = 256; cap >= 64 && !chosen; cap >>= 1) {   // largest pixel tile that leaves room for >= 3 stages
+    for (int cap = int32_boxes && a.cout > 64 ? 128 : 256; cap >= 64 && !chosen; cap >>= 1) {   // largest pixel tile that leaves room for >= 3 stages
       p.pt = pick_pt(P, p.c_tiles, h->sm_count, cap);
       // A weight slab of at most 72 KiB stays resident (the stages then hold activations only): a third less
       // traffic into shared memory per K block.  Where the slab would cost the larger pixel tile its stages, the
@@ -1430,7 +1517,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
         stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
         p.fold = (a.cout <= 64 && p.pt >= 128) ? 1 : 0;
         p.halves = p.pt >= (p.fold ? 256 : 128) ? 2 : 1;
-        out_tile_bytes = p.staged_out ? 4 * p.pt * 32 : 0;
+        out_tile_bytes = int32_boxes ? box_bytes : p.staged_out ? 4 * p.pt * 32 : 0;
         p.lg_bufs = p.pt <= 128 ? 2 : 1;
         res_tile_bytes = p.staged_res ? p.pt * kTileC : 0;
         // residual tiles: as many buffers as accumulators, fewer when a long reduction needs the room for stages
@@ -1530,7 +1617,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     // Fourth shape, *duo*: clusters of two CTAs on adjacent SMs share every MMA (cta_group::2, M = 256): each CTA
     // fetches its own 128 weight rows and HALF of the tile's pixel rows, 32 KiB per K block and SM instead of
     // 48 KiB for the same MMA time.  For the long reductions whose weights stream, which the operand fetch bounds.
-    p.duo = (!pair && !wide && !a.wide && !p.strip && !p.wres && !p.fold && p.pt >= 128 && p.bkb == 128 && a.cout % 256 == 0 &&
+    p.duo = (!pair && !wide && !int32_boxes && !p.strip && !p.wres && !p.fold && p.pt >= 128 && p.bkb == 128 && a.cout % 256 == 0 &&
              k_total >= 2048 && (long long)p.p_tiles * p.c_tiles >= 2LL * h->sm_count) ? 1 : 0;
     if (p.duo) {
       stage_bytes = (kTileC + p.pt / 2) * p.bkb;
@@ -1566,7 +1653,9 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.out = a.out; p.out_bits = a.out_bits; p.out_signed = a.out_signed;
   if (a.wide) {
     p.q_out = a.wide->q; p.qb = a.wide->qb; p.qc = a.wide->qc; p.q_hi = a.wide->q_qmax;
+    p.q_sat = 0;
     p.q_lo = a.wide->q_relu ? (a.wide->q_qmin > 0 ? a.wide->q_qmin : 0) : a.wide->q_qmin;
+    p.q_sat = p.q_lo == 0 && p.q_hi == 255 ? 1 : 0;
   }
   {
     const int lo = a.relu ? (a.qmin > 0 ? a.qmin : 0) : a.qmin;
@@ -1576,7 +1665,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.status = h->dev_status;
 
   const CUtensorMapSwizzle swz = swizzle_for(p.bkb);
-  alignas(64) CUtensorMap map_x, map_w, map_out, map_res;
+  alignas(64) CUtensorMap map_x, map_w, map_out, map_res, map_q;
   p.x_tiled = (!a.pitch_w && a.kh == 1 && a.kw == 1 && a.stride == 1 && a.pad == 0) ? 1 : 0;
   if (p.strip) {
     // activations (C, W, H, N), box = one patch: bkb channels x pitch columns x (rows + 3) rows of one image
@@ -1594,7 +1683,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     if (!encode_im2col_map(&map_x, a, p.bkb, p.pt >> p.duo)) return HQ_ERR_CUDA;
   }
   if (!encode_rows_map(&map_w, a.wgt, a.cout, (long long)a.kh * a.kw * a.cin, p.bkb, p.fold ? 64 : kTileC, swz)) return HQ_ERR_CUDA;
-  map_out = map_w; map_res = map_w;                    // valid placeholders when a path is not staged
+  map_out = map_w; map_res = map_w; map_q = map_w;                    // valid placeholders when a path is not staged
   // (with rtm the residual tile is an MMA operand and, later, the output box: 128-byte swizzle both ways)
   const CUtensorMapSwizzle box_swz = p.rtm ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;
   if (p.strip) {
@@ -1612,6 +1701,12 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
                                        box_swz)) return HQ_ERR_CUDA;
   if (p.staged_res && !encode_rows_map(&map_res, a.res, P, a.cout, kTileC, p.pt, box_swz))
     return HQ_ERR_CUDA;
+
+  if (int32_boxes) {
+    if (a.out && !encode_rows_map(&map_out, a.out, P, 4ll * a.cout, 128, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
+    if (a.res && !encode_rows_map(&map_res, a.res, P, (long long)a.cout * a.res_bits / 8, a.res_bits == 32 ? 128 : 32, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
+    if (p.q_out && !encode_rows_map(&map_q, p.q_out, P, a.cout, 32, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
+  }
 
   const size_t dyn_smem = (size_t)stages * stage_bytes + out_tile_bytes + ((size_t)res_tile_bytes << p.lg_rbufs) + wres_bytes + patch_total +
                           (p.rtm ? 16 * 1024 : 0) + 1024;
@@ -1631,18 +1726,18 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   cudaError_t err;
   if (p.duo) {
     cfg.blockDim = dim3(32 * (2 + kSoloEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
-    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, 1, true>, map_x, map_w, map_out, map_res, p);
+    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, 1, true>, map_x, map_w, map_out, map_res, map_q, p);
   } else if (wide) {
     cfg.blockDim = dim3(32 * 11); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
-    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<8, 1, 1, false, true>, map_x, map_w, map_out, map_res, p);
+    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<8, 1, 1, false, true>, map_x, map_w, map_out, map_res, map_q, p);
   } else if (pair) {
     cfg.blockDim = dim3(32 * (1 + kPairIssuerWarps + kPairEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem;
-    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, map_x, map_w, map_out, map_res, p);
+    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);
   } else {
     // one CTA per SM (it may allocate all 512 tensor-memory columns): never request less than 120 KiB
     cfg.blockDim = dim3(32 * (1 + kSoloIssuerWarps + kSoloEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
-    if (a.wide) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps, false, false, true>, map_x, map_w, map_out, map_res, p);
-    else err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps>, map_x, map_w, map_out, map_res, p);
+    if (int32_boxes) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps, false, false, true>, map_x, map_w, map_out, map_res, map_q, p);
+    else err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);
   }
   return err == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }
