@@ -434,10 +434,21 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
 // What bounds it: nine bytes of HBM traffic per value against three wide multiplies and about fifteen plain instructions.
 // 64 images of 56x56x256: plain loads and stores of a lane (16 KiB in flight per SM) 172-261 us, this form 95-106 us;
 // raw result 110 us with direct stores, 52 us here.
-// FORM 0: every shift of the warp's channels is at least 32 (no 64-bit step).  1: c or rc below 32: bits [c, c + 32) by a funnel
-// shift, and where some value of 16 pixels does not fit 32 bits those 16 again in 64 bits.  2: qc below 32 as well: 64 bits.
+// FORM 0: every shift of the warp's channels is at least 32 (no 64-bit step).  1: c or rc below 32: 64-bit sum of the two terms,
+// saturated.  2: qc below 32 as well.  3: raw.  (The loop works on 16 pixels at a time: with 32 unrolled, and the 64-bit form as
+// a second pass, it ran out of the instruction cache: 2.9 stalls per issue.)
 constexpr int kWideSlots = 3;
 constexpr int kWideBox = 32 * 32 * 4, kWideQBox = 32 * 32;
+// (t >> c) as upper and lower word: c1 = min(c, 32), c2 = c - c1, cm = min(c, 31)
+__device__ __forceinline__ void shift64(long long t, int c1, int c2, int cm, int& up, unsigned& low) {
+  const int hi = (int)(t >> 32);
+  low = (unsigned)((int)__funnelshift_rc((unsigned)t, (unsigned)hi, c1) >> c2);
+  up = hi >> cm;
+}
+// a 64-bit value saturated to INT32
+__device__ __forceinline__ int sat32(int up, unsigned low) {
+  return up == ((int)low >> 31) ? (int)low : (up >> 31) ^ INT_MAX;
+}
 template <int FORM, bool Q>
 __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const ChanConst& k_in, const CUtensorMap* map_res, const CUtensorMap* map_q) {
   const EpiCtx e = e_in;
@@ -448,7 +459,7 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
   const int lane = e.lane;
   const int qb = Q && e.ch_live ? p.qb[e.ch] : 0, qc = Q && e.ch_live ? p.qc[e.ch] : 32;
   const long long qr0 = 1LL << (qc - 1);
-  const int qsh = FORM < 2 ? qc - 32 : qc;
+  const int qsh = qc - 32, qsh1 = min(qc, 32), qsh2 = qc - qsh1, qcm = min(qc, 31);
   const int msh1 = min(k.sh, 32), msh2 = k.sh - msh1, mcm = min(k.sh, 31);
   const int rsh1 = min(k.rsh, 32), rsh2 = k.rsh - rsh1, rcm = min(k.rsh, 31);
   const uint32_t bmask = (1u << p.lg_bufs) - 1u;
@@ -484,88 +495,81 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
   int done = 0, slot = 0;
   uint32_t sph = 0;
   bool ok = true;
-  auto box = [&](const int (&v)[32], int px0) {
-    if (!live) return;
-    if (!RAW) { ok = wait_bar(&ctl.wbox[e.ew][slot], sph); if (!ok) return; }
+  // 16 pixels of a box: h = 0 the first half, 1 the second
+  auto unit = [&](const int (&v)[16], int h) {
     uint8_t* const sp = e.smem_raw + (slots - e.raw) + slot * kWideBox;
-    const uint32_t qbox = qboxes + (uint32_t)((done & 1) * kWideQBox);
-    int* const words = (int*)sp + lane;
+    int* const words = (int*)sp + 512 * h + lane;
+    int y[16];
+    if constexpr (RAW) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      int y[16];
-      if constexpr (RAW) {
+      for (int j = 0; j < 16; ++j) y[j] = v[j] + k.bias;
+    } else {
+      int r[16];
+      if (!res8) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) y[j] = v[16 * h + j] + k.bias;
+        for (int j = 0; j < 16; ++j) r[j] = words[32 * j];
       } else {
-        int r[16];
-        if (!res8) {
+        const uint8_t* const bytes = sp + res_at + 512 * h + lane;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) r[j] = words[(16 * h + j) * 32];
+        for (int j = 0; j < 16; ++j) r[j] = p.res_signed ? (int)(signed char)bytes[32 * j] : (int)bytes[32 * j];
+        __syncwarp();                                // these byte rows may be overwritten by the sums below
+      }
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        long long t, u;
+        asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(v[j]), "r"(k.b), "l"(k.r0));
+        asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(u) : "r"(r[j]), "r"(k.rb), "l"(k.rr0));
+        if constexpr (FORM == 0) {
+          y[j] = ((int)(t >> 32) >> msh2) + ((int)(u >> 32) >> rsh2);                // each within [-2^30, 2^30)
         } else {
-          const uint8_t* const bytes = sp + res_at + lane;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) r[j] = p.res_signed ? (int)(signed char)bytes[(16 * h + j) * 32] : (int)bytes[(16 * h + j) * 32];
-          __syncwarp();                              // these byte rows may be overwritten by the sums below
+          int tu, uu;
+          unsigned tl, ul;
+          shift64(t, msh1, msh2, mcm, tu, tl);
+          shift64(u, rsh1, rsh2, rcm, uu, ul);
+          unsigned low;
+          int up;
+          asm("add.cc.u32 %0, %2, %3;\n\taddc.s32 %1, %4, %5;" : "=r"(low), "=r"(up) : "r"(tl), "r"(ul), "r"(tu), "r"(uu));
+          y[j] = sat32(up, low);
         }
-        int bad = FORM == 2 ? 1 : 0;
-        if constexpr (FORM < 2) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            long long t, u;
-            asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(v[16 * h + j]), "r"(k.b), "l"(k.r0));
-            asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(u) : "r"(r[j]), "r"(k.rb), "l"(k.rr0));
-            if constexpr (FORM == 0) {
-              y[j] = ((int)(t >> 32) >> msh2) + ((int)(u >> 32) >> rsh2);            // each within [-2^30, 2^30)
-            } else {
-              const int th = (int)(t >> 32), uh = (int)(u >> 32);
-              const int t0 = (int)__funnelshift_rc((unsigned)t, (unsigned)th, msh1), u0 = (int)__funnelshift_rc((unsigned)u, (unsigned)uh, rsh1);
-              bad |= ((th >> mcm) ^ (t0 >> 31)) | ((uh >> rcm) ^ (u0 >> 31));
-              asm("add.sat.s32 %0, %1, %2;" : "=r"(y[j]) : "r"(t0 >> msh2), "r"(u0 >> rsh2));
-            }
-            y[j] = min(max(y[j], e.lo), e.hi);
-          }
-        }
-        if (FORM == 2 || (FORM == 1 && __any_sync(0xffffffffu, bad != 0))) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const long long sum = (((long long)v[16 * h + j] * (long long)k.b + k.r0) >> k.sh) + (((long long)r[j] * (long long)k.rb + k.rr0) >> k.rsh);
-            y[j] = (int)(sum < (long long)e.lo ? (long long)e.lo : sum > (long long)e.hi ? (long long)e.hi : sum);
-          }
-        }
-      }
-      if (RAW || sum_out) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) words[(16 * h + j) * 32] = y[j];
-      }
-      if constexpr (Q) {
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          int z[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            long long t;
-            asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(y[4 * g + j]), "r"(qb), "l"(qr0));
-            if constexpr (FORM < 2) z[j] = (int)(t >> 32) >> qsh;
-            else { const long long zz = t >> qsh; z[j] = (int)(zz < -256 ? -256 : zz > 255 ? 255 : zz); }
-          }
-          unsigned w;
-          if (p.q_sat == 1) w = sat_pack4<false>(z[0], z[1], z[2], z[3]);
-          else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) z[j] = min(max(z[j], p.q_lo), p.q_hi);
-            w = __byte_perm(__byte_perm((unsigned)z[0], (unsigned)z[1], 0x0040), __byte_perm((unsigned)z[2], (unsigned)z[3], 0x0040), 0x5410);
-          }
-          w = quad_transpose(w, lane);                                    // four channels of pixel 16 h + 4 g + lane % 4
-          asm volatile("st.shared.b32 [%0], %1;" ::"r"(qbox + (uint32_t)((16 * h + 4 * g + (lane & 3)) * 32 + (lane & ~3))), "r"(w) : "memory");
-        }
+        y[j] = min(max(y[j], e.lo), e.hi);
       }
     }
+    if (RAW || sum_out) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) words[32 * j] = y[j];
+    }
+    if constexpr (Q) {
+      const uint32_t qrow = qboxes + (uint32_t)((done & 1) * kWideQBox + 512 * h + (lane & 3) * 32 + (lane & ~3));
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        int z[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          long long t;
+          asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(y[4 * g + j]), "r"(qb), "l"(qr0));
+          if constexpr (FORM < 2) z[j] = (int)(t >> 32) >> qsh;
+          else { int up; unsigned low; shift64(t, qsh1, qsh2, qcm, up, low); z[j] = sat32(up, low); }
+        }
+        unsigned w;
+        if (p.q_sat == 1) w = sat_pack4<false>(z[0], z[1], z[2], z[3]);
+        else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) z[j] = min(max(z[j], p.q_lo), p.q_hi);
+          w = __byte_perm(__byte_perm((unsigned)z[0], (unsigned)z[1], 0x0040), __byte_perm((unsigned)z[2], (unsigned)z[3], 0x0040), 0x5410);
+        }
+        w = quad_transpose(w, lane);                                      // four channels of pixel 16 h + 4 g + lane % 4
+        asm volatile("st.shared.b32 [%0], %1;" ::"r"(qrow + 128u * g), "r"(w) : "memory");
+      }
+    }
+  };
+  // the finished box leaves, the box after next is fetched
+  auto ship = [&](int px0) {
     fence_async_smem();                              // make this lane's writes visible to the TMA engine
     __syncwarp();
     if (lane == 0) {
       if (px0 < p.P) {
         if (RAW || sum_out) tma_store_2d(e.map_out, slots + (uint32_t)(slot * kWideBox), ch0 * 4, px0);
-        if (Q) tma_store_2d(map_q, qbox, ch0, px0);
+        if (Q) tma_store_2d(map_q, qboxes + (uint32_t)((done & 1) * kWideQBox), ch0, px0);
       }
       tma_store_commit();
       // the store before this one has been read: its slot takes the box after next, and the other byte box is free
@@ -577,38 +581,40 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
     if (++slot == kWideSlots) { slot = 0; sph ^= 1u; }
   };
 
-  int va[32], vb[32];
+  int va[16], vb[16];
   uint32_t tcount = 0, as = 0;
   int p_tile = e.p_tile0;
   if (wait_bar(&ctl.tfull[0], 0)) {
     tc_fence_after();
-    tmem_ld32_issue(t_warp, va);
+    tmem_ld16_issue(t_warp, va);
     bool pending = true;
     while (true) {
       const int px_first = tile_at(p, p_tile) * p.pt + e.col0;
       const bool has_next = p_tile + e.p_step < p.p_tiles;
       const uint32_t nas = (tcount + 1u) & bmask, naph = ((tcount + 1u) >> p.lg_bufs) & 1u;
       const uint32_t t_addr = t_warp + as * p.acc_stride;
-      for (int c = 0; c < nb; c += 2) {
+#pragma unroll 1
+      for (int c = 0; c < nb; ++c) {
+        if (!RAW && live) { ok = wait_bar(&ctl.wbox[e.ew][slot], sph); if (!ok) break; }
         tmem_ld_wait();
-        tie32(va);
-        tmem_ld32_issue(t_addr + 32 * (c + 1), vb);
-        box(va, px_first + 32 * c);
+        tie16(va);
+        tmem_ld16_issue(t_addr + 32 * c + 16, vb);
+        if (live) unit(va, 0);
         tmem_ld_wait();
-        tie32(vb);
+        tie16(vb);
         pending = false;
-        if (c + 2 < nb) { tmem_ld32_issue(t_addr + 32 * (c + 2), va); pending = true; }
+        if (c + 1 < nb) { tmem_ld16_issue(t_addr + 32 * (c + 1), va); pending = true; }
         else {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) release_accumulator(p, ctl, as);
         }
-        box(vb, px_first + 32 * (c + 1));
+        if (live) { unit(vb, 1); ship(px_first + 32 * c); }
       }
       if (!ok || !has_next) break;
       if (!wait_bar(&ctl.tfull[nas], naph)) break;
       tc_fence_after();
-      tmem_ld32_issue(t_warp + nas * p.acc_stride, va);
+      tmem_ld16_issue(t_warp + nas * p.acc_stride, va);
       pending = true;
       p_tile += e.p_step; ++tcount; as = nas;
     }
