@@ -125,7 +125,7 @@ struct SharedCtl {
   unsigned long long drain;
   unsigned long long wfull;              // resident weight slab landed
   unsigned long long pfull[3], pempty[3];  // strip mode: input patches
-  unsigned long long wbox[8][3];         // INT32 results: residual boxes of the epilogue warps (kWideSlots each)
+  unsigned long long wbox[16][3];         // INT32 results: residual boxes of the epilogue warps (kWideSlots each)
   uint32_t tmem_base;
   volatile uint32_t abort_flag;
 };
@@ -427,9 +427,9 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
 //   - a convolution that ends in the INT32 residual add of Fig. 2 (Section 3.3) and the requantization of the next block
 //     (WideArgs): y = clamp(relu(dn(acc + bias, b, c) + dn(res, rb, rc))) to INT32, z = clamp(dn(y, qb, qc)) to bytes;
 //   - a raw INT32 result, acc + bias (FORM 3).
-// A warp works on boxes of 32 pixels x 32 channels, one channel per lane.  The residual box arrives by TMA in one of the
-// warp's own three 4 KiB slots (two boxes ahead), the sums are written over it in place and leave by TMA from there;
-// the requantized bytes are turned round in lane quads and leave from a 1 KiB box.  No CTA-wide barrier, no predicates at the
+// Sixteen warps; a warp works on boxes of 16 pixels x 32 channels, one channel per lane.  The residual box arrives by TMA in one of the
+// warp's own three 2 KiB slots (two boxes ahead), the sums are written over it in place and leave by TMA from there;
+// the requantized bytes are turned round in lane quads and leave from a 512-byte box.  No CTA-wide barrier, no predicates at the
 // tensor's edges (the copies clip), and 64 KiB of loads in flight per SM.
 // What bounds it: nine bytes of HBM traffic per value against three wide multiplies and about fifteen plain instructions.
 // 64 images of 56x56x256: plain loads and stores of a lane (16 KiB in flight per SM) 172-261 us, this form 95-106 us;
@@ -438,7 +438,8 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
 // saturated.  2: qc below 32 as well.  3: raw.  (The loop works on 16 pixels at a time: with 32 unrolled, and the 64-bit form as
 // a second pass, it ran out of the instruction cache: 2.9 stalls per issue.)
 constexpr int kWideSlots = 3;
-constexpr int kWideBox = 32 * 32 * 4, kWideQBox = 32 * 32;
+constexpr int kWideWarps = 16;          // 640 threads: 96 registers each
+constexpr int kWideBox = 16 * 32 * 4, kWideQBox = 16 * 32;
 // (t >> c) as upper and lower word: c1 = min(c, 32), c2 = c - c1, cm = min(c, 31)
 __device__ __forceinline__ void shift64(long long t, int c1, int c2, int cm, int& up, unsigned& low) {
   const int hi = (int)(t >> 32);
@@ -463,13 +464,13 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
   const int msh1 = min(k.sh, 32), msh2 = k.sh - msh1, mcm = min(k.sh, 31);
   const int rsh1 = min(k.rsh, 32), rsh2 = k.rsh - rsh1, rcm = min(k.rsh, 31);
   const uint32_t bmask = (1u << p.lg_bufs) - 1u;
-  const int nb = e.px_per_warp >> 5;                                   // boxes per tile: 2 or 4
+  const int nb = e.px_per_warp >> 4;                                   // boxes per tile: 1 or 2
   const bool sum_out = p.out != nullptr, live = e.warp_live;
   if (e.p_tile0 >= p.p_tiles) return;
   const uint32_t t_warp = e.tmem_base + ((uint32_t)(e.q * 32) << 16) + (uint32_t)e.col0;
   const int ch0 = e.c_tile * kTileC + e.cq * 32;                       // first channel of the warp
   const uint32_t slots = e.out_stage + (uint32_t)(e.ew * kWideSlots * kWideBox);
-  const uint32_t qboxes = e.out_stage + (uint32_t)(kSoloEpilogueWarps * kWideSlots * kWideBox + e.ew * 2 * kWideQBox);
+  const uint32_t qboxes = e.out_stage + (uint32_t)(kWideWarps * kWideSlots * kWideBox + e.ew * 2 * kWideQBox);
   const bool res8 = !RAW && p.res_bits == 8;
   const uint32_t res_bytes = res8 ? kWideQBox : kWideBox, res_at = res8 ? kWideBox - kWideQBox : 0;   // bytes lie at the slot's end
   const unsigned long long pol = policy_evict_first();
@@ -485,7 +486,7 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
     const uint32_t bar = smem_u32(&ctl.wbox[e.ew][pf_slot]);
     mbar_expect_tx(bar, res_bytes);
     tma_load_2d_hint(slots + (uint32_t)(pf_slot * kWideBox) + res_at, map_res, bar, res8 ? ch0 : ch0 * 4,
-                     tile_at(p, pf_tile) * p.pt + e.col0 + 32 * pf_sub, pol);
+                     tile_at(p, pf_tile) * p.pt + e.col0 + 16 * pf_sub, pol);
     ++issued;
     if (++pf_slot == kWideSlots) pf_slot = 0;
     if (++pf_sub == nb) { pf_sub = 0; pf_tile += e.p_step; }
@@ -495,27 +496,27 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
   int done = 0, slot = 0;
   uint32_t sph = 0;
   bool ok = true;
-  // 16 pixels of a box: h = 0 the first half, 1 the second
-  auto unit = [&](const int (&v)[16], int h) {
+  // 8 pixels of a box: its h-th half
+  auto unit = [&](const int (&v)[8], int h) {
     uint8_t* const sp = e.smem_raw + (slots - e.raw) + slot * kWideBox;
-    int* const words = (int*)sp + 512 * h + lane;
-    int y[16];
+    int* const words = (int*)sp + 256 * h + lane;
+    int y[8];
     if constexpr (RAW) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) y[j] = v[j] + k.bias;
+      for (int j = 0; j < 8; ++j) y[j] = v[j] + k.bias;
     } else {
-      int r[16];
+      int r[8];
       if (!res8) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) r[j] = words[32 * j];
+        for (int j = 0; j < 8; ++j) r[j] = words[32 * j];
       } else {
-        const uint8_t* const bytes = sp + res_at + 512 * h + lane;
+        const uint8_t* const bytes = sp + res_at + 256 * h + lane;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) r[j] = p.res_signed ? (int)(signed char)bytes[32 * j] : (int)bytes[32 * j];
+        for (int j = 0; j < 8; ++j) r[j] = p.res_signed ? (int)(signed char)bytes[32 * j] : (int)bytes[32 * j];
         __syncwarp();                                // these byte rows may be overwritten by the sums below
       }
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
+      for (int j = 0; j < 8; ++j) {
         long long t, u;
         asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(v[j]), "r"(k.b), "l"(k.r0));
         asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(u) : "r"(r[j]), "r"(k.rb), "l"(k.rr0));
@@ -536,12 +537,12 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
     }
     if (RAW || sum_out) {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) words[32 * j] = y[j];
+      for (int j = 0; j < 8; ++j) words[32 * j] = y[j];
     }
     if constexpr (Q) {
-      const uint32_t qrow = qboxes + (uint32_t)((done & 1) * kWideQBox + 512 * h + (lane & 3) * 32 + (lane & ~3));
+      const uint32_t qrow = qboxes + (uint32_t)((done & 1) * kWideQBox + 256 * h + (lane & 3) * 32 + (lane & ~3));
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
+      for (int g = 0; g < 2; ++g) {
         int z[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -557,7 +558,7 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
           for (int j = 0; j < 4; ++j) z[j] = min(max(z[j], p.q_lo), p.q_hi);
           w = __byte_perm(__byte_perm((unsigned)z[0], (unsigned)z[1], 0x0040), __byte_perm((unsigned)z[2], (unsigned)z[3], 0x0040), 0x5410);
         }
-        w = quad_transpose(w, lane);                                      // four channels of pixel 16 h + 4 g + lane % 4
+        w = quad_transpose(w, lane);                                      // four channels of pixel 8 h + 4 g + lane % 4
         asm volatile("st.shared.b32 [%0], %1;" ::"r"(qrow + 128u * g), "r"(w) : "memory");
       }
     }
@@ -581,12 +582,12 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
     if (++slot == kWideSlots) { slot = 0; sph ^= 1u; }
   };
 
-  int va[16], vb[16];
+  int va[8], vb[8];
   uint32_t tcount = 0, as = 0;
   int p_tile = e.p_tile0;
   if (wait_bar(&ctl.tfull[0], 0)) {
     tc_fence_after();
-    tmem_ld16_issue(t_warp, va);
+    tmem_ld8_issue(t_warp, va);
     bool pending = true;
     while (true) {
       const int px_first = tile_at(p, p_tile) * p.pt + e.col0;
@@ -597,24 +598,25 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
       for (int c = 0; c < nb; ++c) {
         if (!RAW && live) { ok = wait_bar(&ctl.wbox[e.ew][slot], sph); if (!ok) break; }
         tmem_ld_wait();
-        tie16(va);
-        tmem_ld16_issue(t_addr + 32 * c + 16, vb);
+        tie8(va);
+        tmem_ld8_issue(t_addr + 16 * c + 8, vb);
         if (live) unit(va, 0);
         tmem_ld_wait();
-        tie16(vb);
+        tie8(vb);
         pending = false;
-        if (c + 1 < nb) { tmem_ld16_issue(t_addr + 32 * (c + 1), va); pending = true; }
+        if (c + 1 < nb) { tmem_ld8_issue(t_addr + 16 * (c + 1), va); pending = true; }
         else {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) release_accumulator(p, ctl, as);
         }
-        if (live) { unit(vb, 1); ship(px_first + 32 * c); }
+        if (live) unit(vb, 1);
+        if (live) ship(px_first + 16 * c);
       }
       if (!ok || !has_next) break;
       if (!wait_bar(&ctl.tfull[nas], naph)) break;
       tc_fence_after();
-      tmem_ld16_issue(t_warp + nas * p.acc_stride, va);
+      tmem_ld8_issue(t_warp + nas * p.acc_stride, va);
       pending = true;
       p_tile += e.p_step; ++tcount; as = nas;
     }
@@ -826,7 +828,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     }
     mbar_init(smem_u32(&ctl.drain), p.ni);
     mbar_init(smem_u32(&ctl.wfull), 1);
-    if constexpr (WIDE) for (int s = 0; s < 8 * kWideSlots; ++s) mbar_init(smem_u32(&ctl.wbox[s / kWideSlots][s % kWideSlots]), 1);
+    if constexpr (WIDE) for (int s = 0; s < kWideWarps * kWideSlots; ++s) mbar_init(smem_u32(&ctl.wbox[s / kWideSlots][s % kWideSlots]), 1);
     for (int s = 0; s < 3; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), p.ni); }
     ctl.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1422,7 +1424,7 @@ bool hq_conv_tc_init() {
          cudaFuncSetAttribute(conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               112 * 1024) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<8, 1, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAttr) == cudaSuccess &&
-         cudaFuncSetAttribute(conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+         cudaFuncSetAttribute(conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               kSmemAttr) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<kSoloEpilogueWarps, 1, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               kSmemAttr) == cudaSuccess;
@@ -1479,7 +1481,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // INT32 results through TMA boxes (epilogue_loop_wide): every residual add, and raw results but for the long reductions
   // that the two-CTA shape serves better (and rows that are not whole 16-byte pieces)
   const bool int32_boxes = a.wide || (a.out_bits == 32 && !a.res && a.cout % 4 == 0 && k_total < 2048);
-  const int box_bytes = kSoloEpilogueWarps * (kWideSlots * kWideBox + (a.wide && a.wide->q ? 2 * kWideQBox : 0));
+  const int box_bytes = kWideWarps * (kWideSlots * kWideBox + (a.wide && a.wide->q ? 2 * kWideQBox : 0));
   // (measured: with the weight slab resident the one-CTA shape catches up for K >= 128; the pair shape still
   // wins on the fused-residual expansions with the shortest reduction, and loses where a tile carries little
   // epilogue work, e.g. 64 output channels.  Where the layer is large enough for 256-pixel tiles and its residual
@@ -1522,7 +1524,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
         if (!p.wres) { if (keep_w) continue; wres_bytes = 0; }
         stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
         p.fold = (a.cout <= 64 && p.pt >= 128) ? 1 : 0;
-        p.halves = p.pt >= (p.fold ? 256 : 128) ? 2 : 1;
+        p.halves = int32_boxes ? 4 : p.pt >= (p.fold ? 256 : 128) ? 2 : 1;
         out_tile_bytes = int32_boxes ? box_bytes : p.staged_out ? 4 * p.pt * 32 : 0;
         p.lg_bufs = p.pt <= 128 ? 2 : 1;
         res_tile_bytes = p.staged_res ? p.pt * kTileC : 0;
@@ -1709,9 +1711,9 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     return HQ_ERR_CUDA;
 
   if (int32_boxes) {
-    if (a.out && !encode_rows_map(&map_out, a.out, P, 4ll * a.cout, 128, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
-    if (a.res && !encode_rows_map(&map_res, a.res, P, (long long)a.cout * a.res_bits / 8, a.res_bits == 32 ? 128 : 32, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
-    if (p.q_out && !encode_rows_map(&map_q, p.q_out, P, a.cout, 32, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
+    if (a.out && !encode_rows_map(&map_out, a.out, P, 4ll * a.cout, 128, 16, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
+    if (a.res && !encode_rows_map(&map_res, a.res, P, (long long)a.cout * a.res_bits / 8, a.res_bits == 32 ? 128 : 32, 16, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
+    if (p.q_out && !encode_rows_map(&map_q, p.q_out, P, a.cout, 32, 16, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
   }
 
   const size_t dyn_smem = (size_t)stages * stage_bytes + out_tile_bytes + ((size_t)res_tile_bytes << p.lg_rbufs) + wres_bytes + patch_total +
@@ -1741,8 +1743,8 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);
   } else {
     // one CTA per SM (it may allocate all 512 tensor-memory columns): never request less than 120 KiB
-    cfg.blockDim = dim3(32 * (1 + kSoloIssuerWarps + kSoloEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
-    if (int32_boxes) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps, false, false, true>, map_x, map_w, map_out, map_res, map_q, p);
+    cfg.blockDim = dim3(32 * (1 + kSoloIssuerWarps + (int32_boxes ? kWideWarps : kSoloEpilogueWarps))); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
+    if (int32_boxes) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, true>, map_x, map_w, map_out, map_res, map_q, p);
     else err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);
   }
   return err == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
