@@ -432,8 +432,8 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
 // the requantized bytes are turned round in lane quads and leave from a 512-byte box.  No CTA-wide barrier, no predicates at the
 // tensor's edges (the copies clip), and 64 KiB of loads in flight per SM.
 // What bounds it: nine bytes of HBM traffic per value against three wide multiplies and about fifteen plain instructions.
-// 64 images of 56x56x256: plain loads and stores of a lane (16 KiB in flight per SM) 172-261 us, this form 95-106 us;
-// raw result 110 us with direct stores, 52 us here.
+// 64 images of 56x56x256 (461 MB): loads and stores by the lanes (16 KiB in flight per SM) 172-261 us; boxes on eight warps
+// 131-135 us, on sixteen 113-119 us (4.0 TB/s, issue slots 47 % busy); raw result 110 us with direct stores, 43 us here.
 // FORM 0: every shift of the warp's channels is at least 32 (no 64-bit step).  1: c or rc below 32: 64-bit sum of the two terms,
 // saturated.  2: qc below 32 as well.  3: raw.  (The loop works on 16 pixels at a time: with 32 unrolled, and the 64-bit form as
 // a second pass, it ran out of the instruction cache: 2.9 stalls per issue.)
