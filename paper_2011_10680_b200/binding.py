@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 
 import numpy as np
 
@@ -104,6 +105,21 @@ def lib():
     return _lib
 
 
+_packed = None
+
+
+def _packed_calls():
+    """hq_conv2d and hq_linear taking their structures as byte strings."""
+    global _packed
+    if _packed is None:
+        assert len(_PACK_TENSOR(*[0] * 7)) == C.sizeof(hq_tensor) and len(_PACK_CONV(*[0] * 17)) == C.sizeof(hq_conv_desc)
+        fns = [lib()["hq_conv2d"], lib()["hq_linear"]]           # function objects of their own
+        for fn in fns:
+            fn.argtypes, fn.restype = [C.c_void_p, C.c_char_p, C.c_char_p, C.c_char_p, C.c_void_p], C.c_int32
+        _packed = fns
+    return _packed
+
+
 def ilp_solve(omega, size, bops, latency, size_limit: int = -1, bops_limit: int = -1, latency_limit: int = -1):
     """hq_ilp_solve on host arrays of shape [n_layers, 2] (int64).  Returns (status, choices, objective)."""
     tabs = [np.ascontiguousarray(t, dtype=np.int64) for t in (omega, size, bops, latency)]
@@ -127,19 +143,42 @@ def _check(code: int, where: str):
         raise HqError(code, where)
 
 
+_raw_stream = None
+
+
 def _stream():
-    import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """Handle of torch's current stream.  (A small call is bound by the host: asking for the raw handle takes 0.3 us, the
+    stream object that torch.cuda.current_stream() builds 3.4.)"""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+        _raw_stream = (lambda: raw(device())) if raw else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _raw_stream()
 
 
 def tensor_of(t, c: int, bits: int, is_signed: int) -> hq_tensor:
     """Describe a torch CUDA tensor of shape (n, h, w, c_stored) as an hq_tensor with logical channels c."""
-    n, h, w = t.shape[0], t.shape[1], t.shape[2]
+    n, h, w = t.shape[:3]
     return hq_tensor(t.data_ptr(), n, h, w, c, bits, is_signed)
 
 
 def _dy(b, c) -> hq_dyadic:
     return hq_dyadic(b.data_ptr() if b is not None else None, c.data_ptr() if c is not None else None)
+
+
+# The same structures as byte strings: one native call instead of a ctypes object and a conversion per field.
+_PACK_TENSOR = struct.Struct("@P6i").pack
+_PACK_CONV = struct.Struct("@7i7P3i4x").pack
+
+
+def _ptr(t) -> int:
+    return t.data_ptr() if t is not None else 0
+
+
+def _packed_tensor(t, c, bits, is_signed) -> bytes:
+    n, h, w = t.shape[:3]
+    return _PACK_TENSOR(t.data_ptr(), n, h, w, c, bits, is_signed)
 
 
 def to_device(a):
@@ -223,14 +262,12 @@ class Handle:
     # ---- one call per C entry point --------------------------------------------------------
     def conv2d(self, x, in_bits, in_signed, cin, wgt, cout, kh, kw, stride, pad, bias, b, c, out, out_bits, out_signed,
                res=None, res_bits=0, res_signed=0, rb=None, rc=None, relu=1, qmin=0, qmax=255, linear=False):
-        tin = tensor_of(x, cin, in_bits, in_signed)
-        tout = tensor_of(out, cout, out_bits, out_signed)
+        # (the residual's structure is referenced by address: it has to live until the call returns)
         tres = tensor_of(res, cout, res_bits, res_signed) if res is not None else None
-        d = hq_conv_desc(kh, kw, stride, pad, cin, cout, in_bits, wgt.data_ptr(),
-                         bias.data_ptr() if bias is not None else None, _dy(b, c),
-                         C.pointer(tres) if tres is not None else None, _dy(rb, rc), relu, qmin, qmax)
-        fn = lib().hq_linear if linear else lib().hq_conv2d
-        return fn(self._h, C.byref(tin), C.byref(d), C.byref(tout), _stream())
+        d = _PACK_CONV(kh, kw, stride, pad, cin, cout, in_bits, wgt.data_ptr(), _ptr(bias), _ptr(b), _ptr(c),
+                       C.addressof(tres) if tres is not None else 0, _ptr(rb), _ptr(rc), relu, qmin, qmax)
+        fn = _packed_calls()[1 if linear else 0]
+        return fn(self._h, _packed_tensor(x, cin, in_bits, in_signed), d, _packed_tensor(out, cout, out_bits, out_signed), _stream())
 
     def residual_add(self, main, main_bits, main_signed, mb, mc, res, res_bits, res_signed, rb, rc, ch,
                      relu, qmin, qmax, out, out_bits, out_signed):
