@@ -11,8 +11,8 @@
 //     pixels (integer sums: any split is exact);
 //   - weights do not depend on the previous kernel, so their TMA copies are issued before griddepcontrol.wait, as are
 //     barrier set-up, tensor-memory allocation and the per-channel constants;
-//   - activations come by TMA (tiled or im2col); where no tensor map can describe the fetch (packed 4-bit values, channel
-//     counts that are not a multiple of 32, tensors below 128 KiB without room behind them) the eight epilogue warps gather
+//   - activations come by TMA (tiled or im2col); where no tensor map can describe the fetch (packed 4-bit values, tensors
+//     below 128 KiB without room behind them) the eight epilogue warps gather
 //     them with 16-byte loads into the same swizzled layout: zeros for padding taps, nibbles widened on the way, no patch matrix;
 //   - the epilogue turns 4 x 4 bytes round inside lane quads with two shuffles and writes words: no staging box and no
 //     store whose completion has to be awaited;
@@ -50,7 +50,7 @@ struct SmallParams {
   int32_t h, w, cin, wo, howo, stride, pad, kh, kw;
   int32_t P, C, K;                               // output pixels, output channels, reduction length (values)
   int32_t bkb, nkb, lg_split, stages;            // bytes of K per stage (gather: 128); K blocks of the layer; log2 of the cluster size; stages per CTA
-  int32_t x_mode, cchunks;                       // kXGather / kXTiled / kXIm2col; K blocks per filter tap (TMA modes)
+  int32_t x_mode, cchunks, tail_steps;           // kXGather / kXTiled / kXIm2col; K blocks per filter tap and MMA steps of its last one (TMA modes)
   int32_t pt, lg_cols, c_tiles, fold;            // pixels per tile (MMA N); log2 of the pixels a CTA finishes; channel tiles; folded rows
   int32_t x_bits, x_signed;
   uint32_t part_off;                             // partial sums of a cluster, from the 1024-aligned base
@@ -324,8 +324,10 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
       auto load_w = [&](int i, int s) {
         const uint32_t bar = smem_u32(&ctl.wfull[s]), dst = tiles + (uint32_t)s * stage_bytes;
         mbar_expect_tx(bar, w_bytes);
-        tma_load_2d(dst, &map_w, bar, (kb0 + i) * p.bkb, row);
-        tma_load_2d(dst + w_bytes / 2, &map_w, bar, (kb0 + i) * p.bkb, row2);
+        int wx = (kb0 + i) * p.bkb;
+        if (!GATHER) { const int tap = (kb0 + i) / p.cchunks; wx = tap * p.cin + (kb0 + i - tap * p.cchunks) * p.bkb; }
+        tma_load_2d(dst, &map_w, bar, wx, row);
+        tma_load_2d(dst + w_bytes / 2, &map_w, bar, wx, row2);
       };
       const int px0 = p_tile * p.pt;
       const int img = (int)p.by_howo.div((uint32_t)px0), rem = px0 - img * p.howo, oh = (int)p.by_wo.div((uint32_t)rem), ow = rem - oh * p.wo;
@@ -377,9 +379,10 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
         tc_fence_after();
         const uint32_t a = tiles + (uint32_t)s * stage_bytes;
         uint64_t adesc = hi | (uint64_t)((a >> 4) & 0x3FFF), bdesc = hi | (uint64_t)(((a + w_bytes) >> 4) & 0x3FFF);
-        // (the last block may end inside: whole 32-byte steps beyond K are left out, a partial step meets zero weights)
-        const int left = p.K - (kb0 + i) * p.bkb;
-        const int steps = (min(left, p.bkb) + 31) >> 5;
+        // (a block may reach past the channels: whole 32-byte steps beyond them are left out, a partial step meets zeros)
+        int steps;
+        if (GATHER) steps = (min(p.K - (kb0 + i) * p.bkb, p.bkb) + 31) >> 5;
+        else steps = (kb0 + i + 1) % p.cchunks == 0 ? p.tail_steps : p.bkb >> 5;
         for (int q = 0; q < steps; ++q, adesc += 2, bdesc += 2) mma_i8(tmem_base, adesc, bdesc, idesc, (i | q) ? 1u : 0u);
         mma_commit(smem_u32(i + 1 == L ? &ctl.tfull : &ctl.empty[s]));
         if (++s == p.stages) { s = 0; ph ^= 1; }
@@ -611,10 +614,10 @@ SmallShape small_shape(const ConvArgs& a, int sm_count) {
   ConvArgs b8 = a;
   b8.in_bits = 8;
   const bool packed = a.in_bits == 4, rows_map = a.kh == 1 && a.kw == 1 && a.stride == 1 && a.pad == 0;
-  s.x_mode = packed || a.cin % 32 != 0 || !hq_conv_tc_supported(b8) ? kXGather
+  s.x_mode = packed || !hq_conv_tc_supported(b8) ? kXGather
            : rows_map ? kXTiled : !hq_conv_tc_small_im2col(a) ? kXIm2col : kXGather;
-  s.bkb = s.x_mode == kXGather || a.cin % 128 == 0 ? 128 : a.cin % 64 == 0 ? 64 : 32;
-  s.nkb = (int)(((long long)a.kh * a.kw * a.cin + s.bkb - 1) / s.bkb);
+  s.bkb = s.x_mode == kXGather ? 128 : hq_conv_bkb(a.cin);
+  s.nkb = s.x_mode == kXGather ? (int)(((long long)a.kh * a.kw * a.cin + s.bkb - 1) / s.bkb) : a.kh * a.kw * ((a.cin + s.bkb - 1) / s.bkb);
   // Pixel tile and split of the reduction: 64 pixels, fewer while that still doubles the CTAs without exceeding one per SM
   // (the epilogue of a tile is the longest piece of the chain, and half as long on half the pixels).
   for (s.pt = 64; ; s.pt >>= 1) {
@@ -672,7 +675,8 @@ hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t str
   p.x = a.in; p.h = a.h; p.w = a.w; p.cin = a.cin; p.wo = a.wo; p.howo = a.ho * a.wo;
   p.stride = a.stride; p.pad = a.pad; p.kh = a.kh; p.kw = a.kw;
   p.P = (int32_t)((long long)a.n * a.ho * a.wo); p.C = a.cout; p.K = a.kh * a.kw * a.cin;
-  p.x_mode = s.x_mode; p.bkb = s.bkb; p.cchunks = a.cin / s.bkb;
+  p.x_mode = s.x_mode; p.bkb = s.bkb; p.cchunks = (a.cin + s.bkb - 1) / s.bkb;
+  p.tail_steps = (a.cin - (p.cchunks - 1) * s.bkb + 31) >> 5;
   p.nkb = s.nkb; p.lg_split = s.lg_split; p.stages = s.stages; p.pt = s.pt; p.c_tiles = s.c_tiles;
   while ((1 << p.lg_cols) < (s.pt >> s.lg_split)) ++p.lg_cols;
   p.fold = s.fold;

@@ -65,7 +65,9 @@ constexpr int kPairIssuerWarps = 1;
 struct TcParams {
   int32_t P, C;          // output pixels (n*ho*wo) and output channels
   int32_t howo, wo, stride, pad, kw;
-  int32_t cchunks;       // K blocks per filter tap
+  int32_t cin;
+  int32_t cchunks;       // K blocks per filter tap; the last one may reach past the channels (the copies fill zeros there)
+  int32_t tail_steps;    // 32-byte MMA steps of a tap's last K block
   int32_t bkb;           // bytes of K per stage (32, 64 or 128) = swizzle span
   int32_t k_blocks;      // kh * kw * cchunks
   int32_t pt;            // pixel tile = MMA N: 64, 128 or 256
@@ -882,11 +884,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         mbar_expect_tx(bar, (uint32_t)p.k_blocks * w_bytes);
         for (int kb = 0; kb < p.k_blocks; ++kb) {
           const uint32_t w_dst = tiles + p.wres_off + (uint32_t)kb * w_bytes;
+          const int tap = kb / p.cchunks, wx = tap * p.cin + (kb - tap * p.cchunks) * p.bkb;
           if (p.fold) {
-            tma_load_2d(w_dst, &map_w, bar, kb * p.bkb, 0);
-            tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, kb * p.bkb, 0);
+            tma_load_2d(w_dst, &map_w, bar, wx, 0);
+            tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx, 0);
           } else {
-            tma_load_2d(w_dst, &map_w, bar, kb * p.bkb, c_tile * kTileC);
+            tma_load_2d(w_dst, &map_w, bar, wx, c_tile * kTileC);
           }
         }
       }
@@ -939,7 +942,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           oh -= d_oh; if (oh < 0) { oh += ho; --img; }
           img -= d_img;
         }
-        int chunk = 0, tap_s = 0, tap_r = 0;
+        int chunk = 0, tap_s = 0, tap_r = 0, wx = 0;     // wx: the block's first byte in a weight row
         // The residual tile of this output tile is fetched as soon as its buffer is free, but this thread only
         // blocks for the buffer after the tile's last operand block is on its way: the buffer comes back when the
         // epilogue of an earlier tile ends, and the operand copies must not queue behind that.
@@ -968,8 +971,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             if (rank == 0) mbar_expect_tx(bar, 2u * stage_bytes);
             if (p.x_tiled) tma_load_2d_2cta(w_dst + x_off, &map_x, bar, chunk * p.bkb, p0 + half_off);
             else tma_load_im2col_2cta(w_dst + x_off, &map_x, bar, chunk * p.bkb, cw, chh, img_now, (uint16_t)tap_s, (uint16_t)tap_r);
-            tma_load_2d_2cta(w_dst, &map_w, bar, kb * p.bkb, c_tile * kTileC);
-            if (++chunk == p.cchunks) { chunk = 0; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
+            tma_load_2d_2cta(w_dst, &map_w, bar, wx + chunk * p.bkb, c_tile * kTileC);
+            if (++chunk == p.cchunks) { chunk = 0; wx += p.cin; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
             if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1u; }
             if (res_due && kb + 1 == p.k_blocks && !residual(true)) { ok = false; break; }
             continue;
@@ -983,12 +986,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           if (p.wres) {
             // weights are resident
           } else if (p.fold) {   // 64-row box, twice: accumulator lanes 64-127 repeat lanes 0-63
-            tma_load_2d(w_dst, &map_w, bar, kb * p.bkb, 0);
-            tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, kb * p.bkb, 0);
+            tma_load_2d(w_dst, &map_w, bar, wx + chunk * p.bkb, 0);
+            tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx + chunk * p.bkb, 0);
           } else {
-            tma_load_2d(w_dst, &map_w, bar, kb * p.bkb, c_tile * kTileC);
+            tma_load_2d(w_dst, &map_w, bar, wx + chunk * p.bkb, c_tile * kTileC);
           }
-          if (++chunk == p.cchunks) { chunk = 0; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
+          if (++chunk == p.cchunks) { chunk = 0; wx += p.cin; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
           if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1u; }
           if (res_due && kb + 1 == p.k_blocks && !residual(true)) { ok = false; break; }
         }
@@ -1073,17 +1076,20 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         if (!mbar_wait(smem_u32(&ctl.tempty[as]), aph ^ 1u, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + as * p.acc_stride;
+        int chunk = 0;
         for (int kb = 0; kb < p.k_blocks; ++kb) {
+          int nsteps = ksteps;
+          if (++chunk == p.cchunks) { chunk = 0; nsteps = p.tail_steps; }
           if (kb > 0 && !mbar_wait(smem_u32(&ctl.full[s]), ph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) { ok = false; break; }
           const uint32_t w_addr = tiles + s * stage_bytes;
           const uint32_t a_addr = p.wres ? tiles + p.wres_off + (uint32_t)kb * w_bytes : w_addr;
           uint64_t adesc = desc_hi | (uint64_t)((a_addr >> 4) & 0x3FFF);
           uint64_t bdesc = desc_hi | (uint64_t)(((w_addr + x_off) >> 4) & 0x3FFF);
           if constexpr (DUO) {
-            for (int k = 0; k < ksteps; ++k, adesc += 2, bdesc += 2)
+            for (int k = 0; k < nsteps; ++k, adesc += 2, bdesc += 2)
               mma_i8_2cta(d_tmem, adesc, bdesc, idesc, (kb | k) ? 1u : 0u);
           } else {
-            for (int k = 0; k < ksteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
+            for (int k = 0; k < nsteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
               mma_i8(d_tmem, adesc, bdesc, idesc, (kb | k) ? 1u : 0u);
           }
           // the accumulator's barrier first on the last K block: the epilogue is the one waiting
@@ -1151,7 +1157,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           }
           uint64_t adesc = desc_hi | (uint64_t)((a_addr >> 4) & 0x3FFF);
           uint64_t bdesc = desc_hi | (uint64_t)((b_addr >> 4) & 0x3FFF);
-          for (int k = 0; k < ksteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
+          const int nsteps = p.tail_steps != ksteps && b % p.cchunks == p.cchunks - 1 ? p.tail_steps : ksteps;
+          for (int k = 0; k < nsteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
             mma_i8(d_tmem, adesc, bdesc, idesc, (b | k) ? 1u : 0u);
           if (b == 0 && ni > 1) mbar_arrive(smem_u32(&ctl.tstart[as]));   // the overwriting MMA is on its way
           // the accumulator's barrier first on this issuer's last block: the epilogue is the one waiting
@@ -1432,7 +1439,7 @@ bool hq_conv_tc_init() {
 
 bool hq_conv_tc_supported(const ConvArgs& a) {
   if (a.in_bits != 8) return false;
-  if (a.cin % 32 != 0) return false;
+  if (a.cin % 16 != 0) return false;
   if (a.kh > 255 || a.kw > 255 || a.pad > 127 || a.stride > 8) return false;
   if ((long long)a.n * a.ho * a.wo >= (1ll << 31) - 256) return false;
   if ((long long)a.kh * a.kw * a.cin >= (1ll << 24)) return false;
@@ -1467,9 +1474,9 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.rev = h->tile_order ? 1 : 0;
   p.P = (int32_t)P; p.C = a.cout; p.howo = a.ho * a.wo; p.wo = a.wo;
   p.stride = a.stride; p.pad = a.pad; p.kw = a.kw;
-  p.bkb = (a.cin % 128 == 0) ? 128 : (a.cin % 64 == 0) ? 64 : 32;
-  p.cchunks = a.cin / p.bkb;
-  p.k_blocks = a.kh * a.kw * p.cchunks;
+  auto set_bkb = [&](int bkb) { p.bkb = bkb; p.cchunks = (a.cin + bkb - 1) / bkb; p.k_blocks = a.kh * a.kw * p.cchunks; };
+  p.cin = a.cin;
+  set_bkb(hq_conv_bkb(a.cin));
   p.c_tiles = (a.cout + kTileC - 1) / kTileC;
   if (p.c_tiles > h->sm_count) return HQ_ERR_UNSUPPORTED;
   // outputs and 8-bit residuals whose rows are 16-byte multiples travel through TMA
@@ -1491,7 +1498,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   int stages = 0, stage_bytes = 0, res_tile_bytes = 0, out_tile_bytes = 0, wres_bytes = 0;
   if (pair) {
     // 128-pixel tiles, two accumulator buffers (256 columns), K blocks of at most 64 bytes
-    if (p.bkb > 64) { p.bkb = 64; p.cchunks = a.cin / p.bkb; p.k_blocks = a.kh * a.kw * p.cchunks; }
+    if (p.bkb > 64) set_bkb(64);
     p.pt = pick_pt(P, p.c_tiles, 2 * h->sm_count, 128);
     wres_bytes = p.k_blocks * kTileC * p.bkb;
     p.wres = wres_bytes <= 16 * 1024 ? 1 : 0;              // short reductions: the weight slab stays resident
@@ -1507,9 +1514,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     if (stages < 3 || p.pt < 128) pair = false;
   }
   if (!pair) {
-    p.bkb = (a.cin % 128 == 0) ? 128 : (a.cin % 64 == 0) ? 64 : 32;
-    p.cchunks = a.cin / p.bkb;
-    p.k_blocks = a.kh * a.kw * p.cchunks;
+    set_bkb(hq_conv_bkb(a.cin));
     const int smem_budget = kSmemBudget;                // dynamic bytes after the 1024-byte alignment slack
     // staging: 8 warps x pt/2 pixel rows x 32 bytes (reserved at the 8-bit size), residual 2 or 4 x [pt][128]
     bool chosen = false;
@@ -1643,6 +1648,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     }
   }
   p.acc_stride = p.rtm ? 2 * p.pt : p.pt;
+  p.tail_steps = (a.cin - (p.cchunks - 1) * p.bkb + 31) >> 5;
   { const long long bound = k_total * 255 * 128; int bits = 0; while ((1LL << bits) <= bound) ++bits; p.acc_bits = bits; }
   p.tmem_cols = (uint32_t)(p.acc_stride << p.lg_bufs);  // 512 columns, or 256 for the smallest tile
   if (stages > kMaxStages) stages = kMaxStages;

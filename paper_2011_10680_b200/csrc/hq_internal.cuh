@@ -130,6 +130,13 @@ struct EltArgs {
   uint32_t* status;          // the handle's device status word (bounded waits report here), or NULL
 };
 
+// Bytes of K per stage of the tensor-core convolutions: the shortest power of two up to 128 that holds a tap's channels, else
+// 128 with the last block reaching past them (the copies fill zeros, the MMA steps beyond the channels are left out, and what
+// the weight box picks up of the next tap meets nothing).  An SM takes in one operand row per two cycles whatever its length, so
+// the rows have to be long: 3x3 over 96 channels in 32-byte rows 82 us, over 192 in 64-byte rows 42 us (35x35 and 17x17, 256
+// images); in 128-byte rows 58 and 36 us.  5x5 over 48 channels as a patch matrix (three launches) 161 us, fetched directly 135 us.
+inline int hq_conv_bkb(int cin) { return cin > 64 ? 128 : cin > 32 ? 64 : 32; }
+
 cudaError_t hq_launch_conv_cuda_core(const ConvArgs& a, cudaStream_t s);
 bool hq_conv_tc_init();
 bool hq_conv_tc_supported(const ConvArgs& a);

@@ -99,3 +99,34 @@ def test_fused_int32_stream_add_large_tiles():
     finally:
         net.close()
         hq.close()
+
+
+@pytest.mark.parametrize("path", [2, 4])
+@pytest.mark.parametrize("cfg", [
+    # n, h, w, cin, cout, k, stride, pad, bits, residual
+    (9, 20, 20, 48, 64, 5, 1, 2, 8, False),      # one 64-byte block per tap, 16 bytes of it past the channels
+    (9, 20, 20, 96, 96, 3, 1, 1, 8, False),      # 96 of 128
+    (5, 20, 20, 144, 192, 3, 2, 1, 8, False),    # a full block and 16 of 128
+    (9, 20, 20, 192, 256, 1, 1, 0, 8, True),     # tiled rows, residual
+    (12, 30, 30, 16, 128, 3, 1, 1, 8, False),    # half a 32-byte block
+    (4, 20, 20, 288, 256, 3, 1, 1, 8, False),    # long reduction, two-CTA shape on path 3
+    (9, 20, 20, 48, 64, 5, 1, 2, 4, False),      # widened 4-bit operands
+])
+def test_conv_channels_that_do_not_fill_a_block(cfg, path):
+    """K blocks that reach past the channels of a tap, in both tensor-core kernels."""
+    from oracle import hqref
+    from paper_2011_10680_b200 import binding, build
+    build.build()
+    n, h, w, cin, cout, k, stride, pad, bits, residual = cfg
+    case = inputs.conv_case(600, n, h, w, cin, cout, k, stride, pad, bits=bits, residual=residual, c_range=(38, 44))
+    ref = hqref.conv_case(case)
+    hq = binding.Handle(0)
+    try:
+        for p in ((2, 3) if path == 2 else (4,)):
+            hq.set_conv_path(p)
+            st, out = hq.conv_case(case)
+            assert st == binding.HQ_OK, binding.status_string(st)
+            hq.sync()
+            assert np.array_equal(out.cpu().numpy().view(ref.dtype).reshape(ref.shape), ref)
+    finally:
+        hq.close()
