@@ -170,7 +170,9 @@ struct hq_network {
   // ADD layers with an INT32 result that run behind the convolution producing their main operand (see plan_wide_adds):
   // the convolution's layer or -1; the REQUANT layer done along with it or -1; whether somebody else reads the sum
   std::vector<int32_t> wide_conv, wide_requant;
-  std::vector<char> wide_sum_read, run_by_add;   // run_by_add: conv / requant layers that such an ADD runs
+  std::vector<char> wide_sum_read, run_by_add;   // run_by_add: layers that such an ADD, or a CONCAT, runs
+  std::vector<int32_t> pool_branch;  // CONCAT layers: the branch whose 3x3 window sums are rescaled straight into it, or -1
+  std::vector<void*> concat_narrow;  // CONCAT layers: the narrow pairs of the 8- and 4-bit branches (owned)
   std::vector<char> tile_order;      // per conv / linear / concat layer: tensors walked from the last pixel to the first (see plan_tile_orders)
   void* scratch;                     // patch matrix of the lowered first layer (owned)
   size_t scratch_bytes;
@@ -257,12 +259,39 @@ static void plan_wide_adds(hq_network* net) {
   }
 }
 
+// A window-sum layer (3x3, stride 1, pad 1) of an 8-bit tensor that only a concatenation reads is rescaled straight into its
+// channels of the concatenated tensor; the INT32 sums are not stored (but with layer taps, which need every tensor).
+static void plan_pool_branches(hq_network* net) {
+  const int n = (int)net->layers.size();
+  net->pool_branch.assign(n, -1);
+  for (int i = 0; i < n; ++i) {
+    const hq_layer& l = net->layers[i];
+    if (l.op != HQ_OP_CONCAT) continue;
+    for (int k = 0, off = 0; k < l.n_in; off += net->outs[l.ins[k]].c, ++k) {
+      const int j = l.ins[k];
+      const hq_layer& sp = net->layers[j];
+      if (sp.op != HQ_OP_SUMPOOL || sp.pool_k != 3 || sp.pool_stride != 1 || sp.pool_pad != 1 || sp.in0 < 0) continue;
+      if (net->stored_wide[sp.in0] || !hq_sumpool_concat_applies(net->outs[sp.in0], net->outs[i], off)) continue;
+      int readers = 0;
+      for (int m = j + 1; m < n; ++m) {
+        const hq_layer& r = net->layers[m];
+        if (r.op == HQ_OP_CONCAT) { for (int q = 0; q < r.n_in; ++q) readers += r.ins[q] == j; }
+        else readers += (r.in0 == j) + (((r.op == HQ_OP_CONV || r.op == HQ_OP_ADD) && r.in1 == j) ? 1 : 0);
+      }
+      if (readers != 1 || net->pool_branch[i] >= 0) continue;
+      net->pool_branch[i] = k;
+      net->run_by_add[j] = 1;
+    }
+  }
+}
+
 // Kernels of one pass: one per layer, plus the helpers of convolutions that run in a lowered form.
 static void count_launches(hq_network* net) {
   net->launches = (int32_t)net->layers.size();
   for (size_t i = 0; i < net->layers.size(); ++i) {
     const hq_layer& l = net->layers[i];
     if (net->run_by_add[i]) { net->launches -= 1; continue; }
+    if (l.op == HQ_OP_CONCAT && net->pool_branch[i] >= 0) net->launches += 1;
     if (l.op != HQ_OP_CONV) continue;
     const hq_conv_desc& d = l.conv;
     const hq_tensor& o = net->outs[i];
@@ -638,7 +667,21 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
       if (hq_launch_residual_narrow(l.rescale1.b, l.rescale1.c, net->outs[l.in1].is_signed, ch, buf1, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
     }
   }
-  if (st == HQ_OK) { plan_wide_adds(net); plan_tile_orders(net); count_launches(net); }
+  if (st == HQ_OK) { plan_wide_adds(net); plan_pool_branches(net); plan_tile_orders(net); count_launches(net); }
+  // narrow pairs of the concatenations' stored branches (a one-off search per channel)
+  net->concat_narrow.assign(n_layers, nullptr);
+  for (int i = 0; st == HQ_OK && i < n_layers; ++i) {
+    const hq_layer& l = net->layers[i];
+    if (l.op != HQ_OP_CONCAT) continue;
+    hq_tensor br[HQ_CONCAT_MAX_BRANCHES];
+    for (int k = 0; k < l.n_in; ++k) br[k] = net->outs[l.ins[k]];
+    hq_tensor o = net->outs[i];
+    void* buf = net_alloc(net, (size_t)o.c * 16, i);
+    if (!buf) { st = HQ_ERR_WORKSPACE; break; }
+    if (cudaMemsetAsync(buf, 0, (size_t)o.c * 16, nullptr) != cudaSuccess ||
+        hq_concat_requant_planned(h, l.n_in, br, l.rescales, l.relu, l.qmin, l.qmax, &o, nullptr, ConcatPlan{-1, buf, true}) != HQ_OK) continue;   // (a call the kernels decline is declined when it runs)
+    net->concat_narrow[i] = buf;
+  }
   if (st == HQ_OK && cudaDeviceSynchronize() != cudaSuccess) st = HQ_ERR_CUDA;
   if (st != HQ_OK) { hq_network_destroy(net); return st; }
   *out = net;
@@ -715,7 +758,13 @@ static hq_status run_layers(hq_network* net, const hq_tensor* images, hq_tensor*
         for (int k = 0; k < l.n_in; ++k) br[k] = net->outs[l.ins[k]];
         const int32_t callers_order = h->tile_order;
         h->tile_order = net->tile_order[i];
-        st = hq_concat_requant(h, l.n_in, br, l.rescales, l.relu, l.qmin, l.qmax, &o, s);
+        const int pool = fuse ? net->pool_branch[i] : -1;
+        if (pool >= 0) {
+          int off = 0;
+          for (int k = 0; k < pool; ++k) off += br[k].c;
+          st = hq_launch_sumpool_concat(h, net->outs[net->layers[l.ins[pool]].in0], l.rescales[pool], l.relu, l.qmin, l.qmax, o, off, s);
+        }
+        if (st == HQ_OK) st = hq_concat_requant_planned(h, l.n_in, br, l.rescales, l.relu, l.qmin, l.qmax, &o, s, ConcatPlan{pool, net->concat_narrow[i], false});
         h->tile_order = callers_order;
         break;
       }

@@ -49,6 +49,7 @@ __global__ void __launch_bounds__(128) concat_narrow_kernel(const __grid_constan
   int4 res = make_int4(0, 0, 0, 0);
   if (a.br[i].bits != 32) {
     const int k = oc - a.br[i].ch_off;
+    if (k < 0 || k >= a.br[i].ch) return;              // channels of a branch that is not part of this call
     const long long b = a.br[i].b[k];
     const int c = a.br[i].c[k];
     const int r_lo = a.br[i].is_signed ? -128 : 0;
@@ -488,6 +489,11 @@ inline bool al16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 extern "C" hq_status hq_concat_requant(hq_handle* h, int32_t n_branches, const hq_tensor* branches,
                                        const hq_dyadic* rescale, int32_t relu, int32_t qmin, int32_t qmax,
                                        hq_tensor* out, void* stream) {
+  return hq_concat_requant_planned(h, n_branches, branches, rescale, relu, qmin, qmax, out, stream, ConcatPlan{-1, nullptr, false});
+}
+
+hq_status hq_concat_requant_planned(hq_handle* h, int32_t n_branches, const hq_tensor* branches, const hq_dyadic* rescale, int32_t relu,
+                                    int32_t qmin, int32_t qmax, hq_tensor* out, void* stream, const ConcatPlan& plan) {
   if (!h || !branches || !rescale || !out || !out->data) return HQ_ERR_INVALID_ARG;
   if (n_branches < 1 || n_branches > HQ_CONCAT_MAX_BRANCHES) return HQ_ERR_INVALID_ARG;
   if (out->bits != 8 && out->bits != 4) return HQ_ERR_INVALID_ARG;
@@ -512,6 +518,7 @@ extern "C" hq_status hq_concat_requant(hq_handle* h, int32_t n_branches, const h
     if (t.bits == 4 && (t.c & 1)) return HQ_ERR_INVALID_ARG;
     if (out->bits == 4 && (t.c & 1)) return HQ_ERR_UNSUPPORTED;   // a byte of the output would span two branches
     if (!al16(t.data)) return HQ_ERR_ALIGNMENT;
+    if (i == plan.skip) { off += t.c; continue; }
     const bool four = t.c % 4 == 0 && out->c % 2 == 0;
     int pieces = 1;
     if (four && t.c > 1024) {
@@ -564,8 +571,14 @@ extern "C" hq_status hq_concat_requant(hq_handle* h, int32_t n_branches, const h
   // launch on the same stream, repaid by the cheaper arithmetic).
   a.narrow = nullptr;
   bool any_narrow = false;
-  for (int i = 0; i < n_branches; ++i) any_narrow = any_narrow || branches[i].bits != 32;
-  if (any_narrow && h->narrow_pairs && out->c <= 2 * kNarrowChannels && a.pixels * out->c >= (1ll << 22)) {
+  for (int i = 0; i < n_branches; ++i) any_narrow = any_narrow || (i != plan.skip && branches[i].bits != 32);
+  if (plan.prepare) {
+    if (any_narrow) concat_narrow_kernel<<<(out->c + 3) / 4, 128, 0, (cudaStream_t)stream>>>(a, (int4*)plan.narrow);
+    return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
+  }
+  if (plan.narrow) {
+    a.narrow = any_narrow ? (const int4*)plan.narrow : nullptr;
+  } else if (any_narrow && h->narrow_pairs && out->c <= 2 * kNarrowChannels && a.pixels * out->c >= (1ll << 22)) {
     int4* tab = (int4*)h->narrow_pairs;
     concat_narrow_kernel<<<(out->c + 3) / 4, 128, 0, (cudaStream_t)stream>>>(a, tab);
     if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;

@@ -178,6 +178,16 @@ cudaError_t hq_launch_expire_wait(uint32_t* status, int budget_ms, cudaStream_t 
 cudaError_t hq_launch_pack4(const void* in, long long values, void* out, int sm_count, cudaStream_t s);
 // Grow the handle's scratch buffer (not allowed while `s` is capturing).
 hq_status hq_reserve_workspace(hq_handle* h, size_t bytes, cudaStream_t s);
+// hq_concat_requant as a network runs it: `skip` is a branch written by somebody else (-1: none); `narrow` the branches' narrow
+// pairs, out->c x 16 bytes (NULL: a large call works them out itself), only computed with `prepare`.
+struct ConcatPlan { int32_t skip; void* narrow; bool prepare; };
+hq_status hq_concat_requant_planned(hq_handle* h, int32_t n_branches, const hq_tensor* branches, const hq_dyadic* rescale, int32_t relu,
+                                    int32_t qmin, int32_t qmax, hq_tensor* out, void* stream, const ConcatPlan& plan);
+// 3x3 / stride 1 / pad 1 window sums of an 8-bit tensor rescaled by `r` straight into channels [ch_off, ch_off + in->c) of an
+// 8-bit concatenation (sumpool.cu); false: the shapes do not allow it.
+bool hq_sumpool_concat_applies(const hq_tensor& in, const hq_tensor& out, int32_t ch_off);
+hq_status hq_launch_sumpool_concat(hq_handle* h, const hq_tensor& in, hq_dyadic r, int32_t relu, int32_t qmin, int32_t qmax,
+                                   const hq_tensor& out, int32_t ch_off, cudaStream_t s);
 cudaError_t hq_launch_residual_add(const EltArgs& a, int sm_count, cudaStream_t s);
 cudaError_t hq_launch_avgpool(const void* in, int n, int h, int w, int ch, int in_bits, int in_signed,
                               const int32_t* b, const int32_t* c, int qmin, int qmax,

@@ -152,7 +152,110 @@ __global__ void __launch_bounds__(256) sumpool3_rows_kernel(const __grid_constan
   }
 }
 
+// The same walk over an 8-bit input, ending in the concatenation of the module: the sums are rescaled by their branch's dyadic
+// pair (Appendix E, dn(S_i / (9 S_a))) and written to their channel range of the output row.  The INT32 tensor between the
+// two (four bytes written and read per value) goes away: what is left is one byte in (three reads of a byte from L1 / L2) and
+// one byte out per value.
+struct SumCatArgs {
+  SumPoolArgs s;
+  const int32_t* b; const int32_t* c;
+  unsigned char* out; int32_t out_ch, ch_off, lo, hi, sat;    // sat: the clamp is that of u8
+};
+template <int SIGNED>
+__global__ void __launch_bounds__(256) sumpool3_concat_kernel(const __grid_constant__ SumCatArgs p, int strip_rows, int strips) {
+  hq_pdl_entry();
+  const SumPoolArgs& a = p.s;
+  const int cg = a.ch >> 2;
+  const int col = blockIdx.x * 256 + threadIdx.x;
+  if (col >= a.w * cg) return;
+  const int ow = col / cg, g = col - ow * cg;
+  const int img = blockIdx.y / strips, strip = blockIdx.y - img * strips;
+  const int r0 = strip * strip_rows, r1 = min(r0 + strip_rows, a.h);
+  const bool left = ow > 0, right = ow + 1 < a.w;
+  const long long img_row0 = (long long)img * a.h;
+  const unsigned* __restrict__ in = (const unsigned*)a.in;
+  constexpr unsigned kBias = SIGNED ? 0x80808080u : 0u;
+  int b[4], c[4];
+  long long add[4];
+  bool fast = true;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    b[i] = __ldg(p.b + 4 * g + i); c[i] = __ldg(p.c + 4 * g + i);
+    add[i] = (1LL << (c[i] - 1)) - (SIGNED ? 9LL * 128 * b[i] : 0);
+    fast = fast && c[i] >= 32;
+  }
+  auto hsum = [&](int ih, unsigned& lo, unsigned& hi) {
+    unsigned v0 = 0, v1 = 0, v2 = 0;
+    if (ih >= 0 && ih < a.h) {
+      const unsigned* row = in + ((img_row0 + ih) * a.w + ow) * cg + g;
+      v1 = __ldg(row);
+      if (left) v0 = __ldg(row - cg);
+      if (right) v2 = __ldg(row + cg);
+    }
+    v0 ^= kBias; v1 ^= kBias; v2 ^= kBias;
+    lo = (v0 & 0x00FF00FFu) + (v1 & 0x00FF00FFu) + (v2 & 0x00FF00FFu);
+    hi = ((v0 >> 8) & 0x00FF00FFu) + ((v1 >> 8) & 0x00FF00FFu) + ((v2 >> 8) & 0x00FF00FFu);
+  };
+  unsigned char* outp = p.out + ((img_row0 + r0) * a.w + ow) * p.out_ch + p.ch_off + 4 * g;
+  const long long out_step = (long long)a.w * p.out_ch;
+  unsigned l0, h0, l1, h1;
+  hsum(r0 - 1, l0, h0);
+  hsum(r0, l1, h1);
+#pragma unroll 4
+  for (int oh = r0; oh < r1; ++oh, outp += out_step) {
+    unsigned l2, h2;
+    hsum(oh + 1, l2, h2);
+    const unsigned lo = l0 + l1 + l2, hi = h0 + h1 + h2;
+    const int q[4] = {(int)(lo & 0xFFFFu), (int)(hi & 0xFFFFu), (int)(lo >> 16), (int)(hi >> 16)};
+    int y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      long long t;
+      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(q[i]), "r"(b[i]), "l"(add[i]));     // (the bias of signed bytes is in `add`)
+      if (fast) y[i] = (int)(t >> 32) >> (c[i] - 32);
+      else { t >>= c[i]; y[i] = (int)(t < -256 ? -256 : t > 255 ? 255 : t); }
+    }
+    unsigned w23, w;
+    if (!p.sat) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) y[i] = min(max(y[i], p.lo), p.hi) & 0xFF;
+    }
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w23) : "r"(y[3]), "r"(y[2]), "r"(0));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(y[1]), "r"(y[0]), "r"(w23));
+    *(unsigned*)outp = w;
+    l0 = l1; h0 = h1; l1 = l2; h1 = h2;
+  }
+}
+
+// strips of rows: long enough that the two extra input rows per strip matter little, short enough to fill the GPU
+int strip_rows_for(int n, int h, long long cols, int sm_count) {
+  int rows = 8;
+  while (rows > 2 && (cols + 255) / 256 * n * ((h + rows - 1) / rows) < 16LL * sm_count) rows >>= 1;
+  return rows;
+}
+
 }  // namespace
+
+bool hq_sumpool_concat_applies(const hq_tensor& in, const hq_tensor& out, int32_t ch_off) {
+  return in.bits == 8 && out.bits == 8 && in.c % 4 == 0 && out.c % 4 == 0 && ch_off % 4 == 0 && in.h == out.h && in.w == out.w &&
+         (long long)in.n * ((in.h + 1) / 2) <= 65535;
+}
+
+hq_status hq_launch_sumpool_concat(hq_handle* h, const hq_tensor& in, hq_dyadic r, int32_t relu, int32_t qmin, int32_t qmax,
+                                   const hq_tensor& out, int32_t ch_off, cudaStream_t s) {
+  if (!r.b || !r.c) return HQ_ERR_INVALID_ARG;
+  SumCatArgs p{};
+  p.s.in = in.data; p.s.n = in.n; p.s.h = in.h; p.s.w = in.w; p.s.ch = in.c;
+  p.b = r.b; p.c = r.c; p.out = (unsigned char*)out.data; p.out_ch = out.c; p.ch_off = ch_off;
+  p.lo = relu ? (qmin > 0 ? qmin : 0) : qmin; p.hi = qmax;
+  p.sat = p.lo == 0 && p.hi == 255 ? 1 : 0;
+  const long long cols = (long long)in.w * (in.c / 4);
+  const int rows = strip_rows_for(in.n, in.h, cols, h->sm_count), strips = (in.h + rows - 1) / rows;
+  const dim3 grid((unsigned)((cols + 255) / 256), (unsigned)(in.n * strips));
+  if (in.is_signed) hq_launch_pdl(sumpool3_concat_kernel<1>, grid, 256, 0, s, p, rows, strips);
+  else hq_launch_pdl(sumpool3_concat_kernel<0>, grid, 256, 0, s, p, rows, strips);
+  return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
+}
 
 extern "C" hq_status hq_sumpool(hq_handle* h, const hq_tensor* in, int32_t k, int32_t stride, int32_t pad,
                                 hq_tensor* out, void* stream) {
@@ -172,10 +275,8 @@ extern "C" hq_status hq_sumpool(hq_handle* h, const hq_tensor* in, int32_t k, in
   a.vec = in->c % 4 != 0 ? 0 : in->bits == 32 ? 1 : in->bits == 8 ? 2 : 0;
   if (a.n == 0) return HQ_OK;
   if (a.vec && k == 3 && stride == 1 && pad == 1) {
-    // strips of rows: long enough that the two extra input rows per strip matter little, short enough to fill the GPU
     const long long cols3 = (long long)a.w * (a.ch / 4);
-    int strip_rows = 8;
-    while (strip_rows > 2 && (cols3 + 255) / 256 * a.n * ((a.h + strip_rows - 1) / strip_rows) < 16LL * h->sm_count) strip_rows >>= 1;
+    const int strip_rows = strip_rows_for(a.n, a.h, cols3, h->sm_count);
     const int strips = (a.h + strip_rows - 1) / strip_rows;
     if ((cols3 + 255) / 256 <= 0x7fffffffLL && (long long)a.n * strips <= 65535) {
       const dim3 grid3((unsigned)((cols3 + 255) / 256), (unsigned)(a.n * strips));

@@ -130,3 +130,31 @@ def test_conv_channels_that_do_not_fill_a_block(cfg, path):
             assert np.array_equal(out.cpu().numpy().view(ref.dtype).reshape(ref.shape), ref)
     finally:
         hq.close()
+
+
+@pytest.mark.parametrize("signed,shift", [(False, None), (True, None), (True, 28), (False, 31)])
+def test_fused_pooling_branch(signed, shift):
+    """Graph replay rescales the window sums of a pooling branch straight into the concatenation: unsigned and signed module
+    inputs, shifts on both sides of 32, a branch at either end; ragged last strip (9 rows).  Oracle through the layer taps."""
+    from paper_2011_10680_b200 import binding, build
+    from test_gpu_parity import run_network_and_compare
+    build.build()
+    bd = inputs._Builder(31)
+    bd.scale[-1], bd.shape[-1], bd.bits[-1] = 2.0 ** -4, (20, 20, 3), 8
+    x = bd.conv(-1, 48, 3, 2, 0, 8, relu=not signed, out_bits=8, out_signed=signed)
+    for last in (True, False):
+        m = bd.conv(x, 36, 1, 1, 0, 8, relu=True, out_bits=8)
+        p = bd.sumpool(x, 3, 1, 1)
+        x = bd.concat([m, p] if last else [p, m])
+        if shift:
+            k = bd.layers[x]["ins"].index(p)
+            bd.layers[x]["cs"][k][::3] = shift
+    x = bd.avgpool(x)
+    bd.conv(x, 16, 1, 1, 0, 8, relu=False, out_bits=32, op="linear")
+    t = dict(layers=bd.layers, image_hw=20, classes=16, depth=0, conv_bits=[8], shapes=[bd.shape[i] for i in range(len(bd.layers))],
+             bits=[bd.bits[i] for i in range(len(bd.layers))])
+    hq = binding.Handle(0)
+    try:
+        run_network_and_compare(hq, t, batch=3, seed=6)
+    finally:
+        hq.close()
