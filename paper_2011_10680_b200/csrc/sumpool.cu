@@ -161,70 +161,82 @@ struct SumCatArgs {
   const int32_t* b; const int32_t* c;
   unsigned char* out; int32_t out_ch, ch_off, lo, hi, sat;    // sat: the clamp is that of u8
 };
-template <int SIGNED>
-__global__ void __launch_bounds__(256) sumpool3_concat_kernel(const __grid_constant__ SumCatArgs p, int strip_rows, int strips) {
-  hq_pdl_entry();
+// Bound by the integer pipe: about 12 instructions per value with running pointers, byte permutes and the form of the shift chosen
+// outside the loop (256 x 35x35x288: 114 us, 127 us with the address and bounds arithmetic of sumpool3_rows_kernel, 31 instructions a value).
+template <int SIGNED, bool FAST>
+__device__ __forceinline__ void sumpool3_concat_column(const SumCatArgs& p, int ow, int g, int img, int r0, int r1) {
   const SumPoolArgs& a = p.s;
   const int cg = a.ch >> 2;
-  const int col = blockIdx.x * 256 + threadIdx.x;
-  if (col >= a.w * cg) return;
-  const int ow = col / cg, g = col - ow * cg;
-  const int img = blockIdx.y / strips, strip = blockIdx.y - img * strips;
-  const int r0 = strip * strip_rows, r1 = min(r0 + strip_rows, a.h);
   const bool left = ow > 0, right = ow + 1 < a.w;
-  const long long img_row0 = (long long)img * a.h;
-  const unsigned* __restrict__ in = (const unsigned*)a.in;
+  const long long pixel = ((long long)img * a.h + r0) * a.w + ow;
   constexpr unsigned kBias = SIGNED ? 0x80808080u : 0u;
-  int b[4], c[4];
+  int b[4], sh[4];
   long long add[4];
-  bool fast = true;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    b[i] = __ldg(p.b + 4 * g + i); c[i] = __ldg(p.c + 4 * g + i);
-    add[i] = (1LL << (c[i] - 1)) - (SIGNED ? 9LL * 128 * b[i] : 0);
-    fast = fast && c[i] >= 32;
+    const int c = __ldg(p.c + 4 * g + i);
+    b[i] = __ldg(p.b + 4 * g + i); sh[i] = FAST ? c - 32 : c;
+    add[i] = (1LL << (c - 1)) - (SIGNED ? 9LL * 128 * b[i] : 0);       // the bias of signed bytes comes off here
   }
-  auto hsum = [&](int ih, unsigned& lo, unsigned& hi) {
+  const unsigned* row = (const unsigned*)a.in + (pixel - a.w) * cg + g;      // the row above the strip (read only where it exists)
+  const long long row_step = (long long)a.w * cg;
+  int ih = r0 - 1;
+  // the row's three-pixel sum as (bytes 0, 2) and (bytes 1, 3) in 16-bit lanes
+  auto hsum = [&](unsigned& even, unsigned& odd) {
+    const bool in = (unsigned)ih < (unsigned)a.h;
     unsigned v0 = 0, v1 = 0, v2 = 0;
-    if (ih >= 0 && ih < a.h) {
-      const unsigned* row = in + ((img_row0 + ih) * a.w + ow) * cg + g;
-      v1 = __ldg(row);
-      if (left) v0 = __ldg(row - cg);
-      if (right) v2 = __ldg(row + cg);
-    }
-    v0 ^= kBias; v1 ^= kBias; v2 ^= kBias;
-    lo = (v0 & 0x00FF00FFu) + (v1 & 0x00FF00FFu) + (v2 & 0x00FF00FFu);
-    hi = ((v0 >> 8) & 0x00FF00FFu) + ((v1 >> 8) & 0x00FF00FFu) + ((v2 >> 8) & 0x00FF00FFu);
+    if (in) v1 = __ldg(row);
+    if (in && left) v0 = __ldg(row - cg);
+    if (in && right) v2 = __ldg(row + cg);
+    if (SIGNED) { v0 ^= kBias; v1 ^= kBias; v2 ^= kBias; }
+    even = __byte_perm(v0, 0u, 0x4240) + __byte_perm(v1, 0u, 0x4240) + __byte_perm(v2, 0u, 0x4240);
+    odd = __byte_perm(v0, 0u, 0x4341) + __byte_perm(v1, 0u, 0x4341) + __byte_perm(v2, 0u, 0x4341);
+    row += row_step; ++ih;
   };
-  unsigned char* outp = p.out + ((img_row0 + r0) * a.w + ow) * p.out_ch + p.ch_off + 4 * g;
+  unsigned char* out = p.out + pixel * p.out_ch + p.ch_off + 4 * g;
   const long long out_step = (long long)a.w * p.out_ch;
-  unsigned l0, h0, l1, h1;
-  hsum(r0 - 1, l0, h0);
-  hsum(r0, l1, h1);
+  unsigned e0, o0, e1, o1;
+  hsum(e0, o0);
+  hsum(e1, o1);
 #pragma unroll 4
-  for (int oh = r0; oh < r1; ++oh, outp += out_step) {
-    unsigned l2, h2;
-    hsum(oh + 1, l2, h2);
-    const unsigned lo = l0 + l1 + l2, hi = h0 + h1 + h2;
-    const int q[4] = {(int)(lo & 0xFFFFu), (int)(hi & 0xFFFFu), (int)(lo >> 16), (int)(hi >> 16)};
+  for (int n = r1 - r0; n > 0; --n) {
+    unsigned e2, o2;
+    hsum(e2, o2);
+    const unsigned even = e0 + e1 + e2, odd = o0 + o1 + o2;
+    const int q[4] = {(int)(even & 0xFFFFu), (int)(odd & 0xFFFFu), (int)(even >> 16), (int)(odd >> 16)};
     int y[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       long long t;
-      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(q[i]), "r"(b[i]), "l"(add[i]));     // (the bias of signed bytes is in `add`)
-      if (fast) y[i] = (int)(t >> 32) >> (c[i] - 32);
-      else { t >>= c[i]; y[i] = (int)(t < -256 ? -256 : t > 255 ? 255 : t); }
+      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(q[i]), "r"(b[i]), "l"(add[i]));
+      if (FAST) y[i] = (int)(t >> 32) >> sh[i];
+      else { t >>= sh[i]; y[i] = (int)(t < -256 ? -256 : t > 255 ? 255 : t); }
     }
-    unsigned w23, w;
     if (!p.sat) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) y[i] = min(max(y[i], p.lo), p.hi) & 0xFF;
     }
+    unsigned w23, w;
     asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w23) : "r"(y[3]), "r"(y[2]), "r"(0));
     asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(y[1]), "r"(y[0]), "r"(w23));
-    *(unsigned*)outp = w;
-    l0 = l1; h0 = h1; l1 = l2; h1 = h2;
+    *(unsigned*)out = w;
+    out += out_step;
+    e0 = e1; o0 = o1; e1 = e2; o1 = o2;
   }
+}
+template <int SIGNED>
+__global__ void __launch_bounds__(256) sumpool3_concat_kernel(const __grid_constant__ SumCatArgs p, int strip_rows, int strips) {
+  hq_pdl_entry();
+  const int cg = p.s.ch >> 2;
+  const int col = blockIdx.x * 256 + threadIdx.x;
+  if (col >= p.s.w * cg) return;
+  const int ow = col / cg, g = col - ow * cg;
+  const int img = blockIdx.y / strips, r0 = (blockIdx.y - img * strips) * strip_rows, r1 = min(r0 + strip_rows, p.s.h);
+  bool fast = true;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) fast = fast && __ldg(p.c + 4 * g + i) >= 32;
+  if (__all_sync(__activemask(), fast)) sumpool3_concat_column<SIGNED, true>(p, ow, g, img, r0, r1);
+  else sumpool3_concat_column<SIGNED, false>(p, ow, g, img, r0, r1);
 }
 
 // strips of rows: long enough that the two extra input rows per strip matter little, short enough to fill the GPU
@@ -250,7 +262,10 @@ hq_status hq_launch_sumpool_concat(hq_handle* h, const hq_tensor& in, hq_dyadic 
   p.lo = relu ? (qmin > 0 ? qmin : 0) : qmin; p.hi = qmax;
   p.sat = p.lo == 0 && p.hi == 255 ? 1 : 0;
   const long long cols = (long long)in.w * (in.c / 4);
-  const int rows = strip_rows_for(in.n, in.h, cols, h->sm_count), strips = (in.h + rows - 1) / rows;
+  int rows = strip_rows_for(in.n, in.h, cols, h->sm_count);
+  // (arithmetic weighs more here than in the plain sums: strips twice as long where they still make 16 blocks per SM)
+  if (rows == 8 && (cols + 255) / 256 * in.n * ((in.h + 17) / 18) >= 16LL * h->sm_count) rows = in.h <= 18 ? in.h : 18;
+  const int strips = (in.h + rows - 1) / rows;
   const dim3 grid((unsigned)((cols + 255) / 256), (unsigned)(in.n * strips));
   if (in.is_signed) hq_launch_pdl(sumpool3_concat_kernel<1>, grid, 256, 0, s, p, rows, strips);
   else hq_launch_pdl(sumpool3_concat_kernel<0>, grid, 256, 0, s, p, rows, strips);
