@@ -453,6 +453,7 @@ static hq_status residual_add_impl(hq_handle* h, const hq_tensor* main_t, hq_dya
       return HQ_ERR_CUDA;
     a.m_narrow = base;
     a.r_narrow = base1;
+    a.narrow_fresh = 1;
   }
   return hq_launch_residual_add(a, h->sm_count, s) == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }

@@ -108,6 +108,7 @@ struct TcParams {
   const int32_t* bias; const int32_t* b; const int32_t* c;
   const void* res; int32_t res_bits, res_signed; const int32_t* rb; const int32_t* rc;
   const int4* res_narrow;   // optional per-channel {m, a, s, valid} from residual_narrow_kernel
+  int32_t w_fresh;          // 1: the weights are written by the kernel launched just before this one
   int32_t narrow_fresh;     // 1: the pairs are written by the kernel launched just before this one
   int32_t relu, qmin, qmax;
   void* out; int32_t out_bits;
@@ -879,6 +880,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       int ow = px_first - img * p.howo - oh * p.wo;
       const int step = p_step * p.pt;
       const int d_img = step / p.howo, d_oh = (step - d_img * p.howo) / p.wo, d_ow = step - d_img * p.howo - d_oh * p.wo;
+      if (p.w_fresh) asm volatile("griddepcontrol.wait;" ::: "memory");
       if (p.wres) {              // the channel tile's weights for every K block, once
         const uint32_t bar = smem_u32(&ctl.wfull);
         mbar_expect_tx(bar, (uint32_t)p.k_blocks * w_bytes);
@@ -1376,6 +1378,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 struct NarrowJob { const int32_t* rb; const int32_t* rc; int is_signed; int4* out; };
 
 __global__ void __launch_bounds__(128) residual_narrow_kernel(NarrowJob j0, NarrowJob j1, int n) {
+  hq_pdl_entry();
   // one warp per channel: lane l checks the inputs l, l + 32, ... for both candidate multipliers; warps past the
   // first n channels serve the second job (the other operand of an element-wise call), if there is one
   int ch = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1662,7 +1665,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.bias = a.bias; p.b = a.b; p.c = a.c;
   p.res = a.res; p.res_bits = a.res_bits; p.res_signed = a.res_signed; p.rb = a.rb; p.rc = a.rc;
   p.res_narrow = (a.res && a.res_bits == 8) ? (const int4*)a.res_narrow : nullptr;
-  p.narrow_fresh = a.res_narrow_fresh;
+  p.narrow_fresh = a.res_narrow_fresh; p.w_fresh = a.wgt_fresh;
   p.relu = a.relu; p.qmin = a.qmin; p.qmax = a.qmax;
   p.out = a.out; p.out_bits = a.out_bits; p.out_signed = a.out_signed;
   if (a.wide) {
@@ -1767,7 +1770,7 @@ cudaError_t hq_launch_residual_narrow2(const int32_t* b0, const int32_t* c0, int
   if (channels <= 0) return cudaSuccess;
   const NarrowJob j0{b0, c0, signed0, (int4*)out0}, j1{b1, c1, signed1, (int4*)out1};
   const int warps = out1 ? 2 * channels : channels;
-  residual_narrow_kernel<<<(warps + 3) / 4, 128, 0, s>>>(j0, j1, channels);
+  hq_launch_pdl(residual_narrow_kernel, (warps + 3) / 4, 128, 0, s, j0, j1, channels);
   return cudaGetLastError();
 }
 

@@ -394,28 +394,23 @@ __device__ __forceinline__ bool ebar_wait(unsigned bar, unsigned parity, EltPipe
   return true;
 }
 
+// One chunk of the pipeline below into its slot (one thread).
+template <bool RES>
+__device__ __forceinline__ void requant8_issue(const EltArgs& a, long long chunk, unsigned slot, EltPipe* pipe, unsigned char* stage) {
+  constexpr unsigned chunk_bytes = (RES ? 4 : 8) * 256 * 4, stage_bytes = RES ? 2u * chunk_bytes : chunk_bytes;
+  const unsigned bar = esmem(&pipe->full[slot]);
+  ebar_expect_tx(bar, stage_bytes);
+  ebulk_load(esmem(stage + slot * stage_bytes), (const unsigned char*)a.main_t + chunk * chunk_bytes, chunk_bytes, bar);
+  if (RES) ebulk_load(esmem(stage + slot * stage_bytes + chunk_bytes), (const unsigned char*)a.res + chunk * chunk_bytes, chunk_bytes, bar);
+}
+
 template <bool RES, bool MSIGNED, bool RSIGNED, bool OUT4, bool SLOW, int SATP, bool NARROW>
 __device__ __forceinline__ void requant8_chunks(const EltArgs& a, const Dy8 (&m)[4], const Dy8 (&r)[4], int wx, long long total,
-                                                int lo, int hi, EltPipe* pipe, unsigned char* stage) {
+                                                int lo, int hi, EltPipe* pipe, unsigned char* stage, unsigned issued) {
   constexpr int T = 256, U = RES ? 4 : 8;
   constexpr unsigned chunk_bytes = U * T * 4, stage_bytes = RES ? 2u * chunk_bytes : chunk_bytes;
   const int tid = threadIdx.x, lane = tid & 31;
   const long long n_chunks = total / (U * T);
-  const unsigned char* mg = (const unsigned char*)a.main_t;
-  const unsigned char* rg = (const unsigned char*)a.res;
-  auto issue = [&](long long chunk, unsigned slot) {
-    const unsigned bar = esmem(&pipe->full[slot]);
-    ebar_expect_tx(bar, stage_bytes);
-    ebulk_load(esmem(stage + slot * stage_bytes), mg + chunk * chunk_bytes, chunk_bytes, bar);
-    if (RES) ebulk_load(esmem(stage + slot * stage_bytes + chunk_bytes), rg + chunk * chunk_bytes, chunk_bytes, bar);
-  };
-  unsigned issued = 0;                                   // thread 0: chunks handed to the copy engine so far
-  if (tid == 0) {
-    for (int k = 0; k < kEltStages - 1; ++k) {
-      const long long chunk = blockIdx.x + (long long)k * gridDim.x;
-      if (chunk < n_chunks) { issue(chunk, (unsigned)k); ++issued; }
-    }
-  }
   unsigned it = 0;
   bool ok = true;
   for (long long chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x, ++it) {
@@ -426,7 +421,7 @@ __device__ __forceinline__ void requant8_chunks(const EltArgs& a, const Dy8 (&m)
         const unsigned it2 = it + kEltStages - 1, s2 = it2 % kEltStages, use = it2 / kEltStages;
         // the slot's previous use must have been read by every warp (a fresh barrier passes at once)
         ok = ebar_wait(esmem(&pipe->empty[s2]), (use & 1u) ^ 1u, pipe, a.status);
-        if (ok) { issue(nxt, s2); ++issued; }
+        if (ok) { requant8_issue<RES>(a, nxt, s2, pipe, stage); ++issued; }
       }
     }
     unsigned w = 1u;
@@ -466,7 +461,7 @@ __device__ __forceinline__ void requant8_chunks(const EltArgs& a, const Dy8 (&m)
 
 template <bool RES, bool MSIGNED, bool RSIGNED, bool OUT4, int SATP>
 __global__ void __launch_bounds__(256, RES ? 3 : 5) requant8_staged_kernel(EltArgs a, int words, int lo, int hi) {
-  hq_pdl_entry();
+  if (!a.narrow_fresh) hq_pdl_entry();
   extern __shared__ __align__(128) unsigned char stage[];
   __shared__ EltPipe pipe;
   const int tid = threadIdx.x;
@@ -478,6 +473,16 @@ __global__ void __launch_bounds__(256, RES ? 3 : 5) requant8_staged_kernel(EltAr
   __syncthreads();
   const int wx = tid & (words - 1);           // word (4 channels) of the pixel; words is a power of two <= 256
   const long long total = a.pixels * words;
+  unsigned issued = 0;                                   // thread 0: chunks handed to the copy engine so far
+  if (tid == 0) {
+    for (int k = 0; k < kEltStages - 1; ++k) {
+      const long long chunk = blockIdx.x + (long long)k * gridDim.x;
+      if (chunk < total / (256 * (RES ? 4 : 8))) { requant8_issue<RES>(a, chunk, (unsigned)k, &pipe, stage); ++issued; }
+    }
+  }
+  // The launch just before is the search for narrow pairs, which itself waited for everything before it: the operands may be
+  // fetched while it runs, only the pairs (and the output, whose readers it waited for) have to wait.
+  if (a.narrow_fresh) hq_pdl_entry();
   Dy8 m[4], r[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -514,14 +519,14 @@ __global__ void __launch_bounds__(256, RES ? 3 : 5) requant8_staged_kernel(EltAr
     if (nib) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) { nm[i].sh -= 4; m[i].sh -= 4; }
-      if (narrow) requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, 4, true>(a, nm, nr, wx, total, lo, hi, &pipe, stage);
-      else requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, 4, false>(a, m, r, wx, total, lo, hi, &pipe, stage);
+      if (narrow) requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, 4, true>(a, nm, nr, wx, total, lo, hi, &pipe, stage, issued);
+      else requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, 4, false>(a, m, r, wx, total, lo, hi, &pipe, stage, issued);
       return;
     }
   }
-  if (narrow) requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, SATP, true>(a, nm, nr, wx, total, lo, hi, &pipe, stage);
-  else if (slow) requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, true, 0, false>(a, m, r, wx, total, lo, hi, &pipe, stage);
-  else requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, SATP, false>(a, m, r, wx, total, lo, hi, &pipe, stage);
+  if (narrow) requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, SATP, true>(a, nm, nr, wx, total, lo, hi, &pipe, stage, issued);
+  else if (slow) requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, true, 0, false>(a, m, r, wx, total, lo, hi, &pipe, stage, issued);
+  else requant8_chunks<RES, MSIGNED, RSIGNED, OUT4, false, SATP, false>(a, m, r, wx, total, lo, hi, &pipe, stage, issued);
 }
 
 template <bool RES, bool MSIGNED, bool RSIGNED, bool OUT4, int SATP>

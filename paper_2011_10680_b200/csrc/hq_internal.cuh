@@ -113,6 +113,7 @@ struct ConvArgs {
                              // to one byte per value; for the first-layer form the virtual-channel weights and constants
   const WideArgs* wide;      // non-NULL: the convolution ends in the INT32 residual add (see WideArgs)
   int32_t in_slack;          // nonzero: the allocation behind `in` goes on for at least kIm2colMinTensorBytes + one image
+  int32_t wgt_fresh;         // nonzero: the weights are written by the launch just before: nothing of them is fetched ahead of it
   int32_t pad_after_delta;   // padding after the last row/column minus `pad`
   // byte pitches of the activation tensor along W, H and N when it is not dense (0: dense NHWC).  A W pitch
   // below cin bytes makes neighbouring "pixels" overlap: a pixel is then a window of adjacent stored pixels.
@@ -126,6 +127,7 @@ struct EltArgs {
   void* out; int32_t out_bits;
   // optional narrow pairs {m, a, s, valid} per channel for 8-bit operands (see hq_launch_residual_narrow), or NULL
   const void* m_narrow; const void* r_narrow;
+  int32_t narrow_fresh;      // nonzero: they are written by the launch just before (residual_narrow_kernel)
   int32_t overlap;           // set by the launcher: this launch overlaps its neighbours (hq_pdl_entry)
   uint32_t* status;          // the handle's device status word (bounded waits report here), or NULL
 };

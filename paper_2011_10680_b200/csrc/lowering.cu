@@ -324,19 +324,25 @@ __device__ __forceinline__ uint4 widen4_vec(uint2 v) {
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// 8 packed bytes -> 16 bytes; element 2j = low nibble of byte j.  Four independent loads per thread and trip.
+// 8 packed bytes -> 16 bytes; element 2j = low nibble of byte j.  Four independent loads per thread and trip.  Two tensors per
+// launch: the first `blocks1` blocks widen the second one (a layer's weights beside its activations).
+struct WidenJob { const uint2* in; long long n_vec; uint4* out; };
 template <bool SIGNED>
-__global__ void __launch_bounds__(256) widen4_kernel(const uint2* __restrict__ in, long long n_vec, uint4* __restrict__ out) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  for (; i + 3 * stride < n_vec; i += 4 * stride) {
+__device__ __forceinline__ void widen4_walk(const WidenJob& j, long long i, long long stride) {
+  for (; i + 3 * stride < j.n_vec; i += 4 * stride) {
     uint2 v[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = __ldg(in + i + u * stride);
+    for (int u = 0; u < 4; ++u) v[u] = __ldg(j.in + i + u * stride);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) out[i + u * stride] = widen4_vec<SIGNED>(v[u]);
+    for (int u = 0; u < 4; ++u) j.out[i + u * stride] = widen4_vec<SIGNED>(v[u]);
   }
-  for (; i < n_vec; i += stride) out[i] = widen4_vec<SIGNED>(__ldg(in + i));
+  for (; i < j.n_vec; i += stride) j.out[i] = widen4_vec<SIGNED>(__ldg(j.in + i));
+}
+template <bool SIGNED>
+__global__ void __launch_bounds__(256) widen4_kernel(WidenJob x, WidenJob w, int blocks1) {
+  hq_pdl_entry();
+  if ((int)blockIdx.x < blocks1) widen4_walk<true>(w, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)blocks1 * blockDim.x);
+  else widen4_walk<SIGNED>(x, (long long)(blockIdx.x - blocks1) * blockDim.x + threadIdx.x, (long long)(gridDim.x - blocks1) * blockDim.x);
 }
 
 // One byte per value -> two values per byte (low nibble first); 8 bytes in, 4 bytes out per thread and step.
@@ -350,14 +356,16 @@ __global__ void __launch_bounds__(256) pack4_kernel(const uint2* __restrict__ in
   }
 }
 
-cudaError_t launch_widen4(const void* in, long long elems, int is_signed, void* out, int sm_count, cudaStream_t s) {
-  const long long n_vec = elems / 16;                  // callers guarantee a multiple of 16 elements
-  if (n_vec == 0) return cudaSuccess;
-  long long blocks = (n_vec + 255) / 256;
+// `wgt` (signed, w_elems values) may be NULL.  Callers guarantee multiples of 16 elements.
+cudaError_t launch_widen4(const void* in, long long elems, int is_signed, void* out, const void* wgt, long long w_elems, void* wout,
+                          int sm_count, cudaStream_t s) {
+  const WidenJob x{(const uint2*)in, elems / 16, (uint4*)out}, w{(const uint2*)wgt, wgt ? w_elems / 16 : 0, (uint4*)wout};
   const long long cap = (long long)sm_count * 16;
-  const int grid = (int)(blocks < cap ? blocks : cap);
-  if (is_signed) widen4_kernel<true><<<grid, 256, 0, s>>>((const uint2*)in, n_vec, (uint4*)out);
-  else widen4_kernel<false><<<grid, 256, 0, s>>>((const uint2*)in, n_vec, (uint4*)out);
+  auto blocks_for = [&](long long n_vec) { const long long b = (n_vec + 255) / 256; return (int)(b < cap ? b : cap); };
+  const int blocks1 = blocks_for(w.n_vec), grid = blocks1 + blocks_for(x.n_vec);
+  if (grid == 0) return cudaSuccess;
+  if (is_signed) hq_launch_pdl(widen4_kernel<true>, grid, 256, 0, s, x, w, blocks1);
+  else hq_launch_pdl(widen4_kernel<false>, grid, 256, 0, s, x, w, blocks1);
   return cudaGetLastError();
 }
 
@@ -391,11 +399,9 @@ hq_status hq_launch_conv_widen4(hq_handle* h, const ConvArgs& a, void* scratch, 
   const long long x = (long long)a.n * a.h * a.w * a.cin, w = (long long)a.cout * a.kh * a.kw * a.cin;
   unsigned char* xw = (unsigned char*)scratch;
   unsigned char* ww = xw + (x + 255) / 256 * 256;
-  // (weights first: the convolution fetches resident weights without waiting for the launch just before it)
-  if (!a.wgt_widened && launch_widen4(a.wgt, w, 1, ww, h->sm_count, s) != cudaSuccess) return HQ_ERR_CUDA;
-  if (launch_widen4(a.in, x, a.in_signed, xw, h->sm_count, s) != cudaSuccess) return HQ_ERR_CUDA;
+  if (launch_widen4(a.in, x, a.in_signed, xw, a.wgt_widened ? nullptr : a.wgt, w, ww, h->sm_count, s) != cudaSuccess) return HQ_ERR_CUDA;
   ConvArgs t = a;
-  t.in = xw; t.wgt = a.wgt_widened ? a.wgt_widened : ww; t.in_bits = 8;
+  t.in = xw; t.wgt = a.wgt_widened ? a.wgt_widened : ww; t.in_bits = 8; t.wgt_fresh = a.wgt_widened ? 0 : 1;
   const hq_status st = hq_launch_conv_tc(h, t, s);
   if (st != HQ_ERR_UNSUPPORTED || !hq_conv_lowering_applies(t)) return st;
   return hq_launch_conv_lowered(h, t, xw + widen4_copy_bytes(a), s);      // declined by the direct kernel: patch matrix
@@ -410,7 +416,7 @@ cudaError_t hq_launch_pack4(const void* in, long long values, void* out, int sm_
 }
 
 cudaError_t hq_launch_widen_weights(const void* wgt, long long values, void* out, int sm_count, cudaStream_t s) {
-  return launch_widen4(wgt, values, 1, out, sm_count, s);
+  return launch_widen4(wgt, values, 1, out, nullptr, 0, nullptr, sm_count, s);
 }
 
 // ------------------------------------------------------------------------------------------------
