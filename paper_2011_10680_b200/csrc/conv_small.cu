@@ -45,7 +45,7 @@ FastDiv fast_div(uint32_t d) {
 }
 
 struct SmallParams {
-  FastDiv by_c_tiles, by_howo, by_wo, by_cin, by_kw;
+  FastDiv by_cchunks, by_c_tiles, by_howo, by_wo, by_cin, by_kw;
   const void* x; const void* w4;                 // activations; packed 4-bit weights (NULL: weights by TMA)
   int32_t h, w, cin, wo, howo, stride, pad, kh, kw;
   int32_t P, C, K;                               // output pixels, output channels, reduction length (values)
@@ -321,17 +321,20 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
     // before the convolution that reads them); activations, in the TMA modes, after it.
     if (elect_one()) {
       const int row = p.fold ? c_tile * 64 : c_tile * kTileC, row2 = p.fold ? row : row + 64;
-      auto load_w = [&](int i, int s) {
+      // (K blocks are loaded in order: the weight column advances by a block, and by a tap's channels at its end)
+      const int wtap = GATHER ? 0 : (int)p.by_cchunks.div((uint32_t)kb0);
+      int wchunk = kb0 - wtap * p.cchunks, tap_x = wtap * p.cin, wx = GATHER ? kb0 * 128 : tap_x + wchunk * p.bkb;
+      auto load_w = [&](int s) {
         const uint32_t bar = smem_u32(&ctl.wfull[s]), dst = tiles + (uint32_t)s * stage_bytes;
         mbar_expect_tx(bar, w_bytes);
-        int wx = (kb0 + i) * p.bkb;
-        if (!GATHER) { const int tap = (kb0 + i) / p.cchunks; wx = tap * p.cin + (kb0 + i - tap * p.cchunks) * p.bkb; }
         tma_load_2d(dst, &map_w, bar, wx, row);
         tma_load_2d(dst + w_bytes / 2, &map_w, bar, wx, row2);
+        wx += p.bkb;
+        if (!GATHER && ++wchunk == p.cchunks) { wchunk = 0; tap_x += p.cin; wx = tap_x; }
       };
       const int px0 = p_tile * p.pt;
       const int img = (int)p.by_howo.div((uint32_t)px0), rem = px0 - img * p.howo, oh = (int)p.by_wo.div((uint32_t)rem), ow = rem - oh * p.wo;
-      const int tap0 = p.x_mode == kXIm2col ? kb0 / p.cchunks : 0;
+      const int tap0 = p.x_mode == kXIm2col ? (int)p.by_cchunks.div((uint32_t)kb0) : 0;
       int chunk = kb0 - tap0 * p.cchunks, tr = (int)p.by_kw.div((uint32_t)tap0), ts = tap0 - tr * p.kw;
       auto load_x = [&](int s) {
         const uint32_t bar = smem_u32(&ctl.xfull[s]), dst = tiles + (uint32_t)s * stage_bytes + w_bytes;
@@ -341,7 +344,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
         if (++chunk == p.cchunks) { chunk = 0; if (++ts == p.kw) { ts = 0; ++tr; } }
       };
       const int ahead = L < p.stages ? L : p.stages;
-      if (!p.w4) for (int i = 0; i < ahead; ++i) load_w(i, i);
+      if (!p.w4) for (int i = 0; i < ahead; ++i) load_w(i);
       if constexpr (!GATHER) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         for (int i = 0; i < ahead; ++i) load_x(i);
@@ -349,7 +352,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
       int issued = ahead;
       for (int i = ahead, s = 0, ph = 0; i < L && !(p.w4 && GATHER); ++i, ++issued) {
         if (!mbar_wait(smem_u32(&ctl.empty[s]), (uint32_t)ph, &ctl, p.status, HQ_DEV_TIMEOUT_PRODUCER)) break;
-        if (!p.w4) load_w(i, s);
+        if (!p.w4) load_w(s);
         if (!GATHER) load_x(s);
         if (++s == p.stages) { s = 0; ph ^= 1; }
       }
@@ -373,6 +376,8 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
       const uint32_t idesc = (2u << 4) | (1u << 7) | ((uint32_t)(p.x_signed ? 1 : 0) << 10) | ((uint32_t)(p.pt >> 3) << 17) |
                              ((uint32_t)(kTileC >> 4) << 24);
       const uint64_t hi = smem_desc(0, p.bkb);
+      const int full_steps = p.bkb >> 5;
+      int chunk = GATHER ? 0 : kb0 - (int)p.by_cchunks.div((uint32_t)kb0) * p.cchunks;
       for (int i = 0, s = 0, ph = 0; i < L; ++i) {
         if (!p.w4 && !mbar_wait(smem_u32(&ctl.wfull[s]), (uint32_t)ph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) break;
         if (!mbar_wait(smem_u32(&ctl.xfull[s]), (uint32_t)ph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) break;
@@ -382,7 +387,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
         // (a block may reach past the channels: whole 32-byte steps beyond them are left out, a partial step meets zeros)
         int steps;
         if (GATHER) steps = (min(p.K - (kb0 + i) * p.bkb, p.bkb) + 31) >> 5;
-        else steps = (kb0 + i + 1) % p.cchunks == 0 ? p.tail_steps : p.bkb >> 5;
+        else { steps = full_steps; if (++chunk == p.cchunks) { chunk = 0; steps = p.tail_steps; } }
         for (int q = 0; q < steps; ++q, adesc += 2, bdesc += 2) mma_i8(tmem_base, adesc, bdesc, idesc, (i | q) ? 1u : 0u);
         mma_commit(smem_u32(i + 1 == L ? &ctl.tfull : &ctl.empty[s]));
         if (++s == p.stages) { s = 0; ph ^= 1; }
@@ -671,6 +676,7 @@ hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t str
   if (s.p_tiles == 0) return HQ_OK;
   SmallParams p{};
   p.by_c_tiles = fast_div((uint32_t)s.c_tiles); p.by_howo = fast_div((uint32_t)(a.ho * a.wo)); p.by_wo = fast_div((uint32_t)a.wo);
+  p.by_cchunks = fast_div((uint32_t)((a.cin + s.bkb - 1) / s.bkb));
   p.by_cin = fast_div((uint32_t)a.cin); p.by_kw = fast_div((uint32_t)a.kw);
   p.x = a.in; p.h = a.h; p.w = a.w; p.cin = a.cin; p.wo = a.wo; p.howo = a.ho * a.wo;
   p.stride = a.stride; p.pad = a.pad; p.kh = a.kh; p.kw = a.kw;

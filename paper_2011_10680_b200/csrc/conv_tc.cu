@@ -36,6 +36,8 @@
 // Every wait on an mbarrier is bounded: after the budget the waiter records a code in the
 // handle's status word, raises a CTA-wide abort flag and every role leaves its loop, drains what
 // it has in flight (again bounded), and the CTA frees its tensor memory and returns.
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace {
@@ -108,7 +110,6 @@ struct TcParams {
   const int32_t* bias; const int32_t* b; const int32_t* c;
   const void* res; int32_t res_bits, res_signed; const int32_t* rb; const int32_t* rc;
   const int4* res_narrow;   // optional per-channel {m, a, s, valid} from residual_narrow_kernel
-  int32_t w_fresh;          // 1: the weights are written by the kernel launched just before this one
   int32_t narrow_fresh;     // 1: the pairs are written by the kernel launched just before this one
   int32_t relu, qmin, qmax;
   void* out; int32_t out_bits;
@@ -880,19 +881,20 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       int ow = px_first - img * p.howo - oh * p.wo;
       const int step = p_step * p.pt;
       const int d_img = step / p.howo, d_oh = (step - d_img * p.howo) / p.wo, d_ow = step - d_img * p.howo - d_oh * p.wo;
-      if (p.w_fresh) asm volatile("griddepcontrol.wait;" ::: "memory");
       if (p.wres) {              // the channel tile's weights for every K block, once
         const uint32_t bar = smem_u32(&ctl.wfull);
         mbar_expect_tx(bar, (uint32_t)p.k_blocks * w_bytes);
+        int wx = 0, tap_x = 0, left = p.cchunks;
         for (int kb = 0; kb < p.k_blocks; ++kb) {
           const uint32_t w_dst = tiles + p.wres_off + (uint32_t)kb * w_bytes;
-          const int tap = kb / p.cchunks, wx = tap * p.cin + (kb - tap * p.cchunks) * p.bkb;
           if (p.fold) {
             tma_load_2d(w_dst, &map_w, bar, wx, 0);
             tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx, 0);
           } else {
             tma_load_2d(w_dst, &map_w, bar, wx, c_tile * kTileC);
           }
+          wx += p.bkb;
+          if (--left == 0) { left = p.cchunks; tap_x += p.cin; wx = tap_x; }
         }
       }
       // The resident weights above do not wait for the previous kernel: weights are never written by the launch
@@ -944,7 +946,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           oh -= d_oh; if (oh < 0) { oh += ho; --img; }
           img -= d_img;
         }
-        int chunk = 0, tap_s = 0, tap_r = 0, wx = 0;     // wx: the block's first byte in a weight row
+        int chunk = 0, tap_s = 0, tap_r = 0, wx = 0, tap_x = 0;     // wx: the block's first byte in a weight row
         // The residual tile of this output tile is fetched as soon as its buffer is free, but this thread only
         // blocks for the buffer after the tile's last operand block is on its way: the buffer comes back when the
         // epilogue of an earlier tile ends, and the operand copies must not queue behind that.
@@ -973,8 +975,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             if (rank == 0) mbar_expect_tx(bar, 2u * stage_bytes);
             if (p.x_tiled) tma_load_2d_2cta(w_dst + x_off, &map_x, bar, chunk * p.bkb, p0 + half_off);
             else tma_load_im2col_2cta(w_dst + x_off, &map_x, bar, chunk * p.bkb, cw, chh, img_now, (uint16_t)tap_s, (uint16_t)tap_r);
-            tma_load_2d_2cta(w_dst, &map_w, bar, wx + chunk * p.bkb, c_tile * kTileC);
-            if (++chunk == p.cchunks) { chunk = 0; wx += p.cin; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
+            tma_load_2d_2cta(w_dst, &map_w, bar, wx, c_tile * kTileC);
+            wx += p.bkb;
+            if (++chunk == p.cchunks) { chunk = 0; tap_x += p.cin; wx = tap_x; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
             if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1u; }
             if (res_due && kb + 1 == p.k_blocks && !residual(true)) { ok = false; break; }
             continue;
@@ -988,12 +991,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           if (p.wres) {
             // weights are resident
           } else if (p.fold) {   // 64-row box, twice: accumulator lanes 64-127 repeat lanes 0-63
-            tma_load_2d(w_dst, &map_w, bar, wx + chunk * p.bkb, 0);
-            tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx + chunk * p.bkb, 0);
+            tma_load_2d(w_dst, &map_w, bar, wx, 0);
+            tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx, 0);
           } else {
-            tma_load_2d(w_dst, &map_w, bar, wx + chunk * p.bkb, c_tile * kTileC);
+            tma_load_2d(w_dst, &map_w, bar, wx, c_tile * kTileC);
           }
-          if (++chunk == p.cchunks) { chunk = 0; wx += p.cin; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
+          wx += p.bkb;
+          if (++chunk == p.cchunks) { chunk = 0; tap_x += p.cin; wx = tap_x; if (++tap_s == p.kw) { tap_s = 0; ++tap_r; } }
           if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1u; }
           if (res_due && kb + 1 == p.k_blocks && !residual(true)) { ok = false; break; }
         }
@@ -1066,11 +1070,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       bool ok = true;
       const uint64_t desc_hi = smem_desc(0, p.bkb);           // everything but the start address
       const int ksteps = p.bkb >> 5;
+      const bool tail = p.tail_steps != ksteps;              // a tap's last block holds fewer steps
       if (p.wres && !mbar_wait(smem_u32(&ctl.wfull), 0, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) ok = false;
       // One issuer, plain form: the lean loop (the hand-over chain of short reductions is latency bound, every
       // instruction on it counts).
       const bool lean = ni == 1 && !p.strip;
-      for (int p_tile = p_tile0; p_tile < p.p_tiles && ok && lean; p_tile += p_step, ++tcount) {
+      auto lean_tiles = [&](auto tail_tag) {
+        constexpr bool TAIL = decltype(tail_tag)::value;
+      for (int p_tile = p_tile0; p_tile < p.p_tiles && ok; p_tile += p_step, ++tcount) {
         const uint32_t as = tcount & bmask, aph = (tcount >> p.lg_bufs) & 1u;
         // The operands of the tile's first K block have usually landed long ago; looking at them first
         // keeps that check off the path between the epilogue's hand-back and the first MMA.
@@ -1081,7 +1088,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         int chunk = 0;
         for (int kb = 0; kb < p.k_blocks; ++kb) {
           int nsteps = ksteps;
-          if (++chunk == p.cchunks) { chunk = 0; nsteps = p.tail_steps; }
+          if (TAIL && ++chunk == p.cchunks) { chunk = 0; nsteps = p.tail_steps; }
           if (kb > 0 && !mbar_wait(smem_u32(&ctl.full[s]), ph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) { ok = false; break; }
           const uint32_t w_addr = tiles + s * stage_bytes;
           const uint32_t a_addr = p.wres ? tiles + p.wres_off + (uint32_t)kb * w_bytes : w_addr;
@@ -1115,6 +1122,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           commit(smem_u32(&ctl.tfull[as]));
         }
       }
+      };
+      if (lean) { if (tail) lean_tiles(std::true_type{}); else lean_tiles(std::false_type{}); }
       for (int p_tile = p_tile0; p_tile < p.p_tiles && ok && !lean; p_tile += p_step, ++tcount) {
         const uint32_t as = tcount & bmask, aph = (tcount >> p.lg_bufs) & 1u;
         const uint32_t d_tmem = tmem_base + as * p.pt;
@@ -1159,8 +1168,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           }
           uint64_t adesc = desc_hi | (uint64_t)((a_addr >> 4) & 0x3FFF);
           uint64_t bdesc = desc_hi | (uint64_t)((b_addr >> 4) & 0x3FFF);
-          const int nsteps = p.tail_steps != ksteps && b % p.cchunks == p.cchunks - 1 ? p.tail_steps : ksteps;
-          for (int k = 0; k < nsteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
+          for (int k = 0; k < ksteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
             mma_i8(d_tmem, adesc, bdesc, idesc, (b | k) ? 1u : 0u);
           if (b == 0 && ni > 1) mbar_arrive(smem_u32(&ctl.tstart[as]));   // the overwriting MMA is on its way
           // the accumulator's barrier first on this issuer's last block: the epilogue is the one waiting
@@ -1504,7 +1512,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     if (p.bkb > 64) set_bkb(64);
     p.pt = pick_pt(P, p.c_tiles, 2 * h->sm_count, 128);
     wres_bytes = p.k_blocks * kTileC * p.bkb;
-    p.wres = wres_bytes <= 16 * 1024 ? 1 : 0;              // short reductions: the weight slab stays resident
+    p.wres = wres_bytes <= 16 * 1024 && !a.wgt_fresh ? 1 : 0;              // short reductions: the weight slab stays resident
     if (!p.wres) wres_bytes = 0;
     stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
     p.fold = (a.cout <= 64 && p.pt >= 128) ? 1 : 0;
@@ -1528,7 +1536,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       // tile wins and the weights travel with the stages.
       for (int keep_w = 1; keep_w >= 0 && !chosen; --keep_w) {
         wres_bytes = p.k_blocks * kTileC * p.bkb;
-        p.wres = (keep_w && wres_bytes <= 72 * 1024) ? 1 : 0;
+        p.wres = (keep_w && wres_bytes <= 72 * 1024 && !a.wgt_fresh) ? 1 : 0;     // (resident weights are fetched ahead of the previous launch's end)
         if (!p.wres) { if (keep_w) continue; wres_bytes = 0; }
         stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
         p.fold = (a.cout <= 64 && p.pt >= 128) ? 1 : 0;
@@ -1568,7 +1576,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       const long long tiles_all = (long long)a.n * tpi * p.c_tiles;
       const size_t patch = (size_t)(rows + 3) * (1u << lg_wp) * bkb, wb = (size_t)kTileC * bkb;
       const size_t slab = (size_t)9 * cchunks * wb;
-      const bool keep_w = slab <= 72 * 1024;
+      const bool keep_w = slab <= 72 * 1024 && !a.wgt_fresh;
       const size_t room = (size_t)kSmemBudget - 32 * 1024 - (keep_w ? slab : 0);
       int npatch = 0, wstages = 0;
       if (keep_w) { npatch = (int)(room / patch); if (npatch > 3) npatch = 3; }
@@ -1620,7 +1628,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       out_tile_bytes = 0;
       res_tile_bytes = p.pt * kTileC;
       wres_bytes = p.k_blocks * kTileC * p.bkb;
-      p.wres = wres_bytes <= 72 * 1024 ? 1 : 0;
+      p.wres = wres_bytes <= 72 * 1024 && !a.wgt_fresh ? 1 : 0;
       if (!p.wres) wres_bytes = 0;
       stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
       // four residual / output tiles when they leave room for three operand stages: a tile is held from its load to
@@ -1639,7 +1647,9 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       stage_bytes = (kTileC + p.pt / 2) * p.bkb;
       stages = (kSmemBudget - out_tile_bytes - (res_tile_bytes << p.lg_rbufs)) / stage_bytes;
     }
-    const int issuers = pair ? kPairIssuerWarps : wide ? 1 : (p.strip || p.wres) ? kSoloIssuerWarps : 1;
+    // (the dealt loop knows whole K blocks only: channels that do not fill their last block take the single issuer)
+    const bool tail = a.cin % p.bkb > 0 && a.cin % p.bkb <= p.bkb - 32;
+    const int issuers = pair ? kPairIssuerWarps : wide ? 1 : (p.strip || (p.wres && !tail)) ? kSoloIssuerWarps : 1;
     p.ni = p.k_blocks < issuers ? p.k_blocks : issuers;
     if (!(p.strip && p.wres)) {
       while (p.ni > 1 && stages < p.ni) --p.ni;
@@ -1665,7 +1675,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.bias = a.bias; p.b = a.b; p.c = a.c;
   p.res = a.res; p.res_bits = a.res_bits; p.res_signed = a.res_signed; p.rb = a.rb; p.rc = a.rc;
   p.res_narrow = (a.res && a.res_bits == 8) ? (const int4*)a.res_narrow : nullptr;
-  p.narrow_fresh = a.res_narrow_fresh; p.w_fresh = a.wgt_fresh;
+  p.narrow_fresh = a.res_narrow_fresh;
   p.relu = a.relu; p.qmin = a.qmin; p.qmax = a.qmax;
   p.out = a.out; p.out_bits = a.out_bits; p.out_signed = a.out_signed;
   if (a.wide) {
