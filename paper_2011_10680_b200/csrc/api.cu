@@ -87,6 +87,10 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
     const hq_status st4 = hq_launch_conv_small(h, a, s);
     if (st4 != HQ_ERR_UNSUPPORTED || h->conv_path == 4) return st4;
   }
+  if (h->conv_path == 0 && a.wgt_widened && hq_conv_pairs_applies(a, h->sm_count)) {
+    const hq_status st5 = hq_launch_conv_pairs(h, a, s);
+    if (st5 != HQ_ERR_UNSUPPORTED) return st5;
+  }
   const bool tc_ok = hq_conv_tc_supported(a);
   const bool force_tc = h->conv_path >= 2;
   if (force_tc && !tc_ok && !hq_conv_widen4_applies(a)) return HQ_ERR_UNSUPPORTED;
@@ -546,6 +550,13 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
             if (!wbuf) { st = HQ_ERR_WORKSPACE; break; }
             net->wgt_widened[i] = wbuf;
             if (hq_launch_widen_weights(d.w, wvals, wbuf, h->sm_count, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
+          } else if (l.in1 < 0 && !hq_conv_small_wanted(a, h->sm_count) && hq_conv_pairs_applies(a, h->sm_count)) {
+            a.wgt = d.w; a.bias = d.bias; a.b = d.requant.b; a.c = d.requant.c;
+            if (!a.b || !a.c) break;
+            void* wbuf = net_alloc(net, hq_conv_pairs_prepared_bytes(), i);
+            if (!wbuf) { st = HQ_ERR_WORKSPACE; break; }
+            net->wgt_widened[i] = wbuf;
+            if (hq_prepare_conv_pairs(a, wbuf, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
           } else if (hq_conv_s2d_applies(a)) {
             const size_t need = hq_conv_s2d_bytes(a);
             if (need > net->scratch_bytes) net->scratch_bytes = need;

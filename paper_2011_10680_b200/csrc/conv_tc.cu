@@ -98,6 +98,8 @@ struct TcParams {
   int32_t lg_wp, rows;   // log2 of the position pitch; output rows per tile (pt = rows << lg_wp)
   int32_t tpi;           // tiles per image = ceil(ho / rows)
   int32_t ho;            // output (= input) height
+  int32_t pairs;         // 1: strip mode over pixel pairs (lowering.cu): twelve blocks (filter row, pixel of four) of 64 bytes
+  int32_t w_blocks;      // K blocks of the resident weight slab
   int32_t npatch;        // patch buffers (2 or 3)
   uint32_t patch_bytes, patch_off;   // bytes of one patch [(rows+3) << lg_wp][bkb]; offset from the 1024-aligned base
   uint32_t tmem_cols;
@@ -883,9 +885,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       const int d_img = step / p.howo, d_oh = (step - d_img * p.howo) / p.wo, d_ow = step - d_img * p.howo - d_oh * p.wo;
       if (p.wres) {              // the channel tile's weights for every K block, once
         const uint32_t bar = smem_u32(&ctl.wfull);
-        mbar_expect_tx(bar, (uint32_t)p.k_blocks * w_bytes);
+        mbar_expect_tx(bar, (uint32_t)p.w_blocks * w_bytes);
         int wx = 0, tap_x = 0, left = p.cchunks;
-        for (int kb = 0; kb < p.k_blocks; ++kb) {
+        for (int kb = 0; kb < p.w_blocks; ++kb) {
           const uint32_t w_dst = tiles + p.wres_off + (uint32_t)kb * w_bytes;
           if (p.fold) {
             tma_load_2d(w_dst, &map_w, bar, wx, 0);
@@ -1069,8 +1071,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       const uint32_t bmask = (1u << p.lg_bufs) - 1u;
       bool ok = true;
       const uint64_t desc_hi = smem_desc(0, p.bkb);           // everything but the start address
-      const int ksteps = p.bkb >> 5;
-      const bool tail = p.tail_steps != ksteps;              // a tap's last block holds fewer steps
+      const int ksteps = p.pairs ? 2 : p.bkb >> 5;
+      const bool tail = !p.pairs && p.tail_steps != ksteps;              // a tap's last block holds fewer steps
       if (p.wres && !mbar_wait(smem_u32(&ctl.wfull), 0, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) ok = false;
       // One issuer, plain form: the lean loop (the hand-over chain of short reductions is latency bound, every
       // instruction on it counts).
@@ -1137,7 +1139,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             // The start is then not aligned to the swizzle pattern's eight rows, which needs nothing more: the
             // pattern is a function of the shared-memory address, for the copy that wrote the patch and for the
             // MMA that reads it alike (the descriptor's base-offset field stays 0; a phase there gives wrong sums).
-            const int chunk = b / 9, tap = b - 9 * chunk, tr = tap / 3, ts = tap - 3 * tr;
+            const int chunk = p.pairs ? 0 : b / 9, tap = b - 9 * chunk, tr = p.pairs ? b >> 2 : tap / 3, ts = p.pairs ? b & 3 : tap - 3 * tr;
             if (chunk != cur_chunk) {
               if (cur_chunk >= 0) mma_commit(smem_u32(&ctl.pempty[ps]));    // my MMAs on the previous patch
               cur_chunk = chunk;
@@ -1146,7 +1148,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
               if (!mbar_wait(smem_u32(&ctl.pfull[ps]), (pidx / (uint32_t)p.npatch) & 1u, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) { ok = false; break; }
             }
             b_addr = tiles + p.patch_off + ps * p.patch_bytes + (uint32_t)(((tr << p.lg_wp) + ts) * p.bkb);
-            if (p.wres) {
+            if (p.pairs) {
+              // pixel ts - 1 of the pair: second half of the pair before, the pair itself, first half of the pair after
+              b_addr = tiles + p.patch_off + ps * p.patch_bytes + (uint32_t)(((tr << p.lg_wp) + ((ts + 1) >> 1)) * 128 + (((ts + 1) & 1) << 6));
+              a_addr = tiles + p.wres_off + (uint32_t)(2 * tr + (ts >> 1)) * w_bytes + (uint32_t)((ts & 1) << 6);
+            } else if (p.wres) {
               a_addr = tiles + p.wres_off + (uint32_t)(tap * p.cchunks + chunk) * w_bytes;
             } else {
               if (!mbar_wait(smem_u32(&ctl.full[s]), ph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) { ok = false; break; }
@@ -1575,18 +1581,19 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       const int cchunks = a.cin / bkb, rows = 256 >> lg_wp, tpi = (a.h + rows - 1) / rows;
       const long long tiles_all = (long long)a.n * tpi * p.c_tiles;
       const size_t patch = (size_t)(rows + 3) * (1u << lg_wp) * bkb, wb = (size_t)kTileC * bkb;
-      const size_t slab = (size_t)9 * cchunks * wb;
-      const bool keep_w = slab <= 72 * 1024 && !a.wgt_fresh;
+      const size_t slab = (size_t)(a.pairs ? 6 : 9 * cchunks) * wb;
+      const bool keep_w = (slab <= 72 * 1024 && !a.wgt_fresh) || a.pairs;
       const size_t room = (size_t)kSmemBudget - 32 * 1024 - (keep_w ? slab : 0);
       int npatch = 0, wstages = 0;
       if (keep_w) { npatch = (int)(room / patch); if (npatch > 3) npatch = 3; }
       else if (room >= 2 * patch + 3 * wb) { npatch = 2; wstages = (int)((room - 2 * patch) / wb); }
       // measured: with the weights streaming through the stage ring the strip form is no faster than the plain
       // one (both are bound by what the SM can take in per cycle), so it is used where the weights stay resident
-      if (((tiles_all >= 2LL * h->sm_count && keep_w) || h->conv_path == 3) && npatch >= 2) {
+      if (((tiles_all >= 2LL * h->sm_count && keep_w) || h->conv_path == 3 || a.pairs) && npatch >= 2) {
         p.strip = 1; p.lg_wp = lg_wp; p.rows = rows; p.tpi = tpi; p.ho = a.h; p.npatch = npatch;
         p.patch_bytes = (uint32_t)patch;
-        p.bkb = bkb; p.cchunks = cchunks; p.k_blocks = 9 * cchunks;
+        p.bkb = bkb; p.cchunks = cchunks; p.k_blocks = a.pairs ? 12 : 9 * cchunks;
+        p.pairs = a.pairs;
         p.pt = 256; p.lg_bufs = 1; p.lg_rbufs = 1; p.halves = 2;
         p.fold = a.cout <= 64 ? 1 : 0;
         p.wres = keep_w ? 1 : 0;
@@ -1603,7 +1610,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // The direct kernel fetches activations through an im2col-mode map unless the layer is 1x1 / stride 1 / unpadded
   // (tiled map) or takes the strip form (tiled map over padded patches).  That mode is not used on tensors below
   // 128 KiB (hq_conv_tc_small_im2col); such a layer is declined here and runs in its lowered form.
-  if (!p.strip && hq_conv_tc_small_im2col(a)) return HQ_ERR_UNSUPPORTED;
+  if ((!p.strip && hq_conv_tc_small_im2col(a)) || (a.pairs && !p.strip)) return HQ_ERR_UNSUPPORTED;
   p.x_signed = a.in_signed;
   bool wide = false;
   {
@@ -1661,6 +1668,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     }
   }
   p.acc_stride = p.rtm ? 2 * p.pt : p.pt;
+  p.w_blocks = p.pairs ? 6 : p.k_blocks;
   p.tail_steps = (a.cin - (p.cchunks - 1) * p.bkb + 31) >> 5;
   { const long long bound = k_total * 255 * 128; int bits = 0; while ((1LL << bits) <= bound) ++bits; p.acc_bits = bits; }
   p.tmem_cols = (uint32_t)(p.acc_stride << p.lg_bufs);  // 512 columns, or 256 for the smallest tile
@@ -1709,7 +1717,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   } else {
     if (!encode_im2col_map(&map_x, a, p.bkb, p.pt >> p.duo)) return HQ_ERR_CUDA;
   }
-  if (!encode_rows_map(&map_w, a.wgt, a.cout, (long long)a.kh * a.kw * a.cin, p.bkb, p.fold ? 64 : kTileC, swz)) return HQ_ERR_CUDA;
+  if (!encode_rows_map(&map_w, a.wgt, a.cout, p.pairs ? 6 * 128 : (long long)a.kh * a.kw * a.cin, p.bkb, p.fold ? 64 : kTileC, swz)) return HQ_ERR_CUDA;
   map_out = map_w; map_res = map_w; map_q = map_w;                    // valid placeholders when a path is not staged
   // (with rtm the residual tile is an MMA operand and, later, the output box: 128-byte swizzle both ways)
   const CUtensorMapSwizzle box_swz = p.rtm ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;

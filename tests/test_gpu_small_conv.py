@@ -158,3 +158,25 @@ def test_fused_pooling_branch(signed, shift):
         run_network_and_compare(hq, t, batch=3, seed=6)
     finally:
         hq.close()
+
+
+@pytest.mark.parametrize("hw,batch,signed", [(56, 11, False), (50, 13, True), (26, 41, False)])
+def test_conv_over_pixel_pairs(hw, batch, signed):
+    """3x3 layers of 64 channels in the pixel-pair form of a network: full and ragged tiles, both pitches, signed outputs."""
+    from paper_2011_10680_b200 import binding, build
+    from test_gpu_parity import run_network_and_compare
+    build.build()
+    bd = inputs._Builder(hw)
+    bd.scale[-1], bd.shape[-1], bd.bits[-1] = 2.0 ** -4, (2 * hw, 2 * hw, 3), 8
+    x = bd.conv(-1, 64, 3, 2, 1, 8, relu=True, out_bits=8)
+    x = bd.conv(x, 64, 3, 1, 1, 8, relu=not signed, out_bits=8, out_signed=signed)
+    x = bd.conv(x, 64, 3, 1, 1, 8, relu=True, out_bits=8)
+    x = bd.avgpool(x)
+    bd.conv(x, 16, 1, 1, 0, 8, relu=False, out_bits=32, op="linear")
+    t = dict(layers=bd.layers, image_hw=2 * hw, classes=16, depth=0, conv_bits=[8], shapes=[bd.shape[i] for i in range(len(bd.layers))],
+             bits=[bd.bits[i] for i in range(len(bd.layers))])
+    hq = binding.Handle(0)
+    try:
+        run_network_and_compare(hq, t, batch=batch, seed=6)
+    finally:
+        hq.close()
