@@ -725,7 +725,8 @@ static hq_status run_layers(hq_network* net, const hq_tensor* images, hq_tensor*
         if (in_wide) { d.w_bits = 8; d.w = net->wgt_widened[i]; }
         const int32_t callers_order = h->tile_order;
         h->tile_order = net->tile_order[i];
-        if (l.op == HQ_OP_LINEAR) { in.c = in.h * in.w * in.c; in.h = 1; in.w = 1; st = hq_linear(h, &in, &d, &o, s); }
+        if (l.op == HQ_OP_LINEAR) { in.c = in.h * in.w * in.c; in.h = 1; in.w = 1; 
+          st = d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0 ? conv_common(h, &in, &d, &o, s, nullptr, 0, nullptr, nullptr, l.in0 >= 0) : HQ_ERR_INVALID_ARG; }
         else st = conv_common(h, &in, &d, &o, s, net->scratch, net->scratch_bytes, net->res_narrow[i], in_wide ? nullptr : net->wgt_widened[i], l.in0 >= 0);
         h->tile_order = callers_order;
         break;

@@ -52,7 +52,7 @@ struct SmallParams {
   int32_t bkb, nkb, lg_split, stages;            // bytes of K per stage (gather: 128); K blocks of the layer; log2 of the cluster size; stages per CTA
   int32_t x_mode, cchunks, tail_steps;           // kXGather / kXTiled / kXIm2col; K blocks per filter tap and MMA steps of its last one (TMA modes)
   int32_t pt, lg_cols, c_tiles, fold;            // pixels per tile (MMA N); log2 of the pixels a CTA finishes; channel tiles; folded rows
-  int32_t x_bits, x_signed;
+  int32_t x_bits, x_signed, params_late;         // params_late: weights and constants may be the previous launch's output
   uint32_t part_off;                             // partial sums of a cluster, from the 1024-aligned base
   uint32_t tmem_cols;
   const int32_t* bias; const int32_t* b; const int32_t* c;
@@ -314,6 +314,8 @@ __global__ void __launch_bounds__(kSmallThreads, 2) conv_small_kernel(const __gr
   tc_fence_after();
   if (p.lg_split) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // waited for before the first remote store
   const uint32_t tmem_base = ctl.tmem_base;
+  // A call of its own may follow the kernel that wrote its weights and constants: nothing is read ahead of that one's end.
+  if (p.params_late) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
@@ -686,7 +688,7 @@ hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t str
   p.nkb = s.nkb; p.lg_split = s.lg_split; p.stages = s.stages; p.pt = s.pt; p.c_tiles = s.c_tiles;
   while ((1 << p.lg_cols) < (s.pt >> s.lg_split)) ++p.lg_cols;
   p.fold = s.fold;
-  p.x_bits = a.in_bits; p.x_signed = a.in_signed;
+  p.x_bits = a.in_bits; p.x_signed = a.in_signed; p.params_late = a.in_slack ? 0 : 1;      // (a network's parameters are older)
   const void* wgt = (a.in_bits == 4 && a.wgt_widened) ? a.wgt_widened : a.wgt;
   if (a.in_bits == 4 && !a.wgt_widened) p.w4 = a.wgt;
   const int stage_bytes = (kTileC + s.pt) * s.bkb;

@@ -331,7 +331,7 @@ bool hq_conv_pairs_applies(const ConvArgs& a, int sm_count) {
       a.out_bits != 8 || (a.w & 1) || a.n >= 65536) return false;
   const int wp = a.w / 2, lg = wp >= 11 && wp <= 14 ? 4 : wp >= 23 && wp <= 30 ? 5 : 0;
   const int rows = lg ? 256 >> lg : 1;
-  return lg && 2LL * a.n * ((a.h + rows - 1) / rows) >= sm_count;
+  return lg && 4LL * a.n * ((a.h + rows - 1) / rows) >= sm_count;
 }
 size_t hq_conv_pairs_prepared_bytes() { return 128 * kPairK + 3 * 128 * 4; }
 cudaError_t hq_prepare_conv_pairs(const ConvArgs& a, void* buf, cudaStream_t s) {
