@@ -307,7 +307,7 @@ static void count_launches(hq_network* net) {
     if (hq_conv_small_wanted(a, net->h->sm_count)) continue;
     if (a.in_bits == 4) net->launches += hq_conv_widen4_applies(a) ? 1 : 0;     // activations widened (weights were when the network was built)
     else if (hq_conv_s2d_applies(a)) net->launches += 1;                          // space-to-depth copy
-    else if ((!hq_conv_tc_supported(a) || hq_conv_tc_small_im2col(a)) && hq_conv_lowering_applies(a)) net->launches += 2;   // padded weights, patch matrix
+    else if ((!hq_conv_tc_supported(a) || hq_conv_tc_declines(a)) && hq_conv_lowering_applies(a)) net->launches += 2;   // padded weights, patch matrix
   }
 }
 
@@ -565,7 +565,7 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
             if (!wbuf) { st = HQ_ERR_WORKSPACE; break; }
             net->wgt_widened[i] = wbuf;
             if (hq_prepare_conv_s2d(a, wbuf, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
-          } else if ((!hq_conv_tc_supported(a) || hq_conv_tc_small_im2col(a)) && hq_conv_lowering_applies(a)) {
+          } else if ((!hq_conv_tc_supported(a) || hq_conv_tc_declines(a)) && hq_conv_lowering_applies(a)) {
             const size_t need = hq_conv_lowering_bytes(a);
             if (need > net->scratch_bytes) net->scratch_bytes = need;
           }

@@ -40,6 +40,7 @@ struct ConcatArgs {
 // tries the two neighbouring multipliers against the 64-bit definition for every r and records the one that agrees
 // everywhere (valid = 1), else valid = 0 and the channel keeps the wide form.  c >= 41 makes the term 0 for every r.
 __global__ void __launch_bounds__(128) concat_narrow_kernel(const __grid_constant__ ConcatArgs a, int4* out) {
+  hq_pdl_entry();
   const int oc = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (oc >= a.out_ch) return;
   int i = 0;
@@ -580,7 +581,7 @@ hq_status hq_concat_requant_planned(hq_handle* h, int32_t n_branches, const hq_t
     a.narrow = any_narrow ? (const int4*)plan.narrow : nullptr;
   } else if (any_narrow && h->narrow_pairs && out->c <= 2 * kNarrowChannels && a.pixels * out->c >= (1ll << 22)) {
     int4* tab = (int4*)h->narrow_pairs;
-    concat_narrow_kernel<<<(out->c + 3) / 4, 128, 0, (cudaStream_t)stream>>>(a, tab);
+    hq_launch_pdl(concat_narrow_kernel, (out->c + 3) / 4, 128, 0, (cudaStream_t)stream, a, tab);
     if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;
     a.narrow = tab;
   }

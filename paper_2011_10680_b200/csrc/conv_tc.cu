@@ -1481,6 +1481,19 @@ bool hq_conv_tc_small_im2col(const ConvArgs& a) {
   return span < kIm2colMinTensorBytes;
 }
 
+// Filters over channel counts that are not a multiple of 32: the direct kernel fetches every tap's short row anew for every
+// tile of output channels, the patch matrix pays once for long rows.  In cycles per output pixel and SM, from launches of both
+// forms: a direct row costs 5 (up to 64 bytes) or 7, a patch row 7, building the matrix K / 16.  Direct: 5x5 over 48 channels to 64
+// 135 us against 161; patches: 3x3 over 48 channels to 1664 66 us against 81.
+static bool prefers_patches(const ConvArgs& a) {
+  if (a.cin % 32 == 0 || a.kh * a.kw == 1 || a.pitch_w || a.pairs || !hq_conv_lowering_applies(a)) return false;
+  const long long K = (long long)a.kh * a.kw * a.cin, tiles = (a.cout + kTileC - 1) / kTileC;
+  const int bkb = hq_conv_bkb(a.cin);
+  const long long direct_rows = (long long)a.kh * a.kw * ((a.cin + bkb - 1) / bkb), patch_rows = (K + 127) / 128;
+  return tiles * (direct_rows * (bkb < 128 ? 5 : 7) - 7 * patch_rows) > K / 16;
+}
+bool hq_conv_tc_declines(const ConvArgs& a) { return hq_conv_tc_small_im2col(a) || prefers_patches(a); }
+
 hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream) {
   if (!hq_conv_tc_supported(a)) return HQ_ERR_UNSUPPORTED;
   if (!load_driver_entry_points()) return HQ_ERR_CUDA;
@@ -1610,7 +1623,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // The direct kernel fetches activations through an im2col-mode map unless the layer is 1x1 / stride 1 / unpadded
   // (tiled map) or takes the strip form (tiled map over padded patches).  That mode is not used on tensors below
   // 128 KiB (hq_conv_tc_small_im2col); such a layer is declined here and runs in its lowered form.
-  if ((!p.strip && hq_conv_tc_small_im2col(a)) || (a.pairs && !p.strip)) return HQ_ERR_UNSUPPORTED;
+  if ((!p.strip && hq_conv_tc_declines(a)) || (a.pairs && !p.strip)) return HQ_ERR_UNSUPPORTED;
   p.x_signed = a.in_signed;
   bool wide = false;
   {

@@ -146,6 +146,7 @@ bool hq_conv_tc_supported(const ConvArgs& a);
 // True for a layer the direct kernel declines although its shape is supported: it would fetch a tensor below
 // 128 KiB through an im2col-mode map.  Such a layer runs in its lowered (patch-matrix) form.
 bool hq_conv_tc_small_im2col(const ConvArgs& a);
+bool hq_conv_tc_declines(const ConvArgs& a);      // ... or whose patch matrix is cheaper than its short rows
 // Tensor-core path; returns HQ_OK, HQ_ERR_UNSUPPORTED (nothing was launched) or HQ_ERR_CUDA.
 hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t s);
 // One tile per CTA, reduction split over a cluster: small problems (conv_small.cu).  Same status convention.

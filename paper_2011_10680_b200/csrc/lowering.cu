@@ -436,7 +436,7 @@ static size_t widen4_copy_bytes(const ConvArgs& a) {
 size_t hq_conv_widen4_bytes(const ConvArgs& a) {
   ConvArgs t = a;
   t.in_bits = 8;
-  const bool lowered = (!hq_conv_tc_supported(t) || hq_conv_tc_small_im2col(t)) && hq_conv_lowering_applies(t);
+  const bool lowered = (!hq_conv_tc_supported(t) || hq_conv_tc_declines(t)) && hq_conv_lowering_applies(t);
   return widen4_copy_bytes(a) + (lowered ? hq_conv_lowering_bytes(t) : 0);
 }
 
