@@ -32,6 +32,7 @@ struct ConcatArgs {
   void* out;
   const int4* narrow;   // per OUTPUT channel {m, a, s, valid} from concat_narrow_kernel (8-/4-bit branches), or NULL
   int32_t sat;          // 1: relu and the clamp bounds equal a saturating conversion to the 8-bit output type
+  int32_t overlap;      // 1: this launch overlaps its neighbours (hq_pdl_entry)
   int32_t rev;          // 1: pixels are walked from the last to the first (the handle's tile order): same results
 };
 
@@ -40,7 +41,6 @@ struct ConcatArgs {
 // tries the two neighbouring multipliers against the 64-bit definition for every r and records the one that agrees
 // everywhere (valid = 1), else valid = 0 and the channel keeps the wide form.  c >= 41 makes the term 0 for every r.
 __global__ void __launch_bounds__(128) concat_narrow_kernel(const __grid_constant__ ConcatArgs a, int4* out) {
-  hq_pdl_entry();
   const int oc = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (oc >= a.out_ch) return;
   int i = 0;
@@ -470,7 +470,7 @@ __device__ __forceinline__ int concat_my_branch(const ConcatArgs& a, int width) 
 
 // Branches in the four-channel form (few registers, many warps per SM) ...
 __global__ void __launch_bounds__(256, 4) concat_requant_kernel(const __grid_constant__ ConcatArgs a) {
-  hq_pdl_entry();
+  if (a.overlap) hq_pdl_entry();
   const int i = concat_my_branch(a, 4);
   if (a.br[i].bits == 32) concat_w4<32>(a, i);
   else if (a.br[i].bits == 8) concat_w4<8>(a, i);
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(256, 4) concat_requant_kernel(const __grid_con
 
 // ... and the others (ragged or very wide branches) in the sixteen-channel form, in a launch of their own.
 __global__ void __launch_bounds__(256, 2) concat_requant_wide_kernel(const __grid_constant__ ConcatArgs a) {
-  hq_pdl_entry();
+  if (a.overlap) hq_pdl_entry();
   concat_branch<16>(a, concat_my_branch(a, 16));
 }
 
@@ -571,6 +571,7 @@ hq_status hq_concat_requant_planned(hq_handle* h, int32_t n_branches, const hq_t
   // A large call first works out the narrow pairs of its 8- and 4-bit branches in the handle's buffer (one small
   // launch on the same stream, repaid by the cheaper arithmetic).
   a.narrow = nullptr;
+  a.overlap = 1;
   bool any_narrow = false;
   for (int i = 0; i < n_branches; ++i) any_narrow = any_narrow || (i != plan.skip && branches[i].bits != 32);
   if (plan.prepare) {
@@ -581,11 +582,12 @@ hq_status hq_concat_requant_planned(hq_handle* h, int32_t n_branches, const hq_t
     a.narrow = any_narrow ? (const int4*)plan.narrow : nullptr;
   } else if (any_narrow && h->narrow_pairs && out->c <= 2 * kNarrowChannels && a.pixels * out->c >= (1ll << 22)) {
     int4* tab = (int4*)h->narrow_pairs;
-    hq_launch_pdl(concat_narrow_kernel, (out->c + 3) / 4, 128, 0, (cudaStream_t)stream, a, tab);
+    concat_narrow_kernel<<<(out->c + 3) / 4, 128, 0, (cudaStream_t)stream>>>(a, tab);
     if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;
     a.narrow = tab;
+    a.overlap = a.pixels * out->c >= (1ll << 24) ? 1 : 0;      // (behind a search of its own a smaller call loses 5 % by it)
   }
-  if (blocks4) hq_launch_pdl(concat_requant_kernel, (unsigned)blocks4, 256, 0, (cudaStream_t)stream, a);
-  if (blocks16) hq_launch_pdl(concat_requant_wide_kernel, (unsigned)blocks16, 256, 0, (cudaStream_t)stream, a);
+  if (blocks4) hq_launch_pdl_if(a.overlap != 0, concat_requant_kernel, (unsigned)blocks4, 256, 0, (cudaStream_t)stream, a);
+  if (blocks16) hq_launch_pdl_if(a.overlap != 0, concat_requant_wide_kernel, (unsigned)blocks16, 256, 0, (cudaStream_t)stream, a);
   return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }

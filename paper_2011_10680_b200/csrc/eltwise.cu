@@ -273,7 +273,7 @@ __device__ __forceinline__ void requant8_flat(const EltArgs& a, const Dy8 (&m)[4
 
 template <bool RES, bool MSIGNED, bool RSIGNED, bool OUT4, int SATP, bool FLAT>
 __global__ void __launch_bounds__(256) requant8_kernel(EltArgs a, int words, int lo, int hi) {
-  hq_pdl_entry();
+  if (a.overlap) hq_pdl_entry();
   // word (4 channels) of the pixel
   const int wx = FLAT ? (int)(threadIdx.x & (unsigned)(words - 1)) : (int)(blockIdx.x * blockDim.x + threadIdx.x);
   if (wx >= words) return;
@@ -539,9 +539,9 @@ cudaError_t launch_requant8_form(const EltArgs& a, dim3 grid, dim3 block, int wo
       hq_launch_pdl(requant8_staged_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP>, sm_count * (RES ? 3 : 5), 256, smem, s, a, words, lo, hi);
       return cudaGetLastError();
     }
-    hq_launch_pdl(requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, true>, (unsigned)(blocks < cap ? blocks : cap), 256, 0, s, a, words, lo, hi);
+    hq_launch_pdl_if(a.overlap != 0, requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, true>, (unsigned)(blocks < cap ? blocks : cap), 256, 0, s, a, words, lo, hi);
   } else {
-    hq_launch_pdl(requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, false>, grid, block, 0, s, a, words, lo, hi);
+    hq_launch_pdl_if(a.overlap != 0, requant8_kernel<RES, MSIGNED, RSIGNED, OUT4, SATP, false>, grid, block, 0, s, a, words, lo, hi);
   }
   return cudaGetLastError();
 }
@@ -660,9 +660,9 @@ __global__ void __launch_bounds__(256) residual_add_out32_kernel(EltArgs a) {
 // The same for channel counts that are a multiple of four, operands of 8 or 32 bits: a thread owns four channels
 // (their pairs stay in registers: the launch makes the thread count a multiple of the quads per pixel), reads
 // 16 bytes of an INT32 operand (4 of an 8-bit one) and writes 16 bytes per step, two steps in flight.
-template <int MB, int RB>   // operand bits: 8 or 32; RB = 0: no second operand
+template <int MB, int RB, bool OVERLAP>   // operand bits: 8 or 32; RB = 0: no second operand
 __global__ void __launch_bounds__(256) residual_add_out32_vec_kernel(EltArgs a) {
-  if (a.overlap) hq_pdl_entry();
+  if constexpr (OVERLAP) hq_pdl_entry();
   const long long quads = a.pixels * (a.ch >> 2);
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -699,6 +699,12 @@ __global__ void __launch_bounds__(256) residual_add_out32_vec_kernel(EltArgs a) 
   };
   for (; i + stride < quads; i += 2 * stride) { one(i); one(i + stride); }
   if (i < quads) one(i);
+}
+
+template <int MB, int RB>
+void launch_add_out32(const EltArgs& a, int grid, cudaStream_t s) {
+  if (a.overlap) hq_launch_pdl(residual_add_out32_vec_kernel<MB, RB, true>, grid, 256, 0, s, a);
+  else residual_add_out32_vec_kernel<MB, RB, false><<<grid, 256, 0, s>>>(a);
 }
 
 // Any channel count: one thread per output byte (one element at 8 bit, two at 4 bit).
@@ -1016,12 +1022,12 @@ cudaError_t hq_launch_residual_add(const EltArgs& args, int sm_count, cudaStream
       if (blocks >= mult) {
         const int g = (int)blocks;
         const int rbits = a.res ? a.res_bits : 0;
-        if (a.main_bits == 32 && rbits == 32) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<32, 32>, g, 256, 0, s, a);
-        else if (a.main_bits == 32 && rbits == 8) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<32, 8>, g, 256, 0, s, a);
-        else if (a.main_bits == 32) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<32, 0>, g, 256, 0, s, a);
-        else if (rbits == 32) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<8, 32>, g, 256, 0, s, a);
-        else if (rbits == 8) hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<8, 8>, g, 256, 0, s, a);
-        else hq_launch_pdl_if(a.overlap != 0, residual_add_out32_vec_kernel<8, 0>, g, 256, 0, s, a);
+        if (a.main_bits == 32 && rbits == 32) launch_add_out32<32, 32>(a, g, s);
+        else if (a.main_bits == 32 && rbits == 8) launch_add_out32<32, 8>(a, g, s);
+        else if (a.main_bits == 32) launch_add_out32<32, 0>(a, g, s);
+        else if (rbits == 32) launch_add_out32<8, 32>(a, g, s);
+        else if (rbits == 8) launch_add_out32<8, 8>(a, g, s);
+        else launch_add_out32<8, 0>(a, g, s);
         return cudaGetLastError();
       }
     }
