@@ -109,13 +109,17 @@ _packed = None
 
 
 def _packed_calls():
-    """hq_conv2d and hq_linear taking their structures as byte strings."""
+    """hq_conv2d, hq_linear and hq_concat_requant taking their structures as byte strings."""
     global _packed
     if _packed is None:
         assert len(_PACK_TENSOR(*[0] * 7)) == C.sizeof(hq_tensor) and len(_PACK_CONV(*[0] * 17)) == C.sizeof(hq_conv_desc)
         fns = [lib()["hq_conv2d"], lib()["hq_linear"]]           # function objects of their own
         for fn in fns:
             fn.argtypes, fn.restype = [C.c_void_p, C.c_char_p, C.c_char_p, C.c_char_p, C.c_void_p], C.c_int32
+        cat = lib()["hq_concat_requant"]
+        cat.argtypes = [C.c_void_p, C.c_int32, C.c_char_p, C.c_char_p, C.c_int32, C.c_int32, C.c_int32, C.c_char_p, C.c_void_p]
+        cat.restype = C.c_int32
+        fns.append(cat)
         _packed = fns
     return _packed
 
@@ -285,10 +289,10 @@ class Handle:
     def concat_requant(self, branches, relu, qmin, qmax, out, out_bits, out_signed):
         """`branches`: list of dicts {x, bits, signed, ch, b, c} of CUDA tensors; `out`: (n, h, w, sum ch)."""
         n = len(branches)
-        ts = (hq_tensor * n)(*[tensor_of(br["x"], br["ch"], br["bits"], br["signed"]) for br in branches])
-        ds = (hq_dyadic * n)(*[_dy(br["b"], br["c"]) for br in branches])
-        to = tensor_of(out, out.shape[3] * (2 if out_bits == 4 else 1), out_bits, out_signed)
-        return lib().hq_concat_requant(self._h, n, ts, ds, relu, qmin, qmax, C.byref(to), _stream())
+        ts = b"".join([_packed_tensor(br["x"], br["ch"], br["bits"], br["signed"]) for br in branches])
+        ds = struct.pack("@%dP" % (2 * n), *[_ptr(br[k]) for br in branches for k in ("b", "c")])
+        to = _packed_tensor(out, out.shape[3] * (2 if out_bits == 4 else 1), out_bits, out_signed)
+        return _packed_calls()[2](self._h, n, ts, ds, relu, qmin, qmax, to, _stream())
 
     def sumpool(self, x, ch, bits, signed, k, stride, pad, out):
         ti = tensor_of(x, ch, bits, signed)

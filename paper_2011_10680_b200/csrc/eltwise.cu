@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(256) residual_add_out32_kernel(EltArgs a) {
 // (their pairs stay in registers: the launch makes the thread count a multiple of the quads per pixel), reads
 // 16 bytes of an INT32 operand (4 of an 8-bit one) and writes 16 bytes per step, two steps in flight.
 template <int MB, int RB, bool OVERLAP>   // operand bits: 8 or 32; RB = 0: no second operand
-__global__ void __launch_bounds__(256) residual_add_out32_vec_kernel(EltArgs a) {
+__global__ void __launch_bounds__(256, 4) residual_add_out32_vec_kernel(EltArgs a) {
   if constexpr (OVERLAP) hq_pdl_entry();
   const long long quads = a.pixels * (a.ch >> 2);
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -684,10 +684,7 @@ __global__ void __launch_bounds__(256) residual_add_out32_vec_kernel(EltArgs a) 
       for (int j = 0; j < 4; ++j) v[j] = is_signed ? (int)(signed char)(t >> (8 * j)) : (int)((t >> (8 * j)) & 0xFFu);
     }
   };
-  auto one = [&](long long q) {
-    int m[4], r[4] = {0, 0, 0, 0};
-    load(a.main_t, MB, a.main_signed, q, m);
-    if (RB) load(a.res, RB, a.res_signed, q, r);
+  auto finish = [&](long long q, const int (&m)[4], const int (&r)[4]) {
     int y[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -697,8 +694,22 @@ __global__ void __launch_bounds__(256) residual_add_out32_vec_kernel(EltArgs a) 
     }
     ((int4*)a.out)[q] = make_int4(y[0], y[1], y[2], y[3]);
   };
-  for (; i + stride < quads; i += 2 * stride) { one(i); one(i + stride); }
-  if (i < quads) one(i);
+  // both steps' operands are requested before either is used
+  for (; i + stride < quads; i += 2 * stride) {
+    int m0[4], m1[4], r0[4] = {0, 0, 0, 0}, r1[4] = {0, 0, 0, 0};
+    load(a.main_t, MB, a.main_signed, i, m0);
+    if (RB) load(a.res, RB, a.res_signed, i, r0);
+    load(a.main_t, MB, a.main_signed, i + stride, m1);
+    if (RB) load(a.res, RB, a.res_signed, i + stride, r1);
+    finish(i, m0, r0);
+    finish(i + stride, m1, r1);
+  }
+  if (i < quads) {
+    int m[4], r[4] = {0, 0, 0, 0};
+    load(a.main_t, MB, a.main_signed, i, m);
+    if (RB) load(a.res, RB, a.res_signed, i, r);
+    finish(i, m, r);
+  }
 }
 
 template <int MB, int RB>
