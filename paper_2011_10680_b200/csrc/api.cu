@@ -235,7 +235,7 @@ static void plan_wide_adds(hq_network* net) {
     const int j = l.in0;
     const hq_layer& cv = net->layers[j];
     const hq_tensor& o = net->outs[j];
-    if (cv.op != HQ_OP_CONV || o.bits != 32 || cv.in1 >= 0 || cv.in0 < 0 || o.c % 16 != 0 || net->outs[l.in1].bits == 4) continue;
+    if (cv.op != HQ_OP_CONV || o.bits != 32 || cv.in1 >= 0 || cv.in0 < 0 || net->outs[l.in1].bits == 4) continue;
     if (!l.rescale0.b || !l.rescale0.c || !l.rescale1.b || !l.rescale1.c) continue;
     bool alone = true;
     for (int m = j + 1; m < n; ++m) alone = alone && (m == i || !reads(m, j));
@@ -244,7 +244,7 @@ static void plan_wide_adds(hq_network* net) {
     a.n = in.n; a.h = in.h; a.w = in.w; a.cin = in.c; a.in_bits = net->stored_wide[cv.in0] ? 8 : in.bits; a.cout = o.c;
     a.kh = cv.conv.kh; a.kw = cv.conv.kw; a.stride = cv.conv.stride; a.pad = cv.conv.pad; a.ho = o.h; a.wo = o.w; a.out_bits = 32;
     a.in_slack = 1;
-    if (!alone || !hq_conv_tc_supported(a) || (o.c + 127) / 128 > net->h->sm_count) continue;
+    if (!alone || !hq_conv_wide_applies(a, net->h->sm_count)) continue;
     net->wide_conv[i] = j;
     net->run_by_add[j] = 1;
     net->wide_sum_read[i] = i == n - 1;

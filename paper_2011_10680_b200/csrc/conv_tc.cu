@@ -1494,6 +1494,12 @@ static bool prefers_patches(const ConvArgs& a) {
 }
 bool hq_conv_tc_declines(const ConvArgs& a) { return hq_conv_tc_small_im2col(a) || prefers_patches(a); }
 
+bool hq_conv_wide_applies(const ConvArgs& a, int sm_count) {
+  // (the smallest tile with its weights in the stages always leaves room for three of them beside the boxes)
+  static_assert(kSmemBudget - kWideWarps * (kWideSlots * kWideBox + 2 * kWideQBox) >= 3 * (kTileC + 64) * 128, "stages of the INT32 shape");
+  return hq_conv_tc_supported(a) && !hq_conv_tc_declines(a) && a.cout % 16 == 0 && (a.cout + kTileC - 1) / kTileC <= sm_count;
+}
+
 hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream) {
   if (!hq_conv_tc_supported(a)) return HQ_ERR_UNSUPPORTED;
   if (!load_driver_entry_points()) return HQ_ERR_CUDA;

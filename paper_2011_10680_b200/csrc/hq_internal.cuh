@@ -147,6 +147,9 @@ bool hq_conv_tc_supported(const ConvArgs& a);
 // 128 KiB through an im2col-mode map.  Such a layer runs in its lowered (patch-matrix) form.
 bool hq_conv_tc_small_im2col(const ConvArgs& a);
 bool hq_conv_tc_declines(const ConvArgs& a);      // ... or whose patch matrix is cheaper than its short rows
+// The layer can end in the INT32 residual add (ConvArgs::wide): there is no other kernel for that, so the launcher takes
+// exactly these.
+bool hq_conv_wide_applies(const ConvArgs& a, int sm_count);
 // Tensor-core path; returns HQ_OK, HQ_ERR_UNSUPPORTED (nothing was launched) or HQ_ERR_CUDA.
 hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t s);
 // One tile per CTA, reduction split over a cluster: small problems (conv_small.cu).  Same status convention.
