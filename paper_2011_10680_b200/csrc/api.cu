@@ -251,7 +251,8 @@ static void plan_wide_adds(hq_network* net) {
     for (int m = i + 1; m < n; ++m) {
       if (!reads(m, i)) continue;
       const hq_layer& r = net->layers[m];
-      const bool bytes = net->outs[m].bits == 8 || net->stored_wide[m];
+      // (a clamp outside the type is refused when the layer runs, by itself)
+      const bool bytes = (net->outs[m].bits == 8 || net->stored_wide[m]) && type_range_ok(8, net->outs[m].is_signed, r.qmin, r.qmax);
       if (net->wide_requant[i] < 0 && r.op == HQ_OP_REQUANT && bytes && m != n - 1 && r.rescale0.b && r.rescale0.c) {
         net->wide_requant[i] = m;
         net->run_by_add[m] = 1;
