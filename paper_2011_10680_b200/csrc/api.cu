@@ -36,7 +36,7 @@ inline long long tensor_bytes(int n, int h, int w, int c, int bits) {
 hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, hq_tensor* out, void* stream,
                       void* scratch = nullptr, size_t scratch_bytes = 0, const void* res_narrow = nullptr,
                       const void* wgt_widened = nullptr, bool in_slack = false, const WideArgs* wide = nullptr,
-                      bool wide_sum = true) {
+                      bool wide_sum = true, bool pairs = false) {
   if (!h || !d) return HQ_ERR_INVALID_ARG;
   hq_status st = check_tensor(in, true, true, false);
   if (st != HQ_OK) return st;
@@ -87,7 +87,7 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
     const hq_status st4 = hq_launch_conv_small(h, a, s);
     if (st4 != HQ_ERR_UNSUPPORTED || h->conv_path == 4) return st4;
   }
-  if (h->conv_path == 0 && a.wgt_widened && hq_conv_pairs_applies(a, h->sm_count)) {
+  if (h->conv_path == 0 && pairs) {
     const hq_status st5 = hq_launch_conv_pairs(h, a, s);
     if (st5 != HQ_ERR_UNSUPPORTED) return st5;
   }
@@ -170,6 +170,7 @@ struct hq_network {
   std::vector<void*> res_narrow;     // per conv layer with a fused 8-bit residual: its narrow residual pairs (owned)
   std::vector<void*> narrow0, narrow1; // per ADD / REQUANT layer with 8-bit operands: narrow pairs of the two branches (owned)
   std::vector<void*> wgt_widened;    // per 4-bit conv layer on the tensor-core path: its weights, one byte per value (owned)
+  std::vector<char> pairs;           // per conv layer: it runs over pixel pairs (hq_conv_pairs_applies)
   std::vector<char> stored_wide;     // per layer: its 4-bit output is kept one value per byte (all consumers are such convs)
   // ADD layers with an INT32 result that run behind the convolution producing their main operand (see plan_wide_adds):
   // the convolution's layer or -1; the REQUANT layer done along with it or -1; whether somebody else reads the sum
@@ -517,6 +518,7 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
   net->bytes.resize(n_layers);
   net->res_narrow.assign(n_layers, nullptr);
   net->wgt_widened.assign(n_layers, nullptr);
+  net->pairs.assign(n_layers, 0);
   net->stored_wide.assign(n_layers, 0);
   net->narrow0.assign(n_layers, nullptr);
   net->narrow1.assign(n_layers, nullptr);
@@ -543,6 +545,7 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
           ConvArgs a{};
           a.n = batch; a.h = in.h; a.w = in.w; a.cin = in.c; a.in_bits = in.bits; a.cout = d.cout; a.kh = d.kh; a.kw = d.kw;
           a.stride = d.stride; a.pad = d.pad; a.ho = o.h; a.wo = o.w; a.out_bits = o.bits; a.in_slack = l.in0 >= 0;
+          net->pairs[i] = l.in1 < 0 && !hq_conv_small_wanted(a, h->sm_count) && hq_conv_pairs_applies(a, h->sm_count);
           if (hq_conv_widen4_applies(a)) {
             const size_t need = hq_conv_widen4_bytes(a);
             if (need > net->scratch_bytes) net->scratch_bytes = need;
@@ -551,13 +554,6 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
             if (!wbuf) { st = HQ_ERR_WORKSPACE; break; }
             net->wgt_widened[i] = wbuf;
             if (hq_launch_widen_weights(d.w, wvals, wbuf, h->sm_count, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
-          } else if (l.in1 < 0 && !hq_conv_small_wanted(a, h->sm_count) && hq_conv_pairs_applies(a, h->sm_count)) {
-            a.wgt = d.w; a.bias = d.bias; a.b = d.requant.b; a.c = d.requant.c;
-            if (!a.b || !a.c) break;
-            void* wbuf = net_alloc(net, hq_conv_pairs_prepared_bytes(), i);
-            if (!wbuf) { st = HQ_ERR_WORKSPACE; break; }
-            net->wgt_widened[i] = wbuf;
-            if (hq_prepare_conv_pairs(a, wbuf, nullptr) != cudaSuccess) { st = HQ_ERR_CUDA; break; }
           } else if (hq_conv_s2d_applies(a)) {
             const size_t need = hq_conv_s2d_bytes(a);
             if (need > net->scratch_bytes) net->scratch_bytes = need;
@@ -728,7 +724,8 @@ static hq_status run_layers(hq_network* net, const hq_tensor* images, hq_tensor*
         h->tile_order = net->tile_order[i];
         if (l.op == HQ_OP_LINEAR) { in.c = in.h * in.w * in.c; in.h = 1; in.w = 1; 
           st = d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0 ? conv_common(h, &in, &d, &o, s, nullptr, 0, nullptr, nullptr, l.in0 >= 0) : HQ_ERR_INVALID_ARG; }
-        else st = conv_common(h, &in, &d, &o, s, net->scratch, net->scratch_bytes, net->res_narrow[i], in_wide ? nullptr : net->wgt_widened[i], l.in0 >= 0);
+        else st = conv_common(h, &in, &d, &o, s, net->scratch, net->scratch_bytes, net->res_narrow[i], in_wide ? nullptr : net->wgt_widened[i], l.in0 >= 0, nullptr, true,
+                              net->pairs[i] != 0);
         h->tile_order = callers_order;
         break;
       }

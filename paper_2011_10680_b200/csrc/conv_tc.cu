@@ -889,7 +889,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         int wx = 0, tap_x = 0, left = p.cchunks;
         for (int kb = 0; kb < p.w_blocks; ++kb) {
           const uint32_t w_dst = tiles + p.wres_off + (uint32_t)kb * w_bytes;
-          if (p.fold) {
+          if (p.pairs) {           // block (filter row, half of the four pixels): rows of output 2q, then of output 2q + 1
+            tma_load_3d(w_dst, &map_w, bar, (kb & 1) * 128, kb >> 1, 0);
+            tma_load_3d(w_dst + 64 * 128, &map_w, bar, (kb & 1) * 128 - 64, kb >> 1, 0);
+          } else if (p.fold) {
             tma_load_2d(w_dst, &map_w, bar, wx, 0);
             tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx, 0);
           } else {
@@ -1265,10 +1268,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     // per-channel constants, once per kernel
     ChanConst k{};
     uint32_t fast = (p.out_bits != 32) ? 1u : 0u;
-    k.bias = (ch_live && p.bias) ? p.bias[ch] : 0;
+    const int pch = p.pairs ? ch & 63 : ch;       // (pixel pairs: both outputs of a pair have the layer's channels)
+    k.bias = (ch_live && p.bias) ? p.bias[pch] : 0;
     if (p.out_bits != 32) {
-      k.b = ch_live ? p.b[ch] : 0;
-      const int cc = ch_live ? p.c[ch] : 32;
+      k.b = ch_live ? p.b[pch] : 0;
+      const int cc = ch_live ? p.c[pch] : 32;
       k.sh = cc;
       k.r0 = (long long)k.bias * (long long)k.b + (1LL << (cc - 1));
       if (p.res) {
@@ -1736,7 +1740,14 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   } else {
     if (!encode_im2col_map(&map_x, a, p.bkb, p.pt >> p.duo)) return HQ_ERR_CUDA;
   }
-  if (!encode_rows_map(&map_w, a.wgt, a.cout, p.pairs ? 6 * 128 : (long long)a.kh * a.kw * a.cin, p.bkb, p.fold ? 64 : kTileC, swz)) return HQ_ERR_CUDA;
+  if (p.pairs) {
+    // weights (filter row of 3 x 64 bytes, 3 rows, 64 channels), box = 128 bytes of one filter row of every channel
+    const cuuint64_t dims[3] = {192, 3, 64}, strides[2] = {192, 576};
+    const cuuint32_t box[3] = {128, 1, 64}, estr[3] = {1, 1, 1};
+    if (g_encode_tiled(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(a.wgt), dims, strides, box, estr,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return HQ_ERR_CUDA;
+  } else if (!encode_rows_map(&map_w, a.wgt, a.cout, (long long)a.kh * a.kw * a.cin, p.bkb, p.fold ? 64 : kTileC, swz)) return HQ_ERR_CUDA;
   map_out = map_w; map_res = map_w; map_q = map_w;                    // valid placeholders when a path is not staged
   // (with rtm the residual tile is an MMA operand and, later, the output box: 128-byte swizzle both ways)
   const CUtensorMapSwizzle box_swz = p.rtm ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;

@@ -112,7 +112,7 @@ struct ConvArgs {
   const void* wgt_widened;   // weights as the lowered form wants them, prepared once by a network, or NULL: 4-bit weights widened
                              // to one byte per value; for the first-layer form the virtual-channel weights and constants
   const WideArgs* wide;      // non-NULL: the convolution ends in the INT32 residual add (see WideArgs)
-  int32_t pairs;             // nonzero: the pixel-pair form (hq_conv_pairs_applies): "pixels" are pairs, "channels" those of both
+  int32_t pairs;             // nonzero: the pixel-pair form (hq_conv_pairs_applies): "pixels" are pairs, "channels" those of both; weights and constants are the layer's own
   int32_t in_slack;          // nonzero: a layer inside a network; the allocation behind `in` goes on for at least kIm2colMinTensorBytes + one image
   int32_t wgt_fresh;         // nonzero: the weights are written by the launch just before: they are not kept resident (fetched ahead of its end)
   int32_t pad_after_delta;   // padding after the last row/column minus `pad`
@@ -174,10 +174,8 @@ size_t hq_conv_s2d_bytes(const ConvArgs& a);
 hq_status hq_launch_conv_s2d(hq_handle* h, const ConvArgs& a, void* scratch, cudaStream_t s);
 size_t hq_conv_s2d_prepared_bytes(const ConvArgs& a);
 cudaError_t hq_prepare_conv_s2d(const ConvArgs& a, void* buf, cudaStream_t s);
-// 3x3 / stride 1 layers over 64 channels, 64 to 64, as convolutions over pixel pairs; weights prepared once by a network.
+// 3x3 / stride 1 layers over 64 channels, 64 to 64, as convolutions over pixel pairs (inside networks).
 bool hq_conv_pairs_applies(const ConvArgs& a, int sm_count);
-size_t hq_conv_pairs_prepared_bytes();
-cudaError_t hq_prepare_conv_pairs(const ConvArgs& a, void* buf, cudaStream_t s);
 hq_status hq_launch_conv_pairs(hq_handle* h, const ConvArgs& a, cudaStream_t s);
 // 4-bit operands: widen to bytes in scratch, then the tensor-core kernel.
 bool hq_conv_widen4_applies(const ConvArgs& a);

@@ -305,27 +305,12 @@ hq_status hq_launch_conv_s2d(hq_handle* h, const ConvArgs& a, void* scratch, cud
 // 3x3 / stride 1 / pad 1, 64 channels to 64, as a convolution over PIXEL PAIRS (128 bytes): virtual channel o*64 + ch of pair q is
 // channel ch of output 2q + o, the same byte of the NHWC output read as rows of 128.  An output pair reads the four pixels
 // 2q-1 .. 2q+2 of three rows: virtual weight row (o, ch), position t = 0..3 is w[ch][r][t - o] (zero outside 0..2), K = 3*4*64.
+// Nothing is prepared for that: 128 bytes of a virtual row are 128 bytes of the filter row's 192 from 128 h - 64 o on, zeros
+// beyond its ends, which is what a copy of the weight tensor itself with that (negative or overhanging) start delivers.
 // Against the plain form, whose 64 channels fill half of the accumulator lanes (the weight rows are loaded twice): all 128 lanes
 // do work of their own, 24 instead of 36 MMAs per 512 pixels, and half as many operand rows of twice the length.
-// Measured per launch in the strip form of conv_tc.cu, 56x56: 256 images 58.7 -> 37 us.
+// Measured per launch in the strip form of conv_tc.cu, 56x56: 256 images 59 -> 50 us.
 // ------------------------------------------------------------------------------------------------
-namespace {
-constexpr int kPairK = 3 * 4 * 64;
-__global__ void pair_weights_kernel(const signed char* __restrict__ w, signed char* __restrict__ out, const int32_t* __restrict__ bias,
-                                    const int32_t* __restrict__ b, const int32_t* __restrict__ c, int32_t* __restrict__ consts) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 128 * kPairK) return;
-  const int ci = i & 63, t = (i >> 6) & 3, v = i / kPairK, r = (i - v * kPairK) >> 8;
-  const int o = v >> 6, ch = v & 63, s = t - o;
-  out[i] = s >= 0 && s < 3 ? w[((ch * 3 + r) * 3 + s) * 64 + ci] : (signed char)0;
-  if (i < 128) {
-    consts[i] = bias ? bias[i & 63] : 0;
-    consts[128 + i] = b[i & 63];
-    consts[256 + i] = c[i & 63];
-  }
-}
-}  // namespace
-
 bool hq_conv_pairs_applies(const ConvArgs& a, int sm_count) {
   if (a.in_bits != 8 || a.cin != 64 || a.cout != 64 || a.kh != 3 || a.kw != 3 || a.stride != 1 || a.pad != 1 || a.pitch_w || a.res || a.wide ||
       a.out_bits != 8 || (a.w & 1) || a.n >= 65536) return false;
@@ -333,17 +318,9 @@ bool hq_conv_pairs_applies(const ConvArgs& a, int sm_count) {
   const int rows = lg ? 256 >> lg : 1;
   return lg && 4LL * a.n * ((a.h + rows - 1) / rows) >= sm_count;
 }
-size_t hq_conv_pairs_prepared_bytes() { return 128 * kPairK + 3 * 128 * 4; }
-cudaError_t hq_prepare_conv_pairs(const ConvArgs& a, void* buf, cudaStream_t s) {
-  pair_weights_kernel<<<(128 * kPairK + 255) / 256, 256, 0, s>>>((const signed char*)a.wgt, (signed char*)buf, a.bias, a.b, a.c,
-                                                               (int32_t*)((unsigned char*)buf + 128 * kPairK));
-  return cudaGetLastError();
-}
 hq_status hq_launch_conv_pairs(hq_handle* h, const ConvArgs& a, cudaStream_t s) {
   ConvArgs t = a;
-  const int32_t* consts = (const int32_t*)((const unsigned char*)a.wgt_widened + 128 * kPairK);
-  t.pairs = 1; t.wgt = a.wgt_widened; t.wgt_widened = nullptr; t.w = a.w / 2; t.wo = a.wo / 2; t.cin = 128; t.cout = 128;
-  t.bias = consts; t.b = consts + 128; t.c = consts + 256;
+  t.pairs = 1; t.w = a.w / 2; t.wo = a.wo / 2; t.cin = 128; t.cout = 128;
   return hq_launch_conv_tc(h, t, s);
 }
 

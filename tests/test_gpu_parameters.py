@@ -1,6 +1,9 @@
 """When parameters are read, and which layers a network may run behind others: everything against the CPU oracle, bit-exact."""
 from __future__ import annotations
 
+import copy
+
+import numpy as np
 import pytest
 
 from paper_2011_10680_b200 import inputs
@@ -18,6 +21,20 @@ def hq():
     h = binding.Handle(0)
     yield h
     h.close()
+
+
+def _table(bd, image_hw, classes=16):
+    x = bd.avgpool(len(bd.layers) - 1)
+    bd.conv(x, classes, 1, 1, 0, 8, relu=False, out_bits=32, op="linear")
+    ids = range(len(bd.layers))
+    return dict(layers=bd.layers, image_hw=image_hw, classes=classes, depth=0, conv_bits=[8], shapes=[bd.shape[i] for i in ids],
+                bits=[bd.bits[i] for i in ids])
+
+
+def _builder(seed, image_hw):
+    bd = inputs._Builder(seed)
+    bd.scale[-1], bd.shape[-1], bd.bits[-1] = 2.0 ** -4, (image_hw, image_hw, 3), 8
+    return bd
 
 
 def test_int32_add_behind_a_convolution_of_short_rows(hq):
@@ -45,3 +62,45 @@ def test_a_clamp_outside_its_type_is_refused_behind_an_int32_add(hq):
                 hq.sync()
         finally:
             net.close()
+
+
+def _rewrite_and_compare(hq, table, batch, change):
+    """Run a network, overwrite the parameters of some layers in place, run it again: the new values count."""
+    from oracle.network import run_network
+    from paper_2011_10680_b200 import binding
+    images = inputs.random_images(21, batch, table["image_hw"])
+    changed = copy.deepcopy(table)
+    change(changed["layers"])
+    want = [run_network(t, images)[-1] for t in (table, changed)]
+    assert not np.array_equal(*want)
+    net, other = binding.Network(hq, table, batch), binding.Network(hq, changed, batch)
+    try:
+        d_img = binding.to_device(images)
+        logits = binding.alloc_out(*net.logits_shape, 32, 1)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for ref in want:
+                assert net.run(d_img, logits, None) == binding.HQ_OK
+                hq.sync()
+                assert np.array_equal(logits.cpu().numpy().reshape(ref.shape), ref)
+                for mine, theirs in zip(net._keep, other._keep):
+                    for key, tensor in mine.items():
+                        if tensor is not None:
+                            tensor.copy_(theirs[key])
+                torch.cuda.synchronize()
+        net.check_guards()
+    finally:
+        net.close()
+        other.close()
+
+
+@pytest.mark.parametrize("hw,batch", [(56, 11), (26, 41)])
+def test_pixel_pair_layers_follow_their_parameters(hq, hw, batch):
+    """3x3 layers over 64 channels in the pixel-pair form of a network: weights, bias and pairs are read at every run."""
+    bd = _builder(hw, 2 * hw)
+    x = bd.conv(-1, 64, 3, 2, 1, 8, relu=True, out_bits=8)
+    bd.conv(x, 64, 3, 1, 1, 8, relu=True, out_bits=8)
+
+    def change(layers):
+        l = layers[1]
+        l["wgt"], l["bias"], l["b"], l["c"] = np.ascontiguousarray(l["wgt"][::-1]), l["bias"][::-1].copy(), np.roll(l["b"], 1), np.roll(l["c"], 1)
+    _rewrite_and_compare(hq, _table(bd, 2 * hw), batch, change)
