@@ -10,6 +10,8 @@
 // pointers and keeps several pixels in flight; neighbouring lanes read neighbouring pieces of the dense branch
 // tensor and write neighbouring words of the output row.  The pixel loop is compiled per operand signedness, form
 // of the arithmetic and output type and chosen once per thread.  Integer arithmetic only.
+#include <climits>
+
 #include "hq_internal.cuh"
 
 namespace {
@@ -30,7 +32,7 @@ struct ConcatArgs {
   int32_t n_br, out_ch, out_bits, relu, qmin, qmax;
   long long pixels;
   void* out;
-  const int4* narrow;   // per OUTPUT channel {m, a, s, valid} from concat_narrow_kernel (8-/4-bit branches), or NULL
+  const int4* narrow;   // per OUTPUT channel {m, a, s, tag} from concat_narrow_kernel (8-/4-bit branches), or NULL
   int32_t sat;          // 1: relu and the clamp bounds equal a saturating conversion to the 8-bit output type
   int32_t overlap;      // 1: this launch overlaps its neighbours (hq_pdl_entry)
   int32_t rev;          // 1: pixels are walked from the last to the first (the handle's tile order): same results
@@ -39,7 +41,12 @@ struct ConcatArgs {
 // Narrow multiply-add pairs for the 8- and 4-bit branches.  A stored 8-bit value r has 256 possible values, so
 // dn(r, b, c) can often be written (r*m + a) >> s in 32-bit arithmetic (on unsigned words for unsigned operands), m ~ b / 2^8: one warp per output channel
 // tries the two neighbouring multipliers against the 64-bit definition for every r and records the one that agrees
-// everywhere (valid = 1), else valid = 0 and the channel keeps the wide form.  c >= 41 makes the term 0 for every r.
+// everywhere, else tag = 0 and the channel keeps the wide form.  c >= 41 makes the term 0 for every r.
+// A network searches once, when it is built, and its caller may rewrite b and c in place afterwards: an entry names the pair
+// it was found for (tag = b with the top bit set, s = c - 8, or 0 for c >= 41) and is used for that pair only.
+__device__ __forceinline__ int narrow_tag(int b) { return b | INT_MIN; }
+__device__ __forceinline__ bool narrow_is_for(const int4& n, int b, int c) { return n.w == narrow_tag(b) && (c >= 41 ? n.z == 0 : n.z > 0 && n.z == c - 8); }
+
 __global__ void __launch_bounds__(128) concat_narrow_kernel(const __grid_constant__ ConcatArgs a, int4* out) {
   const int oc = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (oc >= a.out_ch) return;
@@ -55,7 +62,7 @@ __global__ void __launch_bounds__(128) concat_narrow_kernel(const __grid_constan
     const int c = a.br[i].c[k];
     const int r_lo = a.br[i].is_signed ? -128 : 0;
     if (c >= 41) {
-      res = make_int4(0, 0, 0, 1);                     // |r*b| < 2^39 <= 2^(c-2)
+      res = make_int4(0, 0, 0, narrow_tag((int)b));    // |r*b| < 2^39 <= 2^(c-2)
     } else if (c >= 9 && c <= 38) {
       const int s = c - 8, add = 1 << (s - 1);
       const long long m0 = b >> 8, m1 = m0 + 1;
@@ -72,8 +79,8 @@ __global__ void __launch_bounds__(128) concat_narrow_kernel(const __grid_constan
       }
       ok0 = __all_sync(0xffffffffu, ok0);
       ok1 = __all_sync(0xffffffffu, ok1);
-      if (ok0) res = make_int4((int)m0, add, s, 1);
-      else if (ok1) res = make_int4((int)m1, add, s, 1);
+      if (ok0) res = make_int4((int)m0, add, s, narrow_tag((int)b));
+      else if (ok1) res = make_int4((int)m1, add, s, narrow_tag((int)b));
     }
   }
   if (lane == 0) out[oc] = res;
@@ -179,7 +186,7 @@ __device__ __forceinline__ void concat_branch(const ConcatArgs& a, const int i) 
   bool narrow = a.narrow != nullptr && bits != 32 && nk == N;
   if (narrow) {
 #pragma unroll
-    for (int j = 0; j < N; ++j) narrow = narrow && __ldg(&a.narrow[off + j].w) != 0;
+    for (int j = 0; j < N; ++j) narrow = narrow && narrow_is_for(__ldg(a.narrow + off + j), bb[j], ss[j]);
     if (narrow) {
 #pragma unroll
       for (int j = 0; j < N; ++j) { const int4 t = __ldg(a.narrow + off + j); bb[j] = t.x; hh[j] = t.y; ss[j] = t.z; }
@@ -406,7 +413,7 @@ __device__ __forceinline__ void concat_w4(const ConcatArgs& a, const int i) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) same = same && __ldg(a.br[i].b + kc + j) == b0 && __ldg(a.br[i].c + kc + j) == c0;
     const int4 n0 = __ldg(a.narrow + a.br[i].ch_off);
-    if (__syncthreads_and(same && n0.w != 0)) {
+    if (__syncthreads_and(same && narrow_is_for(n0, b0, c0))) {
       if (is_signed) { if (a.sat) concat_uniform8<true, 0>(a, i, n0.x, n0.y, n0.z, lo, hi); else concat_uniform8<true, 1>(a, i, n0.x, n0.y, n0.z, lo, hi); }
       else { if (a.sat) concat_uniform8<false, 0>(a, i, n0.x, n0.y, n0.z, lo, hi); else concat_uniform8<false, 1>(a, i, n0.x, n0.y, n0.z, lo, hi); }
       return;
@@ -425,7 +432,7 @@ __device__ __forceinline__ void concat_w4(const ConcatArgs& a, const int i) {
   bool narrow = a.narrow != nullptr && BITS != 32;
   if (narrow) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) narrow = narrow && __ldg(&a.narrow[off + j].w) != 0;
+    for (int j = 0; j < 4; ++j) narrow = narrow && narrow_is_for(__ldg(a.narrow + off + j), bb[j], ss[j]);
     if (narrow) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) { const int4 t = __ldg(a.narrow + off + j); bb[j] = t.x; hh[j] = t.y; ss[j] = t.z; }

@@ -104,3 +104,25 @@ def test_pixel_pair_layers_follow_their_parameters(hq, hw, batch):
         l = layers[1]
         l["wgt"], l["bias"], l["b"], l["c"] = np.ascontiguousarray(l["wgt"][::-1]), l["bias"][::-1].copy(), np.roll(l["b"], 1), np.roll(l["c"], 1)
     _rewrite_and_compare(hq, _table(bd, 2 * hw), batch, change)
+
+
+@pytest.mark.parametrize("batch", [2, 21])
+@pytest.mark.parametrize("shifts", [None, (45, 8)])
+def test_concatenations_follow_their_pairs(hq, batch, shifts):
+    """The pairs of a concatenation's branches are read at every run, below and above the size that works with narrow pairs;
+    from a pair that scales everything to zero to one with the same multiplier and the smallest shift without a narrow form."""
+    bd = _builder(41, 42)
+    x = bd.conv(-1, 48, 3, 1, 0, 8, relu=True, out_bits=8)
+    cat = bd.concat([bd.conv(x, 80, 1, 1, 0, 8, relu=True, out_bits=8), x])
+    if shifts:
+        for c in bd.layers[cat]["cs"]:
+            c[::2] = shifts[0]
+
+    def change(layers):
+        if shifts:
+            for c in layers[cat]["cs"]:
+                c[::2] = shifts[1]
+            return
+        layers[cat]["bs"] = [np.roll(b, 3) for b in layers[cat]["bs"]]
+        layers[cat]["cs"] = [c + 1 for c in layers[cat]["cs"]]
+    _rewrite_and_compare(hq, _table(bd, 42), batch, change)
