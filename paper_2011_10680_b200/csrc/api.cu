@@ -64,6 +64,9 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
   }
   ConvArgs a{};
   a.in_slack = in_slack ? 1 : 0;
+  // A caller may write parameters on the stream and call at once.  (A network's own layers follow its first launch, which has
+  // waited for whatever came before it.)
+  a.params_late = in_slack ? 0 : 1;
   a.in = in->data; a.n = in->n; a.h = in->h; a.w = in->w; a.cin = in->c; a.in_bits = in->bits; a.in_signed = in->is_signed;
   a.wgt = d->w; a.wgt_widened = wgt_widened; a.cout = d->cout; a.kh = d->kh; a.kw = d->kw; a.stride = d->stride; a.pad = d->pad;
   a.bias = d->bias; a.b = d->requant.b; a.c = d->requant.c;
@@ -112,6 +115,7 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
         hq_launch_residual_narrow(a.rb, a.rc, a.res_signed, a.cout, h->narrow_pairs, s) == cudaSuccess) {
       a.res_narrow = h->narrow_pairs;
       a.res_narrow_fresh = 1;
+      a.params_late = 0;                       // (that launch has waited for the one before it)
     }
     const hq_status st = hq_launch_conv_tc(h, a, s);
     if (st != HQ_ERR_UNSUPPORTED) return st;

@@ -688,7 +688,7 @@ hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t str
   p.nkb = s.nkb; p.lg_split = s.lg_split; p.stages = s.stages; p.pt = s.pt; p.c_tiles = s.c_tiles;
   while ((1 << p.lg_cols) < (s.pt >> s.lg_split)) ++p.lg_cols;
   p.fold = s.fold;
-  p.x_bits = a.in_bits; p.x_signed = a.in_signed; p.params_late = a.in_slack ? 0 : 1;      // (a network's parameters are older)
+  p.x_bits = a.in_bits; p.x_signed = a.in_signed; p.params_late = a.params_late;
   const void* wgt = (a.in_bits == 4 && a.wgt_widened) ? a.wgt_widened : a.wgt;
   if (a.in_bits == 4 && !a.wgt_widened) p.w4 = a.wgt;
   const int stage_bytes = (kTileC + s.pt) * s.bkb;

@@ -113,6 +113,7 @@ struct TcParams {
   const void* res; int32_t res_bits, res_signed; const int32_t* rb; const int32_t* rc;
   const int4* res_narrow;   // optional per-channel {m, a, s, valid} from residual_narrow_kernel
   int32_t narrow_fresh;     // 1: the pairs are written by the kernel launched just before this one
+  int32_t params_late;      // 1: so may be weights, bias or pairs (see ConvArgs)
   int32_t relu, qmin, qmax;
   void* out; int32_t out_bits;
   void* q_out; const int32_t* qb; const int32_t* qc; int32_t q_lo, q_hi, q_sat;   // wide: the stream requantized to bytes, or NULL
@@ -862,8 +863,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   // resources.  The threads that read what the previous kernel wrote -- the producer lane (activations and
   // residual tiles by TMA) and epilogue warps that load a residual directly -- wait for that grid to complete
   // first; the other roles only consume what arrives behind the producer's barriers.  The next kernel's CTAs
-  // may start filling SMs as ours leave.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // may start filling SMs as ours leave.  Weights and constants are read ahead of that inside a network; a call of its own
+  // (params_late) may follow the kernel that wrote them: its producer and epilogue wait before they read those too, and the
+  // next kernel is let in after the producer's wait only (a network's second layer would read its own parameters at once).
+  if (!p.params_late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -883,6 +886,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       int ow = px_first - img * p.howo - oh * p.wo;
       const int step = p_step * p.pt;
       const int d_img = step / p.howo, d_oh = (step - d_img * p.howo) / p.wo, d_ow = step - d_img * p.howo - d_oh * p.wo;
+      if (p.params_late) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      }
       if (p.wres) {              // the channel tile's weights for every K block, once
         const uint32_t bar = smem_u32(&ctl.wfull);
         mbar_expect_tx(bar, (uint32_t)p.w_blocks * w_bytes);
@@ -902,8 +909,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           if (--left == 0) { left = p.cchunks; tap_x += p.cin; wx = tap_x; }
         }
       }
-      // The resident weights above do not wait for the previous kernel: weights are never written by the launch
-      // immediately before this one (the helper kernels that prepare weights are always followed by another launch).
+      // The resident weights above do not wait for the previous kernel unless it may have written them (params_late; the
+      // helper kernels that prepare weights are always followed by another launch).
       // Everything below reads activations, which the previous kernel may still be writing.
       asm volatile("griddepcontrol.wait;" ::: "memory");
       const unsigned long long pol_first = policy_evict_first();
@@ -1236,6 +1243,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const bool ch_live = ch < p.C;
     const bool warp_live = (c_tile * kTileC + cq * 32) < p.C; // warp-uniform
     const int lo = p.relu ? (p.qmin > 0 ? p.qmin : 0) : p.qmin, hi = p.qmax;
+    if (p.params_late) asm volatile("griddepcontrol.wait;" ::: "memory");     // (the constants below)
 
     if constexpr (WIDE) {
       if (half < p.halves) {
@@ -1707,6 +1715,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.res = a.res; p.res_bits = a.res_bits; p.res_signed = a.res_signed; p.rb = a.rb; p.rc = a.rc;
   p.res_narrow = (a.res && a.res_bits == 8) ? (const int4*)a.res_narrow : nullptr;
   p.narrow_fresh = a.res_narrow_fresh;
+  p.params_late = a.params_late;
   p.relu = a.relu; p.qmin = a.qmin; p.qmax = a.qmax;
   p.out = a.out; p.out_bits = a.out_bits; p.out_signed = a.out_signed;
   if (a.wide) {

@@ -153,6 +153,7 @@ hq_status hq_launch_conv_lowered(hq_handle* h, const ConvArgs& a, void* scratch,
   }
   ConvArgs t = a;
   t.in = patches; t.h = a.ho; t.w = a.wo; t.cin = Kp; t.wgt = wpad; t.kh = t.kw = 1; t.stride = 1; t.pad = 0;
+  t.params_late = 0;                     // (the padded weights are two launches old)
   return hq_launch_conv_tc(h, t, s);
 }
 
@@ -262,6 +263,7 @@ ConvArgs s2d_conv_args(const ConvArgs& a, const void* scratch) {
   t.pitch_w = 32; t.pitch_h = (long long)wp * 16; t.pitch_n = (long long)hp * wp * 16;
   t.cout = 2 * a.cout; t.wo = a.wo / 2;
   t.bias = consts; t.b = consts + 2 * a.cout; t.c = consts + 4 * a.cout;
+  t.params_late = 0;                     // (prepared before the launch that copies the image)
   return t;
 }
 }  // namespace
@@ -424,7 +426,7 @@ hq_status hq_launch_conv_widen4(hq_handle* h, const ConvArgs& a, void* scratch, 
   unsigned char* ww = xw + (x + 255) / 256 * 256;
   if (launch_widen4(a.in, x, a.in_signed, xw, a.wgt_widened ? nullptr : a.wgt, w, ww, h->sm_count, s) != cudaSuccess) return HQ_ERR_CUDA;
   ConvArgs t = a;
-  t.in = xw; t.wgt = a.wgt_widened ? a.wgt_widened : ww; t.in_bits = 8; t.wgt_fresh = a.wgt_widened ? 0 : 1;
+  t.in = xw; t.wgt = a.wgt_widened ? a.wgt_widened : ww; t.in_bits = 8; t.wgt_fresh = a.wgt_widened ? 0 : 1; t.params_late = 0;
   const hq_status st = hq_launch_conv_tc(h, t, s);
   if (st != HQ_ERR_UNSUPPORTED || !hq_conv_lowering_applies(t)) return st;
   return hq_launch_conv_lowered(h, t, xw + widen4_copy_bytes(a), s);      // declined by the direct kernel: patch matrix

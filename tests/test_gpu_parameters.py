@@ -126,3 +126,71 @@ def test_concatenations_follow_their_pairs(hq, batch, shifts):
         layers[cat]["bs"] = [np.roll(b, 3) for b in layers[cat]["bs"]]
         layers[cat]["cs"] = [c + 1 for c in layers[cat]["cs"]]
     _rewrite_and_compare(hq, _table(bd, 42), batch, change)
+
+
+@pytest.mark.parametrize("writer", ["library", "torch"])
+@pytest.mark.parametrize("cfg", [
+    # path, n, hw, cin, cout, k, bits, residual
+    (2, 4, 28, 64, 128, 3, 8, False),      # resident weights
+    (2, 8, 28, 64, 64, 3, 8, False),       # the same in strips
+    (2, 49, 28, 64, 256, 1, 8, True),      # residual through tensor memory
+    (2, 13, 14, 256, 256, 3, 8, False),    # weights that travel with the stages
+    (2, 8, 28, 64, 64, 3, 4, False),       # packed operands, widened in the launch before
+    (0, 3, 17, 3, 32, 3, 8, False),        # patch matrix
+    (4, 1, 14, 64, 64, 3, 8, False),       # the kernel for small problems
+    (4, 1, 14, 64, 64, 3, 4, True),
+])
+def test_single_calls_follow_parameters_written_just_before(hq, cfg, writer):
+    """Weights, bias and pairs that the launch right before a call on the same stream has written, by an element-wise call of
+    the library (whose launch lets the next one start early) or by a copy kernel: no call may read them before it ended."""
+    from oracle import hqref
+    from paper_2011_10680_b200 import binding
+    path, n, hw, cin, cout, k, bits, residual = cfg
+    cases = [inputs.conv_case(700 + i, n, hw, hw, cin, cout, k, 1, k // 2, bits=bits, residual=residual, c_range=(39, 44)) for i in range(4)]
+    for case in cases:                     # one set of activations, four sets of parameters
+        case["x"], case["res"] = cases[0]["x"], cases[0]["res"]
+    dev = binding.upload_case(cases[0])
+    names = [f for f in ("wgt", "bias", "b", "c", "rb", "rc") if dev[f] is not None]
+    one = torch.full((max(cin, cout),), 1 << 30, dtype=torch.int32, device="cuda")
+    thirty = torch.full_like(one, 30)      # dn(v, 2^30, 30) = v
+    sources = []
+    for case in cases:
+        src = {f: binding.to_device(case[f]) for f in names}
+        if writer == "library":            # weights as one signed byte per value
+            w = case["wgt"] if bits == 8 else inputs.unpack4(case["wgt"], True).astype(np.int8)
+            src["wgt"] = binding.to_device(np.ascontiguousarray(w))
+        sources.append(src)
+
+    def write(src, f):
+        if writer == "torch":
+            dev[f].copy_(src[f])
+        elif f == "wgt":
+            lo, hi = (-128, 127) if bits == 8 else (-8, 7)
+            st = hq.residual_add(src[f], 8, 1, one, thirty, None, 0, 0, None, None, cin, 0, lo, hi, dev[f], bits, 1)
+            assert st == binding.HQ_OK, binding.status_string(st)
+        else:
+            shape = (1, 1, 1, cout)
+            st = hq.residual_add(src[f].view(shape), 32, 1, one, thirty, None, 0, 0, None, None, cout, 0, -(1 << 31), (1 << 31) - 1,
+                                 dev[f].view(shape), 32, 1)
+            assert st == binding.HQ_OK, binding.status_string(st)
+
+    refs = [hqref.conv_case(case) for case in cases]
+    outs = [binding.alloc_out(cases[0]["n"], cases[0]["ho"], cases[0]["wo"], cout, 8, cases[0]["out_signed"]) for _ in range(4 * len(names))]
+    hq.set_conv_path(path)
+    try:
+        # every parameter in turn is the last one written before the call
+        for r, last in enumerate(names):
+            for i, src in enumerate(sources):
+                for f in names:
+                    if f != last:
+                        write(src, f)
+                write(src, last)
+                st, _ = hq.conv_case(cases[0], dev, outs[4 * r + i])
+                assert st == binding.HQ_OK, binding.status_string(st)
+        hq.sync()
+    finally:
+        hq.set_conv_path(0)
+    for r, last in enumerate(names):
+        for i, ref in enumerate(refs):
+            got = outs[4 * r + i].cpu().numpy().view(ref.dtype).reshape(ref.shape)
+            assert np.array_equal(got, ref), (last, i, int((got != ref).sum()), ref.size)
