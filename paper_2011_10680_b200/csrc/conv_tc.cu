@@ -1549,7 +1549,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     if (p.bkb > 64) set_bkb(64);
     p.pt = pick_pt(P, p.c_tiles, 2 * h->sm_count, 128);
     wres_bytes = p.k_blocks * kTileC * p.bkb;
-    p.wres = wres_bytes <= 16 * 1024 && !a.wgt_fresh ? 1 : 0;              // short reductions: the weight slab stays resident
+    p.wres = wres_bytes <= 16 * 1024 ? 1 : 0;              // short reductions: the weight slab stays resident
     if (!p.wres) wres_bytes = 0;
     stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
     p.fold = (a.cout <= 64 && p.pt >= 128) ? 1 : 0;
@@ -1573,7 +1573,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       // tile wins and the weights travel with the stages.
       for (int keep_w = 1; keep_w >= 0 && !chosen; --keep_w) {
         wres_bytes = p.k_blocks * kTileC * p.bkb;
-        p.wres = (keep_w && wres_bytes <= 72 * 1024 && !a.wgt_fresh) ? 1 : 0;     // (resident weights are fetched ahead of the previous launch's end)
+        p.wres = (keep_w && wres_bytes <= 72 * 1024) ? 1 : 0;
         if (!p.wres) { if (keep_w) continue; wres_bytes = 0; }
         stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
         p.fold = (a.cout <= 64 && p.pt >= 128) ? 1 : 0;
@@ -1613,7 +1613,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       const long long tiles_all = (long long)a.n * tpi * p.c_tiles;
       const size_t patch = (size_t)(rows + 3) * (1u << lg_wp) * bkb, wb = (size_t)kTileC * bkb;
       const size_t slab = (size_t)(a.pairs ? 6 : 9 * cchunks) * wb;
-      const bool keep_w = (slab <= 72 * 1024 && !a.wgt_fresh) || a.pairs;
+      const bool keep_w = slab <= 72 * 1024 || a.pairs;
       const size_t room = (size_t)kSmemBudget - 32 * 1024 - (keep_w ? slab : 0);
       int npatch = 0, wstages = 0;
       if (keep_w) { npatch = (int)(room / patch); if (npatch > 3) npatch = 3; }
@@ -1666,7 +1666,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       out_tile_bytes = 0;
       res_tile_bytes = p.pt * kTileC;
       wres_bytes = p.k_blocks * kTileC * p.bkb;
-      p.wres = wres_bytes <= 72 * 1024 && !a.wgt_fresh ? 1 : 0;
+      p.wres = wres_bytes <= 72 * 1024 ? 1 : 0;
       if (!p.wres) wres_bytes = 0;
       stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
       // four residual / output tiles when they leave room for three operand stages: a tile is held from its load to

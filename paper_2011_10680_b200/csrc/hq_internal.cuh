@@ -114,7 +114,6 @@ struct ConvArgs {
   const WideArgs* wide;      // non-NULL: the convolution ends in the INT32 residual add (see WideArgs)
   int32_t pairs;             // nonzero: the pixel-pair form (hq_conv_pairs_applies): "pixels" are pairs, "channels" those of both; weights and constants are the layer's own
   int32_t in_slack;          // nonzero: a layer inside a network; the allocation behind `in` goes on for at least kIm2colMinTensorBytes + one image
-  int32_t wgt_fresh;         // nonzero: the weights are written by the launch just before: they are not kept resident (fetched ahead of its end)
   int32_t params_late;       // nonzero: weights, bias or pairs may be written by the launch just before: nothing is read ahead of its end
   int32_t pad_after_delta;   // padding after the last row/column minus `pad`
   // byte pitches of the activation tensor along W, H and N when it is not dense (0: dense NHWC).  A W pitch

@@ -426,7 +426,7 @@ hq_status hq_launch_conv_widen4(hq_handle* h, const ConvArgs& a, void* scratch, 
   unsigned char* ww = xw + (x + 255) / 256 * 256;
   if (launch_widen4(a.in, x, a.in_signed, xw, a.wgt_widened ? nullptr : a.wgt, w, ww, h->sm_count, s) != cudaSuccess) return HQ_ERR_CUDA;
   ConvArgs t = a;
-  t.in = xw; t.wgt = a.wgt_widened ? a.wgt_widened : ww; t.in_bits = 8; t.wgt_fresh = a.wgt_widened ? 0 : 1; t.params_late = 0;
+  t.in = xw; t.wgt = a.wgt_widened ? a.wgt_widened : ww; t.in_bits = 8; t.params_late = a.wgt_widened ? 0 : 1;
   const hq_status st = hq_launch_conv_tc(h, t, s);
   if (st != HQ_ERR_UNSUPPORTED || !hq_conv_lowering_applies(t)) return st;
   return hq_launch_conv_lowered(h, t, xw + widen4_copy_bytes(a), s);      // declined by the direct kernel: patch matrix

@@ -132,10 +132,11 @@ def test_concatenations_follow_their_pairs(hq, batch, shifts):
 @pytest.mark.parametrize("cfg", [
     # path, n, hw, cin, cout, k, bits, residual
     (2, 4, 28, 64, 128, 3, 8, False),      # resident weights
-    (2, 8, 28, 64, 64, 3, 8, False),       # the same in strips
+    (3, 8, 28, 64, 64, 3, 8, False),       # the same in strips
     (2, 49, 28, 64, 256, 1, 8, True),      # residual through tensor memory
     (2, 13, 14, 256, 256, 3, 8, False),    # weights that travel with the stages
-    (2, 8, 28, 64, 64, 3, 4, False),       # packed operands, widened in the launch before
+    (3, 8, 28, 64, 64, 3, 4, False),       # packed operands, widened in the launch before, in strips
+    (2, 4, 28, 64, 128, 3, 4, True),       # ... and in resident blocks
     (0, 3, 17, 3, 32, 3, 8, False),        # patch matrix
     (4, 1, 14, 64, 64, 3, 8, False),       # the kernel for small problems
     (4, 1, 14, 64, 64, 3, 4, True),
