@@ -485,7 +485,7 @@ hq_status hq_avgpool_requant(hq_handle* h, const hq_tensor* in, hq_dyadic r, int
   if (!type_range_ok(out->bits, out->is_signed, qmin, qmax)) return HQ_ERR_INVALID_ARG;
   if ((long long)in->h * in->w > (1LL << 23)) return HQ_ERR_UNSUPPORTED;   // INT32 sum of 8-bit values
   return hq_launch_avgpool(in->data, in->n, in->h, in->w, in->c, in->bits, in->is_signed, r.b, r.c, qmin, qmax,
-                           out->data, out->bits, (cudaStream_t)stream) == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
+                           out->data, out->bits, h->sm_count, (cudaStream_t)stream) == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }
 
 hq_status hq_maxpool(hq_handle* h, const hq_tensor* in, int32_t k, int32_t stride, int32_t pad, hq_tensor* out,

@@ -660,19 +660,19 @@ bool hq_conv_small_init() {
          cudaFuncSetAttribute(conv_small_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 110 * 1024) == cudaSuccess;
 }
 
-bool hq_conv_small_supported(const ConvArgs& a) {
+bool hq_conv_small_supported(const ConvArgs& a, int sm_count) {
   if (!(a.in_bits == 8 || a.in_bits == 4) || a.cin % 16 != 0 || a.pitch_w) return false;
   if ((long long)a.n * a.ho * a.wo >= (1ll << 31) - 64 || (long long)a.kh * a.kw * a.cin >= (1ll << 24)) return false;
   if ((long long)a.kh * a.w * a.cin >= (1ll << 31)) return false;
   if (a.out_bits == 4 && (a.cout & 1)) return false;
   if (a.res && !(a.res_bits == 8 || a.res_bits == 32)) return false;
   if (((uintptr_t)a.in & 15u) || ((uintptr_t)a.wgt & 15u)) return false;
-  const SmallShape s = small_shape(a, 148);
+  const SmallShape s = small_shape(a, sm_count);
   return ((s.p_tiles * s.c_tiles) << s.lg_split) < (1ll << 31);
 }
 
 hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t stream) {
-  if (!hq_conv_small_supported(a)) return HQ_ERR_UNSUPPORTED;
+  if (!hq_conv_small_supported(a, h->sm_count)) return HQ_ERR_UNSUPPORTED;
   if (!load_driver_entry_points()) return HQ_ERR_CUDA;
   const SmallShape s = small_shape(a, h->sm_count);
   if (s.p_tiles == 0) return HQ_OK;
@@ -730,7 +730,7 @@ hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t str
 //   - and while a CTA has few K blocks to walk: 9 blocks 9.1 -> 6.6 (3x3 128 at 28x28, n = 13), 16 blocks 8.1 -> 8.3 (2048 -> 512 at
 //     7x7, n = 24), 36 blocks 13.3 -> 14.8 (3x3 512 at 7x7, n = 24).
 bool hq_conv_small_wanted(const ConvArgs& a, int sm_count) {
-  if (!hq_conv_small_supported(a)) return false;
+  if (!hq_conv_small_supported(a, sm_count)) return false;
   const SmallShape s = small_shape(a, sm_count);
   const long long ctas = (s.p_tiles * s.c_tiles) << s.lg_split;
   ConvArgs b8 = a;

@@ -1097,13 +1097,13 @@ cudaError_t hq_launch_residual_add(const EltArgs& args, int sm_count, cudaStream
 
 cudaError_t hq_launch_avgpool(const void* in, int n, int h, int w, int ch, int in_bits, int in_signed,
                               const int32_t* b, const int32_t* c, int qmin, int qmax,
-                              void* out, int out_bits, cudaStream_t s) {
+                              void* out, int out_bits, int sm_count, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   if (in_bits == 8 && out_bits == 8 && ch % 16 == 0 && h * w <= 8 * 257 && n <= 65535) {
     const int hw = h * w;
     // eight slices for long sums, and where the blocks leave SMs idle: a thread then reads its pixels in one or two batches
     // (2048 channels at 7x7, one image: two slices 6.9 us, eight 4 us)
-    if (hw >= 128 || (hw >= 16 && (long long)n * ((ch / 16 + 31) / 32) <= 148)) launch_avgpool_vec16<8>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
+    if (hw >= 128 || (hw >= 16 && (long long)n * ((ch / 16 + 31) / 32) <= sm_count)) launch_avgpool_vec16<8>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
     else if (hw >= 64) launch_avgpool_vec16<4>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
     else launch_avgpool_vec16<2>(in, n, hw, ch, in_signed, b, c, qmin, qmax, out, s);
   } else if (in_bits == 8 && out_bits == 8 && ch % 4 == 0 && h * w <= 257 && n <= 65535) {

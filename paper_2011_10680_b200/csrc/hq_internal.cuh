@@ -154,7 +154,7 @@ bool hq_conv_wide_applies(const ConvArgs& a, int sm_count);
 hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t s);
 // One tile per CTA, reduction split over a cluster: small problems (conv_small.cu).  Same status convention.
 bool hq_conv_small_init();
-bool hq_conv_small_supported(const ConvArgs& a);
+bool hq_conv_small_supported(const ConvArgs& a, int sm_count);
 bool hq_conv_small_wanted(const ConvArgs& a, int sm_count);    // the automatic path's choice
 hq_status hq_launch_conv_small(hq_handle* h, const ConvArgs& a, cudaStream_t s);
 // Fills `out` (channels x 16 bytes) with the narrow residual pairs of an 8-bit residual branch.
@@ -201,6 +201,6 @@ hq_status hq_launch_sumpool_concat(hq_handle* h, const hq_tensor& in, hq_dyadic 
 cudaError_t hq_launch_residual_add(const EltArgs& a, int sm_count, cudaStream_t s);
 cudaError_t hq_launch_avgpool(const void* in, int n, int h, int w, int ch, int in_bits, int in_signed,
                               const int32_t* b, const int32_t* c, int qmin, int qmax,
-                              void* out, int out_bits, cudaStream_t s);
+                              void* out, int out_bits, int sm_count, cudaStream_t s);
 cudaError_t hq_launch_maxpool(const void* in, int n, int h, int w, int ch, int bits, int is_signed,
                               int k, int stride, int pad, void* out, int ho, int wo, cudaStream_t s);
