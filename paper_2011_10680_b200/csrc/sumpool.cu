@@ -263,8 +263,10 @@ hq_status hq_launch_sumpool_concat(hq_handle* h, const hq_tensor& in, hq_dyadic 
   p.sat = p.lo == 0 && p.hi == 255 ? 1 : 0;
   const long long cols = (long long)in.w * (in.c / 4);
   int rows = strip_rows_for(in.n, in.h, cols, h->sm_count);
-  // (arithmetic weighs more here than in the plain sums: strips twice as long where they still make 16 blocks per SM)
-  if (rows == 8 && (cols + 255) / 256 * in.n * ((in.h + 17) / 18) >= 16LL * h->sm_count) rows = in.h <= 18 ? in.h : 18;
+  // (arithmetic weighs more here than in the plain sums: equal strips of at most 18 rows, whose two extra input rows are a
+  // ninth of the work instead of a quarter, where they still make 16 blocks per SM)
+  const int long_strips = (in.h + 17) / 18;
+  if (rows == 8 && (cols + 255) / 256 * in.n * long_strips >= 16LL * h->sm_count) rows = (in.h + long_strips - 1) / long_strips;
   const int strips = (in.h + rows - 1) / rows;
   const dim3 grid((unsigned)((cols + 255) / 256), (unsigned)(in.n * strips));
   if (in.is_signed) hq_launch_pdl(sumpool3_concat_kernel<1>, grid, 256, 0, s, p, rows, strips);
