@@ -104,6 +104,52 @@ def layer_work(table, batch):
     return rows
 
 
+def on_tensor_cores(l):
+    """Layers that run a tensor-core convolution kernel: every conv / linear whose channel count the tensor maps take (4-bit
+    operands included: widened, or kept one value per byte inside the network) and the 3-channel stem (space-to-depth
+    form; its two helper kernels are part of the layer's time)."""
+    return l["op"] in ("conv", "linear") and (l["cin"] % 16 == 0 or (l["cin"] == 3 and l["kh"] == 7 and l["stride"] == 2))
+
+
+def launch_work(table, batch):
+    """layer_work by launch: hq_run_network runs some layers of the workload tables inside the launch of another one, and
+    hq_network_time_layers reports the time of all of them on that layer's row.  Such rows (`runs_in`: the other layer) are
+    empty here, and the other row carries their operations and bytes without the tensors that no longer travel.
+      - an INT32 add whose main operand is the raw result of a convolution, with the first requantization of its sum;
+      - 3x3 / stride 1 window sums of an 8-bit tensor that only a concatenation reads."""
+    layers, shapes = table["layers"], table["shapes"]
+    rows = [dict(r, runs_in=None, conv=on_tensor_cores(l)) for r, l in zip(layer_work(table, batch), layers)]
+    readers = {i: [] for i in range(len(layers))}
+    for j, l in enumerate(layers):
+        for t in l["ins"] if l["op"] == "concat" else (l["in0"], l["in1"]):
+            if t >= 0:
+                readers[t].append(j)
+
+    def take(j, i, saved):
+        rows[i]["ops"] += rows[j]["ops"]
+        rows[i]["bytes"] += rows[j]["bytes"] - saved
+        rows[i]["conv"] = rows[i]["conv"] or rows[j]["conv"]
+        rows[j].update(runs_in=i, ops=0, bytes=0, conv=False)
+
+    wide = lambda i: 4 * batch * shapes[i][0] * shapes[i][1] * shapes[i][2]      # bytes of an INT32 tensor
+    for i, l in enumerate(layers):
+        if l["op"] == "add" and l["out_bits"] == 32:
+            j = l["in0"]
+            if layers[j]["op"] != "conv" or layers[j]["out_bits"] != 32 or readers[j] != [i]:
+                continue
+            take(j, i, 2 * wide(j))                                              # neither written nor read back
+            quant = [m for m in readers[i] if layers[m]["op"] == "requant"]
+            if quant:
+                take(quant[0], i, wide(i) * (2 if readers[i] == quant[:1] else 1))
+        elif l["op"] == "concat":
+            for j in l["ins"]:
+                p = layers[j]
+                if p["op"] == "sumpool" and (p["pool_k"], p["pool_stride"], p["pool_pad"]) == (3, 1, 1) and readers[j] == [i]:
+                    take(j, i, 2 * wide(j))
+                    break
+    return rows
+
+
 class ClockSampler:
     """nvidia-smi clock / throttle sampling while the timed region runs."""
     FIELDS = ("clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.hw_slowdown,"
@@ -741,16 +787,11 @@ def main():
 
     if rank == 0:
         hbm_peak, bf16_peak, peak_kind = measured_peaks()
-        work = layer_work(table, batch)
         rows, tc_bytes, tc_ops, tc_ns = [], 0, 0, 0.0
-        for wk, ns, l in zip(work, layer_ns, table["layers"]):
-            # layers that run conv_tc_kernel: every conv / linear with a channel count the tensor maps take (4-bit
-            # operands included: widened, or kept one value per byte inside the network) and the 3-channel stem
-            # (space-to-depth form; its two helper kernels are part of the layer's time)
-            on_tc = l["op"] in ("conv", "linear") and (l["cin"] % 32 == 0 or (l["cin"] == 3 and l["kh"] == 7 and l["stride"] == 2))
-            if on_tc:
+        for wk, ns in zip(launch_work(table, batch), layer_ns):
+            if wk["conv"]:
                 tc_bytes += wk["bytes"]; tc_ops += wk["ops"]; tc_ns += ns
-            rows.append({**wk, "us": ns / 1e3, "tensor_core": on_tc, "gbs": wk["bytes"] / max(ns, 1),
+            rows.append({**wk, "us": ns / 1e3, "tensor_core": wk["conv"], "gbs": wk["bytes"] / max(ns, 1),
                          "tops": wk["ops"] / max(ns, 1) / 1e3})
         if args.layers_out:
             json.dump(rows, open(args.layers_out, "w"), indent=1)
@@ -806,7 +847,7 @@ def main():
                          "algorithmic_bytes_per_step": tc_bytes,
                          "layerwise_frac": lw_nominal / step_ms,
                          "layerwise_roofline_ms": lw_nominal,
-                         "layerwise_note": "sum over layers of max(ops / 4.5 POPS nominal, algorithmic bytes / measured HBM) / ms_per_step",
+                         "layerwise_note": "sum over layers (those inside another launch counted with it) of max(ops / 4.5 POPS nominal, algorithmic bytes / measured HBM) / ms_per_step",
                          "layerwise_frac_measured_i8_peak": (lw_measured / step_ms) if lw_measured else None,
                          "tensor_tops": tensor_tops,
                          "tensor_frac_of_nominal_4500": tensor_tops / NOMINAL_I8_TOPS,

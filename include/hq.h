@@ -199,9 +199,12 @@ hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layer
 hq_status hq_run_network(hq_network* net, const hq_tensor* images, hq_tensor* logits,
                          void* const* layer_taps, void* stream);
 
-/* Measurement aid: run the table once with plain launches and a CUDA event pair around every
- * layer, wait for the stream, and write each layer's device time in nanoseconds to the HOST
- * array ns[n_layers]. */
+/* Measurement aid: run the table once, in the launches of hq_run_network without taps but outside a graph, with a CUDA
+ * event before and behind every layer; wait for the stream, and write each layer's device time in nanoseconds to the
+ * HOST array ns[n_layers].  Layers that run inside the launch of another one report the time between two events with
+ * nothing between them, and that other layer's entry is the time of all of them: a tensor-core convolution to INT32 that only an
+ * ADD with an INT32 result reads as its main operand, with the first REQUANT of that sum, on the ADD's entry; 3x3 / stride 1
+ * window sums of an 8-bit tensor that only a CONCAT reads, on the CONCAT's.  Such layers run alone when taps are asked for. */
 hq_status hq_network_time_layers(hq_network* net, const hq_tensor* images, hq_tensor* logits, int64_t* ns,
                                  void* stream);
 

@@ -401,7 +401,8 @@ class Network:
         return lib().hq_run_network(self._net, C.byref(ti), C.byref(tl), tap_arr, _stream())
 
     def time_layers(self, images, logits):
-        """Per-layer device time in nanoseconds (CUDA events around each layer, plain launches)."""
+        """Per-layer device time in nanoseconds (CUDA events around each layer, plain launches).  A layer that runs inside the
+        launch of another one is on that one's entry (see hq_network_time_layers)."""
         ti = tensor_of(images, images.shape[3], 8, 0)
         last = self.table["layers"][-1]
         tl = hq_tensor(logits.data_ptr(), self.batch, 1, 1, last["cout"], last["out_bits"], last["out_signed"])
