@@ -185,6 +185,10 @@ hq_status hq_maxpool(hq_handle* h, const hq_tensor* in, int32_t k, int32_t strid
  * Fig. 2 dataflow in fused form, first and last layer 8-bit per Appendix H).  `table` is a HOST
  * array; the pointers inside it are DEVICE pointers that must outlive the network.  Activation
  * buffers for `batch` images of image_h x image_w x image_c (8-bit) are allocated here.
+ * Parameters are constants of the network: prepared forms of some are made here and are not made again - 4-bit weights as
+ * bytes, everything of a 7x7 / stride 2 layer over 3 channels, the narrow multiply-add pairs of 8-bit residuals and of the
+ * 8-bit operands of ADD and REQUANT layers.  The others are read at every run.  A caller that changes parameters builds
+ * the network again.
  */
 hq_status hq_network_create(hq_handle* h, const hq_layer* table, int32_t n_layers, int32_t batch,
                             int32_t image_h, int32_t image_w, int32_t image_c, int32_t image_signed,
