@@ -55,6 +55,23 @@ def test_struct_layouts_match_the_header():
     assert ctypes.sizeof(binding.hq_layer) == 352
 
 
+def test_packed_arguments_equal_the_structures():
+    """The byte strings that convolution and concatenation calls pass, against the ctypes structures: the same bytes, and
+    the same treatment of integers that do not fit a field (the library then answers with a status)."""
+    class Tensor:
+        shape = (2, 3, 4, 5)
+
+        def data_ptr(self):
+            return 0x7f1234567890
+    for c, bits, signed in ((5, 8, 0), (10, 4, True), ((1 << 32) + 7, 8, 1), (1 << 31, 32, 0), (-1, 8, 0)):
+        assert binding._packed_tensor(Tensor(), c, bits, signed) == bytes(binding.tensor_of(Tensor(), c, bits, signed))
+    dy = binding.hq_dyadic
+    for qmin, qmax in ((0, 255), (-(1 << 31), (1 << 31) - 1), (1 << 31, (1 << 32) - 1)):
+        ints = (3, 3, 1, 1, 64, 128, 8)
+        want = binding.hq_conv_desc(*ints, 16, 32, dy(48, 64), None, dy(80, 96), 1, qmin, qmax)
+        assert binding._packed_conv(*ints, 16, 32, 48, 64, 0, 80, 96, 1, qmin, qmax) == bytes(want)
+
+
 def test_cuda_sources_have_no_floating_point():
     csrc = os.path.join(ROOT, "paper_2011_10680_b200", "csrc")
     for f in os.listdir(csrc):
