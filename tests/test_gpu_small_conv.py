@@ -109,7 +109,8 @@ def test_fused_int32_stream_add_large_tiles():
     (5, 20, 20, 144, 192, 3, 2, 1, 8, False),    # a full block and 16 of 128
     (9, 20, 20, 192, 256, 1, 1, 0, 8, True),     # tiled rows, residual
     (12, 30, 30, 16, 128, 3, 1, 1, 8, False),    # half a 32-byte block
-    (4, 20, 20, 288, 256, 3, 1, 1, 8, False),    # long reduction, two-CTA shape on path 3
+    (4, 20, 20, 288, 256, 3, 1, 1, 8, False),    # long reduction: two full blocks and 32 of 128
+    (41, 31, 31, 288, 256, 3, 1, 1, 8, False),   # the same with two tiles per SM: the two-CTA shape, a ragged last tile
     (9, 20, 20, 48, 64, 5, 1, 2, 4, False),      # widened 4-bit operands
 ])
 def test_conv_channels_that_do_not_fill_a_block(cfg, path):
