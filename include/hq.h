@@ -118,8 +118,8 @@ hq_status hq_sync(hq_handle* h, void* stream);
  *   otherwise       :  y = dn(t, b[oc], c[oc]);  if residual: y += dn(res, rb[oc], rc[oc]);
  *                      if relu: y = max(y, 0);  out = clamp(y, qmin, qmax), stored at out->bits.
  * in: bits 8 or 4 (== w_bits), signed or unsigned.  out: n, h, w, c must equal the convolution's
- * output extents.  The tensor-core kernels take layers with cin a multiple of 16, directly or - for the
- * 3-channel first layer, thin layers and layers whose input tensor is below 128 KiB - through a lowered form
+ * output extents.  The tensor-core kernels take layers with cin a multiple of 16 directly - a small one whatever the size
+ * of its input - and the 3-channel first layer, other thin layers and some layers of short rows through a lowered form
  * (space-to-depth copy or patch matrix in scratch memory of the handle); other shapes run on the CUDA-core
  * path.  Accumulator overflow beyond INT32
  * is undefined (cannot happen for K = kh*kw*cin <= 66311 with 8-bit operands).

@@ -179,7 +179,7 @@ struct hq_network {
   // ADD layers with an INT32 result that run behind the convolution producing their main operand (see plan_wide_adds):
   // the convolution's layer or -1; the REQUANT layer done along with it or -1; whether somebody else reads the sum
   std::vector<int32_t> wide_conv, wide_requant;
-  std::vector<char> wide_sum_read, run_by_add;   // run_by_add: layers that such an ADD, or a CONCAT, runs
+  std::vector<char> wide_sum_read, runs_inside;   // runs_inside: layers that run inside the launches of such an ADD, or of a CONCAT
   std::vector<int32_t> pool_branch;  // CONCAT layers: the branch whose 3x3 window sums are rescaled straight into it, or -1
   std::vector<void*> concat_narrow;  // CONCAT layers: the narrow pairs of the 8- and 4-bit branches (owned)
   std::vector<char> tile_order;      // per conv / linear / concat layer: tensors walked from the last pixel to the first (see plan_tile_orders)
@@ -215,7 +215,7 @@ static void plan_tile_orders(hq_network* net) {
       const int src = net->layers[i].in0;
       order = src < 0 ? 0 : !net->tile_order[src];
     }
-    if (i + 1 < n && !either_way(i + 1) && net->layers[i + 1].in0 == i && !net->run_by_add[i]) order = 1;
+    if (i + 1 < n && !either_way(i + 1) && net->layers[i + 1].in0 == i && !net->runs_inside[i]) order = 1;
     net->tile_order[i] = order;
   }
 }
@@ -227,7 +227,7 @@ static void plan_tile_orders(hq_network* net) {
 static void plan_wide_adds(hq_network* net) {
   const int n = (int)net->layers.size();
   net->wide_conv.assign(n, -1); net->wide_requant.assign(n, -1);
-  net->wide_sum_read.assign(n, 0); net->run_by_add.assign(n, 0);
+  net->wide_sum_read.assign(n, 0); net->runs_inside.assign(n, 0);
   auto reads = [&](int j, int id) {
     const hq_layer& l = net->layers[j];
     if (l.op == HQ_OP_CONCAT) { for (int k = 0; k < l.n_in; ++k) if (l.ins[k] == id) return true; return false; }
@@ -251,7 +251,7 @@ static void plan_wide_adds(hq_network* net) {
     a.in_slack = 1;
     if (!alone || !hq_conv_wide_applies(a, net->h->sm_count)) continue;
     net->wide_conv[i] = j;
-    net->run_by_add[j] = 1;
+    net->runs_inside[j] = 1;
     net->wide_sum_read[i] = i == n - 1;
     for (int m = i + 1; m < n; ++m) {
       if (!reads(m, i)) continue;
@@ -260,7 +260,7 @@ static void plan_wide_adds(hq_network* net) {
       const bool bytes = (net->outs[m].bits == 8 || net->stored_wide[m]) && type_range_ok(8, net->outs[m].is_signed, r.qmin, r.qmax);
       if (net->wide_requant[i] < 0 && r.op == HQ_OP_REQUANT && bytes && m != n - 1 && r.rescale0.b && r.rescale0.c) {
         net->wide_requant[i] = m;
-        net->run_by_add[m] = 1;
+        net->runs_inside[m] = 1;
       } else {
         net->wide_sum_read[i] = 1;
       }
@@ -290,7 +290,7 @@ static void plan_pool_branches(hq_network* net) {
       }
       if (readers != 1 || net->pool_branch[i] >= 0) continue;
       net->pool_branch[i] = k;
-      net->run_by_add[j] = 1;
+      net->runs_inside[j] = 1;
     }
   }
 }
@@ -300,7 +300,7 @@ static void count_launches(hq_network* net) {
   net->launches = (int32_t)net->layers.size();
   for (size_t i = 0; i < net->layers.size(); ++i) {
     const hq_layer& l = net->layers[i];
-    if (net->run_by_add[i]) { net->launches -= 1; continue; }
+    if (net->runs_inside[i]) { net->launches -= 1; continue; }
     if (l.op == HQ_OP_CONCAT && net->pool_branch[i] >= 0) net->launches += 1;
     if (l.op != HQ_OP_CONV) continue;
     const hq_conv_desc& d = l.conv;
@@ -709,7 +709,7 @@ static hq_status run_layers(hq_network* net, const hq_tensor* images, hq_tensor*
   for (int i = 0; i < n_layers; ++i) {
     if (marks && cudaEventRecord(marks[i], s) != cudaSuccess) return HQ_ERR_CUDA;
     const hq_layer& l = net->layers[i];
-    if (fuse && net->run_by_add[i]) continue;                 // runs with the ADD layer it feeds, or that feeds it
+    if (fuse && net->runs_inside[i]) continue;                 // its ADD or CONCAT layer runs it
     hq_tensor in = (l.in0 == -1) ? *images : net->outs[l.in0];
     hq_tensor o = net->outs[i];
     if (i == n_layers - 1) o.data = logits->data;

@@ -49,7 +49,7 @@ constexpr int kSmemBudget = 224 * 1024;
 constexpr int kSmemAttr = 226 * 1024;
 constexpr int kMaxAccBufs = 4;                                 // accumulator buffers: 4 x 128 or 2 x 256 columns
 constexpr int kMaxResBufs = 8;                                 // residual / output tiles in shared memory
-// Four launch shapes of the same kernel:
+// Launch shapes of the same kernel:
 //   solo  8 epilogue warps, one CTA per SM, up to 512 tensor-memory columns, up to 224 KiB of shared memory;
 //   pair  4 epilogue warps, two CTAs per SM with 256 columns and at most 110 KiB each.  Layers with a short
 //         reduction are bound by the latency of the hand-over chain between the MMA issuer and the epilogue
@@ -57,6 +57,7 @@ constexpr int kMaxResBufs = 8;                                 // residual / out
 //   rtm   ("residual through tensor memory") 8 epilogue warps, one issuer and a store warp, one CTA per SM, 128-pixel
 //         tiles: fused 8-bit residuals with a short reduction.  The residual tile is transposed and widened by an MMA
 //         with the identity matrix, the epilogue works on 16 x 8 fragments and writes with transposing matrix stores.
+//   wide  16 epilogue warps on boxes of 16 pixels: INT32 results, raw or through the residual add (see epilogue_loop_wide).
 //   duo   the solo roles in clusters of two CTAs that share every MMA (cta_group::2): long reductions whose weights
 //         stream; each CTA fetches its own weight rows and half of the pixel rows.
 constexpr int kSoloEpilogueWarps = 8;
@@ -79,7 +80,7 @@ struct TcParams {
   int32_t wres;          // 1: the CTA's whole weight slab [k_blocks][128][bkb] is loaded once and stays in shared memory
   uint32_t wres_off;     // its offset from the 1024-aligned dynamic base
   int32_t fold;          // 1: at most 64 output channels: W rows loaded twice, lane quarters 2-3 share the pixel columns
-  int32_t halves;        // 2: two warps share a lane quarter's pixel columns; 1 for the 64-pixel tile (warps 6-9 idle)
+  int32_t halves;        // warps that share a lane quarter's pixel columns: 2, 4 with INT32 boxes, 1 for the 64-pixel tile (the others idle)
   int32_t lg_rbufs;      // log2 of the residual-tile buffer count (<= lg_bufs; 0 when a long reduction leaves no room)
   int32_t rtm;           // 1: the 8-bit residual tile reaches the epilogue through tensor memory: an MMA with the identity
                          //    matrix as its A operand turns the [pixels][128 channels] byte tile into INT32 columns beside
@@ -1230,14 +1231,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   } else {
     // ------------------------------------------------------------ epilogue (the last EPI_WARPS warps)
     const int q = warp & 3;                       // the TMEM lane quarter this warp may read: channels 32q..32q+31
-    const int ew = warp - (1 + MMA_WARPS);        // 0..7
-    const int half = ew >> 2;                     // which half of its lane quarter's pixel columns this warp owns
+    const int ew = warp - (1 + MMA_WARPS);        // 0 .. EPI_WARPS - 1
+    const int half = ew >> 2;                     // which share (of p.halves) of its lane quarter's pixel columns this warp owns
     // Channel tiles of at most 64 channels are folded: the weight rows are loaded twice, so accumulator
     // lanes 64-127 repeat lanes 0-63, and lane quarters 2-3 take the second half of the pixel columns
     // of channels 0-63 instead of idling on channels that do not exist.
     const int cq = p.fold ? (q & 1) : q;          // which 32 channels of the tile
     const int slices = p.halves << p.fold;        // pixel-column slices per channel quarter
-    const int px_per_warp = p.pt / slices;        // 128 or 64 pixel columns
+    const int px_per_warp = p.pt / slices;        // 128 or 64 pixel columns; 32 or 16 with INT32 boxes
     const int col0 = ((p.fold ? (q >> 1) * p.halves : 0) + half) * px_per_warp;
     const int ch = c_tile * kTileC + cq * 32 + lane;         // this thread's output channel
     const bool ch_live = ch < p.C;
@@ -1273,7 +1274,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         }
       }
     } else {
-    // per-channel constants, once per kernel
+    // per-channel constants, once per kernel (spelled out: through chan_const the loops compile worse, ResNet-50 INT8 2.11 -> 2.25 ms)
     ChanConst k{};
     uint32_t fast = (p.out_bits != 32) ? 1u : 0u;
     const int pch = p.pairs ? ch & 63 : ch;       // (pixel pairs: both outputs of a pair have the layer's channels)
@@ -1483,9 +1484,9 @@ bool hq_conv_tc_supported(const ConvArgs& a) {
 
 // im2col-mode tensor maps over activation tensors smaller than 128 KiB returned wrong tiles on the driver this
 // library was brought up on (the map encoder marks such tensors in a field of the opaque descriptor).  Instead of
-// editing the descriptor, layers that would need such a map are not run by the direct kernel at all: they take the
-// patch-matrix form (lowering.cu), whose 1x1 convolution uses a plain tiled map.  Only small-batch, late-stage
-// layers are affected (every im2col layer of the benchmark configurations is far larger).
+// editing the descriptor, layers that would need such a map are not run by the direct kernel at all: the kernel for small
+// problems gathers their activations (conv_small.cu), and what it does not take goes through the patch-matrix form
+// (lowering.cu), whose 1x1 convolution uses a plain tiled map.  Inside a network the map is declared large enough instead.
 bool hq_conv_tc_small_im2col(const ConvArgs& a) {
   const bool tiled = !a.pitch_w && a.kh == 1 && a.kw == 1 && a.stride == 1 && a.pad == 0;
   if (tiled || a.in_slack) return false;              // (with room behind the tensor the map is declared large enough)
@@ -1640,7 +1641,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   }
   // The direct kernel fetches activations through an im2col-mode map unless the layer is 1x1 / stride 1 / unpadded
   // (tiled map) or takes the strip form (tiled map over padded patches).  That mode is not used on tensors below
-  // 128 KiB (hq_conv_tc_small_im2col); such a layer is declined here and runs in its lowered form.
+  // 128 KiB (hq_conv_tc_small_im2col); such a layer is declined here.
   if ((!p.strip && hq_conv_tc_declines(a)) || (a.pairs && !p.strip)) return HQ_ERR_UNSUPPORTED;
   p.x_signed = a.in_signed;
   bool wide = false;
