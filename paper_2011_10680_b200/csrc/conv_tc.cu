@@ -795,8 +795,10 @@ __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanCo
 // cta_group::2 instructions (a kernel that contains them cannot be launched without clusters).
 // RTM: the instantiation for fused 8-bit residuals that travel through tensor memory; it has one more warp, which
 // stores the finished output tiles.
-// WIDE: the instantiation for INT32 results, raw or through the residual add of Fig. 2 (epilogue_loop_wide).
-template <int EPI_WARPS, int MIN_CTAS, int MMA_WARPS, bool DUO = false, bool RTM = false, bool WIDE = false>
+// WIDE: the instantiations for INT32 results (epilogue_loop_wide), kRaw32 or through the residual add of Fig. 2, kAdd32.  (One for
+// both ran the add 0.6 % slower as soon as the raw form's waits for parameters were in it; the add only runs in networks.)
+constexpr int kRaw32 = 1, kAdd32 = 2;
+template <int EPI_WARPS, int MIN_CTAS, int MMA_WARPS, bool DUO = false, bool RTM = false, int WIDE = 0>
 __global__ void __launch_bounds__(32 * (1 + MMA_WARPS + EPI_WARPS + (RTM ? 1 : 0)), MIN_CTAS)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res,
@@ -867,7 +869,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   // may start filling SMs as ours leave.  Weights and constants are read ahead of that inside a network; a call of its own
   // (params_late) may follow the kernel that wrote them: its producer and epilogue wait before they read those too, and the
   // next kernel is let in after the producer's wait only (a network's second layer would read its own parameters at once).
-  if (!p.params_late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const bool params_late = WIDE != kAdd32 && p.params_late != 0;
+  if (!params_late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -887,7 +890,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       int ow = px_first - img * p.howo - oh * p.wo;
       const int step = p_step * p.pt;
       const int d_img = step / p.howo, d_oh = (step - d_img * p.howo) / p.wo, d_ow = step - d_img * p.howo - d_oh * p.wo;
-      if (p.params_late) {
+      if (params_late) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       }
@@ -1244,7 +1247,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     const bool ch_live = ch < p.C;
     const bool warp_live = (c_tile * kTileC + cq * 32) < p.C; // warp-uniform
     const int lo = p.relu ? (p.qmin > 0 ? p.qmin : 0) : p.qmin, hi = p.qmax;
-    if (p.params_late) asm volatile("griddepcontrol.wait;" ::: "memory");     // (the constants below)
+    if (params_late) asm volatile("griddepcontrol.wait;" ::: "memory");     // (the constants below)
 
     if constexpr (WIDE) {
       if (half < p.halves) {
@@ -1253,7 +1256,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         e.tmem_base = tmem_base; e.lane = lane; e.q = q; e.cq = cq; e.ew = ew; e.half = half;
         e.col0 = col0; e.px_per_warp = px_per_warp; e.ch = ch; e.c_tile = c_tile; e.p_tile0 = p_tile0; e.p_step = p_step;
         e.lo = lo; e.hi = hi; e.ch_live = ch_live; e.warp_live = warp_live;
-        if (!p.res) {
+        if constexpr (WIDE == kRaw32) {
           ChanConst k{};
           k.bias = (ch_live && p.bias) ? p.bias[ch] : 0;
           epilogue_loop_wide<3, false>(e, k, &map_res, &map_q);
@@ -1461,7 +1464,9 @@ bool hq_conv_tc_init() {
          cudaFuncSetAttribute(conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               112 * 1024) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<8, 1, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAttr) == cudaSuccess &&
-         cudaFuncSetAttribute(conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+         cudaFuncSetAttribute(conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kRaw32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              kSmemAttr) == cudaSuccess &&
+         cudaFuncSetAttribute(conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kAdd32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               kSmemAttr) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<kSoloEpilogueWarps, 1, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               kSmemAttr) == cudaSuccess;
@@ -1811,7 +1816,8 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   } else {
     // one CTA per SM (it may allocate all 512 tensor-memory columns): never request less than 120 KiB
     cfg.blockDim = dim3(32 * (1 + kSoloIssuerWarps + (int32_boxes ? kWideWarps : kSoloEpilogueWarps))); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
-    if (int32_boxes) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, true>, map_x, map_w, map_out, map_res, map_q, p);
+    if (a.wide) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kAdd32>, map_x, map_w, map_out, map_res, map_q, p);
+    else if (int32_boxes) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kRaw32>, map_x, map_w, map_out, map_res, map_q, p);
     else err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);
   }
   return err == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
