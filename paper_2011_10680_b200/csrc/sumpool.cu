@@ -161,8 +161,10 @@ struct SumCatArgs {
   const int32_t* b; const int32_t* c;
   unsigned char* out; int32_t out_ch, ch_off, lo, hi, sat;    // sat: the clamp is that of u8
 };
-// Bound by the integer pipe: about 12 instructions per value with running pointers, byte permutes and the form of the shift chosen
-// outside the loop (256 x 35x35x288: 114 us, 127 us with the address and bounds arithmetic of sumpool3_rows_kernel, 31 instructions a value).
+// What bounds it: instructions and the latency of the three reads of a row, together (64 images of 35x35x288: issue slots 50 % busy,
+// ALU pipe 47 %, 28 of 64 warp slots filled at 58 registers, long-scoreboard stalls 9 per issue, DRAM 8 %).  Running pointers, byte
+// permutes and the form of the shift chosen outside the loop: 256 x 35x35x288 in 114 us, 127 us with the address and bounds
+// arithmetic of sumpool3_rows_kernel.
 template <int SIGNED, bool FAST>
 __device__ __forceinline__ void sumpool3_concat_column(const SumCatArgs& p, int ow, int g, int img, int r0, int r1) {
   const SumPoolArgs& a = p.s;
