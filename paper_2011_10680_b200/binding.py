@@ -188,13 +188,10 @@ def _packed_tensor(t, c, bits, is_signed) -> bytes:
         return bytes(tensor_of(t, c, bits, is_signed))
 
 
-def _packed_conv(*v) -> bytes:
-    """hq_conv_desc: seven integers, seven pointers (w, bias, b, c, residual, rb, rc), relu, qmin, qmax."""
-    try:
-        return _PACK_CONV(*v)
-    except struct.error:
-        res = C.cast(C.c_void_p(v[11]), C.POINTER(hq_tensor))
-        return bytes(hq_conv_desc(*v[:9], hq_dyadic(*v[9:11]), res, hq_dyadic(*v[12:14]), *v[14:]))
+def _wrapped_conv(*v) -> bytes:
+    """hq_conv_desc through ctypes: seven integers, seven pointers (w, bias, b, c, residual, rb, rc), relu, qmin, qmax."""
+    res = C.cast(C.c_void_p(v[11]), C.POINTER(hq_tensor))
+    return bytes(hq_conv_desc(*v[:9], hq_dyadic(*v[9:11]), res, hq_dyadic(*v[12:14]), *v[14:]))
 
 
 def to_device(a):
@@ -280,8 +277,12 @@ class Handle:
                res=None, res_bits=0, res_signed=0, rb=None, rc=None, relu=1, qmin=0, qmax=255, linear=False):
         # (the residual's structure is referenced by address: it has to live until the call returns)
         tres = tensor_of(res, cout, res_bits, res_signed) if res is not None else None
-        d = _packed_conv(kh, kw, stride, pad, cin, cout, in_bits, wgt.data_ptr(), _ptr(bias), _ptr(b), _ptr(c),
-                         C.addressof(tres) if tres is not None else 0, _ptr(rb), _ptr(rc), relu, qmin, qmax)
+        v = (kh, kw, stride, pad, cin, cout, in_bits, wgt.data_ptr(), _ptr(bias), _ptr(b), _ptr(c),
+             C.addressof(tres) if tres is not None else 0, _ptr(rb), _ptr(rc), relu, qmin, qmax)
+        try:
+            d = _PACK_CONV(*v)
+        except struct.error:
+            d = _wrapped_conv(*v)
         fn = _packed_calls()[1 if linear else 0]
         return fn(self._h, _packed_tensor(x, cin, in_bits, in_signed), d, _packed_tensor(out, cout, out_bits, out_signed), _stream())
 

@@ -66,10 +66,13 @@ def test_packed_arguments_equal_the_structures():
     for c, bits, signed in ((5, 8, 0), (10, 4, True), ((1 << 32) + 7, 8, 1), (1 << 31, 32, 0), (-1, 8, 0)):
         assert binding._packed_tensor(Tensor(), c, bits, signed) == bytes(binding.tensor_of(Tensor(), c, bits, signed))
     dy = binding.hq_dyadic
-    for qmin, qmax in ((0, 255), (-(1 << 31), (1 << 31) - 1), (1 << 31, (1 << 32) - 1)):
+    for qmin, qmax, fits in ((0, 255, True), (-(1 << 31), (1 << 31) - 1, True), (1 << 31, (1 << 32) - 1, False)):
         ints = (3, 3, 1, 1, 64, 128, 8)
         want = binding.hq_conv_desc(*ints, 16, 32, dy(48, 64), None, dy(80, 96), 1, qmin, qmax)
-        assert binding._packed_conv(*ints, 16, 32, 48, 64, 0, 80, 96, 1, qmin, qmax) == bytes(want)
+        v = (*ints, 16, 32, 48, 64, 0, 80, 96, 1, qmin, qmax)
+        assert binding._wrapped_conv(*v) == bytes(want)
+        if fits:
+            assert binding._PACK_CONV(*v) == bytes(want)
 
 
 def test_cuda_sources_have_no_floating_point():
