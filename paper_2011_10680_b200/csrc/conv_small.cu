@@ -174,7 +174,7 @@ __device__ __forceinline__ void finish_fast8(const SmallEpi& e, const ChanConst&
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int r = RES == 0 ? 0 : (int)hq_prmt(rword, 0u, SIGNED ? 0x8880u + 0x1111u * j : 0x4440u + j);
-    y[j] = requant_fast<RES != 0, SIGNED, PRE ? 2 : 0, RES >= 3, true>(acc[j], r, k);
+    y[j] = requant_fast<RES != 0, SIGNED, PRE ? 2 : 0, RES >= 3>(acc[j], r, k);
   }
   unsigned w;
   if (p.sat == 1) w = sat_pack4<false>(y[0], y[1], y[2], y[3]);

@@ -355,7 +355,7 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
       const long long y = (((long long)acc * (long long)c.b + c.r0) >> c.sh) + (((long long)r * (long long)c.rb + c.rr0) >> c.rsh);
       return hq_clamp_ll(y, p.relu, p.qmin, p.qmax);
     }
-    const int y = requant_fast<true, RSIGNED, SMALL, RN, true>(acc, r, c);
+    const int y = requant_fast<true, RSIGNED, SMALL, RN>(acc, r, c);
     return SAT ? y : min(max(y, e.lo), e.hi);
   };
   // one unit: 16 values per thread -> four words -> one transposing store of 32 pixel rows x 16 channel bytes
@@ -525,9 +525,7 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
       }
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        long long t, u;
-        asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(v[j]), "r"(k.b), "l"(k.r0));
-        asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(u) : "r"(r[j]), "r"(k.rb), "l"(k.rr0));
+        const long long t = hq_mad_wide(v[j], k.b, k.r0), u = hq_mad_wide(r[j], k.rb, k.rr0);
         if constexpr (FORM == 0) {
           y[j] = ((int)(t >> 32) >> msh2) + ((int)(u >> 32) >> rsh2);                // each within [-2^30, 2^30)
         } else {
@@ -554,8 +552,7 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
         int z[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          long long t;
-          asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(y[4 * g + j]), "r"(qb), "l"(qr0));
+          long long t = hq_mad_wide(y[4 * g + j], qb, qr0);
           if constexpr (FORM < 2) z[j] = (int)(t >> 32) >> qsh;
           else { int up; unsigned low; shift64(t, qsh1, qsh2, qcm, up, low); z[j] = sat32(up, low); }
         }

@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(256) requant32_flat_kernel(EltArgs a, int quad
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       if (!slow) {
-        sv[i] = (int)(((long long)acc[i] * (long long)m[i].b + m[i].r0) >> 32) >> m[i].sh;
+        sv[i] = (int)(hq_mad_wide(acc[i], m[i].b, m[i].r0) >> 32) >> m[i].sh;
         if (RES) sv[i] += dn8<RSIGNED>(__byte_perm(rw, 0u, 0x0444u | ((unsigned)i << 12)), r[i]);
       } else {
         const unsigned rbyte = (rw >> (8 * i)) & 0xFFu;

@@ -32,9 +32,15 @@ constexpr long long kIm2colMinTensorBytes = 128 * 1024;   // smaller activation 
 // ------------------------------------------------------------------------------------------
 // Dyadic arithmetic (Eq. 4): dn(q, b, c) = (q*b + 2^(c-1)) >> c, 64-bit product, arithmetic shift.
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ long long hq_dn(int q, int b, int c) {
-  return ((long long)q * (long long)b + (1LL << (c - 1))) >> c;
+// a * b + c as one multiply-add.  Spelled as a product and a sum, which the assembler joins; the fused PTX form (mad.wide) comes
+// out as two multiplies and an add (product, shift by register and pack in a loop: 6.2 against 4.7 cycles per 32 values and
+// scheduler), and plain C++ can become a full 64 x 64-bit multiply when the sign extension of `b` is hoisted out of a loop.
+__device__ __forceinline__ long long hq_mad_wide(int a, int b, long long c) {
+  long long d;
+  asm("{\n\t.reg .s64 m;\n\tmul.wide.s32 m, %1, %2;\n\tadd.s64 %0, m, %3;\n\t}" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
 }
+__device__ __forceinline__ long long hq_dn(int q, int b, int c) { return hq_mad_wide(q, b, 1LL << (c - 1)) >> c; }
 
 // Byte permute with the full PTX selector: bit 3 of a selector nibble replicates the selected byte's sign bit over the
 // target byte.  (The __byte_perm intrinsic keeps three bits per nibble and cannot sign-extend.)

@@ -209,8 +209,7 @@ __device__ __forceinline__ void sumpool3_concat_column(const SumCatArgs& p, int 
     int y[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      long long t;
-      asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t) : "r"(q[i]), "r"(b[i]), "l"(add[i]));
+      long long t = hq_mad_wide(q[i], b[i], add[i]);
       if (FAST) y[i] = (int)(t >> 32) >> sh[i];
       else { t >>= sh[i]; y[i] = (int)(t < -256 ? -256 : t > 255 ? 255 : t); }
     }

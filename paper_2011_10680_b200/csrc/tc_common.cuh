@@ -313,15 +313,10 @@ struct ChanConst {
 // RN: every channel of the warp has a narrow residual pair (m, a, s) with (r*m + a) >> s equal to the residual
 // term for all 256 values of r (found and checked exhaustively by residual_narrow_kernel); rb / rh / rsh hold
 // m / a / s then, and a 32-bit multiply-add replaces the shift, multiply-high and add.
-// SPELLED: the product is written as the 32 x 32 -> 64 multiply-add instruction it is.  In the fragment loop, left
-// to the compiler, the sign extension of k.b is hoisted out of the loop and the product becomes a full 64 x 64
-// multiply (three to four multiply instructions per value); the other loops compile to the short form by themselves.
-template <bool RES, bool RSIGNED, int SMALL, bool RN = false, bool SPELLED = false>
+template <bool RES, bool RSIGNED, int SMALL, bool RN = false>
 __device__ __forceinline__ int requant_fast(int acc, int r, const ChanConst& k) {
   if (SMALL == 2) acc <<= k.pre;
-  long long t1;
-  if (SPELLED) asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(t1) : "r"(acc), "r"(k.b), "l"(k.r0));
-  else t1 = (long long)acc * (long long)k.b + k.r0;
+  const long long t1 = hq_mad_wide(acc, k.b, k.r0);
   int s;
   if (SMALL != 1) {
     s = (int)(t1 >> 32) >> k.sh;                       // c >= 32 (or pre-shifted): |s| < 2^30
