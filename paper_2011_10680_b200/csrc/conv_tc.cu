@@ -54,14 +54,15 @@ constexpr int kMaxResBufs = 8;                                 // residual / out
 //   pair  4 epilogue warps, two CTAs per SM with 256 columns and at most 110 KiB each.  Layers with a short
 //         reduction are bound by the latency of the hand-over chain between the MMA issuer and the epilogue
 //         (barrier, fences, MMA, commit), not by any throughput; two independent CTAs hide each other's chain.
-//   rtm   ("residual through tensor memory") 8 epilogue warps, one issuer and a store warp, one CTA per SM, 128-pixel
-//         tiles: fused 8-bit residuals with a short reduction.  The residual tile is transposed and widened by an MMA
-//         with the identity matrix, the epilogue works on 16 x 8 fragments and writes with transposing matrix stores.
+//   frag  16 epilogue warps in two groups on alternate tiles, two issuers and a store warp, one CTA per SM, 128-pixel tiles
+//         in four accumulators: fused 8-bit residuals with a short reduction.  The epilogue works on 16 x 8 fragments, reads
+//         the residual with transposing matrix loads and writes over it with transposing matrix stores.
 //   wide  16 epilogue warps on boxes of 16 pixels: INT32 results, raw or through the residual add (see epilogue_loop_wide).
 //   duo   the solo roles in clusters of two CTAs that share every MMA (cta_group::2): long reductions whose weights
 //         stream; each CTA fetches its own weight rows and half of the pixel rows.
 constexpr int kSoloEpilogueWarps = 8;
 constexpr int kPairEpilogueWarps = 4;
+constexpr int kFragWarps = 16, kFragIssuers = 2, kFragGroups = 2, kFragAccs = 4;   // the frag shape: epilogue warps, in two groups; issuers; accumulator buffers
 constexpr int kSoloIssuerWarps = 3;     // 1 + 3 + 8 warps = 384 threads: 168 registers per thread remain
 constexpr int kPairIssuerWarps = 1;
 
@@ -82,12 +83,9 @@ struct TcParams {
   int32_t fold;          // 1: at most 64 output channels: W rows loaded twice, lane quarters 2-3 share the pixel columns
   int32_t halves;        // warps that share a lane quarter's pixel columns: 2, 4 with INT32 boxes, 1 for the 64-pixel tile (the others idle)
   int32_t lg_rbufs;      // log2 of the residual-tile buffer count (<= lg_bufs; 0 when a long reduction leaves no room)
-  int32_t rtm;           // 1: the 8-bit residual tile reaches the epilogue through tensor memory: an MMA with the identity
-                         //    matrix as its A operand turns the [pixels][128 channels] byte tile into INT32 columns beside
-                         //    the accumulator, in the accumulator's own layout (see epilogue_loop_frag)
+  int32_t frag;          // 1: the launch shape of epilogue_loop_frag
   int32_t acc_bits;      // |accumulator| < 2^acc_bits for every 8-bit operand pair: ceil(log2(K * 255 * 128 + 1))
-  int32_t acc_stride;    // tensor-memory columns between accumulator buffers: pt, or 2 * pt with rtm
-  uint32_t ident_off;    // rtm: offset of the 128 x 128 identity matrix (16 KiB, 128-byte swizzle) from the 1024-aligned base
+  int32_t acc_stride;    // tensor-memory columns between accumulator buffers
   int32_t duo;           // 1: two CTAs of a cluster (adjacent SMs) share every MMA: 256 channels x 256 pixels per pair
   int32_t ni;            // MMA issuer warps in use: min(issuer warps of the launch shape, k_blocks)
   int32_t lg_bufs;       // log2 of the accumulator / residual buffer count: tile t of a CTA uses buffer t mod 2^lg_bufs
@@ -129,7 +127,7 @@ struct SharedCtl {
   unsigned long long tstart[kMaxAccBufs];   // the tile's first (overwriting) MMA has been issued
   unsigned long long rfull[kMaxResBufs];
   unsigned long long rempty[kMaxResBufs];
-  unsigned long long ofull[kMaxResBufs];    // rtm: every epilogue warp has written its pieces of the output tile
+  unsigned long long ofull[kMaxResBufs];    // frag: every epilogue warp of the tile's group has written its pieces of the output tile
   unsigned long long drain;
   unsigned long long wfull;              // resident weight slab landed
   unsigned long long pfull[3], pempty[3];  // strip mode: input patches
@@ -313,122 +311,102 @@ __device__ __forceinline__ ChanConst chan_const_for(const TcParams& p, int ch, b
   return k;
 }
 
-// Tile loop of the launch shape for fused 8-bit residuals (eight epilogue warps and a store warp, 128-pixel tiles).
+// Tile loop of the frag shape (sixteen epilogue warps, a store warp, 128-pixel tiles).
 //
-// Nothing moves byte by byte here.  The residual tile [128 pixels][128 channels] lands in shared memory by TMA in the
-// 128-byte-swizzled K-major form of an MMA operand, and the MMA issuer multiplies it by the 128 x 128 identity matrix:
-// D2[ch][px] = sum_k I[ch][k] * R[px][k] = R[px][ch], i.e. the tensor core transposes the tile and widens it to INT32
-// in tensor-memory columns next to the accumulator.  An epilogue warp owns 16 accumulator lanes (channels) and reads
-// accumulator and residual with the same 16x256b loads, which hand thread T the values of channels t4, t4 + 8 for
-// pixel pairs -- the fragment of a 16 x 8 matrix.  It applies Eq. 4 and the residual add of Section 3.3 with the
-// constants of its two channels in registers, packs four results into a word with two saturating converts, and one
-// stmatrix (transposing, b8) writes 32 pixels x 16 channels as 16-byte row pieces into the tile the residual came
-// from (the MMA has finished reading it: the accumulator barrier is committed after the identity MMAs).  The loads of
-// the next 32 columns (or of the next tile's first) are in flight while a unit is processed.  Warps do not wait for
-// each other: each arrives on the tile's `ofull` barrier when its pieces are written, and the store warp alone waits
-// there, stores the [128][128] box (128-byte swizzle, as it was loaded) and hands the buffer back.
-// GEN: 64-bit arithmetic for every shift 1..62 (a residual shift below 9, or an INT32 residual).  SMALL: some channel
-// of the warp has c < 32 (common with 4-bit operands, whose accumulators are small): funnel-shift form of Eq. 4.
-template <bool GEN, bool RSIGNED, bool SAT, bool OSIGNED, bool RN, int SMALL = 0>
+// Nothing moves byte by byte here.  A warp reads 16 accumulator lanes with 16x256b loads, which hand thread T the values of
+// lanes t4, t4 + 8 for pixel pairs -- the fragment of a 16 x 8 matrix.  The weight rows lie on the lanes in the order of
+// encode_paired_rows_map, so that the two lanes are neighbouring channels and a matrix element of 16 bits is the channel pair
+// of one pixel: ldmatrix (transposing) delivers the residual tile [128 pixels][128 channels], as TMA left it with the 128-byte
+// swizzle, in exactly the accumulator's fragments, and stmatrix writes the packed results over it in place, 16-byte row pieces
+// of 32 pixels at a time.  The constants of a thread's two channels stay in registers.  Two groups of eight warps take
+// alternate tiles, four accumulators of 128 columns let the MMAs run ahead.  Warps do not wait for each other: each arrives on
+// the tile's `ofull` barrier when its pieces are written, and the store warp alone waits there, stores the [128][128] box and
+// hands the buffer back.  Up to eight residual / output tiles circulate: their loads in flight cover the memory latency.
+//
+// What bounds it: the integer instructions (about 6.5 per 32 values; the residual's byte extraction is one of them).  1x1 64 -> 256
+// at 56x56 / 128 -> 512 at 28x28 / 256 -> 1024 at 14x14 / 512 -> 2048 at 7x7, 256 images, L2 flushed: 101 / 58 / 42 / 34.5 us.  Before:
+// eight warps, the residual widened into tensor memory by an MMA with the identity matrix, two accumulators and one issuer
+// 115 / 65 / 44 / 35.6 us; there the issuer's own instruction latency (2.5 k cycles a tile) set the tile rate, whatever the
+// epilogue did (sixteen warps or a matrix store of another type: the same time).
+// GEN: 64-bit arithmetic for every shift 1..62 (a residual shift below 9).  SMALL: some channel of the warp has c < 32 (common
+// with 4-bit operands, whose accumulators are small): funnel-shift or pre-shift form of Eq. 4.
+template <bool RES, bool GEN, bool RSIGNED, bool SAT, bool OSIGNED, bool RN, int SMALL = 0>
 __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
   const EpiCtx e = e_in;
   const TcParams& p = *e.p;
   SharedCtl& ctl = *e.ctl;
-  const int lane = e.lane, q = e.q, hh = e.half;
+  const int lane = e.lane, q = e.q, hh = (e.ew >> 2) & 1, group = e.ew >> 3;
   const int t4 = lane >> 2;
-  ChanConst k[2];                                   // channels 32 q + 16 hh + 8 r + t4, r = 0, 1
+  ChanConst k[2];                                   // channels 32 q + 16 hh + 2 t4 + r, on lanes 32 q + 16 hh + t4 + 8 r (see encode_paired_rows_map)
 #pragma unroll
-  for (int r = 0; r < 2; ++r) k[r] = chan_const_for(p, e.c_tile * kTileC + 32 * q + 16 * hh + 8 * r + t4, !GEN, RN, SMALL == 2);
-  const uint32_t bmask = (1u << p.lg_bufs) - 1u, rmask = (1u << p.lg_rbufs) - 1u;
+  for (int r = 0; r < 2; ++r) k[r] = chan_const_for(p, e.c_tile * kTileC + 32 * q + 16 * hh + 2 * t4 + r, !GEN, RN, SMALL == 2);
+  const uint32_t rmask = (1u << p.lg_rbufs) - 1u;
   constexpr int units = 4;                          // 32 pixel columns per unit, 128-pixel tiles
   const uint32_t t_lane = e.tmem_base + ((uint32_t)(q * 32 + 16 * hh) << 16);
   // byte offset of this thread's 16-byte piece in a unit's 32 rows: row `lane`, chunk (2 q + hh) ^ (row % 8)
   const uint32_t row_off = (uint32_t)lane * 128u + ((uint32_t)((2 * q + hh) ^ (lane & 7)) << 4);
-  if (e.p_tile0 >= p.p_tiles) return;
   auto wait_bar = [&](unsigned long long* bar, uint32_t ph) -> bool {
     uint32_t w = 1;
     if (lane == 0) w = mbar_wait(smem_u32(bar), ph, &ctl, p.status, HQ_DEV_TIMEOUT_EPILOGUE) ? 1u : 0u;
     return __shfl_sync(0xffffffffu, w, 0) != 0;
   };
-  auto one = [&](int acc, int r, const ChanConst& c) -> int {
+  auto one = [&](int acc, unsigned word, int i, const ChanConst& c) -> int {
+    const int r = !RES ? 0 : (int)hq_prmt(word, 0u, RSIGNED ? 0x8880u + 0x1111u * i : 0x4440u + i);
     if (GEN) {
-      const long long y = (((long long)acc * (long long)c.b + c.r0) >> c.sh) + (((long long)r * (long long)c.rb + c.rr0) >> c.rsh);
+      const long long y = (hq_mad_wide(acc, c.b, c.r0) >> c.sh) + (hq_mad_wide(r, c.rb, c.rr0) >> c.rsh);
       return hq_clamp_ll(y, p.relu, p.qmin, p.qmax);
     }
-    const int y = requant_fast<true, RSIGNED, SMALL, RN>(acc, r, c);
+    const int y = requant_fast<RES, RSIGNED, SMALL, RN>(acc, r, c);
     return SAT ? y : min(max(y, e.lo), e.hi);
   };
   // one unit: 16 values per thread -> four words -> one transposing store of 32 pixel rows x 16 channel bytes
-  auto unit = [&](const int (&va)[16], const int (&vr)[16], uint32_t tile, int u) {
+  auto unit = [&](const int (&v)[16], const unsigned (&r)[4], uint32_t at) {
     unsigned w[4];
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-      const int y0 = one(va[4 * g + 0], vr[4 * g + 0], k[0]), y1 = one(va[4 * g + 1], vr[4 * g + 1], k[0]);
-      const int y2 = one(va[4 * g + 2], vr[4 * g + 2], k[1]), y3 = one(va[4 * g + 3], vr[4 * g + 3], k[1]);
+      // bytes of a word: (pixel 2 q2, even channel), (2 q2, odd), (2 q2 + 1, even), (2 q2 + 1, odd)
+      const int y0 = one(v[4 * g + 0], r[g], 0, k[0]), y1 = one(v[4 * g + 2], r[g], 1, k[1]);
+      const int y2 = one(v[4 * g + 1], r[g], 2, k[0]), y3 = one(v[4 * g + 3], r[g], 3, k[1]);
       w[g] = sat_pack4<OSIGNED>(y0, y1, y2, y3);
     }
-    // this thread names the row of pixel 32 u + lane: 16 bytes at channel offset 32 q + 16 hh of the row (row_off)
-    if (e.warp_live) stmatrix_t_x4(tile + row_off + (uint32_t)u * 4096u, w[0], w[1], w[2], w[3]);
-  };
-  auto issue = [&](uint32_t as, int u, int (&va)[16], int (&vr)[16]) {
-    const uint32_t t_addr = t_lane + as * p.acc_stride + 32 * u;
-    tmem_ld_frag16(t_addr, va);
-    tmem_ld_frag16(t_addr + p.pt, vr);
+    if (e.warp_live) stmatrix_t_x4(at, w[0], w[1], w[2], w[3]);
   };
 
-  int a0[16], r0[16], a1[16], r1[16];
-  uint32_t tcount = 0, as = 0;
-  int p_tile = e.p_tile0;
-  if (!wait_bar(&ctl.tfull[0], 0)) return;          // accumulator AND transposed residual are in tensor memory
-  tc_fence_after();
-  issue(0, 0, a0, r0);
-  bool pending = true;
-  while (true) {
-    const uint32_t rs = tcount & rmask;
-    const uint32_t tile = e.res_stage + rs * e.res_tile_bytes;          // [128 pixels][128 bytes], 128-byte swizzle
-    const bool has_next = p_tile + e.p_step < p.p_tiles;
-    const uint32_t nas = (tcount + 1u) & bmask, naph = ((tcount + 1u) >> p.lg_bufs) & 1u;
-    bool ok = true, next_issued = false;
+  int a0[16], a1[16];
+  unsigned r0[4] = {0u, 0u, 0u, 0u}, r1[4] = {0u, 0u, 0u, 0u};
+  uint32_t tcount = (uint32_t)group;
+  for (int p_tile = e.p_tile0 + group * e.p_step; p_tile < p.p_tiles; p_tile += kFragGroups * e.p_step, tcount += kFragGroups) {
+    const uint32_t as = tcount & (kFragAccs - 1), aph = (tcount / kFragAccs) & 1u;
+    const uint32_t rs = tcount & rmask, rph = (tcount >> p.lg_rbufs) & 1u;
+    const uint32_t at = e.res_stage + rs * e.res_tile_bytes + row_off;  // tile: [128 pixels][128 bytes], 128-byte swizzle
+    if (!wait_bar(&ctl.tfull[as], aph)) break;
+    if (!(RES ? wait_bar(&ctl.rfull[rs], rph) : wait_bar(&ctl.rempty[rs], rph ^ 1u))) break;
+    tc_fence_after();
+    const uint32_t t_addr = t_lane + as * kTileC;
+    tmem_ld_frag16(t_addr, a0);
+    if (RES) ldmatrix_t_x4(at, r0);
 #pragma unroll
     for (int u = 0; u < units; u += 2) {
-      // ---- unit u (registers a0 / r0), while unit u + 1 streams into a1 / r1
       tmem_ld_wait();
-      issue(as, u + 1, a1, r1);
-      unit(a0, r0, tile, u);
-      // ---- unit u + 1, while the next unit streams into a0 / r0
+      tmem_ld_frag16(t_addr + 32 * (u + 1), a1);
+      if (RES) ldmatrix_t_x4(at + (u + 1) * 4096u, r1);
+      unit(a0, r0, at + u * 4096u);
       tmem_ld_wait();
-      pending = false;
       if (u + 2 < units) {
-        issue(as, u + 2, a0, r0);
-        pending = true;
+        tmem_ld_frag16(t_addr + 32 * (u + 2), a0);
+        if (RES) ldmatrix_t_x4(at + (u + 2) * 4096u, r0);
       } else {
-        // every lane has read its last columns of this tile: hand the accumulator buffer back, and start on the next
-        // tile's first unit if that tile is already there (else after this unit's arithmetic)
+        // every lane has read its last columns of this tile: hand the accumulator buffer back
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) release_accumulator(p, ctl, as);
-        if (has_next) {
-          uint32_t there = 0;
-          if (lane == 0) there = mbar_try_wait(smem_u32(&ctl.tfull[nas]), naph) ? 1u : 0u;
-          if (__shfl_sync(0xffffffffu, there, 0)) { tc_fence_after(); issue(nas, 0, a0, r0); pending = true; next_issued = true; }
-        }
+        if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[as]));
       }
-      unit(a1, r1, tile, u + 1);
+      unit(a1, r1, at + (u + 1) * 4096u);
     }
     fence_async_smem();                             // make this lane's pieces visible to the TMA engine
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(&ctl.ofull[rs]));
-    if (!has_next) break;
-    if (!next_issued) {
-      ok = wait_bar(&ctl.tfull[nas], naph);
-      if (!ok) break;
-      tc_fence_after();
-      issue(nas, 0, a0, r0);
-      pending = true;
-    }
-    p_tile += e.p_step; ++tcount; as = nas;
   }
-  if (pending) tmem_ld_wait();
 }
 
 // Tile loop of the instantiation for INT32 results.  Two uses:
@@ -787,16 +765,58 @@ __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanCo
     if (staged_out && lane == 0) tma_store_wait_all();
 }
 
+// MMA issue of the frag shape: issuer `c` of `n` takes the tiles c, c + n, ...  (One thread needs 1-2 k cycles per tile, nearly
+// all of it the latency of its own instructions between one barrier and the next.)  The accumulator's barrier is awaited before
+// the operands': it says that the tile four earlier has been consumed.  A wait for a stage's n-th fill cannot tell it from the
+// (n-2)-nd unless the (n-1)-st is known to have landed, which that barrier shows where the ring holds four tiles: two issuers only there.
+template <int STEPS>
+__device__ __forceinline__ void frag_issue(const TcParams& p, SharedCtl& ctl, int c, int n, uint32_t tiles, uint32_t stage_bytes,
+                                          uint32_t w_bytes, uint32_t tmem_base, int p_tile0, int p_step) {
+  const uint32_t idesc = (2u << 4) | (1u << 7) | ((uint32_t)(p.x_signed ? 1 : 0) << 10) | ((uint32_t)(kTileC >> 3) << 17) |
+                         ((uint32_t)(kTileC >> 4) << 24);
+  const uint64_t hi = smem_desc(0, STEPS * 32);
+  const uint32_t x_off = p.wres ? 0u : w_bytes;
+  const uint32_t nstages = (uint32_t)p.stages;
+  const int k_blocks = p.k_blocks;
+  const bool tail = p.tail_steps != STEPS;
+  if (p.wres && !mbar_wait(smem_u32(&ctl.wfull), 0, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) return;
+  uint32_t s = 0, ph = 0, tcount = (uint32_t)c;
+  auto skip = [&](int blocks) { for (int i = 0; i < blocks; ++i) if (++s == nstages) { s = 0; ph ^= 1u; } };
+  skip(c * k_blocks);
+  for (int p_tile = p_tile0 + c * p_step; p_tile < p.p_tiles; p_tile += n * p_step, tcount += (uint32_t)n) {
+    const uint32_t as = tcount & (kFragAccs - 1), aph = (tcount / kFragAccs) & 1u;
+    const uint32_t d = tmem_base + as * kTileC;
+    if (!mbar_wait(smem_u32(&ctl.tempty[as]), aph ^ 1u, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) return;
+    for (int kb = 0, chunk = 0; kb < k_blocks; ++kb) {
+      if (!mbar_wait(smem_u32(&ctl.full[s]), ph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) return;
+      tc_fence_after();
+      const uint32_t x = tiles + s * stage_bytes, w = p.wres ? tiles + p.wres_off + (uint32_t)kb * w_bytes : x;
+      const uint64_t ad = hi | (uint64_t)((w >> 4) & 0x3FFF), bd = hi | (uint64_t)(((x + x_off) >> 4) & 0x3FFF);
+      const bool last = ++chunk == p.cchunks;
+      if (last) chunk = 0;
+      if (tail && last) {
+        for (int k = 0; k < p.tail_steps; ++k) mma_i8(d, ad + 2 * k, bd + 2 * k, idesc, (kb | k) ? 1u : 0u);
+      } else {
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) mma_i8(d, ad + 2 * k, bd + 2 * k, idesc, k ? 1u : kb ? 1u : 0u);
+      }
+      if (kb + 1 == k_blocks) mma_commit(smem_u32(&ctl.tfull[as]));
+      mma_commit(smem_u32(&ctl.empty[s]));
+      if (++s == nstages) { s = 0; ph ^= 1u; }
+    }
+    skip((n - 1) * k_blocks);
+  }
+}
+
 // ---------------------------------------------------------------- the kernel -----------------
 // DUO: the instantiation that may be launched as clusters of two CTAs sharing their MMAs; only it contains the
 // cta_group::2 instructions (a kernel that contains them cannot be launched without clusters).
-// RTM: the instantiation for fused 8-bit residuals that travel through tensor memory; it has one more warp, which
-// stores the finished output tiles.
+// FRAG: the instantiation of the frag shape; it has one more warp, which stores the finished output tiles.
 // WIDE: the instantiations for INT32 results (epilogue_loop_wide), kRaw32 or through the residual add of Fig. 2, kAdd32.  (One for
 // both ran the add 0.6 % slower as soon as the raw form's waits for parameters were in it; the add only runs in networks.)
 constexpr int kRaw32 = 1, kAdd32 = 2;
-template <int EPI_WARPS, int MIN_CTAS, int MMA_WARPS, bool DUO = false, bool RTM = false, int WIDE = 0>
-__global__ void __launch_bounds__(32 * (1 + MMA_WARPS + EPI_WARPS + (RTM ? 1 : 0)), MIN_CTAS)
+template <int EPI_WARPS, int MIN_CTAS, int MMA_WARPS, bool DUO = false, bool FRAG = false, int WIDE = 0>
+__global__ void __launch_bounds__(32 * (1 + MMA_WARPS + EPI_WARPS + (FRAG ? 1 : 0)), MIN_CTAS)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_res,
                const __grid_constant__ CUtensorMap map_q, const __grid_constant__ TcParams p) {
@@ -825,15 +845,15 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.full[s]), 1); mbar_init(smem_u32(&ctl.empty[s]), 1); }
     for (int s = 0; s < (1 << p.lg_bufs); ++s) {
-      mbar_init(smem_u32(&ctl.tfull[s]), p.ni); mbar_init(smem_u32(&ctl.tempty[s]), (4 * p.halves) << p.duo);
+      mbar_init(smem_u32(&ctl.tfull[s]), FRAG ? 1 : p.ni); mbar_init(smem_u32(&ctl.tempty[s]), (4 * p.halves) << p.duo);
       mbar_init(smem_u32(&ctl.tstart[s]), 1);
     }
     for (int s = 0; s < (1 << p.lg_rbufs); ++s) {
       mbar_init(smem_u32(&ctl.rfull[s]), 1);
-      mbar_init(smem_u32(&ctl.rempty[s]), RTM ? 1 : 4 * p.halves);
-      mbar_init(smem_u32(&ctl.ofull[s]), EPI_WARPS);
+      mbar_init(smem_u32(&ctl.rempty[s]), FRAG ? 1 : 4 * p.halves);
+      mbar_init(smem_u32(&ctl.ofull[s]), EPI_WARPS / kFragGroups);
     }
-    mbar_init(smem_u32(&ctl.drain), p.ni);
+    mbar_init(smem_u32(&ctl.drain), FRAG ? MMA_WARPS : p.ni);
     mbar_init(smem_u32(&ctl.wfull), 1);
     if constexpr (WIDE) for (int s = 0; s < kWideWarps * kWideSlots; ++s) mbar_init(smem_u32(&ctl.wbox[s / kWideSlots][s % kWideSlots]), 1);
     for (int s = 0; s < 3; ++s) { mbar_init(smem_u32(&ctl.pfull[s]), 1); mbar_init(smem_u32(&ctl.pempty[s]), p.ni); }
@@ -841,18 +861,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) { if constexpr (DUO) tmem_alloc2(smem_u32(&ctl.tmem_base), p.tmem_cols); else tmem_alloc(smem_u32(&ctl.tmem_base), p.tmem_cols); }
-  if (p.rtm) {
-    // the identity matrix as a K-major MMA operand, [128 rows][128 bytes] with the 128-byte swizzle: 16-byte chunk
-    // c of row r sits at chunk position c ^ (r % 8); row r holds a single 1 at byte r
-    uint4* ident = (uint4*)(smem_raw + (tiles - raw) + p.ident_off);
-    for (int i = threadIdx.x; i < 1024; i += blockDim.x) {
-      const int r = i >> 3, c = (i & 7) ^ (r & 7);
-      uint32_t word[4] = {0u, 0u, 0u, 0u};
-      if (c == (r >> 4)) word[(r & 15) >> 2] = 1u << (8 * (r & 3));
-      ident[i] = make_uint4(word[0], word[1], word[2], word[3]);
-    }
-    fence_async_smem();
-  }
   tc_fence_before();
   __syncthreads();
   if constexpr (DUO) cluster_sync_all();   // both CTAs' barriers exist before either touches the other's
@@ -903,6 +911,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           } else if (p.fold) {
             tma_load_2d(w_dst, &map_w, bar, wx, 0);
             tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx, 0);
+          } else if constexpr (FRAG) {
+            tma_load_4d(w_dst, &map_w, bar, wx, 0, 0, c_tile * (kTileC / 16));
           } else {
             tma_load_2d(w_dst, &map_w, bar, wx, c_tile * kTileC);
           }
@@ -1006,6 +1016,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           } else if (p.fold) {   // 64-row box, twice: accumulator lanes 64-127 repeat lanes 0-63
             tma_load_2d(w_dst, &map_w, bar, wx, 0);
             tma_load_2d(w_dst + 64 * p.bkb, &map_w, bar, wx, 0);
+          } else if constexpr (FRAG) {
+            tma_load_4d(w_dst, &map_w, bar, wx, 0, 0, c_tile * (kTileC / 16));
           } else {
             tma_load_2d(w_dst, &map_w, bar, wx, c_tile * kTileC);
           }
@@ -1063,7 +1075,21 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     // does not care about the order of the blocks; only the tile's first MMA, which overwrites the accumulator,
     // must come first: whoever issues it signals `tstart` and the others wait for that.
     const int iss = warp - 1;
-    if (iss < p.ni && rank == 0 && elect_one()) {
+    if constexpr (FRAG) {
+      if (elect_one()) {
+        if (iss < p.ni) {
+          if (p.bkb == 128) frag_issue<4>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step);
+          else if (p.bkb == 64) frag_issue<2>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step);
+          else frag_issue<1>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step);
+        }
+        // Drain: all issued MMAs must have completed before tensor memory is freed.
+        mma_commit(smem_u32(&ctl.drain));
+        const unsigned long long t0 = global_ns();
+        while (!mbar_try_wait(smem_u32(&ctl.drain), 0)) {
+          if (global_ns() - t0 > kWaitBudgetNs) { atomicCAS(p.status, 0u, (uint32_t)HQ_DEV_TIMEOUT_DRAIN); break; }
+        }
+      }
+    } else if (iss < p.ni && rank == 0 && elect_one()) {
       // instruction descriptor: D = S32, A = s8 weights, B = u8/s8 activations, both K-major, N = pt,
       // M = 128 (256 over the two CTAs of a pair)
       const uint32_t idesc = (2u << 4) | (1u << 7) | ((uint32_t)(p.x_signed ? 1 : 0) << 10) |
@@ -1108,31 +1134,17 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           uint64_t adesc = desc_hi | (uint64_t)((a_addr >> 4) & 0x3FFF);
           uint64_t bdesc = desc_hi | (uint64_t)(((w_addr + x_off) >> 4) & 0x3FFF);
           if constexpr (DUO) {
-            for (int k = 0; k < nsteps; ++k, adesc += 2, bdesc += 2)
-              mma_i8_2cta(d_tmem, adesc, bdesc, idesc, (kb | k) ? 1u : 0u);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (k < nsteps) mma_i8_2cta(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, k ? 1u : kb ? 1u : 0u);
           } else {
             for (int k = 0; k < nsteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
               mma_i8(d_tmem, adesc, bdesc, idesc, (kb | k) ? 1u : 0u);
           }
           // the accumulator's barrier first on the last K block: the epilogue is the one waiting
-          if (kb + 1 == p.k_blocks && !p.rtm) commit(smem_u32(&ctl.tfull[as]));
+          if (kb + 1 == p.k_blocks) commit(smem_u32(&ctl.tfull[as]));
           commit(smem_u32(&ctl.empty[s]));         // frees the stage when these MMAs have read it
           if (++s == nstages) { s = 0; ph ^= 1u; }
-        }
-        if (p.rtm && ok) {
-          // The residual tile through the tensor core: D2[ch][px] = sum_k I[ch][k] * R[px][k] = R[px][ch], INT32, in the
-          // pt columns after the accumulator.  Four MMAs of 32 channels of K each; the accumulator barrier then stands
-          // for both results, and for the tile in shared memory being free to be overwritten by the outputs.
-          const uint32_t rs = tcount & ((1u << p.lg_rbufs) - 1u), rph = (tcount >> p.lg_rbufs) & 1u;
-          if (!mbar_wait(smem_u32(&ctl.rfull[rs]), rph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) { ok = false; break; }
-          tc_fence_after();
-          const uint64_t hi128 = smem_desc(0, 128);
-          uint64_t adesc = hi128 | (uint64_t)(((tiles + p.ident_off) >> 4) & 0x3FFF);
-          uint64_t bdesc = hi128 | (uint64_t)(((res_stage + rs * res_tile_bytes) >> 4) & 0x3FFF);
-          const uint32_t idesc_r = (2u << 4) | (1u << 7) | ((uint32_t)(p.res_signed ? 1 : 0) << 10) |
-                                   ((uint32_t)(p.pt >> 3) << 17) | ((uint32_t)(kTileC >> 4) << 24);
-          for (int k = 0; k < 4; ++k, adesc += 2, bdesc += 2) mma_i8(d_tmem + p.pt, adesc, bdesc, idesc_r, k ? 1u : 0u);
-          commit(smem_u32(&ctl.tfull[as]));
         }
       }
       };
@@ -1206,8 +1218,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         if (global_ns() - t0 > kWaitBudgetNs) { atomicCAS(p.status, 0u, (uint32_t)HQ_DEV_TIMEOUT_DRAIN); break; }
       }
     }
-  } else if (RTM && warp == 1 + MMA_WARPS + EPI_WARPS) {
-    // ------------------------------------------------------------ store warp (rtm): finished tiles leave by TMA
+  } else if (FRAG && warp == 1 + MMA_WARPS + EPI_WARPS) {
+    // ------------------------------------------------------------ store warp (frag): finished tiles leave by TMA
     if (elect_one()) {
       const uint32_t rmask = (1u << p.lg_rbufs) - 1u;
       uint32_t tcount = 0;
@@ -1325,34 +1337,27 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     e.warp = warp; e.lane = lane; e.q = q; e.cq = cq; e.ew = ew; e.half = half; e.col0 = col0; e.px_per_warp = px_per_warp; e.ch = ch;
     e.c_tile = c_tile; e.p_tile0 = p_tile0; e.p_step = p_step; e.lo = lo; e.hi = hi;
     e.ch_live = ch_live; e.warp_live = warp_live;
-    if (p.rtm) {
-      if constexpr (RTM) {
-        // residual through tensor memory: the fragment loop, in its general form when some channel needs 64-bit steps
-        const bool rn = warp_narrow;
+    if constexpr (FRAG) {
+        const bool rn = warp_narrow, os = p.out_signed != 0, rs = p.res_signed != 0;
+        // (narrow residual pairs only with the plain and the pre-shift form; the funnel-shift form keeps the multiply-high term)
+#define HQ_FRAG(S, OS) do { \
+          if (!p.res) { if (!warp_small) epilogue_loop_frag<false, false, false, S, OS, false, 0>(e); \
+                        else if (warp_pre) epilogue_loop_frag<false, false, false, S, OS, false, 2>(e); \
+                        else epilogue_loop_frag<false, false, false, S, OS, false, 1>(e); } \
+          else if (warp_small && !warp_pre) { if (rs) epilogue_loop_frag<true, false, true, S, OS, false, 1>(e); else epilogue_loop_frag<true, false, false, S, OS, false, 1>(e); } \
+          else if (warp_small) { if (rs) HQ_FRAG_RES(true, S, OS, 2); else HQ_FRAG_RES(false, S, OS, 2); } \
+          else { if (rs) HQ_FRAG_RES(true, S, OS, 0); else HQ_FRAG_RES(false, S, OS, 0); } } while (0)
+#define HQ_FRAG_RES(RS, S, OS, SM) do { if (rn) epilogue_loop_frag<true, false, RS, S, OS, true, SM>(e); \
+                                        else epilogue_loop_frag<true, false, RS, S, OS, false, SM>(e); } while (0)
         if (!fast) {
-          if (p.out_signed) epilogue_loop_frag<true, false, false, true, false>(e); else epilogue_loop_frag<true, false, false, false, false>(e);
-        } else if (warp_small) {
-          // (narrow residual pairs only with the pre-shift form; the funnel-shift form keeps the plain multiply-high term)
-#define HQ_FRAG_SMALL(RS, S, OS) do { if (warp_pre && rn) epilogue_loop_frag<false, false, S, OS, true, 2>(e); \
-                                      else if (warp_pre) epilogue_loop_frag<false, RS, S, OS, false, 2>(e); \
-                                      else epilogue_loop_frag<false, RS, S, OS, false, 1>(e); } while (0)
-          if (p.sat_pack) {
-            if (p.out_signed) { if (p.res_signed) HQ_FRAG_SMALL(true, true, true); else HQ_FRAG_SMALL(false, true, true); }
-            else { if (p.res_signed) HQ_FRAG_SMALL(true, true, false); else HQ_FRAG_SMALL(false, true, false); }
-          } else {
-            if (p.out_signed) { if (p.res_signed) HQ_FRAG_SMALL(true, false, true); else HQ_FRAG_SMALL(false, false, true); }
-            else { if (p.res_signed) HQ_FRAG_SMALL(true, false, false); else HQ_FRAG_SMALL(false, false, false); }
-          }
-#undef HQ_FRAG_SMALL
-        } else if (p.sat_pack) {
-          if (p.out_signed) { if (rn) epilogue_loop_frag<false, false, true, true, true>(e); else if (p.res_signed) epilogue_loop_frag<false, true, true, true, false>(e); else epilogue_loop_frag<false, false, true, true, false>(e); }
-          else { if (rn) epilogue_loop_frag<false, false, true, false, true>(e); else if (p.res_signed) epilogue_loop_frag<false, true, true, false, false>(e); else epilogue_loop_frag<false, false, true, false, false>(e); }
-        } else {
-          if (p.out_signed) { if (rn) epilogue_loop_frag<false, false, false, true, true>(e); else if (p.res_signed) epilogue_loop_frag<false, true, false, true, false>(e); else epilogue_loop_frag<false, false, false, true, false>(e); }
-          else { if (rn) epilogue_loop_frag<false, false, false, false, true>(e); else if (p.res_signed) epilogue_loop_frag<false, true, false, false, false>(e); else epilogue_loop_frag<false, false, false, false, false>(e); }
-        }
-      }
-    } else if (half >= p.halves) {
+          if (os) { if (rs) epilogue_loop_frag<true, true, true, false, true, false>(e); else epilogue_loop_frag<true, true, false, false, true, false>(e); }
+          else { if (rs) epilogue_loop_frag<true, true, true, false, false, false>(e); else epilogue_loop_frag<true, true, false, false, false, false>(e); }
+        } else if (p.sat_pack) { if (os) HQ_FRAG(true, true); else HQ_FRAG(true, false); }
+        else { if (os) HQ_FRAG(false, true); else HQ_FRAG(false, false); }
+#undef HQ_FRAG_RES
+#undef HQ_FRAG
+    } else {
+    if (half >= p.halves) {
       // the 64-pixel tile has one 64-column slice per lane quarter: this warp only took part in the vote above
     } else if (fast && p.staged_out && p.out_bits == 4 && !p.res && !p.strip && lo >= 0 && hi <= 15) {
       // unsigned 4-bit outputs without a residual (the convs inside a 4-bit block)
@@ -1362,8 +1367,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     } else if (fast && p.staged_out && p.out_bits == 8 && (!p.res || p.staged_res)) {
       const int variant = (p.res ? 4 : 0) | ((p.res && p.res_signed) ? 2 : 0) | (p.sat_pack ? 1 : 0);
       switch (variant) {
-#define HQ_FAST8(R, RS, S, OS) do { if (RTM) { \
-                                    } else if (warp_pre && R && warp_narrow) epilogue_loop_fast8<R, RS, S, OS, 2, R>(e, k); \
+#define HQ_FAST8(R, RS, S, OS) do { if (warp_pre && R && warp_narrow) epilogue_loop_fast8<R, RS, S, OS, 2, R>(e, k); \
                                     else if (warp_pre) epilogue_loop_fast8<R, RS, S, OS, 2, false>(e, k); \
                                     else if (warp_small) epilogue_loop_fast8<R, RS, S, OS, 1, false>(e, k); \
                                     else if (R && warp_narrow) epilogue_loop_fast8<R, RS, S, OS, 0, R>(e, k); \
@@ -1378,6 +1382,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
       }
     } else {
       epilogue_loop_general(e, k, fast);
+    }
     }
     }
   }
@@ -1460,7 +1465,7 @@ bool hq_conv_tc_init() {
                               kSmemAttr) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               112 * 1024) == cudaSuccess &&
-         cudaFuncSetAttribute(conv_tc_kernel<8, 1, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAttr) == cudaSuccess &&
+         cudaFuncSetAttribute(conv_tc_kernel<kFragWarps, 1, kFragIssuers, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAttr) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kRaw32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               kSmemAttr) == cudaSuccess &&
          cudaFuncSetAttribute(conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kAdd32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1543,7 +1548,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // (measured: with the weight slab resident the one-CTA shape catches up for K >= 128; the pair shape still
   // wins on the fused-residual expansions with the shortest reduction, and loses where a tile carries little
   // epilogue work, e.g. 64 output channels.  Where the layer is large enough for 256-pixel tiles and its residual
-  // travels by TMA, the rtm shape below is faster still: 64 -> 256 at 56x56, batch 256: 129 -> 122 us.)
+  // travels by TMA, the frag shape below is faster still: 64 -> 256 at 56x56, batch 256: 129 -> 101 us.)
   const bool wide_fits = p.staged_res && a.out_bits == 8 && a.cout > 64 && pick_pt(P, p.c_tiles, h->sm_count, 256) == 256;
   bool pair = !a.wide && k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !wide_fits;
   int stages = 0, stage_bytes = 0, res_tile_bytes = 0, out_tile_bytes = 0, wres_bytes = 0;
@@ -1586,7 +1591,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
         res_tile_bytes = p.staged_res ? p.pt * kTileC : 0;
         // residual tiles: as many buffers as accumulators, fewer when a long reduction needs the room for stages
         // (its epilogue has slack: a single residual buffer only delays the next tile's prefetch)
-        // The rtm shape (below) works in place in the residual tiles and needs no staging box; with the
+        // The frag shape (below) works in place in the residual tiles and needs no staging box; with the
         // weights resident two stages are enough for its short reductions (the epilogue bounds the tile).
         const bool wide_here = p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && p.staged_res && k_total < 1024;
         if (wide_here) out_tile_bytes = 0;
@@ -1653,18 +1658,13 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     // Measured: several issuers pay off where the operands are mostly in shared memory already (strip form,
     // resident weights); where every block waits for 48 KiB from L2 the tile is bound by that stream and the extra
     // issuers only cost a few percent.
-    // Third launch shape, *rtm*, for the fused 8-bit residual with a short reduction on layers large enough for
-    // 256-pixel tiles (here called `wide` for the condition it shares with the tile choice above): the residual tile
-    // goes through the tensor core into tensor memory, see epilogue_loop_frag.  Measured against the shape it replaced
-    // (sixteen warps, one channel per thread, one byte load and one byte store per value, in place in the residual tile):
-    // 1x1 64 -> 256 at 56x56, batch 256, 125 -> 122 us; 128 -> 512 at 28x28 72 -> 70 us; no byte-wise shared-memory
-    // traffic is left, the epilogue is bound by the integer instructions of Eq. 4 and the residual term themselves.
+    // Third launch shape, *frag*, for the fused 8-bit residual with a short reduction on layers large enough for
+    // 256-pixel tiles (here called `wide` for the condition it shares with the tile choice above): see epilogue_loop_frag.
     wide = !pair && !p.strip && p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && p.staged_res && k_total < 1024;
     if (wide) {
-      // 128-pixel tiles, two buffers of (accumulator + transposed residual) = 512 tensor-memory columns; the two
-      // residual tiles double as the output boxes; the identity matrix takes 16 KiB
-      p.rtm = 1; p.halves = 2;
-      p.pt = 128; p.lg_bufs = 1; p.lg_rbufs = 1;
+      // 128-pixel tiles, four accumulators; the residual tiles double as the output boxes
+      p.frag = 1; p.halves = 2;
+      p.pt = 128; p.lg_bufs = 2; p.lg_rbufs = 1;
       p.p_tiles = (int32_t)((P + p.pt - 1) / p.pt);
       out_tile_bytes = 0;
       res_tile_bytes = p.pt * kTileC;
@@ -1672,10 +1672,11 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       p.wres = wres_bytes <= 72 * 1024 ? 1 : 0;
       if (!p.wres) wres_bytes = 0;
       stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
-      // four residual / output tiles when they leave room for three operand stages: a tile is held from its load to
-      // the end of its store, and the loads of the next tiles must be in flight meanwhile to cover the memory latency
-      for (p.lg_rbufs = 2; ; --p.lg_rbufs) {
-        stages = (kSmemBudget - (res_tile_bytes << p.lg_rbufs) - wres_bytes - 16 * 1024) / stage_bytes;
+      // eight residual / output tiles where they leave room for three operand stages, else four: a tile is held from its load
+      // to the end of its store, and the loads of the next tiles must be in flight meanwhile to cover the memory latency (with
+      // arithmetic and matrix stores left out, 1x1 64 -> 256 at 56x56: four tiles 93 us, eight 87)
+      for (p.lg_rbufs = 3; ; --p.lg_rbufs) {
+        stages = (kSmemBudget - (res_tile_bytes << p.lg_rbufs) - wres_bytes) / stage_bytes;
         if (stages >= 3 || p.lg_rbufs == 1) break;
       }
     }
@@ -1690,9 +1691,12 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     }
     // (the dealt loop knows whole K blocks only: channels that do not fill their last block take the single issuer)
     const bool tail = a.cin % p.bkb > 0 && a.cin % p.bkb <= p.bkb - 32;
-    const int issuers = pair ? kPairIssuerWarps : wide ? 1 : (p.strip || (p.wres && !tail)) ? kSoloIssuerWarps : 1;
+    const int issuers = pair ? kPairIssuerWarps : (p.strip || (p.wres && !tail)) ? kSoloIssuerWarps : 1;
     p.ni = p.k_blocks < issuers ? p.k_blocks : issuers;
-    if (!(p.strip && p.wres)) {
+    if (wide) {
+      if (stages > kMaxStages) stages = kMaxStages;
+      p.ni = stages >= kFragAccs * p.k_blocks ? kFragIssuers : 1;           // (see frag_issue)
+    } else if (!(p.strip && p.wres)) {
       while (p.ni > 1 && stages < p.ni) --p.ni;
       if (stages > kMaxStages) stages = kMaxStages;
       // every stage counts more than the third issuer: the bytes in flight set the tile rate of the layers that wait
@@ -1701,7 +1705,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       stages -= stages % p.ni;
     }
   }
-  p.acc_stride = p.rtm ? 2 * p.pt : p.pt;
+  p.acc_stride = p.pt;
   p.w_blocks = p.pairs ? 6 : p.k_blocks;
   p.tail_steps = (a.cin - (p.cchunks - 1) * p.bkb + 31) >> 5;
   { const long long bound = k_total * 255 * 128; int bits = 0; while ((1LL << bits) <= bound) ++bits; p.acc_bits = bits; }
@@ -1713,7 +1717,6 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.res_stage_off = p.out_stage_off + (uint32_t)out_tile_bytes;
   p.wres_off = p.res_stage_off + ((uint32_t)res_tile_bytes << p.lg_rbufs);
   p.patch_off = p.wres_off + (uint32_t)wres_bytes;
-  p.ident_off = p.patch_off + (uint32_t)patch_total;
   p.bias = a.bias; p.b = a.b; p.c = a.c;
   p.res = a.res; p.res_bits = a.res_bits; p.res_signed = a.res_signed; p.rb = a.rb; p.rc = a.rc;
   p.res_narrow = (a.res && a.res_bits == 8) ? (const int4*)a.res_narrow : nullptr;
@@ -1759,10 +1762,12 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     if (g_encode_tiled(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(a.wgt), dims, strides, box, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return HQ_ERR_CUDA;
+  } else if (p.frag) {
+    if (!encode_paired_rows_map(&map_w, a.wgt, a.cout, (long long)a.kh * a.kw * a.cin, p.bkb, swz)) return HQ_ERR_CUDA;
   } else if (!encode_rows_map(&map_w, a.wgt, a.cout, (long long)a.kh * a.kw * a.cin, p.bkb, p.fold ? 64 : kTileC, swz)) return HQ_ERR_CUDA;
   map_out = map_w; map_res = map_w; map_q = map_w;                    // valid placeholders when a path is not staged
-  // (with rtm the residual tile is an MMA operand and, later, the output box: 128-byte swizzle both ways)
-  const CUtensorMapSwizzle box_swz = p.rtm ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;
+  // (with frag the residual tile becomes the output box: 128-byte swizzle both ways)
+  const CUtensorMapSwizzle box_swz = p.frag ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;
   if (p.strip) {
     // output (C, W, H, N), box = 32 positions of the raster: 32 channels x min(pitch, 32) columns x the rows that makes
     const cuuint32_t bw = p.lg_wp >= 5 ? 32u : (1u << p.lg_wp);
@@ -1774,7 +1779,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return HQ_ERR_CUDA;
   } else
-  if (p.staged_out && !encode_rows_map(&map_out, a.out, P, out_row_bytes, p.rtm ? kTileC : a.out_bits == 4 ? 16 : 32, p.rtm ? p.pt : p.pt / (p.halves << p.fold),
+  if (p.staged_out && !encode_rows_map(&map_out, a.out, P, out_row_bytes, p.frag ? kTileC : a.out_bits == 4 ? 16 : 32, p.frag ? p.pt : p.pt / (p.halves << p.fold),
                                        box_swz)) return HQ_ERR_CUDA;
   if (p.staged_res && !encode_rows_map(&map_res, a.res, P, a.cout, kTileC, p.pt, box_swz))
     return HQ_ERR_CUDA;
@@ -1785,8 +1790,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     if (p.q_out && !encode_rows_map(&map_q, p.q_out, P, a.cout, 32, 16, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
   }
 
-  const size_t dyn_smem = (size_t)stages * stage_bytes + out_tile_bytes + ((size_t)res_tile_bytes << p.lg_rbufs) + wres_bytes + patch_total +
-                          (p.rtm ? 16 * 1024 : 0) + 1024;
+  const size_t dyn_smem = (size_t)stages * stage_bytes + out_tile_bytes + ((size_t)res_tile_bytes << p.lg_rbufs) + wres_bytes + patch_total + 1024;
   const long long total_tiles = (long long)p.p_tiles * p.c_tiles;
   // a multiple of c_tiles, so that every CTA keeps one channel tile
   const int slots = pair ? 2 * h->sm_count : h->sm_count;
@@ -1805,8 +1809,8 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     cfg.blockDim = dim3(32 * (2 + kSoloEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
     err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, 1, true>, map_x, map_w, map_out, map_res, map_q, p);
   } else if (wide) {
-    cfg.blockDim = dim3(32 * 11); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
-    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<8, 1, 1, false, true>, map_x, map_w, map_out, map_res, map_q, p);
+    cfg.blockDim = dim3(32 * (2 + kFragIssuers + kFragWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
+    err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kFragWarps, 1, kFragIssuers, false, true>, map_x, map_w, map_out, map_res, map_q, p);
   } else if (pair) {
     cfg.blockDim = dim3(32 * (1 + kPairIssuerWarps + kPairEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem;
     err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);

@@ -237,12 +237,16 @@ __device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, int (&v)[16]) {
         "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr) : "memory");
 }
-// Four 16 x 8 byte matrices, stored transposed: register g of thread T holds, in byte order, the elements
-// (m, n) = (t4, 2 q2), (t4, 2 q2 + 1), (t4 + 8, 2 q2), (t4 + 8, 2 q2 + 1) of matrix g -- the byte-packed form of the
-// fragment above -- and matrix g's column n becomes the 16 contiguous bytes at the address thread 8 g + n supplies.
+// Four 8 x 8 matrices of 16-bit elements, transposed on the way: register g of thread T (t4, q2 as above) holds the elements
+// (t4, 2 q2) and (t4, 2 q2 + 1) of matrix g, whose column n is the 16 contiguous bytes at the address thread 8 g + n supplies.
+// With the weight rows in the order of encode_paired_rows_map an element is two neighbouring channels of one pixel.
 __device__ __forceinline__ void stmatrix_t_x4(uint32_t row_addr, unsigned r0, unsigned r1, unsigned r2, unsigned r3) {
-  asm volatile("stmatrix.sync.aligned.m16n8.x4.trans.shared.b8 [%0], {%1, %2, %3, %4};"
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};"
                ::"r"(row_addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_t_x4(uint32_t row_addr, unsigned (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(row_addr) : "memory");
 }
 // four values -> four bytes (s0 lowest), clamped to the unsigned / signed 8-bit range by two chained saturating packs
 template <bool OSIGNED>
@@ -413,6 +417,20 @@ bool encode_rows_map(CUtensorMap* map, const void* base, long long rows, long lo
   const cuuint32_t box[2] = {(cuuint32_t)ib, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Weight rows in the order the fragment epilogue wants them on the accumulator lanes: of every sixteen output channels the
+// eight even ones first, then the eight odd ones, so that a thread's two lanes (t4, t4 + 8) hold neighbouring channels.  A
+// four-dimensional map walks them in that order: (K bytes, channel pairs, parity, sixteens).  `rows` is a multiple of 16; box:
+// `ib` bytes of 128 rows.
+bool encode_paired_rows_map(CUtensorMap* map, const void* base, long long rows, long long row_bytes, int ib, CUtensorMapSwizzle swz) {
+  const cuuint64_t dims[4] = {(cuuint64_t)row_bytes, 8, 2, (cuuint64_t)(rows / 16)};
+  const cuuint64_t strides[3] = {(cuuint64_t)(2 * row_bytes), (cuuint64_t)row_bytes, (cuuint64_t)(16 * row_bytes)};
+  const cuuint32_t box[4] = {(cuuint32_t)ib, 8, 2, kTileC / 16};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(base), dims, strides, box, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
