@@ -83,7 +83,7 @@ struct TcParams {
   int32_t fold;          // 1: at most 64 output channels: W rows loaded twice, lane quarters 2-3 share the pixel columns
   int32_t halves;        // warps that share a lane quarter's pixel columns: 2, 4 with INT32 boxes, 1 for the 64-pixel tile (the others idle)
   int32_t lg_rbufs;      // log2 of the residual-tile buffer count (<= lg_bufs; 0 when a long reduction leaves no room)
-  int32_t frag;          // 1: the launch shape of epilogue_loop_frag
+  int32_t frag, deal;    // 1: the launch shape of epilogue_loop_frag; its two issuers take alternate K blocks (see frag_issue)
   int32_t acc_bits;      // |accumulator| < 2^acc_bits for every 8-bit operand pair: ceil(log2(K * 255 * 128 + 1))
   int32_t acc_stride;    // tensor-memory columns between accumulator buffers
   int32_t duo;           // 1: two CTAs of a cluster (adjacent SMs) share every MMA: 256 channels x 256 pixels per pair
@@ -385,7 +385,7 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
     const uint32_t t_addr = t_lane + as * kTileC;
     tmem_ld_frag16(t_addr, a0);
     if (RES) ldmatrix_t_x4(at, r0);
-#pragma unroll
+#pragma unroll 1                                    // (unrolled: 103 / 60 instead of 99 / 57 us on the first two layers above)
     for (int u = 0; u < units; u += 2) {
       tmem_ld_wait();
       tmem_ld_frag16(t_addr + 32 * (u + 1), a1);
@@ -765,13 +765,16 @@ __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanCo
     if (staged_out && lane == 0) tma_store_wait_all();
 }
 
-// MMA issue of the frag shape: issuer `c` of `n` takes the tiles c, c + n, ...  (One thread needs 1-2 k cycles per tile, nearly
-// all of it the latency of its own instructions between one barrier and the next.)  The accumulator's barrier is awaited before
-// the operands': it says that the tile four earlier has been consumed.  A wait for a stage's n-th fill cannot tell it from the
-// (n-2)-nd unless the (n-1)-st is known to have landed, which that barrier shows where the ring holds four tiles: two issuers only there.
-template <int STEPS>
+// MMA issue of the frag shape.  One thread needs about 1 k cycles per K block, nearly all of it the latency of its own
+// instructions between one barrier and the next, so two issuers share the work:
+//   - DEAL false: issuer `c` of `n` takes the tiles c, c + n, ...  The accumulator's barrier is awaited before the operands': it
+//     says that the tile four earlier has been consumed.  A wait for a stage's m-th fill cannot tell it from the (m-2)-nd unless
+//     the (m-1)-st is known to have landed, which that barrier shows where the ring holds four tiles (n = 1 otherwise);
+//   - DEAL true: the K blocks of the CTA, numbered through its tiles, alternate between the two issuers.  The stage count is even,
+//     so that a stage always belongs to one issuer; the tile's first, overwriting MMA signals `tstart`, which the other one awaits.
+template <int STEPS, bool DEAL>
 __device__ __forceinline__ void frag_issue(const TcParams& p, SharedCtl& ctl, int c, int n, uint32_t tiles, uint32_t stage_bytes,
-                                          uint32_t w_bytes, uint32_t tmem_base, int p_tile0, int p_step) {
+                                           uint32_t w_bytes, uint32_t tmem_base, int p_tile0, int p_step) {
   const uint32_t idesc = (2u << 4) | (1u << 7) | ((uint32_t)(p.x_signed ? 1 : 0) << 10) | ((uint32_t)(kTileC >> 3) << 17) |
                          ((uint32_t)(kTileC >> 4) << 24);
   const uint64_t hi = smem_desc(0, STEPS * 32);
@@ -779,32 +782,40 @@ __device__ __forceinline__ void frag_issue(const TcParams& p, SharedCtl& ctl, in
   const uint32_t nstages = (uint32_t)p.stages;
   const int k_blocks = p.k_blocks;
   const bool tail = p.tail_steps != STEPS;
+  const int per = DEAL ? 2 : 1, tiles_per = DEAL ? 1 : n;
   if (p.wres && !mbar_wait(smem_u32(&ctl.wfull), 0, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) return;
-  uint32_t s = 0, ph = 0, tcount = (uint32_t)c;
+  uint32_t s = 0, ph = 0, tcount = DEAL ? 0u : (uint32_t)c;
   auto skip = [&](int blocks) { for (int i = 0; i < blocks; ++i) if (++s == nstages) { s = 0; ph ^= 1u; } };
-  skip(c * k_blocks);
-  for (int p_tile = p_tile0 + c * p_step; p_tile < p.p_tiles; p_tile += n * p_step, tcount += (uint32_t)n) {
+  skip(DEAL ? c : c * k_blocks);
+  int kb = DEAL ? c : 0;
+  for (int p_tile = p_tile0 + (DEAL ? 0 : c * p_step); p_tile < p.p_tiles; p_tile += tiles_per * p_step, tcount += (uint32_t)tiles_per) {
     const uint32_t as = tcount & (kFragAccs - 1), aph = (tcount / kFragAccs) & 1u;
     const uint32_t d = tmem_base + as * kTileC;
     if (!mbar_wait(smem_u32(&ctl.tempty[as]), aph ^ 1u, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) return;
-    for (int kb = 0, chunk = 0; kb < k_blocks; ++kb) {
+    bool first = DEAL && kb != 0;
+    for (; kb < k_blocks; kb += per) {
       if (!mbar_wait(smem_u32(&ctl.full[s]), ph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) return;
+      if (DEAL && first) {
+        if (!mbar_wait(smem_u32(&ctl.tstart[as]), aph, &ctl, p.status, HQ_DEV_TIMEOUT_MMA)) return;
+        first = false;
+      }
       tc_fence_after();
       const uint32_t x = tiles + s * stage_bytes, w = p.wres ? tiles + p.wres_off + (uint32_t)kb * w_bytes : x;
       const uint64_t ad = hi | (uint64_t)((w >> 4) & 0x3FFF), bd = hi | (uint64_t)(((x + x_off) >> 4) & 0x3FFF);
-      const bool last = ++chunk == p.cchunks;
-      if (last) chunk = 0;
-      if (tail && last) {
+      if (tail && (kb + 1) % p.cchunks == 0) {
         for (int k = 0; k < p.tail_steps; ++k) mma_i8(d, ad + 2 * k, bd + 2 * k, idesc, (kb | k) ? 1u : 0u);
       } else {
 #pragma unroll
         for (int k = 0; k < STEPS; ++k) mma_i8(d, ad + 2 * k, bd + 2 * k, idesc, k ? 1u : kb ? 1u : 0u);
       }
-      if (kb + 1 == k_blocks) mma_commit(smem_u32(&ctl.tfull[as]));
+      if (DEAL && kb == 0) mbar_arrive(smem_u32(&ctl.tstart[as]));
+      if (kb + per >= k_blocks) mma_commit(smem_u32(&ctl.tfull[as]));
       mma_commit(smem_u32(&ctl.empty[s]));
-      if (++s == nstages) { s = 0; ph ^= 1u; }
+      s += (uint32_t)per;
+      if (s >= nstages) { s -= nstages; ph ^= 1u; }
     }
-    skip((n - 1) * k_blocks);
+    kb -= k_blocks;
+    if (!DEAL) { kb = 0; skip((n - 1) * k_blocks); }
   }
 }
 
@@ -845,7 +856,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&ctl.full[s]), 1); mbar_init(smem_u32(&ctl.empty[s]), 1); }
     for (int s = 0; s < (1 << p.lg_bufs); ++s) {
-      mbar_init(smem_u32(&ctl.tfull[s]), FRAG ? 1 : p.ni); mbar_init(smem_u32(&ctl.tempty[s]), (4 * p.halves) << p.duo);
+      mbar_init(smem_u32(&ctl.tfull[s]), FRAG && !p.deal ? 1 : p.ni); mbar_init(smem_u32(&ctl.tempty[s]), (4 * p.halves) << p.duo);
       mbar_init(smem_u32(&ctl.tstart[s]), 1);
     }
     for (int s = 0; s < (1 << p.lg_rbufs); ++s) {
@@ -1078,9 +1089,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if constexpr (FRAG) {
       if (elect_one()) {
         if (iss < p.ni) {
-          if (p.bkb == 128) frag_issue<4>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step);
-          else if (p.bkb == 64) frag_issue<2>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step);
-          else frag_issue<1>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step);
+#define HQ_ISSUE(STEPS) do { if (p.deal) frag_issue<STEPS, true>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step); \
+                             else frag_issue<STEPS, false>(p, ctl, iss, p.ni, tiles, stage_bytes, w_bytes, tmem_base, p_tile0, p_step); } while (0)
+          if (p.bkb == 128) HQ_ISSUE(4); else if (p.bkb == 64) HQ_ISSUE(2); else HQ_ISSUE(1);
+#undef HQ_ISSUE
         }
         // Drain: all issued MMAs must have completed before tensor memory is freed.
         mma_commit(smem_u32(&ctl.drain));
@@ -1593,7 +1605,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
         // (its epilogue has slack: a single residual buffer only delays the next tile's prefetch)
         // The frag shape (below) works in place in the residual tiles and needs no staging box; with the
         // weights resident two stages are enough for its short reductions (the epilogue bounds the tile).
-        const bool wide_here = p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && p.staged_res && k_total < 1024;
+        const bool wide_here = p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && (p.staged_res || (!a.res && p.wres)) && k_total < 1024;
         if (wide_here) out_tile_bytes = 0;
         const int min_stages = (wide_here && p.wres) ? 2 : 3;
         for (p.lg_rbufs = p.lg_bufs; ; --p.lg_rbufs) {
@@ -1660,7 +1672,8 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     // issuers only cost a few percent.
     // Third launch shape, *frag*, for the fused 8-bit residual with a short reduction on layers large enough for
     // 256-pixel tiles (here called `wide` for the condition it shares with the tile choice above): see epilogue_loop_frag.
-    wide = !pair && !p.strip && p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && p.staged_res && k_total < 1024;
+    wide = !pair && !p.strip && p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 &&
+           (p.staged_res || (!a.res && p.wres && a.cout % 16 == 0)) && k_total < 1024;
     if (wide) {
       // 128-pixel tiles, four accumulators; the residual tiles double as the output boxes
       p.frag = 1; p.halves = 2;
@@ -1675,9 +1688,10 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       // eight residual / output tiles where they leave room for three operand stages, else four: a tile is held from its load
       // to the end of its store, and the loads of the next tiles must be in flight meanwhile to cover the memory latency (with
       // arithmetic and matrix stores left out, 1x1 64 -> 256 at 56x56: four tiles 93 us, eight 87)
-      for (p.lg_rbufs = 3; ; --p.lg_rbufs) {
+      // Without a residual the tiles only carry outputs, and what is in flight are the operand stages: as many as there may be.
+      for (p.lg_rbufs = p.staged_res ? 3 : 2; ; --p.lg_rbufs) {
         stages = (kSmemBudget - (res_tile_bytes << p.lg_rbufs) - wres_bytes) / stage_bytes;
-        if (stages >= 3 || p.lg_rbufs == 1) break;
+        if (stages >= (p.staged_res ? 3 : kMaxStages) || p.lg_rbufs == 1) break;
       }
     }
     // Fourth shape, *duo*: clusters of two CTAs on adjacent SMs share every MMA (cta_group::2, M = 256): each CTA
@@ -1695,7 +1709,10 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     p.ni = p.k_blocks < issuers ? p.k_blocks : issuers;
     if (wide) {
       if (stages > kMaxStages) stages = kMaxStages;
-      p.ni = stages >= kFragAccs * p.k_blocks ? kFragIssuers : 1;           // (see frag_issue)
+      p.ni = kFragIssuers;
+      if (stages < kFragAccs * p.k_blocks) {
+        if (stages >= 4 && p.k_blocks > 1) { p.deal = 1; stages &= ~1; } else p.ni = 1;
+      }
     } else if (!(p.strip && p.wres)) {
       while (p.ni > 1 && stages < p.ni) --p.ni;
       if (stages > kMaxStages) stages = kMaxStages;
