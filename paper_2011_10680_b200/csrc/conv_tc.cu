@@ -262,6 +262,7 @@ __device__ __forceinline__ void epilogue_loop_fast8(const EpiCtx& e_in, const Ch
     for (int c = 0; c < nchunks; c += 2) {
       // ---- chunk c (registers va), while chunk c+1 streams into vb
       tmem_ld_wait();
+      tie(va);
       tmem_ld32_issue(t_addr + (c + 1) * 32, vb);
       if (c == 0) {                               // the previous tile's store must have read the staging box
         if (lane == 0) tma_store_wait_read0();
@@ -270,6 +271,7 @@ __device__ __forceinline__ void epilogue_loop_fast8(const EpiCtx& e_in, const Ch
       chunk(va, res_tile, c);
       // ---- chunk c+1 (registers vb), while the next chunk streams into va
       tmem_ld_wait();
+      tie(vb);
       pending = false;
       if (c + 2 < nchunks) {
         tmem_ld32_issue(t_addr + (c + 2) * 32, va);
@@ -388,10 +390,12 @@ __device__ __forceinline__ void epilogue_loop_frag(const EpiCtx& e_in) {
 #pragma unroll 1                                    // (unrolled: 103 / 60 instead of 99 / 57 us on the first two layers above)
     for (int u = 0; u < units; u += 2) {
       tmem_ld_wait();
+      tie(a0);
       tmem_ld_frag16(t_addr + 32 * (u + 1), a1);
       if (RES) ldmatrix_t_x4(at + (u + 1) * 4096u, r1);
       unit(a0, r0, at + u * 4096u);
       tmem_ld_wait();
+      tie(a1);
       if (u + 2 < units) {
         tmem_ld_frag16(t_addr + 32 * (u + 2), a0);
         if (RES) ldmatrix_t_x4(at + (u + 2) * 4096u, r0);
@@ -581,11 +585,11 @@ __device__ __forceinline__ void epilogue_loop_wide(const EpiCtx& e_in, const Cha
       for (int c = 0; c < nb; ++c) {
         if (!RAW && live) { ok = wait_bar(&ctl.wbox[e.ew][slot], sph); if (!ok) break; }
         tmem_ld_wait();
-        tie8(va);
+        tie(va);
         tmem_ld8_issue(t_addr + 16 * c + 8, vb);
         if (live) unit(va, 0);
         tmem_ld_wait();
-        tie8(vb);
+        tie(vb);
         pending = false;
         if (c + 1 < nb) { tmem_ld8_issue(t_addr + 16 * (c + 1), va); pending = true; }
         else {
@@ -655,7 +659,9 @@ __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanCo
 
       for (int cc0 = 0; cc0 < px_per_warp; cc0 += 32) {
         int v[32];
-        tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + as * p.pt + col0 + cc0, v);
+        tmem_ld32_issue(tmem_base + ((uint32_t)(q * 32) << 16) + as * p.pt + col0 + cc0, v);
+        tmem_ld_wait();
+        tie(v);
         if (!warp_live) continue;
         const int px0 = p_base + cc0;                                     // global pixel of v[0]
 
@@ -968,6 +974,20 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           }
         }
       }
+      if (FRAG && p.wres && p.x_tiled) {
+        // the leanest form for the layers with the most tiles: this thread's instructions are on the tile's path
+        const int k_blocks = p.k_blocks, bkb = p.bkb;
+        for (int p_tile = p_tile0; p_tile < p.p_tiles && ok; p_tile += p_step) {
+          const int p0 = tile_at(p, p_tile) * kTileC;
+          for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+            if (!mbar_wait(smem_u32(&ctl.empty[s]), ph ^ 1u, &ctl, p.status, HQ_DEV_TIMEOUT_PRODUCER)) { ok = false; break; }
+            const uint32_t bar = smem_u32(&ctl.full[s]);
+            mbar_expect_tx(bar, stage_bytes);
+            tma_load_2d_hint(tiles + s * stage_bytes, &map_x, bar, kb * bkb, p0, pol_first);
+            if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1u; }
+          }
+        }
+      } else
       for (int p_tile = p_tile0; p_tile < p.p_tiles && ok && !p.strip; p_tile += p_step, ++tcount) {
         const int p0 = tile_at(p, p_tile) * p.pt;
         const int cw = ow * p.stride - p.pad, chh = oh * p.stride - p.pad, img_now = img;
@@ -984,7 +1004,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         // The residual tile of this output tile is fetched as soon as its buffer is free, but this thread only
         // blocks for the buffer after the tile's last operand block is on its way: the buffer comes back when the
         // epilogue of an earlier tile ends, and the operand copies must not queue behind that.
-        bool res_due = p.staged_res != 0;
+        bool res_due = !FRAG && p.staged_res != 0;                  // (frag: the store warp fetches them)
         auto residual = [&](bool must) -> bool {
           const uint32_t rbuf = tcount & rmask, rph = (tcount >> p.lg_rbufs) & 1u;
           const uint32_t rb = smem_u32(&ctl.rempty[rbuf]);
@@ -1063,7 +1083,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           if (global_ns() - t0 > kWaitBudgetNs) { atomicCAS(p.status, 0u, (uint32_t)HQ_DEV_TIMEOUT_DRAIN); break; }
         }
       }
-      if (p.staged_res) {
+      if (!FRAG && p.staged_res) {
         const uint32_t tiles_done = tcount < rmask + 1u ? tcount : rmask + 1u;
         for (uint32_t j = 0; j < tiles_done; ++j) {
           const uint32_t k = tcount - 1 - j;
@@ -1232,22 +1252,42 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     }
   } else if (FRAG && warp == 1 + MMA_WARPS + EPI_WARPS) {
     // ------------------------------------------------------------ store warp (frag): finished tiles leave by TMA
+    // The buffer of a tile whose store has read it takes the residual of the tile 2^lg_rbufs later at once (one thread less
+    // between the two, and the operand producer, whose own instructions are on the tiles' path, does not see residuals at all).
     if (elect_one()) {
-      const uint32_t rmask = (1u << p.lg_rbufs) - 1u;
-      uint32_t tcount = 0;
+      const uint32_t bufs = 1u << p.lg_rbufs, rmask = bufs - 1u;
+      const bool res = p.staged_res != 0;
+      const unsigned long long pol_first = policy_evict_first();
+      uint32_t tcount = 0, loads = 0;
+      int load_tile = p_tile0;
+      auto next_residual = [&]() {
+        if (load_tile >= p.p_tiles) return;
+        const uint32_t rs = loads & rmask, bar = smem_u32(&ctl.rfull[rs]);
+        mbar_expect_tx(bar, res_tile_bytes);
+        tma_load_2d_hint(res_stage + rs * res_tile_bytes, &map_res, bar, c_tile * kTileC, tile_at(p, load_tile) * kTileC, pol_first);
+        load_tile += p_step; ++loads;
+      };
+      if (res) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");              // the residual is the output of an earlier kernel
+        for (uint32_t i = 0; i < bufs; ++i) next_residual();
+      }
       for (int p_tile = p_tile0; p_tile < p.p_tiles; p_tile += p_step, ++tcount) {
         const uint32_t rs = tcount & rmask, rph = (tcount >> p.lg_rbufs) & 1u;
         if (!mbar_wait(smem_u32(&ctl.ofull[rs]), rph, &ctl, p.status, HQ_DEV_TIMEOUT_EPILOGUE)) break;
-        tma_store_2d(&map_out, res_stage + rs * res_tile_bytes, c_tile * kTileC, tile_at(p, p_tile) * p.pt);
+        tma_store_2d(&map_out, res_stage + rs * res_tile_bytes, c_tile * kTileC, tile_at(p, p_tile) * kTileC);
         tma_store_commit();
-        if (rmask < 3u) {
-          // only two tile buffers: hand this one back as soon as the store has read it
-          tma_store_wait_read0();
-          mbar_arrive(smem_u32(&ctl.rempty[rs]));
-        } else if (tcount > 0) {
-          // the store before this one has read its tile by now: that buffer may be loaded again
-          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-          mbar_arrive(smem_u32(&ctl.rempty[(tcount - 1u) & rmask]));
+        // the store before this one has read its tile by now; with two buffers only, this one is awaited
+        if (bufs < 4u) tma_store_wait_read0();
+        else if (tcount > 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        else continue;
+        if (res) next_residual();
+        else mbar_arrive(smem_u32(&ctl.rempty[(bufs < 4u ? tcount : tcount - 1u) & rmask]));
+      }
+      // every copy this thread started must have landed before the CTA may exit (all consumed unless a wait ran out)
+      for (uint32_t k = tcount; k < loads; ++k) {
+        const unsigned long long t0 = global_ns();
+        while (!mbar_try_wait(smem_u32(&ctl.rfull[k & rmask]), (k >> p.lg_rbufs) & 1u)) {
+          if (global_ns() - t0 > kWaitBudgetNs) { atomicCAS(p.status, 0u, (uint32_t)HQ_DEV_TIMEOUT_DRAIN); break; }
         }
       }
       tma_store_wait_all();
@@ -1562,6 +1602,12 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // epilogue work, e.g. 64 output channels.  Where the layer is large enough for 256-pixel tiles and its residual
   // travels by TMA, the frag shape below is faster still: 64 -> 256 at 56x56, batch 256: 129 -> 101 us.)
   const bool wide_fits = p.staged_res && a.out_bits == 8 && a.cout > 64 && pick_pt(P, p.c_tiles, h->sm_count, 256) == 256;
+  // Without a residual the frag shape takes over where a CTA's weights stay in shared memory, but for longer reductions whose
+  // pixel rows the im2col mode gathers: four blocks of 128 pixels are issued more slowly than two of 256 (256 images, L2 flushed,
+  // 256-pixel tiles against frag: 1x1 64 -> 256 at 56x56 90 / 69 us, 512 -> 128 at 28x28 32.7 / 27.7, 256 -> 128 / 2 28.7 / 22.0, 256 -> 512 / 2
+  // 55.3 / 54.3, 512 -> 1024 / 2 36.8 / 46.1).
+  const bool tiled = !a.pitch_w && a.kh == 1 && a.kw == 1 && a.stride == 1 && a.pad == 0;
+  const bool plain_frag = !a.res && !a.pitch_w && !a.pairs && a.cout % 16 == 0 && (tiled || k_total <= 256);
   bool pair = !a.wide && k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !wide_fits;
   int stages = 0, stage_bytes = 0, res_tile_bytes = 0, out_tile_bytes = 0, wres_bytes = 0;
   if (pair) {
@@ -1605,7 +1651,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
         // (its epilogue has slack: a single residual buffer only delays the next tile's prefetch)
         // The frag shape (below) works in place in the residual tiles and needs no staging box; with the
         // weights resident two stages are enough for its short reductions (the epilogue bounds the tile).
-        const bool wide_here = p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && (p.staged_res || (!a.res && p.wres)) && k_total < 1024;
+        const bool wide_here = p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && (p.staged_res || (plain_frag && p.wres)) && k_total < 1024;
         if (wide_here) out_tile_bytes = 0;
         const int min_stages = (wide_here && p.wres) ? 2 : 3;
         for (p.lg_rbufs = p.lg_bufs; ; --p.lg_rbufs) {
@@ -1673,7 +1719,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     // Third launch shape, *frag*, for the fused 8-bit residual with a short reduction on layers large enough for
     // 256-pixel tiles (here called `wide` for the condition it shares with the tile choice above): see epilogue_loop_frag.
     wide = !pair && !p.strip && p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 &&
-           (p.staged_res || (!a.res && p.wres && a.cout % 16 == 0)) && k_total < 1024;
+           (p.staged_res || (plain_frag && p.wres)) && k_total < 1024;
     if (wide) {
       // 128-pixel tiles, four accumulators; the residual tiles double as the output boxes
       p.frag = 1; p.halves = 2;

@@ -12,6 +12,7 @@ namespace {
 
 constexpr int kTileC = 128;                   // output channels per tile = MMA M = TMEM lanes
 constexpr unsigned long long kWaitBudgetNs = 2000000000ull;   // 2 s per wait
+constexpr uint32_t kSuspendNs = 1000000;      // longest single suspension of a waiting thread (it looks at the abort flag in between)
 
 // ---------------------------------------------------------------- PTX wrappers ---------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -34,6 +35,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
+// The same, with leave for the hardware to keep the thread suspended for up to `ns` while the phase is not complete.
+__device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t ns) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(ns) : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -45,16 +56,13 @@ template <class Ctl>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, Ctl* ctl, uint32_t* status, uint32_t code) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = global_ns();
-  uint32_t spins = 0;
   while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((++spins & 63u) == 0) {
-      if (ctl->abort_flag) return false;
-      if (global_ns() - t0 > kWaitBudgetNs) {
-        ctl->abort_flag = 1;
-        atomicCAS(status, 0u, code);
-        return false;
-      }
+    if (mbar_try_wait_for(bar, parity, kSuspendNs)) return true;
+    if (ctl->abort_flag) return false;
+    if (global_ns() - t0 > kWaitBudgetNs) {
+      ctl->abort_flag = 1;
+      atomicCAS(status, 0u, code);
+      return false;
     }
   }
 }
@@ -194,18 +202,6 @@ __device__ __forceinline__ void tma_load_im2col_2cta(uint32_t dst, const CUtenso
       " [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
       ::"r"(dst), "l"(map), "r"(in_cta(bar, 0)), "r"(c), "r"(w), "r"(h), "r"(n), "h"(off_w), "h"(off_h) : "memory");
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, int (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, int (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -221,10 +217,12 @@ __device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, int (&v)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
 }
-// keeps what is computed from the loaded registers below the wait
-__device__ __forceinline__ void tie8(int (&v)[8]) {
+// Keeps what is computed from the loaded registers below the wait: used above it, they could also be given to something else
+// while the load is still going to write them.
+template <int N>
+__device__ __forceinline__ void tie(int (&v)[N]) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) asm volatile("" : "+r"(v[i]));
+  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(v[i]));
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // 16 lanes x 32 columns in the layout of an MMA accumulator fragment: thread T (t4 = T / 4, q2 = T % 4) receives, for
