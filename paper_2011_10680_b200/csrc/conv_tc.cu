@@ -55,8 +55,9 @@ constexpr int kMaxResBufs = 8;                                 // residual / out
 //         reduction are bound by the latency of the hand-over chain between the MMA issuer and the epilogue
 //         (barrier, fences, MMA, commit), not by any throughput; two independent CTAs hide each other's chain.
 //   frag  16 epilogue warps in two groups on alternate tiles, two issuers and a store warp, one CTA per SM, 128-pixel tiles
-//         in four accumulators: fused 8-bit residuals with a short reduction.  The epilogue works on 16 x 8 fragments, reads
-//         the residual with transposing matrix loads and writes over it with transposing matrix stores.
+//         in four accumulators: fused 8-bit residuals with a short reduction, and 8-bit results without a residual whose
+//         weights stay resident.  The epilogue works on 16 x 8 fragments, reads the residual with transposing matrix loads and
+//         writes over it with transposing matrix stores; the store warp fetches the residual tiles.
 //   wide  16 epilogue warps on boxes of 16 pixels: INT32 results, raw or through the residual add (see epilogue_loop_wide).
 //   duo   the solo roles in clusters of two CTAs that share every MMA (cta_group::2): long reductions whose weights
 //         stream; each CTA fetches its own weight rows and half of the pixel rows.
@@ -325,8 +326,10 @@ __device__ __forceinline__ ChanConst chan_const_for(const TcParams& p, int ch, b
 // the tile's `ofull` barrier when its pieces are written, and the store warp alone waits there, stores the [128][128] box and
 // hands the buffer back.  Up to eight residual / output tiles circulate: their loads in flight cover the memory latency.
 //
-// What bounds it: the integer instructions (about 6.5 per 32 values; the residual's byte extraction is one of them).  1x1 64 -> 256
-// at 56x56 / 128 -> 512 at 28x28 / 256 -> 1024 at 14x14 / 512 -> 2048 at 7x7, 256 images, L2 flushed: 101 / 58 / 42 / 34.5 us.  Before:
+// What bounds it: the integer instructions (about 6.5 per 32 values; the residual's byte extraction is one of them) and, beside
+// them, the instruction latency of the warps that move tiles along (with no arithmetic the first layer below takes 82 us, with no
+// memory traffic 95).  Twenty-four warps in three groups: no faster.  1x1 64 -> 256 at 56x56 / 128 -> 512 at 28x28 / 256 -> 1024 at
+// 14x14 / 512 -> 2048 at 7x7, 256 images, L2 flushed: 97 / 58 / 40 / 31.7 us; without a residual 64 -> 256 90 -> 69 us.  Before:
 // eight warps, the residual widened into tensor memory by an MMA with the identity matrix, two accumulators and one issuer
 // 115 / 65 / 44 / 35.6 us; there the issuer's own instruction latency (2.5 k cycles a tile) set the tile rate, whatever the
 // epilogue did (sixteen warps or a matrix store of another type: the same time).
