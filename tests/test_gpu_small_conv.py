@@ -181,3 +181,54 @@ def test_conv_over_pixel_pairs(hw, batch, signed):
         run_network_and_compare(hq, t, batch=batch, seed=6)
     finally:
         hq.close()
+
+
+FRAGMENT_CASES = [
+    # n, h, w, cin, cout, k, stride, residual, residual signed, relu, c range, rc range
+    (52, 28, 27, 32, 144, 1, 1, True, False, True, (39, 44), (28, 34)),     # one K block of 32 bytes; second channel tile of 16; ragged last pixel tile
+    (52, 28, 27, 64, 256, 1, 1, True, True, False, (39, 44), (28, 34)),     # two issuers on alternate tiles, signed residual and output
+    (52, 28, 27, 96, 160, 1, 1, True, False, True, (39, 44), (28, 34)),     # the last K block reaches past the channels
+    (52, 28, 27, 128, 256, 1, 1, True, False, True, (28, 31), (28, 34)),    # shifts below 32: pre-shift form
+    (52, 28, 27, 64, 256, 1, 1, True, False, True, (14, 40), (28, 34)),     # some shifts too small for it: funnel-shift form
+    (52, 28, 27, 64, 256, 1, 1, True, True, True, (39, 44), (4, 34)),       # residual shifts below 9: 64-bit form
+    (52, 28, 27, 256, 256, 1, 1, True, False, True, (39, 44), (28, 34)),    # K blocks dealt to the two issuers
+    (52, 28, 27, 160, 256, 1, 1, True, False, True, (39, 44), (28, 34)),    # the same with a partial last block
+    (52, 28, 27, 64, 256, 3, 1, True, False, True, (39, 44), (28, 34)),     # nine blocks: the issuers swap roles from tile to tile
+    (26, 28, 27, 512, 512, 1, 1, True, False, True, (40, 45), (28, 34)),    # four blocks, fewer residual tiles
+    (52, 28, 27, 64, 256, 1, 1, False, False, True, (39, 44), None),        # no residual
+    (52, 28, 27, 64, 176, 1, 1, False, False, False, (26, 44), None),       # the same, signed, ragged channels, small shifts
+    (210, 28, 27, 256, 256, 1, 2, False, False, True, (39, 44), None),      # rows gathered in im2col mode
+]
+
+
+@pytest.mark.parametrize("rev", [0, 1])
+@pytest.mark.parametrize("cfg", FRAGMENT_CASES)
+def test_fragment_epilogue_shape(cfg, rev):
+    """The launch shape with four accumulators and two groups of epilogue warps: every number of K blocks per tile, every form of
+    the arithmetic, ragged channel and pixel tiles, both tile orders.  Integers: equal to the oracle."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from oracle import hqref
+    from paper_2011_10680_b200 import binding, build
+    build.build()
+    n, h, w, cin, cout, k, stride, residual, res_signed, relu, c_range, rc_range = cfg
+    case = inputs.conv_case(700, n, h, w, cin, cout, k, stride, k // 2, residual=residual, relu=relu, c_range=c_range)
+    assert case["ho"] * case["wo"] * n * ((cout + 127) // 128) >= 2 * 148 * 256          # large enough for this shape on 148 SMs
+    if residual:
+        g = inputs.rng(701, cin, cout, k)
+        case["rc"] = g.integers(rc_range[0], rc_range[1] + 1, size=cout, dtype=np.int64).astype(np.int32)
+        if res_signed:
+            case["res"], case["res_signed"] = case["res"].view(np.int8), 1
+    hq = binding.Handle(0)
+    try:
+        hq.set_tile_order(rev)
+        dev = binding.upload_case(case)
+        for _ in range(2):                                  # the second call starts while the first one ends
+            st, out = hq.conv_case(case, dev)
+            assert st == binding.HQ_OK, binding.status_string(st)
+        hq.sync()
+        ref = hqref.conv_case(case)
+        got = out.cpu().numpy().view(ref.dtype).reshape(ref.shape)
+        assert np.array_equal(got, ref), (int((got != ref).sum()), ref.size)
+    finally:
+        hq.close()
