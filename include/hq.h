@@ -275,6 +275,25 @@ hq_status hq_set_conv_path(hq_handle* h, int32_t path);
  * (a network chooses the order layer by layer itself and ignores this setting).  (No counterpart in the paper.) */
 hq_status hq_set_tile_order(hq_handle* h, int32_t order);
 
+/* Debug aid (no paper counterpart): the launch shape and buffer counts that the persistent tensor-core kernel takes for the
+ * call hq_conv2d(in, desc, out) on a GPU with `sm_count` SMs, were the call to reach it as it is (automatic path; unpacked
+ * operands, no lowered form).  Host arithmetic: no GPU is needed and no pointer is followed except `residual`.  HQ_ERR_UNSUPPORTED
+ * for what that kernel does not take. */
+typedef enum { HQ_SHAPE_SOLO = 0, HQ_SHAPE_PAIR = 1, HQ_SHAPE_FRAG = 2, HQ_SHAPE_WIDE = 3, HQ_SHAPE_DUO = 4, HQ_SHAPE_STRIP = 5 } hq_shape;
+typedef struct {
+  int32_t shape;             /* hq_shape */
+  int32_t pixel_tile;        /* output pixels per tile */
+  int32_t k_blocks;          /* blocks of the reduction per tile, of block_bytes bytes */
+  int32_t block_bytes;
+  int32_t weights_resident;  /* 1: the channel tile's weights stay in shared memory */
+  int32_t stages;            /* operand stages of the ring (0: everything is resident) */
+  int32_t issuers;           /* threads that issue MMAs */
+  int32_t alternate_tiles;   /* 1: each issuer takes whole tiles in turn; 0: the K blocks of all tiles in turn */
+  int32_t residual_tiles;    /* residual / output tiles in circulation */
+  int32_t shared_bytes;      /* dynamic shared memory of a CTA */
+} hq_conv_plan;
+hq_status hq_conv2d_plan(const hq_tensor* in, const hq_conv_desc* desc, const hq_tensor* out, int32_t sm_count, hq_conv_plan* plan);
+
 /* Self-test of the bounded device-side waits: one thread waits on a barrier that nothing ever signals, for at
  * most `budget_ms` milliseconds (1..2000), then records the expiry in the handle's status word and returns, as
  * every wait inside the kernels does after its own budget.  The next hq_sync reports HQ_ERR_TIMEOUT; the

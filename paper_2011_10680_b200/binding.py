@@ -24,7 +24,7 @@ EXPORTS = [
     "hq_maxpool", "hq_network_create", "hq_run_network", "hq_network_layer_bytes", "hq_network_launch_count",
     "hq_network_destroy", "hq_set_conv_path", "hq_set_tile_order", "hq_status_string", "hq_network_time_layers", "hq_conv2d_noalloc", "hq_expire_wait_selftest",
     "hq_network_check_guards", "hq_conv2d_noalloc_sync", "hq_mma_peak_launch",
-    "hq_ilp_solve", "hq_concat_requant", "hq_sumpool",
+    "hq_ilp_solve", "hq_concat_requant", "hq_sumpool", "hq_conv2d_plan",
 ]
 
 
@@ -48,6 +48,14 @@ class hq_conv_desc(C.Structure):
                 ("cin", C.c_int32), ("cout", C.c_int32), ("w_bits", C.c_int32), ("w", C.c_void_p),
                 ("bias", C.c_void_p), ("requant", hq_dyadic), ("residual", C.POINTER(hq_tensor)),
                 ("res_rescale", hq_dyadic), ("relu", C.c_int32), ("qmin", C.c_int32), ("qmax", C.c_int32)]
+
+
+HQ_SHAPE = ("solo", "pair", "frag", "wide", "duo", "strip")
+
+
+class hq_conv_plan(C.Structure):
+    _fields_ = [(name, C.c_int32) for name in ("shape", "pixel_tile", "k_blocks", "block_bytes", "weights_resident", "stages",
+                                               "issuers", "alternate_tiles", "residual_tiles", "shared_bytes")]
 
 
 class hq_layer(C.Structure):
@@ -92,6 +100,7 @@ def lib():
         L.hq_mma_peak_launch.argtypes = [vp, i32, i32, C.POINTER(C.c_int64), vp]
         L.hq_set_conv_path.argtypes = [vp, i32]
         L.hq_set_tile_order.argtypes = [vp, i32]
+        L.hq_conv2d_plan.argtypes = [TP, DP, TP, i32, C.POINTER(hq_conv_plan)]
         L.hq_expire_wait_selftest.argtypes = [vp, i32, vp]
         L.hq_expire_wait_selftest.restype = i32
         i64p = C.POINTER(C.c_int64)
@@ -329,6 +338,24 @@ class Handle:
                          case["out_bits"], case["out_signed"], dev["res"], case["res_bits"], case["res_signed"],
                          dev["rb"], dev["rc"], case["relu"], case["qmin"], case["qmax"])
         return st, out
+
+
+def conv2d_plan(n, h, w, cin, cout, k, stride, pad, out_bits=8, residual_bits=0, sm_count=148):
+    """hq_conv2d_plan of a layer of these sizes as a dict, `shape` by name; None where the persistent kernel does not take it.
+    Needs neither a GPU nor data."""
+    somewhere = 1 << 20                      # stands for device memory: aligned, not NULL, never read
+    ho, wo = (h + 2 * pad - k) // stride + 1, (w + 2 * pad - k) // stride + 1
+    tin, tout = hq_tensor(somewhere, n, h, w, cin, 8, 0), hq_tensor(somewhere, n, ho, wo, cout, out_bits, int(out_bits == 32))
+    tres = hq_tensor(somewhere, n, ho, wo, cout, residual_bits, int(residual_bits == 32)) if residual_bits else None
+    pair = hq_dyadic(somewhere, somewhere)
+    d = hq_conv_desc(k, k, stride, pad, cin, cout, 8, somewhere, None, pair, C.pointer(tres) if tres is not None else None, pair, 1, 0,
+                     (1 << min(out_bits, 8)) - 1)
+    plan = hq_conv_plan()
+    st = lib().hq_conv2d_plan(C.byref(tin), C.byref(d), C.byref(tout), sm_count, C.byref(plan))
+    if st == HQ_ERR_UNSUPPORTED:
+        return None
+    _check(st, "hq_conv2d_plan")
+    return {**{name: getattr(plan, name) for name, _ in hq_conv_plan._fields_}, "shape": HQ_SHAPE[plan.shape]}
 
 
 def conv2d_noalloc(case: dict, dev: dict, out):

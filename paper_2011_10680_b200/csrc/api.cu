@@ -31,13 +31,9 @@ inline long long tensor_bytes(int n, int h, int w, int c, int bits) {
   return (long long)n * h * w * c * bits / 8;
 }
 
-// `scratch` / `scratch_bytes`: buffer for the lowered first-layer path owned by the caller (a
-// network); NULL means use (and if needed grow) the handle's own buffer.
-hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, hq_tensor* out, void* stream,
-                      void* scratch = nullptr, size_t scratch_bytes = 0, const void* res_narrow = nullptr,
-                      const void* wgt_widened = nullptr, bool in_slack = false, const WideArgs* wide = nullptr,
-                      bool wide_sum = true, bool pairs = false) {
-  if (!h || !d) return HQ_ERR_INVALID_ARG;
+// Checks the arguments of a convolution and describes it to the kernels (`wide`, `wide_sum`: see conv_common).
+hq_status conv_args(const hq_tensor* in, const hq_conv_desc* d, const hq_tensor* out, const WideArgs* wide, bool wide_sum, ConvArgs& a) {
+  if (!d) return HQ_ERR_INVALID_ARG;
   hq_status st = check_tensor(in, true, true, false);
   if (st != HQ_OK) return st;
   st = check_tensor(out, true, true, true);
@@ -62,18 +58,12 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
       if (!d->res_rescale.b || !d->res_rescale.c) return HQ_ERR_INVALID_ARG;
     }
   }
-  ConvArgs a{};
-  a.in_slack = in_slack ? 1 : 0;
-  // A caller may write parameters on the stream and call at once.  (A network's own layers follow its first launch, which has
-  // waited for whatever came before it.)
-  a.params_late = in_slack ? 0 : 1;
   a.in = in->data; a.n = in->n; a.h = in->h; a.w = in->w; a.cin = in->c; a.in_bits = in->bits; a.in_signed = in->is_signed;
-  a.wgt = d->w; a.wgt_widened = wgt_widened; a.cout = d->cout; a.kh = d->kh; a.kw = d->kw; a.stride = d->stride; a.pad = d->pad;
+  a.wgt = d->w; a.cout = d->cout; a.kh = d->kh; a.kw = d->kw; a.stride = d->stride; a.pad = d->pad;
   a.bias = d->bias; a.b = d->requant.b; a.c = d->requant.c;
   if (d->residual && out->bits != 32) {
     a.res = d->residual->data; a.res_bits = d->residual->bits; a.res_signed = d->residual->is_signed;
     a.rb = d->res_rescale.b; a.rc = d->res_rescale.c;
-    a.res_narrow = res_narrow;
   }
   void* out_data = out->data;
   if (wide) {                                  // (a network's fused add: `d` carries the add's pairs, `out` its INT32 result)
@@ -84,6 +74,25 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
   }
   a.relu = d->relu; a.qmin = d->qmin; a.qmax = d->qmax;
   a.out = out_data; a.ho = ho; a.wo = wo; a.out_bits = out->bits; a.out_signed = out->is_signed;
+  return HQ_OK;
+}
+
+// `scratch` / `scratch_bytes`: buffer for the lowered first-layer path owned by the caller (a
+// network); NULL means use (and if needed grow) the handle's own buffer.
+hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, hq_tensor* out, void* stream,
+                      void* scratch = nullptr, size_t scratch_bytes = 0, const void* res_narrow = nullptr,
+                      const void* wgt_widened = nullptr, bool in_slack = false, const WideArgs* wide = nullptr,
+                      bool wide_sum = true, bool pairs = false) {
+  if (!h) return HQ_ERR_INVALID_ARG;
+  ConvArgs a{};
+  const hq_status st = conv_args(in, d, out, wide, wide_sum, a);
+  if (st != HQ_OK) return st;
+  a.in_slack = in_slack ? 1 : 0;
+  // A caller may write parameters on the stream and call at once.  (A network's own layers follow its first launch, which has
+  // waited for whatever came before it.)
+  a.params_late = in_slack ? 0 : 1;
+  a.wgt_widened = wgt_widened;
+  if (a.res && !wide) a.res_narrow = res_narrow;
   cudaStream_t s = (cudaStream_t)stream;
   if (wide) return hq_launch_conv_tc(h, a, s);
   if (h->conv_path == 4 || (h->conv_path == 0 && hq_conv_small_wanted(a, h->sm_count))) {
@@ -111,7 +120,7 @@ hq_status conv_common(hq_handle* h, const hq_tensor* in, const hq_conv_desc* d, 
     // A single large call with an 8-bit residual: its narrow residual pairs are worked out first, in the handle's
     // buffer (a network prepares them once when it is built); one small launch that the cheaper epilogue repays.
     if (a.res && a.res_bits == 8 && !a.res_narrow && a.cout <= kNarrowChannels &&
-        (long long)a.n * ho * wo * a.cout >= (1ll << 25) &&
+        (long long)a.n * a.ho * a.wo * a.cout >= (1ll << 25) &&
         hq_launch_residual_narrow(a.rb, a.rc, a.res_signed, a.cout, h->narrow_pairs, s) == cudaSuccess) {
       a.res_narrow = h->narrow_pairs;
       a.res_narrow_fresh = 1;
@@ -398,6 +407,14 @@ hq_status hq_set_tile_order(hq_handle* h, int32_t order) {
   if (!h || order < 0 || order > 1) return HQ_ERR_INVALID_ARG;
   h->tile_order = order;
   return HQ_OK;
+}
+
+hq_status hq_conv2d_plan(const hq_tensor* in, const hq_conv_desc* desc, const hq_tensor* out, int32_t sm_count, hq_conv_plan* plan) {
+  if (sm_count < 1 || !plan) return HQ_ERR_INVALID_ARG;
+  ConvArgs a{};
+  const hq_status st = conv_args(in, desc, out, nullptr, false, a);
+  if (st != HQ_OK) return st;
+  return a.n ? hq_conv_tc_plan(a, sm_count, plan) : HQ_ERR_UNSUPPORTED;
 }
 
 hq_status hq_expire_wait_selftest(hq_handle* h, int32_t budget_ms, void* stream) {

@@ -1575,21 +1575,25 @@ bool hq_conv_wide_applies(const ConvArgs& a, int sm_count) {
   return hq_conv_tc_supported(a) && !hq_conv_tc_declines(a) && a.cout % 16 == 0 && (a.cout + kTileC - 1) / kTileC <= sm_count;
 }
 
-hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream) {
-  if (!hq_conv_tc_supported(a)) return HQ_ERR_UNSUPPORTED;
-  if (!load_driver_entry_points()) return HQ_ERR_CUDA;
-  const long long P = (long long)a.n * a.ho * a.wo;
-  if (P == 0) return HQ_OK;
-
+namespace {
+// Launch shape of a layer and what it needs: host arithmetic on sizes alone (no pointer is looked at but for being NULL).
+struct TcPlan {
   TcParams p{};
-  p.rev = h->tile_order ? 1 : 0;
+  bool pair = false, int32_boxes = false;
+  int stages = 0, stage_bytes = 0, res_tile_bytes = 0, out_tile_bytes = 0, wres_bytes = 0;
+  size_t patch_total = 0, dyn_smem = 0;
+};
+
+hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t) {
+  TcParams& p = t.p;
+  const long long P = (long long)a.n * a.ho * a.wo;
   p.P = (int32_t)P; p.C = a.cout; p.howo = a.ho * a.wo; p.wo = a.wo;
   p.stride = a.stride; p.pad = a.pad; p.kw = a.kw;
   auto set_bkb = [&](int bkb) { p.bkb = bkb; p.cchunks = (a.cin + bkb - 1) / bkb; p.k_blocks = a.kh * a.kw * p.cchunks; };
   p.cin = a.cin;
   set_bkb(hq_conv_bkb(a.cin));
   p.c_tiles = (a.cout + kTileC - 1) / kTileC;
-  if (p.c_tiles > h->sm_count) return HQ_ERR_UNSUPPORTED;
+  if (p.c_tiles > sm_count) return HQ_ERR_UNSUPPORTED;
   // outputs and 8-bit residuals whose rows are 16-byte multiples travel through TMA
   const long long out_row_bytes = (long long)a.cout * a.out_bits / 8;
   p.staged_out = (a.out_bits != 32 && out_row_bytes % 16 == 0) ? 1 : 0;
@@ -1599,24 +1603,26 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // INT32 results through TMA boxes (epilogue_loop_wide): every residual add, and raw results but for the long reductions
   // that the two-CTA shape serves better (and rows that are not whole 16-byte pieces)
   const bool int32_boxes = a.wide || (a.out_bits == 32 && !a.res && a.cout % 4 == 0 && k_total < 2048);
+  t.int32_boxes = int32_boxes;
   const int box_bytes = kWideWarps * (kWideSlots * kWideBox + (a.wide && a.wide->q ? 2 * kWideQBox : 0));
   // (measured: with the weight slab resident the one-CTA shape catches up for K >= 128; the pair shape still
   // wins on the fused-residual expansions with the shortest reduction, and loses where a tile carries little
   // epilogue work, e.g. 64 output channels.  Where the layer is large enough for 256-pixel tiles and its residual
   // travels by TMA, the frag shape below is faster still: 64 -> 256 at 56x56, batch 256: 129 -> 101 us.)
-  const bool wide_fits = p.staged_res && a.out_bits == 8 && a.cout > 64 && pick_pt(P, p.c_tiles, h->sm_count, 256) == 256;
+  const bool wide_fits = p.staged_res && a.out_bits == 8 && a.cout > 64 && pick_pt(P, p.c_tiles, sm_count, 256) == 256;
   // Without a residual the frag shape takes over where a CTA's weights stay in shared memory, but for longer reductions whose
   // pixel rows the im2col mode gathers: four blocks of 128 pixels are issued more slowly than two of 256 (256 images, L2 flushed,
   // 256-pixel tiles against frag: 1x1 64 -> 256 at 56x56 90 / 69 us, 512 -> 128 at 28x28 32.7 / 27.7, 256 -> 128 / 2 28.7 / 22.0, 256 -> 512 / 2
   // 55.3 / 54.3, 512 -> 1024 / 2 36.8 / 46.1).
   const bool tiled = !a.pitch_w && a.kh == 1 && a.kw == 1 && a.stride == 1 && a.pad == 0;
   const bool plain_frag = !a.res && !a.pitch_w && !a.pairs && a.cout % 16 == 0 && (tiled || k_total <= 256);
-  bool pair = !a.wide && k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !wide_fits;
-  int stages = 0, stage_bytes = 0, res_tile_bytes = 0, out_tile_bytes = 0, wres_bytes = 0;
+  bool& pair = t.pair;
+  pair = !a.wide && k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !wide_fits;
+  int &stages = t.stages, &stage_bytes = t.stage_bytes, &res_tile_bytes = t.res_tile_bytes, &out_tile_bytes = t.out_tile_bytes, &wres_bytes = t.wres_bytes;
   if (pair) {
     // 128-pixel tiles, two accumulator buffers (256 columns), K blocks of at most 64 bytes
     if (p.bkb > 64) set_bkb(64);
-    p.pt = pick_pt(P, p.c_tiles, 2 * h->sm_count, 128);
+    p.pt = pick_pt(P, p.c_tiles, 2 * sm_count, 128);
     wres_bytes = p.k_blocks * kTileC * p.bkb;
     p.wres = wres_bytes <= 16 * 1024 ? 1 : 0;              // short reductions: the weight slab stays resident
     if (!p.wres) wres_bytes = 0;
@@ -1636,7 +1642,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     // staging: 8 warps x pt/2 pixel rows x 32 bytes (reserved at the 8-bit size), residual 2 or 4 x [pt][128]
     bool chosen = false;
     for (int cap = int32_boxes && a.cout > 64 ? 128 : 256; cap >= 64 && !chosen; cap >>= 1) {   // largest pixel tile that leaves room for >= 3 stages
-      p.pt = pick_pt(P, p.c_tiles, h->sm_count, cap);
+      p.pt = pick_pt(P, p.c_tiles, sm_count, cap);
       // A weight slab of at most 72 KiB stays resident (the stages then hold activations only): a third less
       // traffic into shared memory per K block.  Where the slab would cost the larger pixel tile its stages, the
       // tile wins and the weights travel with the stages.
@@ -1670,7 +1676,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   // row offset into the patch), so the activations enter shared memory once instead of nine times.  The tile is
   // 256 positions of a raster whose pitch is the next power of two above the padded width; worth it while at
   // least three quarters of a pitch are real columns.
-  size_t patch_total = 0;
+  size_t& patch_total = t.patch_total;
   {
     int lg_wp = 0;
     if (a.w >= 11 && a.w <= 14) lg_wp = 4; else if (a.w >= 23 && a.w <= 30) lg_wp = 5; else if (a.w >= 47 && a.w <= 62) lg_wp = 6;
@@ -1689,7 +1695,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
       else if (room >= 2 * patch + 3 * wb) { npatch = 2; wstages = (int)((room - 2 * patch) / wb); }
       // measured: with the weights streaming through the stage ring the strip form is no faster than the plain
       // one (both are bound by what the SM can take in per cycle), so it is used where the weights stay resident
-      if (((tiles_all >= 2LL * h->sm_count && keep_w) || h->conv_path == 3 || a.pairs) && npatch >= 2) {
+      if (((tiles_all >= 2LL * sm_count && keep_w) || conv_path == 3 || a.pairs) && npatch >= 2) {
         p.strip = 1; p.lg_wp = lg_wp; p.rows = rows; p.tpi = tpi; p.ho = a.h; p.npatch = npatch;
         p.patch_bytes = (uint32_t)patch;
         p.bkb = bkb; p.cchunks = cchunks; p.k_blocks = a.pairs ? 12 : 9 * cchunks;
@@ -1747,7 +1753,7 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
     // fetches its own 128 weight rows and HALF of the tile's pixel rows, 32 KiB per K block and SM instead of
     // 48 KiB for the same MMA time.  For the long reductions whose weights stream, which the operand fetch bounds.
     p.duo = (!pair && !wide && !int32_boxes && !p.strip && !p.wres && !p.fold && p.pt >= 128 && p.bkb == 128 && a.cout % 256 == 0 &&
-             k_total >= 2048 && (long long)p.p_tiles * p.c_tiles >= 2LL * h->sm_count) ? 1 : 0;
+             k_total >= 2048 && (long long)p.p_tiles * p.c_tiles >= 2LL * sm_count) ? 1 : 0;
     if (p.duo) {
       stage_bytes = (kTileC + p.pt / 2) * p.bkb;
       stages = (kSmemBudget - out_tile_bytes - (res_tile_bytes << p.lg_rbufs)) / stage_bytes;
@@ -1783,6 +1789,35 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   p.res_stage_off = p.out_stage_off + (uint32_t)out_tile_bytes;
   p.wres_off = p.res_stage_off + ((uint32_t)res_tile_bytes << p.lg_rbufs);
   p.patch_off = p.wres_off + (uint32_t)wres_bytes;
+  t.dyn_smem = (size_t)stages * stage_bytes + out_tile_bytes + ((size_t)res_tile_bytes << p.lg_rbufs) + wres_bytes + patch_total + 1024;
+  return HQ_OK;
+}
+}  // namespace
+
+hq_status hq_conv_tc_plan(const ConvArgs& a, int sm_count, hq_conv_plan* out) {
+  if (!hq_conv_tc_supported(a)) return HQ_ERR_UNSUPPORTED;
+  TcPlan t;
+  const hq_status st = plan_conv_tc(a, sm_count, 0, t);
+  if (st != HQ_OK) return st;
+  const TcParams& p = t.p;
+  out->shape = p.frag ? HQ_SHAPE_FRAG : p.duo ? HQ_SHAPE_DUO : t.pair ? HQ_SHAPE_PAIR : t.int32_boxes ? HQ_SHAPE_WIDE : p.strip ? HQ_SHAPE_STRIP : HQ_SHAPE_SOLO;
+  out->pixel_tile = p.pt; out->k_blocks = p.k_blocks; out->block_bytes = p.bkb; out->weights_resident = p.wres;
+  out->stages = p.stages; out->issuers = p.ni; out->alternate_tiles = p.frag && !p.deal;
+  out->residual_tiles = p.frag || p.staged_res ? 1 << p.lg_rbufs : 0;
+  out->shared_bytes = (int32_t)t.dyn_smem;
+  return HQ_OK;
+}
+
+hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream) {
+  if (!hq_conv_tc_supported(a)) return HQ_ERR_UNSUPPORTED;
+  if (!load_driver_entry_points()) return HQ_ERR_CUDA;
+  const long long P = (long long)a.n * a.ho * a.wo;
+  if (P == 0) return HQ_OK;
+  TcPlan t;
+  const hq_status planned = plan_conv_tc(a, h->sm_count, h->conv_path, t);
+  if (planned != HQ_OK) return planned;
+  TcParams& p = t.p;
+  p.rev = h->tile_order ? 1 : 0;
   p.bias = a.bias; p.b = a.b; p.c = a.c;
   p.res = a.res; p.res_bits = a.res_bits; p.res_signed = a.res_signed; p.rb = a.rb; p.rc = a.rc;
   p.res_narrow = (a.res && a.res_bits == 8) ? (const int4*)a.res_narrow : nullptr;
@@ -1845,21 +1880,21 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return HQ_ERR_CUDA;
   } else
-  if (p.staged_out && !encode_rows_map(&map_out, a.out, P, out_row_bytes, p.frag ? kTileC : a.out_bits == 4 ? 16 : 32, p.frag ? p.pt : p.pt / (p.halves << p.fold),
+  if (p.staged_out && !encode_rows_map(&map_out, a.out, P, (long long)a.cout * a.out_bits / 8, p.frag ? kTileC : a.out_bits == 4 ? 16 : 32, p.frag ? p.pt : p.pt / (p.halves << p.fold),
                                        box_swz)) return HQ_ERR_CUDA;
   if (p.staged_res && !encode_rows_map(&map_res, a.res, P, a.cout, kTileC, p.pt, box_swz))
     return HQ_ERR_CUDA;
 
-  if (int32_boxes) {
+  if (t.int32_boxes) {
     if (a.out && !encode_rows_map(&map_out, a.out, P, 4ll * a.cout, 128, 16, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
     if (a.res && !encode_rows_map(&map_res, a.res, P, (long long)a.cout * a.res_bits / 8, a.res_bits == 32 ? 128 : 32, 16, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
     if (p.q_out && !encode_rows_map(&map_q, p.q_out, P, a.cout, 32, 16, CU_TENSOR_MAP_SWIZZLE_NONE)) return HQ_ERR_CUDA;
   }
 
-  const size_t dyn_smem = (size_t)stages * stage_bytes + out_tile_bytes + ((size_t)res_tile_bytes << p.lg_rbufs) + wres_bytes + patch_total + 1024;
+  const size_t dyn_smem = t.dyn_smem;
   const long long total_tiles = (long long)p.p_tiles * p.c_tiles;
   // a multiple of c_tiles, so that every CTA keeps one channel tile
-  const int slots = pair ? 2 * h->sm_count : h->sm_count;
+  const int slots = t.pair ? 2 * h->sm_count : h->sm_count;
   const int grid = (int)(total_tiles <= slots ? total_tiles : (slots / p.c_tiles) * p.c_tiles);
   // Launched with programmatic stream serialization: the grid may begin (barrier set-up, tensor-memory
   // allocation) while the previous kernel drains; the kernel waits for it before reading any input.
@@ -1874,17 +1909,17 @@ hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t stream
   if (p.duo) {
     cfg.blockDim = dim3(32 * (2 + kSoloEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
     err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, 1, true>, map_x, map_w, map_out, map_res, map_q, p);
-  } else if (wide) {
+  } else if (p.frag) {
     cfg.blockDim = dim3(32 * (2 + kFragIssuers + kFragWarps)); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
     err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kFragWarps, 1, kFragIssuers, false, true>, map_x, map_w, map_out, map_res, map_q, p);
-  } else if (pair) {
+  } else if (t.pair) {
     cfg.blockDim = dim3(32 * (1 + kPairIssuerWarps + kPairEpilogueWarps)); cfg.dynamicSmemBytes = dyn_smem;
     err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kPairEpilogueWarps, 2, kPairIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);
   } else {
     // one CTA per SM (it may allocate all 512 tensor-memory columns): never request less than 120 KiB
-    cfg.blockDim = dim3(32 * (1 + kSoloIssuerWarps + (int32_boxes ? kWideWarps : kSoloEpilogueWarps))); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
+    cfg.blockDim = dim3(32 * (1 + kSoloIssuerWarps + (t.int32_boxes ? kWideWarps : kSoloEpilogueWarps))); cfg.dynamicSmemBytes = dyn_smem < 120 * 1024 ? 120 * 1024 : dyn_smem;
     if (a.wide) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kAdd32>, map_x, map_w, map_out, map_res, map_q, p);
-    else if (int32_boxes) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kRaw32>, map_x, map_w, map_out, map_res, map_q, p);
+    else if (t.int32_boxes) err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kWideWarps, 1, kSoloIssuerWarps, false, false, kRaw32>, map_x, map_w, map_out, map_res, map_q, p);
     else err = cudaLaunchKernelEx(&cfg, conv_tc_kernel<kSoloEpilogueWarps, 1, kSoloIssuerWarps>, map_x, map_w, map_out, map_res, map_q, p);
   }
   return err == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;

@@ -158,6 +158,7 @@ bool hq_conv_tc_declines(const ConvArgs& a);      // ... or whose patch matrix i
 bool hq_conv_wide_applies(const ConvArgs& a, int sm_count);
 // Tensor-core path; returns HQ_OK, HQ_ERR_UNSUPPORTED (nothing was launched) or HQ_ERR_CUDA.
 hq_status hq_launch_conv_tc(hq_handle* h, const ConvArgs& a, cudaStream_t s);
+hq_status hq_conv_tc_plan(const ConvArgs& a, int sm_count, hq_conv_plan* out);     // what it would launch; host arithmetic only
 // One tile per CTA, reduction split over a cluster: small problems (conv_small.cu).  Same status convention.
 bool hq_conv_small_init();
 bool hq_conv_small_supported(const ConvArgs& a, int sm_count);
