@@ -776,11 +776,13 @@ __device__ __noinline__ void epilogue_loop_general(const EpiCtx& e, const ChanCo
 
 // MMA issue of the frag shape.  One thread needs about 1 k cycles per K block, nearly all of it the latency of its own
 // instructions between one barrier and the next, so two issuers share the work:
-//   - DEAL false: issuer `c` of `n` takes the tiles c, c + n, ...  The accumulator's barrier is awaited before the operands': it
-//     says that the tile four earlier has been consumed.  A wait for a stage's m-th fill cannot tell it from the (m-2)-nd unless
-//     the (m-1)-st is known to have landed, which that barrier shows where the ring holds four tiles (n = 1 otherwise);
-//   - DEAL true: the K blocks of the CTA, numbered through its tiles, alternate between the two issuers.  The stage count is even,
-//     so that a stage always belongs to one issuer; the tile's first, overwriting MMA signals `tstart`, which the other one awaits.
+//   - DEAL false: issuer `c` of `n` takes the tiles c, c + n, ...  The stage count is a multiple of n * k_blocks;
+//   - DEAL true: the K blocks of the CTA, numbered through its tiles, alternate between the two issuers, whose number divides
+//     the stage count; the tile's first, overwriting MMA signals `tstart`, which the other one awaits.
+// Either way a stage belongs to one issuer for the whole launch.  It has to: a wait for a stage's m-th fill looks at a parity and
+// cannot tell it from the (m-2)-nd, so the waiting thread must have seen the (m-1)-st itself.  (No other barrier shows that one: copies
+// land out of order, and with five stages of one-block tiles the fill before is the other issuer's, five tiles back, while the
+// accumulator's barrier speaks of the tile four back.)
 template <int STEPS, bool DEAL>
 __device__ __forceinline__ void frag_issue(const TcParams& p, SharedCtl& ctl, int c, int n, uint32_t tiles, uint32_t stage_bytes,
                                            uint32_t w_bytes, uint32_t tmem_base, int p_tile0, int p_step) {
@@ -1765,9 +1767,10 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
     if (wide) {
       if (stages > kMaxStages) stages = kMaxStages;
       p.ni = kFragIssuers;
-      if (stages < kFragAccs * p.k_blocks) {
-        if (stages >= 4 && p.k_blocks > 1) { p.deal = 1; stages &= ~1; } else p.ni = 1;
-      }
+      // (a stage has to stay with one issuer, see frag_issue)
+      if (stages >= kFragAccs * p.k_blocks) stages -= stages % (kFragIssuers * p.k_blocks);
+      else if (stages >= 4 && p.k_blocks > 1) { p.deal = 1; stages -= stages % kFragIssuers; }
+      else p.ni = 1;
     } else if (!(p.strip && p.wres)) {
       while (p.ni > 1 && stages < p.ni) --p.ni;
       if (stages > kMaxStages) stages = kMaxStages;

@@ -1,0 +1,54 @@
+"""Launch plans of the persistent convolution kernel: host arithmetic, checked without a GPU over the sizes the kernel takes."""
+from __future__ import annotations
+
+import itertools
+
+import pytest
+
+from paper_2011_10680_b200 import binding, build
+
+SMS = 148
+PIXELS = (52, 28, 27)                        # 39312 pixels: 256-pixel tiles of two channel tiles fill the SMs twice
+
+
+@pytest.fixture(scope="module", autouse=True)
+def library():
+    build.build()
+
+
+def all_plans():
+    """Every K-block size and count, one to five channel tiles, with and without a residual, whole and ragged channels."""
+    small, large = (2, 14, 14), PIXELS
+    for cin, (k, stride), cout, res, out_bits, (n, h, w) in itertools.product(
+            [*range(16, 529, 16), 640, 768, 896, 1008, 1024, 2048], [(1, 1), (1, 2), (3, 1), (3, 2)], [64, 128, 144, 256, 512, 640],
+            [0, 8, 32], [8, 4, 32], [small, large]):
+        if res and out_bits != 8:
+            continue
+        plan = binding.conv2d_plan(n * stride * stride, h, w, cin, cout, k, stride, k // 2, out_bits, res, SMS)
+        if plan is not None:
+            yield (n, h, w, cin, cout, k, stride, res, out_bits), plan
+
+
+def test_a_stage_belongs_to_one_issuer():
+    """An issuer waits for the fill of a stage by its parity, so it has to have seen the fill before: whatever a stage
+    holds, from one end of the launch to the other, goes to the same issuer.  Otherwise a copy that is overtaken by the
+    next tiles lets the other issuer multiply what was there before."""
+    seen = set()
+    for layer, plan in all_plans():
+        stages, issuers, blocks = plan["stages"], plan["issuers"], plan["k_blocks"]
+        if issuers < 2 or not stages:
+            continue
+        seen.add((plan["shape"], stages, issuers, blocks, plan["alternate_tiles"]))
+    assert {("frag", 1), ("frag", 0), ("solo", 0)} <= {(s[0], s[4]) for s in seen}
+    for shape, stages, issuers, blocks, alternate in seen:
+        owner = {}
+        for block in range(4 * stages * issuers * blocks):
+            issuer = (block // blocks if alternate else block) % issuers
+            assert owner.setdefault(block % stages, issuer) == issuer, (shape, stages, issuers, blocks, alternate)
+
+
+def test_plans_fit_the_sm():
+    for layer, plan in all_plans():
+        assert plan["shared_bytes"] <= 227 * 1024, (layer, plan)
+        assert plan["stages"] >= 2 or plan["shape"] == "strip", (layer, plan)
+        assert plan["issuers"] <= max(1, plan["stages"]) or plan["shape"] == "strip", (layer, plan)
