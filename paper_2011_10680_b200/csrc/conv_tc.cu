@@ -819,7 +819,7 @@ __device__ __forceinline__ void frag_issue(const TcParams& p, SharedCtl& ctl, in
 #pragma unroll
         for (int k = 0; k < STEPS; ++k) mma_i8(d, ad + 2 * k, bd + 2 * k, idesc, k ? 1u : kb ? 1u : 0u);
       }
-      if (DEAL && kb == 0) mbar_arrive(smem_u32(&ctl.tstart[as]));
+      if (DEAL && kb == 0) { tc_fence_before(); mbar_arrive(smem_u32(&ctl.tstart[as])); }    // (the other issuer fences behind its wait)
       if (kb + per >= k_blocks) mma_commit(smem_u32(&ctl.tfull[as]));
       mma_commit(smem_u32(&ctl.empty[s]));
       s += (uint32_t)per;
@@ -1236,7 +1236,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
           uint64_t bdesc = desc_hi | (uint64_t)((b_addr >> 4) & 0x3FFF);
           for (int k = 0; k < ksteps; ++k, adesc += 2, bdesc += 2)     // 32 bytes of K per instruction
             mma_i8(d_tmem, adesc, bdesc, idesc, (b | k) ? 1u : 0u);
-          if (b == 0 && ni > 1) mbar_arrive(smem_u32(&ctl.tstart[as]));   // the overwriting MMA is on its way
+          if (b == 0 && ni > 1) { tc_fence_before(); mbar_arrive(smem_u32(&ctl.tstart[as])); }   // the overwriting MMA is on its way
           // the accumulator's barrier first on this issuer's last block: the epilogue is the one waiting
           if (b + (int)ni >= p.k_blocks) mma_commit(smem_u32(&ctl.tfull[as]));
           if (ring) {

@@ -2,6 +2,8 @@
 from __future__ import annotations
 
 import itertools
+import os
+import re
 
 import pytest
 
@@ -52,3 +54,15 @@ def test_plans_fit_the_sm():
         assert plan["shared_bytes"] <= 227 * 1024, (layer, plan)
         assert plan["stages"] >= 2 or plan["shape"] == "strip", (layer, plan)
         assert plan["issuers"] <= max(1, plan["stages"]) or plan["shape"] == "strip", (layer, plan)
+
+
+def test_signals_between_tensor_core_threads_are_fenced():
+    """What one thread's tensor-core operations did is ordered before another's only by a pair of fences around the barrier: every
+    arrival that says "my MMA is issued" or "my loads are done" has its half directly ahead of it."""
+    path = os.path.join(os.path.dirname(build.__file__), "csrc", "conv_tc.cu")
+    code = re.sub(r"//[^\n]*", "", open(path).read())
+    code = re.sub(r"\s+", " ", code)
+    arrivals = list(re.finditer(r"mbar_arrive\(smem_u32\(&ctl\.(tstart|tempty)\[", code))
+    assert {m.group(1) for m in arrivals} == {"tstart", "tempty"}
+    for m in arrivals:
+        assert re.search(r"tc_fence_before\(\); (__syncwarp\(\); )?(if \(lane == 0\) )?$", code[:m.start()]), code[m.start() - 80:m.end() + 10]
