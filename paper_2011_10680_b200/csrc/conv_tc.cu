@@ -1742,13 +1742,15 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
       p.wres = wres_bytes <= 72 * 1024 ? 1 : 0;
       if (!p.wres) wres_bytes = 0;
       stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
-      // eight residual / output tiles where they leave room for three operand stages, else four: a tile is held from its load
-      // to the end of its store, and the loads of the next tiles must be in flight meanwhile to cover the memory latency (with
-      // arithmetic and matrix stores left out, 1x1 64 -> 256 at 56x56: four tiles 93 us, eight 87)
+      // Eight residual / output tiles where a tile is one or two K blocks, else four: a tile is held from its load to the end of its
+      // store, and the loads of the next tiles must be in flight meanwhile to cover the memory latency (1x1 64 -> 256 at 56x56, 256
+      // images, with residual: four tiles 134 us a call, eight 128; 256 -> 1024 at 14x14 the same either way).  Longer tiles cover it by
+      // themselves and need the room for stages: with the three that eight tiles leave, the second issuer has none of its own (3x3 64 -> 256
+      // at 28x28: eight tiles 85 us, four 79; 1x1 384 -> 768, 128 images: 62 / 54; 768 -> 1024 at 14x14, weights streaming: 74 / 68).
       // Without a residual the tiles only carry outputs, and what is in flight are the operand stages: as many as there may be.
-      for (p.lg_rbufs = p.staged_res ? 3 : 2; ; --p.lg_rbufs) {
+      for (p.lg_rbufs = p.staged_res && p.k_blocks <= 2 ? 3 : 2; ; --p.lg_rbufs) {
         stages = (kSmemBudget - (res_tile_bytes << p.lg_rbufs) - wres_bytes) / stage_bytes;
-        if (stages >= (p.staged_res ? 3 : kMaxStages) || p.lg_rbufs == 1) break;
+        if (p.staged_res || stages >= kMaxStages || p.lg_rbufs == 1) break;
       }
     }
     // Fourth shape, *duo*: clusters of two CTAs on adjacent SMs share every MMA (cta_group::2, M = 256): each CTA

@@ -49,6 +49,14 @@ def test_a_stage_belongs_to_one_issuer():
             assert owner.setdefault(block % stages, issuer) == issuer, (shape, stages, issuers, blocks, alternate)
 
 
+def test_fragment_shape_has_stages_for_both_issuers():
+    """The residual tiles must not take the room of the operand stages: one issuer alone sets the tile rate of this shape."""
+    plans = [(layer, plan) for layer, plan in all_plans() if plan["shape"] == "frag"]
+    assert {plan["weights_resident"] for _, plan in plans} == {0, 1}
+    for layer, plan in plans:
+        assert plan["stages"] >= 4 and plan["issuers"] == 2, (layer, plan)
+
+
 def test_plans_fit_the_sm():
     for layer, plan in all_plans():
         assert plan["shared_bytes"] <= 227 * 1024, (layer, plan)
