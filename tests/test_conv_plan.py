@@ -57,6 +57,21 @@ def test_fragment_shape_has_stages_for_both_issuers():
         assert plan["stages"] >= 4 and plan["issuers"] == 2, (layer, plan)
 
 
+def test_cases_of_the_fragment_shape_take_the_plans_they_name():
+    from test_gpu_small_conv import FRAGMENT_CASES
+    dealt = set()
+    for n, h, w, cin, cout, k, stride, residual, _, _, _, _, (blocks, stages, issue, tiles, resident) in FRAGMENT_CASES:
+        plan = binding.conv2d_plan(n, h, w, cin, cout, k, stride, k // 2, 8, 8 if residual else 0, SMS)
+        got = (plan["shape"], plan["issuers"], plan["k_blocks"], plan["stages"], "tiles" if plan["alternate_tiles"] else "blocks",
+               plan["residual_tiles"], plan["weights_resident"])
+        assert got == ("frag", 2, blocks, stages, issue, tiles, resident), (cin, cout, k, got)
+        if issue == "blocks":
+            dealt.add(blocks % 2)
+        pixels, channel_tiles = n * ((h - 1) // stride + 1) * ((w - 1) // stride + 1), (cout + 127) // 128
+        assert pixels % 128 and pixels // 128 // (SMS // channel_tiles) >= 20            # tiles per CTA: eight buffers come round twice
+    assert dealt == {0, 1}
+
+
 def test_plans_fit_the_sm():
     for layer, plan in all_plans():
         assert plan["shared_bytes"] <= 227 * 1024, (layer, plan)

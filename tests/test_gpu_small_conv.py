@@ -184,20 +184,25 @@ def test_conv_over_pixel_pairs(hw, batch, signed):
 
 
 FRAGMENT_CASES = [
-    # n, h, w, cin, cout, k, stride, residual, residual signed, relu, c range, rc range
-    (52, 28, 27, 32, 144, 1, 1, True, False, True, (39, 44), (28, 34)),     # one K block of 32 bytes; second channel tile of 16; ragged last pixel tile
-    (52, 28, 27, 64, 256, 1, 1, True, True, False, (39, 44), (28, 34)),     # two issuers on alternate tiles, signed residual and output
-    (52, 28, 27, 96, 160, 1, 1, True, False, True, (39, 44), (28, 34)),     # the last K block reaches past the channels
-    (52, 28, 27, 128, 256, 1, 1, True, False, True, (28, 31), (28, 34)),    # shifts below 32: pre-shift form
-    (52, 28, 27, 64, 256, 1, 1, True, False, True, (14, 40), (28, 34)),     # some shifts too small for it: funnel-shift form
-    (52, 28, 27, 64, 256, 1, 1, True, True, True, (39, 44), (4, 34)),       # residual shifts below 9: 64-bit form
-    (52, 28, 27, 256, 256, 1, 1, True, False, True, (39, 44), (28, 34)),    # K blocks dealt to the two issuers
-    (52, 28, 27, 160, 256, 1, 1, True, False, True, (39, 44), (28, 34)),    # the same with a partial last block
-    (52, 28, 27, 64, 256, 3, 1, True, False, True, (39, 44), (28, 34)),     # nine blocks: the issuers swap roles from tile to tile
-    (26, 28, 27, 512, 512, 1, 1, True, False, True, (40, 45), (28, 34)),    # four blocks, fewer residual tiles
-    (52, 28, 27, 64, 256, 1, 1, False, False, True, (39, 44), None),        # no residual
-    (52, 28, 27, 64, 176, 1, 1, False, False, False, (26, 44), None),       # the same, signed, ragged channels, small shifts
-    (210, 28, 27, 256, 256, 1, 2, False, False, True, (39, 44), None),      # rows gathered in im2col mode
+    # n, h, w, cin, cout, k, stride, residual, residual signed, relu, c range, rc range,
+    #   plan on 148 SMs: K blocks, stages, MMA issue (whole tiles in turn / K blocks dealt in turn), residual or output tiles, weights resident
+    (258, 28, 27, 32, 144, 1, 1, True, False, True, (39, 44), (28, 34), (1, 8, "tiles", 8, 1)),     # blocks of 32 bytes; second channel tile of 16; ragged last pixel tile
+    (258, 28, 27, 64, 256, 1, 1, True, True, False, (39, 44), (28, 34), (1, 8, "tiles", 8, 1)),     # signed residual and output
+    (258, 28, 27, 96, 160, 1, 1, True, False, True, (39, 44), (28, 34), (1, 4, "tiles", 8, 1)),     # the last K block reaches past the channels
+    (258, 28, 27, 128, 256, 1, 1, True, False, True, (28, 31), (28, 34), (1, 4, "tiles", 8, 1)),    # shifts below 32: pre-shift form
+    (258, 28, 27, 64, 256, 1, 1, True, False, True, (14, 40), (28, 34), (1, 8, "tiles", 8, 1)),     # some shifts too small for it: funnel-shift form
+    (258, 28, 27, 64, 256, 1, 1, True, True, True, (39, 44), (4, 34), (1, 8, "tiles", 8, 1)),       # residual shifts below 9: 64-bit form
+    (258, 28, 27, 256, 256, 1, 1, True, False, True, (39, 44), (28, 34), (2, 4, "blocks", 8, 1)),   # each issuer keeps one block of every tile
+    (258, 28, 27, 160, 256, 1, 1, True, False, True, (39, 44), (28, 34), (2, 4, "blocks", 8, 1)),   # the same with a partial last block
+    (258, 28, 27, 320, 256, 1, 1, True, False, True, (39, 44), (28, 34), (3, 6, "blocks", 4, 1)),   # three blocks: the issuers swap roles from tile to tile
+    (258, 28, 27, 64, 256, 3, 1, True, False, True, (39, 44), (28, 34), (9, 8, "blocks", 4, 1)),    # nine blocks, rows gathered in im2col mode
+    (258, 28, 27, 32, 256, 3, 1, True, True, True, (39, 44), (28, 34), (9, 8, "blocks", 4, 1)),     # nine blocks of 32 bytes
+    (130, 28, 27, 512, 512, 1, 1, True, False, True, (40, 45), (28, 34), (4, 6, "blocks", 4, 1)),   # four blocks
+    (130, 28, 27, 640, 512, 1, 1, True, False, True, (40, 45), (28, 34), (5, 4, "blocks", 4, 0)),   # five blocks, weights in the stages
+    (258, 28, 27, 64, 256, 1, 1, False, False, True, (39, 44), None, (1, 8, "tiles", 4, 1)),        # no residual
+    (258, 28, 27, 64, 176, 1, 1, False, False, False, (26, 44), None, (1, 8, "tiles", 4, 1)),       # the same, signed, ragged channels, small shifts
+    (980, 28, 27, 256, 256, 1, 2, False, False, True, (39, 44), None, (2, 8, "tiles", 4, 1)),       # the same, rows gathered in im2col mode
+    (258, 28, 27, 384, 256, 1, 1, False, False, True, (39, 44), None, (3, 8, "blocks", 2, 1)),      # three blocks without a residual, two output tiles
 ]
 
 
@@ -205,30 +210,34 @@ FRAGMENT_CASES = [
 @pytest.mark.parametrize("cfg", FRAGMENT_CASES)
 def test_fragment_epilogue_shape(cfg, rev):
     """The launch shape with four accumulators and two groups of epilogue warps: every number of K blocks per tile, every form of
-    the arithmetic, ragged channel and pixel tiles, both tile orders.  Integers: equal to the oracle."""
+    the arithmetic, ragged channel and pixel tiles, both tile orders, and enough tiles that every ring of buffers comes round twice
+    (two distinct images, repeated: the output must repeat with them).  Integers: equal to the oracle.  That each case takes
+    the plan it names is checked without a GPU (test_conv_plan.py)."""
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA device")
     from oracle import hqref
     from paper_2011_10680_b200 import binding, build
     build.build()
-    n, h, w, cin, cout, k, stride, residual, res_signed, relu, c_range, rc_range = cfg
-    case = inputs.conv_case(700, n, h, w, cin, cout, k, stride, k // 2, residual=residual, relu=relu, c_range=c_range)
-    assert case["ho"] * case["wo"] * n * ((cout + 127) // 128) >= 2 * 148 * 256          # large enough for this shape on 148 SMs
+    n, h, w, cin, cout, k, stride, residual, res_signed, relu, c_range, rc_range, _ = cfg
+    case = inputs.conv_case(700, 2, h, w, cin, cout, k, stride, k // 2, residual=residual, relu=relu, c_range=c_range)
     if residual:
         g = inputs.rng(701, cin, cout, k)
         case["rc"] = g.integers(rc_range[0], rc_range[1] + 1, size=cout, dtype=np.int64).astype(np.int32)
         if res_signed:
             case["res"], case["res_signed"] = case["res"].view(np.int8), 1
+    big = dict(case, n=n, x=np.tile(case["x"], (n // 2, 1, 1, 1)))
+    if residual:
+        big["res"] = np.tile(case["res"], (n // 2, 1, 1, 1))
+    ref = hqref.conv_case(case)
     hq = binding.Handle(0)
     try:
         hq.set_tile_order(rev)
-        dev = binding.upload_case(case)
+        dev = binding.upload_case(big)
         for _ in range(2):                                  # the second call starts while the first one ends
-            st, out = hq.conv_case(case, dev)
+            st, out = hq.conv_case(big, dev)
             assert st == binding.HQ_OK, binding.status_string(st)
         hq.sync()
-        ref = hqref.conv_case(case)
-        got = out.cpu().numpy().view(ref.dtype).reshape(ref.shape)
-        assert np.array_equal(got, ref), (int((got != ref).sum()), ref.size)
+        got = out.cpu().numpy().view(ref.dtype).reshape(n // 2, *ref.shape)
+        assert np.array_equal(got, np.broadcast_to(ref, got.shape)), (int((got != ref).sum()), got.size)
     finally:
         hq.close()
