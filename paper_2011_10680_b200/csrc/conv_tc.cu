@@ -1946,15 +1946,14 @@ cudaError_t hq_launch_residual_narrow2(const int32_t* b0, const int32_t* c0, int
 }
 
 namespace {
-// The wait of the kernels above in miniature: poll an mbarrier, give up after the budget, say so in the status word.
+// The wait of the kernels above, on a barrier that nothing signals: it gives up after the budget and says so in the status word.
 __global__ void expire_wait_kernel(uint32_t* status, unsigned long long budget_ns) {
-  __shared__ unsigned long long bar;
-  mbar_init(smem_u32(&bar), 1);
+  struct Ctl { unsigned long long bar; volatile uint32_t abort_flag; };
+  __shared__ Ctl ctl;
+  ctl.abort_flag = 0;
+  mbar_init(smem_u32(&ctl.bar), 1);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  const unsigned long long t0 = global_ns();
-  while (!mbar_try_wait(smem_u32(&bar), 0)) {
-    if (global_ns() - t0 > budget_ns) { atomicCAS(status, 0u, (uint32_t)HQ_DEV_TIMEOUT_EPILOGUE); break; }
-  }
+  mbar_wait(smem_u32(&ctl.bar), 0, &ctl, status, (uint32_t)HQ_DEV_TIMEOUT_EPILOGUE, budget_ns);
 }
 }  // namespace
 

@@ -53,13 +53,14 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // Bounded wait.  Returns false when the budget ran out or another role already aborted.
 template <class Ctl>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, Ctl* ctl, uint32_t* status, uint32_t code) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, Ctl* ctl, uint32_t* status, uint32_t code,
+                                          unsigned long long budget_ns = kWaitBudgetNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = global_ns();
   while (true) {
     if (mbar_try_wait_for(bar, parity, kSuspendNs)) return true;
     if (ctl->abort_flag) return false;
-    if (global_ns() - t0 > kWaitBudgetNs) {
+    if (global_ns() - t0 > budget_ns) {
       ctl->abort_flag = 1;
       atomicCAS(status, 0u, code);
       return false;
