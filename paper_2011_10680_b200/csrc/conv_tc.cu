@@ -326,13 +326,14 @@ __device__ __forceinline__ ChanConst chan_const_for(const TcParams& p, int ch, b
 // the tile's `ofull` barrier when its pieces are written, and the store warp alone waits there, stores the [128][128] box and
 // hands the buffer back.  Up to eight residual / output tiles circulate: their loads in flight cover the memory latency.
 //
-// What bounds it: the integer instructions (about 6.5 per 32 values; the residual's byte extraction is one of them) and, beside
-// them, the instruction latency of the warps that move tiles along (with no arithmetic the first layer below takes 82 us, with no
-// memory traffic 95).  Twenty-four warps in three groups: no faster.  1x1 64 -> 256 at 56x56 / 128 -> 512 at 28x28 / 256 -> 1024 at
-// 14x14 / 512 -> 2048 at 7x7, 256 images, L2 flushed: 97 / 58 / 40 / 31.7 us; without a residual 64 -> 256 90 -> 69 us.  Before:
-// eight warps, the residual widened into tensor memory by an MMA with the identity matrix, two accumulators and one issuer
-// 115 / 65 / 44 / 35.6 us; there the issuer's own instruction latency (2.5 k cycles a tile) set the tile rate, whatever the
-// epilogue did (sixteen warps or a matrix store of another type: the same time).
+// What bounds it: instructions and their latency together.  All warps execute 10.2 warp instructions per 32 values (5.3 without a
+// residual) in 52 % (46 %) of the issue slots, no unit is saturated, tensor pipe 5 %, DRAM 30 % (counters at 128 images); 1x1 64 -> 256 at
+// 56x56, 256 images, L2 flushed, takes 97 us, with no arithmetic 82, with no memory traffic 95.  Twenty-four warps in three groups: no
+// faster.  Inside ResNet-50 at 256 images, us a layer:
+// 1x1 64 -> 256 at 56x56 / 128 -> 512 at 28x28 / 256 -> 1024 at 14x14 / 512 -> 2048 at 7x7 with residual 94 / 55 / 34 / 25, 64 -> 256 without 67.  The
+// shape before this one - eight warps, the residual widened into tensor memory by an MMA with the identity matrix, two accumulators, one
+// issuer, multiply-adds of three instructions - took 122 / 70 / 42 / 33 and, for the last, the solo shape 88; the issuer's own instruction
+// latency (2.5 k cycles a tile) set its tile rate, whatever the epilogue did (sixteen warps or another matrix store: the same).
 // GEN: 64-bit arithmetic for every shift 1..62 (a residual shift below 9).  SMALL: some channel of the warp has c < 32 (common
 // with 4-bit operands, whose accumulators are small): funnel-shift or pre-shift form of Eq. 4.
 template <bool RES, bool GEN, bool RSIGNED, bool SAT, bool OSIGNED, bool RN, int SMALL = 0>
@@ -1610,8 +1611,8 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
   // (measured: with the weight slab resident the one-CTA shape catches up for K >= 128; the pair shape still
   // wins on the fused-residual expansions with the shortest reduction, and loses where a tile carries little
   // epilogue work, e.g. 64 output channels.  Where the layer is large enough for 256-pixel tiles and its residual
-  // travels by TMA, the frag shape below is faster still: 64 -> 256 at 56x56, batch 256: 129 -> 101 us.)
-  const bool wide_fits = p.staged_res && a.out_bits == 8 && a.cout > 64 && pick_pt(P, p.c_tiles, sm_count, 256) == 256;
+  // travels by TMA, the frag shape below is faster still: 64 -> 256 at 56x56, batch 256: 129 -> 97 us.)
+  const bool frag_fits = p.staged_res && a.out_bits == 8 && a.cout > 64 && pick_pt(P, p.c_tiles, sm_count, 256) == 256;
   // Without a residual the frag shape takes over where a CTA's weights stay in shared memory, but for longer reductions whose
   // pixel rows the im2col mode gathers: four blocks of 128 pixels are issued more slowly than two of 256 (256 images, L2 flushed,
   // 256-pixel tiles against frag: 1x1 64 -> 256 at 56x56 90 / 69 us, 512 -> 128 at 28x28 32.7 / 27.7, 256 -> 128 / 2 28.7 / 22.0, 256 -> 512 / 2
@@ -1619,7 +1620,7 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
   const bool tiled = !a.pitch_w && a.kh == 1 && a.kw == 1 && a.stride == 1 && a.pad == 0;
   const bool plain_frag = !a.res && !a.pitch_w && !a.pairs && a.cout % 16 == 0 && (tiled || k_total <= 256);
   bool& pair = t.pair;
-  pair = !a.wide && k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !wide_fits;
+  pair = !a.wide && k_total <= 64 && a.res != nullptr && a.res_bits == 8 && a.cout >= 128 && !frag_fits;
   int &stages = t.stages, &stage_bytes = t.stage_bytes, &res_tile_bytes = t.res_tile_bytes, &out_tile_bytes = t.out_tile_bytes, &wres_bytes = t.wres_bytes;
   if (pair) {
     // 128-pixel tiles, two accumulator buffers (256 columns), K blocks of at most 64 bytes
@@ -1662,9 +1663,9 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
         // (its epilogue has slack: a single residual buffer only delays the next tile's prefetch)
         // The frag shape (below) works in place in the residual tiles and needs no staging box; with the
         // weights resident two stages are enough for its short reductions (the epilogue bounds the tile).
-        const bool wide_here = p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && (p.staged_res || (plain_frag && p.wres)) && k_total < 1024;
-        if (wide_here) out_tile_bytes = 0;
-        const int min_stages = (wide_here && p.wres) ? 2 : 3;
+        const bool frag_here = p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 && (p.staged_res || (plain_frag && p.wres)) && k_total < 1024;
+        if (frag_here) out_tile_bytes = 0;
+        const int min_stages = (frag_here && p.wres) ? 2 : 3;
         for (p.lg_rbufs = p.lg_bufs; ; --p.lg_rbufs) {
           stages = (smem_budget - out_tile_bytes - (res_tile_bytes << p.lg_rbufs) - wres_bytes) / stage_bytes;
           if (stages >= min_stages || p.lg_rbufs == 0 || !res_tile_bytes || k_total < 1024) break;
@@ -1720,7 +1721,7 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
   // 128 KiB (hq_conv_tc_small_im2col); such a layer is declined here.
   if ((!p.strip && hq_conv_tc_declines(a)) || (a.pairs && !p.strip)) return HQ_ERR_UNSUPPORTED;
   p.x_signed = a.in_signed;
-  bool wide = false;
+  bool frag = false;
   {
     // issuer warps in use: at most one per K block; where the blocks travel through the stage ring, the stage count
     // becomes a multiple of it (every stage then belongs to one issuer)
@@ -1728,10 +1729,10 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
     // resident weights); where every block waits for 48 KiB from L2 the tile is bound by that stream and the extra
     // issuers only cost a few percent.
     // Third launch shape, *frag*, for the fused 8-bit residual with a short reduction on layers large enough for
-    // 256-pixel tiles (here called `wide` for the condition it shares with the tile choice above): see epilogue_loop_frag.
-    wide = !pair && !p.strip && p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 &&
+    // 256-pixel tiles (the condition it shares with the tile choice above): see epilogue_loop_frag.
+    frag = !pair && !p.strip && p.pt == 256 && !p.fold && p.staged_out && a.out_bits == 8 &&
            (p.staged_res || (plain_frag && p.wres)) && k_total < 1024;
-    if (wide) {
+    if (frag) {
       // 128-pixel tiles, four accumulators; the residual tiles double as the output boxes
       p.frag = 1; p.halves = 2;
       p.pt = 128; p.lg_bufs = 2; p.lg_rbufs = 1;
@@ -1743,10 +1744,11 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
       if (!p.wres) wres_bytes = 0;
       stage_bytes = ((p.wres ? 0 : kTileC) + p.pt) * p.bkb;
       // Eight residual / output tiles where a tile is one or two K blocks, else four: a tile is held from its load to the end of its
-      // store, and the loads of the next tiles must be in flight meanwhile to cover the memory latency (1x1 64 -> 256 at 56x56, 256
-      // images, with residual: four tiles 134 us a call, eight 128; 256 -> 1024 at 14x14 the same either way).  Longer tiles cover it by
-      // themselves and need the room for stages: with the three that eight tiles leave, the second issuer has none of its own (3x3 64 -> 256
-      // at 28x28: eight tiles 85 us, four 79; 1x1 384 -> 768, 128 images: 62 / 54; 768 -> 1024 at 14x14, weights streaming: 74 / 68).
+      // store, and the loads of the next tiles must be in flight meanwhile to cover the memory latency (inside ResNet-50 at 256 images,
+      // four / eight tiles: 128 -> 512 at 28x28 65 / 55 us, 256 -> 1024 at 14x14 39 / 34; a call of 64 -> 256 at 56x56 134 / 128).  Longer
+      // tiles cover it by themselves and need the room for stages: with the three that eight tiles leave, the second issuer has none
+      // of its own (calls of 256 images, eight / four tiles: 3x3 64 -> 256 at 28x28 85 / 79 us; 1x1 768 -> 1024 at 14x14, weights streaming,
+      // 74 / 68; 384 -> 768 at 28x28, 128 images, 62 / 54).
       // Without a residual the tiles only carry outputs, and what is in flight are the operand stages: as many as there may be.
       for (p.lg_rbufs = p.staged_res && p.k_blocks <= 2 ? 3 : 2; ; --p.lg_rbufs) {
         stages = (kSmemBudget - (res_tile_bytes << p.lg_rbufs) - wres_bytes) / stage_bytes;
@@ -1756,7 +1758,7 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
     // Fourth shape, *duo*: clusters of two CTAs on adjacent SMs share every MMA (cta_group::2, M = 256): each CTA
     // fetches its own 128 weight rows and HALF of the tile's pixel rows, 32 KiB per K block and SM instead of
     // 48 KiB for the same MMA time.  For the long reductions whose weights stream, which the operand fetch bounds.
-    p.duo = (!pair && !wide && !int32_boxes && !p.strip && !p.wres && !p.fold && p.pt >= 128 && p.bkb == 128 && a.cout % 256 == 0 &&
+    p.duo = (!pair && !frag && !int32_boxes && !p.strip && !p.wres && !p.fold && p.pt >= 128 && p.bkb == 128 && a.cout % 256 == 0 &&
              k_total >= 2048 && (long long)p.p_tiles * p.c_tiles >= 2LL * sm_count) ? 1 : 0;
     if (p.duo) {
       stage_bytes = (kTileC + p.pt / 2) * p.bkb;
@@ -1766,7 +1768,7 @@ hq_status plan_conv_tc(const ConvArgs& a, int sm_count, int conv_path, TcPlan& t
     const bool tail = a.cin % p.bkb > 0 && a.cin % p.bkb <= p.bkb - 32;
     const int issuers = pair ? kPairIssuerWarps : (p.strip || (p.wres && !tail)) ? kSoloIssuerWarps : 1;
     p.ni = p.k_blocks < issuers ? p.k_blocks : issuers;
-    if (wide) {
+    if (frag) {
       if (stages > kMaxStages) stages = kMaxStages;
       p.ni = kFragIssuers;
       // (a stage has to stay with one issuer, see frag_issue)
